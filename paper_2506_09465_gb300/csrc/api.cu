@@ -132,11 +132,11 @@ void free_all(Ctx* c) {
                   c->d_pcg_iters, c->d_scalar, c->d_adj, c->d_mg, c->d_mg_diag, c->d_mg_dinv, c->d_mg_cx,
                   c->d_mg_cy, c->d_mg_cz, c->d_mg_cinv, c->d_mg_b, c->d_mg_x, c->d_mg_t, c->d_mg_r, c->d_fd_q, c->d_fd_lam,
                   c->d_inst_beg, c->d_inst_end, c->d_inst_next, c->d_cost_prefix, c->d_window, c->d_wmax,
-                  c->d_group_mag, c->d_mag, c->d_wall_unit, c->d_all_beg, c->d_all_end, c->d_all_cost_prefix,
+                  c->d_group_mag, c->d_mag, c->d_wall_unit,
                   c->d_all_group_mag, c->d_R32, c->d_W32, c->d_F32, c->d_m2, c->d_wallTf,
                   c->d_pslot_off, c->d_phome_off, c->d_pnband, c->d_pnwall, c->d_px, c->d_pband, c->d_phome,
                   c->d_pcount, c->d_pfcount, c->d_phome_w, c->d_wemit, c->d_DY, c->d_EY, c->d_GX, c->d_Fd,
-                  c->d_all_real, c->d_defer, c->d_defer_n};
+                  c->d_all_real, c->d_defer, c->d_defer_n, c->d_land_fwd, c->d_land_all};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (c->h_pinned) cudaFreeHost(c->h_pinned);
@@ -337,14 +337,19 @@ iugkp_status rebuild_forward_groups(Ctx* c) {
     window[k] = make_int2((int)((X - len) / 2), (int)len);
     if (len < X) c->sync_partial = true;
   }
-  void* olds[] = {c->d_inst_beg, c->d_inst_end, c->d_cost_prefix, c->d_window, c->d_group_mag};
+  void* olds[] = {c->d_inst_beg, c->d_inst_end, c->d_cost_prefix, c->d_window, c->d_group_mag, c->d_land_fwd};
   for (void* p : olds)
     if (p) cudaFree(p);
+  c->d_land_fwd = nullptr;
   c->d_inst_beg = c->d_inst_end = nullptr;
   c->d_cost_prefix = nullptr;
   c->d_window = nullptr;
   c->d_group_mag = nullptr;
   if ((s = upload(c, &c->d_group_mag, gmag)) != IUGKP_OK) return s;
+  std::vector<LandGroup> lg;
+  land_tasks(c, c->h_groups_fwd, lg, c->land_fwd_tasks, c->land_fwd_qch);
+  if (c->fwd_particles == 0) c->land_fwd_tasks = 0;  // the all-zero placeholder group
+  if ((s = upload(c, &c->d_land_fwd, lg)) != IUGKP_OK) return s;
   if ((s = upload(c, &c->d_inst_beg, beg)) != IUGKP_OK) return s;
   if ((s = upload(c, &c->d_inst_end, end)) != IUGKP_OK) return s;
   if ((s = upload(c, &c->d_cost_prefix, prefix)) != IUGKP_OK) return s;
@@ -742,14 +747,12 @@ iugkp_status iugkp_create_batch(int n, const iugkp_grid* g, const double* const*
   }
   if ((s = rebuild_forward_groups(c)) != IUGKP_OK) return bail(s);
   {
-    std::vector<long long> beg, end;
-    std::vector<double> prefix;
     std::vector<unsigned> gmag;
-    staged_tables(c, c->h_groups_all, beg, end, prefix, c->all_cost_total, gmag);
-    UP(c->d_all_beg, beg);
-    UP(c->d_all_end, end);
-    UP(c->d_all_cost_prefix, prefix);
+    for (const Group& g : c->h_groups_all) gmag.push_back(div_magic(g.n_emitters));
     UP(c->d_all_group_mag, gmag);
+    std::vector<LandGroup> lg;
+    land_tasks(c, c->h_groups_all, lg, c->land_all_tasks, c->land_all_qch);
+    UP(c->d_land_all, lg);
   }
   {
     std::vector<unsigned> mag((size_t)5 * n);
@@ -783,8 +786,8 @@ iugkp_status iugkp_create_batch(int n, const iugkp_grid* g, const double* const*
     const long long cap = std::min<long long>(c->total_particles / 32 + 65536, 1ll << 31);
     c->defer_cap = (unsigned)cap;
     if ((s = dalloc(c, &c->d_defer, (size_t)cap)) != IUGKP_OK) return bail(s);
-    if ((s = dalloc(c, &c->d_defer_n, 1)) != IUGKP_OK) return bail(s);
-    if (cudaMemset(c->d_defer_n, 0, sizeof(unsigned)) != cudaSuccess) {
+    if ((s = dalloc(c, &c->d_defer_n, 4)) != IUGKP_OK) return bail(s);
+    if (cudaMemset(c->d_defer_n, 0, 4 * sizeof(unsigned)) != cudaSuccess) {
       cudaGetLastError();
       fail(c, IUGKP_ECUDA, "clear of the replay queue");
       return bail(IUGKP_ECUDA);
@@ -948,6 +951,36 @@ iugkp_status sweep_async(Ctx* c, const double* T, unsigned epoch, double* R, dou
     CK(launch_sweep_staged(c, a, s), "staged sweep launch");
   else
     CK(launch_sweep(c, a, s), "sweep launch");
+  return IUGKP_OK;
+}
+
+// Every axis short enough for the landing sweeps' FP32 cell coordinates.
+bool land_sizes(const Ctx* c) {
+  for (const InstDesc& in : c->h_inst)
+    for (int a = 0; a < in.dim; ++a)
+      if (in.n[a] >= (1 << 23)) return false;
+  return true;
+}
+
+// A sweep of which only the real collisions are read (the macro update and the correction take
+// R alone): R into c->d_R, no W, no faces, no walls, no event counts.
+iugkp_status sweep_real_async(Ctx* c, const double* T, unsigned epoch, cudaStream_t s) {
+  if (!staged_path(c) || !land_sizes(c))
+    return sweep_async(c, T, epoch, c->d_R, nullptr, nullptr, nullptr, nullptr, s);
+  if (c->opt.tally == IUGKP_TALLY_STAGED_K32) {
+    if (!c->d_R32) return fail(c, IUGKP_EINVAL, "compensated tally buffers missing");
+  } else {
+    CK(cudaMemsetAsync(c->d_R, 0, (size_t)c->nb * c->total_cells * sizeof(double), s), "clear R");
+  }
+  SweepArgs a = base_args(c);
+  a.groups = c->d_groups_fwd;
+  a.n_groups = (int)c->h_groups_fwd.size();
+  a.total_particles = c->fwd_particles;
+  a.T = T;
+  a.R = c->d_R;
+  a.counters = c->d_counters;
+  a.epoch = epoch;
+  CK(launch_land(c, a, false, s), "landing sweep launch");
   return IUGKP_OK;
 }
 
@@ -1236,10 +1269,12 @@ iugkp_status iugkp_check_fp32_walk(double* out6) {
 namespace {
 
 // One IUGKP iteration cur -> nxt without host round trips: sweep, macro update, Newton
-// correction (CG status checked on the device), residual sums into res_dev[0..1].
-iugkp_status iteration_async(Ctx* c, const double* cur, double* nxt, unsigned epoch, double* res_dev,
+// correction (CG status checked on the device), residual sums into res_dev[0..1]. The update
+// reads R alone, so the sweep tallies nothing else but, on request, the faces (into c->d_F).
+iugkp_status iteration_async(Ctx* c, const double* cur, double* nxt, unsigned epoch, bool want_F, double* res_dev,
                              cudaStream_t s) {
-  iugkp_status st = sweep_async(c, cur, epoch, c->d_R, c->d_W, c->d_F, c->d_wall, c->d_counters, s);
+  iugkp_status st = want_F ? sweep_async(c, cur, epoch, c->d_R, nullptr, c->d_F, nullptr, nullptr, s)
+                           : sweep_real_async(c, cur, epoch, s);
   if (st != IUGKP_OK) return st;
   CK(launch_macro(c, c->d_R, nullptr, nxt, nullptr, s), "macro");
   if (c->opt.newton) {
@@ -1275,8 +1310,8 @@ iugkp_status solve_graph(Ctx* c, double* T, double tol, int max_iter, cudaStream
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   CK(cudaStreamBeginCapture(gs, cudaStreamCaptureModeThreadLocal), "begin capture");
-  iugkp_status st = iteration_async(c, T, c->d_T2, epoch, c->d_res_block, gs);
-  if (st == IUGKP_OK) st = iteration_async(c, c->d_T2, T, epoch, c->d_res_block + 2, gs);
+  iugkp_status st = iteration_async(c, T, c->d_T2, epoch, false, c->d_res_block, gs);
+  if (st == IUGKP_OK) st = iteration_async(c, c->d_T2, T, epoch, false, c->d_res_block + 2, gs);
   cudaError_t ce = cudaStreamEndCapture(gs, &graph);
   if (st != IUGKP_OK) {
     if (graph) cudaGraphDestroy(graph);
@@ -1330,7 +1365,7 @@ iugkp_status iugkp_solve_steady(iugkp_ctx* ctx, double* T_inout_dev, double tol,
   iugkp_status st;
   while (it < max_iter) {
     const unsigned epoch = c->opt.draws == IUGKP_DRAWS_FROZEN ? c->opt.epoch0 : c->opt.epoch0 + (unsigned)it;
-    if ((st = sweep_async(c, cur, epoch, c->d_R, c->d_W, c->d_F, c->d_wall, c->d_counters, s)) != IUGKP_OK) return st;
+    if ((st = sweep_real_async(c, cur, epoch, s)) != IUGKP_OK) return st;
     CK(launch_macro(c, c->d_R, nullptr, nxt, nullptr, s), "macro");
     if (c->opt.newton) {
       CK(launch_newton(c, cur, nxt, c->d_R, s), "newton");
@@ -1448,7 +1483,7 @@ iugkp_status iugkp_average(iugkp_ctx* ctx, double* T_inout_dev, int n_steps, uns
   double* nxt = c->d_T2;
   for (int k = 0; k < n_steps; ++k) {
     // the solve's update with fresh draws: epoch_first + k
-    iugkp_status st = iteration_async(c, cur, nxt, epoch_first + (unsigned)k, c->d_scalar + 4, s);
+    iugkp_status st = iteration_async(c, cur, nxt, epoch_first + (unsigned)k, F_mean_dev != nullptr, c->d_scalar + 4, s);
     if (st != IUGKP_OK) return st;
     CK(launch_welford(c, nxt, T_mean_dev, m2, c->total_cells, k + 1, s), "welford");
     if (F_mean_dev) CK(launch_welford(c, c->d_F, F_mean_dev, nullptr, c->total_faces, k + 1, s), "flux mean");
@@ -1463,11 +1498,12 @@ iugkp_status iugkp_average(iugkp_ctx* ctx, double* T_inout_dev, int n_steps, uns
 
 namespace {
 
-// The adjoint re-trace: the staged kernel for the FP32 walk with staged tallies (the
+// The adjoint re-trace: the landing kernels for the FP32 walk with staged tallies (the
 // fast path), else the plain one-thread-per-particle kernel.
 cudaError_t adjoint_sweep(Ctx* c, const SweepArgs& a, cudaStream_t s) {
-  if (c->opt.tally != IUGKP_TALLY_FP64 && c->opt.precision == IUGKP_TRACK_FP32 && c->total_particles < (1ll << 31))
-    return launch_adjoint_staged(c, a, s);
+  if (c->opt.tally != IUGKP_TALLY_FP64 && c->opt.precision == IUGKP_TRACK_FP32 && c->total_particles < (1ll << 31) &&
+      land_sizes(c))
+    return launch_land(c, a, true, s);
   return launch_adjoint(c, a, s);
 }
 

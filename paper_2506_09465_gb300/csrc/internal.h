@@ -186,17 +186,16 @@ struct Ctx {
   unsigned long long* d_wmax = nullptr;  // [n_inst] bit patterns of the largest weight
   unsigned* d_group_mag = nullptr;   // [forward groups] division magic of the emitter count
   double* d_wall_unit = nullptr;     // [n_inst * 6] power entering per face per unit wall T
-  // adjoint re-trace over all groups (staged kernel)
-  long long* d_all_beg = nullptr;
-  long long* d_all_end = nullptr;
-  double* d_all_cost_prefix = nullptr;
-  double all_cost_total = 0.0;
-  unsigned* d_all_group_mag = nullptr;
-  int adj_blocks_per_sm = 1;
+  unsigned* d_all_group_mag = nullptr;  // [all groups] the same for the adjoint re-trace
   // particles the staged FP32 walk left to the FP64 replay (sweep and adjoint re-trace)
   uint2* d_defer = nullptr;
-  unsigned* d_defer_n = nullptr;
+  unsigned* d_defer_n = nullptr;     // [4] queue length, unused, 64-bit claim counter of the landing sweeps
   unsigned defer_cap = 0;
+  // landing sweeps (land.cu): tasks of the forward groups and of every group (adjoint)
+  LandGroup* d_land_fwd = nullptr;
+  LandGroup* d_land_all = nullptr;
+  unsigned land_fwd_tasks = 0, land_all_tasks = 0;
+  int land_fwd_qch = 1, land_all_qch = 1;
   unsigned* d_mag = nullptr;         // [n_inst * 5]: division magics of n_x, n_y, n(o1) for walls normal to x, y, z
   int staged_cap = 0;           // x-faces per shared-memory window
   int staged_blocks_per_sm = 1;
@@ -226,7 +225,9 @@ cudaError_t launch_pcg_check(const Ctx* c, cudaStream_t s);
 cudaError_t launch_axpy_grad(const Ctx* c, const double* at, const double* g, double* lam_half, cudaStream_t s);
 cudaError_t launch_sweep_staged(const Ctx* c, const SweepArgs& a, cudaStream_t s);
 cudaError_t configure_staged(Ctx* c);
-cudaError_t launch_adjoint_staged(const Ctx* c, const SweepArgs& a, cudaStream_t s);
+cudaError_t launch_k32_finalize(const Ctx* c, const float2* src, double* dst, long long n, cudaStream_t s);
+cudaError_t launch_land(const Ctx* c, const SweepArgs& a, bool adj, cudaStream_t s);
+void land_tasks(const Ctx* c, const std::vector<Group>& groups, std::vector<LandGroup>& out, unsigned& n_tasks, int& qch);
 cudaError_t launch_replay(const Ctx* c, const SweepArgs& a, const StagedArgs& S, cudaStream_t s);
 cudaError_t launch_adjoint_replay(const Ctx* c, const SweepArgs& a, cudaStream_t s);
 cudaError_t launch_walk_bounds(unsigned long long* out, cudaStream_t s);

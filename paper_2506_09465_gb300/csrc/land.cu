@@ -1,0 +1,548 @@
+// Landing sweeps: the sweep where only the real collisions are asked for (R alone: the steady
+// and averaging loops) and the adjoint re-trace. Same particles and draws as the staged sweep
+// (sweep_staged.cu; arXiv 2506.09465 Sec. 3.1 steps (1)-(3), Sec. 3.2 null collisions).
+//
+// A particle's path from emission to its end is one straight segment, so a candidate at path
+// length D lies, along axis a, X_a = xi_a + g_a D cells from the emission cell's low face
+// (g_a = s_a / h_a): its cell is floor(X_a), and it lies outside the domain exactly when the
+// segment met a wall before it. Nothing else is needed where no face is tallied: no distances
+// to faces (one reciprocal and one quotient per axis), no counts, no exit.
+//
+// FP32 against FP64: g_a is within 3.5 2^-23 of its FP64 value (square root 0.75, sincospif
+// 0.73, their product 0.5, 1 / h and its product 1.5, in units of 2^-23; walk_bounds_kernel
+// measures the first two), D within eD (walk32.cuh), and the sum is rounded once, so X_a is
+// within |g_a| D 2^-21 + |g_a| eD + 2^-24 of the FP64 walk's position. LAND_REL and LAND_ABS
+// take twice and four times that. A candidate within the bound of a face or a wall is left to
+// the FP64 replay, so every real collision is the FP64 walk's. The walls are tested by the
+// differences X - lo and X - hi, which are exact where X is near the wall (adding tol to the
+// wall's coordinate would round by more than tol on a wide grid).
+#include <cuda_runtime.h>
+
+#include <algorithm>
+
+#include "device.cuh"
+#include "internal.h"
+#include "staged.h"
+#include "walk32.cuh"
+
+namespace iugkp {
+
+namespace {
+
+constexpr float LAND_REL = 0x1p-20f;
+constexpr float LAND_ABS = 0x1p-22f;
+constexpr float FLOOR_MAGIC = 12582912.f;  // 1.5 2^23: a round-down add leaves floor(X) in the low bits, |X| < 2^22
+
+// Position of a candidate along one axis: its cell offset and whether it lies within tol of a
+// face (either side).
+__device__ __forceinline__ int floor_near(float X, float tol, bool& near) {
+  const float Y = __fadd_rd(X, FLOOR_MAGIC);
+  const float fr = X - (Y - FLOOR_MAGIC);
+  near |= fminf(fr, 1.f - fr) <= tol;
+  return __float_as_int(Y) - 0x4B400000;
+}
+
+// Cell of an emitter of kind `kind` (0: cells; 1 + w: faces of wall w), and for a wall the
+// index of its face within the instance.
+template <int DIM>
+__device__ __forceinline__ void emitter_cell(const InstDesc& in, const StagedArgs& S, int k, int kind, int e, int (&c)[3],
+                                             uint32_t& id) {
+  const int n0 = in.n[0], n1 = in.n[1], n2 = in.n[2];
+  c[0] = c[1] = c[2] = 0;
+  if (kind == 0) {
+    id = (uint32_t)e;
+    if (DIM == 1) {
+      c[0] = e;
+      return;
+    }
+    const int r = (int)udiv((unsigned)e, (unsigned)n0, S.mag_n0[k]);
+    c[0] = e - r * n0;
+    c[1] = r;
+    if (DIM == 3) {
+      c[2] = (int)udiv((unsigned)r, (unsigned)n1, S.mag_n1[k]);
+      c[1] = r - c[2] * n1;
+    }
+    return;
+  }
+  const int wl = kind - 1, a = wl >> 1, side = wl & 1;
+  // faces of wall a run over (o1, o2) = ((a+1)%3, (a+2)%3), o1 fastest
+  const int no1 = a == 0 ? n1 : (a == 1 ? n2 : n0);
+  const int j2 = (int)udiv((unsigned)e, (unsigned)no1, S.mag_wall[k * 3 + a]);
+  const int j1 = e - j2 * no1;
+  long long face;
+  if (a == 0) {
+    c[0] = side ? n0 - 1 : 0;
+    c[1] = j1;
+    c[2] = j2;
+    face = in.fax_off[0] + (side ? n0 : 0) + (long long)(n0 + 1) * (j1 + (long long)n1 * j2);
+  } else if (a == 1) {
+    c[0] = j2;
+    c[1] = side ? n1 - 1 : 0;
+    c[2] = j1;
+    face = in.fax_off[1] + j2 + (long long)n0 * ((side ? n1 : 0) + (long long)(n1 + 1) * j1);
+  } else {
+    c[0] = j1;
+    c[1] = j2;
+    c[2] = side ? n2 - 1 : 0;
+    face = in.fax_off[2] + j1 + (long long)n0 * (j2 + (long long)n1 * (side ? n2 : 0));
+  }
+  id = (uint32_t)(in.ncells + face);
+}
+
+// Direction and fractions within the emission cell from the stream's first block(s); st.j is
+// set to the first uniform after the emission.
+template <int DIM>
+__device__ __forceinline__ void emit_segment(Stream& st, int kind, float (&xi)[3], float (&s)[3]) {
+  xi[0] = xi[1] = xi[2] = 0.5f;
+  s[0] = s[1] = s[2] = 0.f;
+  if (kind == 0) {
+    float u_mu, u_phi = 0.5f;
+    xi[0] = word_uniform<float>(st.buf.x);
+    if (DIM == 1) {
+      u_mu = word_uniform<float>(st.buf.y);
+    } else if (DIM == 2) {
+      xi[1] = word_uniform<float>(st.buf.y);
+      u_mu = word_uniform<float>(st.buf.z);
+      u_phi = word_uniform<float>(st.buf.w);
+    } else {
+      xi[1] = word_uniform<float>(st.buf.y);
+      xi[2] = word_uniform<float>(st.buf.z);
+      u_mu = word_uniform<float>(st.buf.w);
+      st.load_block(1);
+      u_phi = word_uniform<float>(st.buf.x);
+    }
+    const float mu = 2.f * u_mu - 1.f;
+    s[0] = mu;
+    if (DIM >= 2) {
+      const float sn = sqrtf(fmaf(-mu, mu, 1.f));
+      float sp, cp;
+      sincospif(2.f * u_phi, &sp, &cp);
+      s[1] = sn * cp;
+      s[2] = sn * sp;
+    }
+    st.j = thermal_uniforms(DIM);
+    return;
+  }
+  const int wl = kind - 1, a = wl >> 1, side = wl & 1;
+  float u_n, u_phi = 0.5f, t0 = 0.5f, t1 = 0.5f;
+  if (DIM == 1) {
+    u_n = word_uniform<float>(st.buf.x);
+  } else {
+    t0 = word_uniform<float>(st.buf.x);
+    if (DIM == 2) {
+      u_n = word_uniform<float>(st.buf.y);
+      u_phi = word_uniform<float>(st.buf.z);
+    } else {
+      t1 = word_uniform<float>(st.buf.y);
+      u_n = word_uniform<float>(st.buf.z);
+      u_phi = word_uniform<float>(st.buf.w);
+    }
+  }
+  const float mn = sqrtf(u_n), sn = DIM >= 2 ? sqrtf(1.f - u_n) : 0.f;
+  float sp = 0.f, cp = 0.f;
+  if (DIM >= 2) sincospif(2.f * u_phi, &sp, &cp);
+  const float nrm = side ? -mn : mn, ta = sn * cp, tb = sn * sp, edge = side ? 1.f : 0.f;
+  if (a == 0) {
+    s[0] = nrm; s[1] = ta; s[2] = tb;
+    xi[0] = edge; xi[1] = t0; xi[2] = t1;
+  } else if (a == 1) {
+    s[1] = nrm; s[2] = ta; s[0] = tb;
+    xi[1] = edge; xi[0] = t0; xi[2] = t1;
+  } else {
+    s[2] = nrm; s[0] = ta; s[1] = tb;
+    xi[2] = edge; xi[0] = t0; xi[1] = t1;
+  }
+  st.j = wall_uniforms(DIM);
+}
+
+template <bool K32>
+__device__ __forceinline__ void deposit(const SweepArgs& A, const StagedArgs& S, long long j, double w) {
+  if (K32) tally_k32(&S.R32[j], w);
+  else atomicAdd(&A.R[j], w);
+}
+
+// Bands whose every candidate is real: one candidate per particle, no chain. A lane keeps its
+// emitter for qch particles in a row, so the cell coordinates, the weight, the first Philox
+// rounds (the counter's emitter word does not change) and, in the adjoint, the gathered sum stay
+// in registers; the lanes of a warp hold neighbouring emitters. Tasks (a tile of emitters x a
+// run of particle numbers) are claimed one at a time by each warp.
+template <int DIM, bool ADJ, bool K32>
+__global__ void __launch_bounds__(LAND_NT) land_kernel(SweepArgs A, StagedArgs S, LandArgs L) {
+  const int lane = threadIdx.x & 31;
+  unsigned t_beg = 1, t_end = 0;  // tasks of the cached group
+  LandGroup G;
+  for (;;) {
+    unsigned task = 0;
+    if (lane == 0) task = (unsigned)atomicAdd(L.next, 1ull);
+    task = __shfl_sync(0xffffffffu, task, 0);
+    if (task >= L.n_tasks) return;
+    if (task < t_beg || task >= t_end) {
+      int lo = 0, hi = L.n_groups - 1;
+      while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (L.groups[mid].task0 <= task) lo = mid;
+        else hi = mid - 1;
+      }
+      G = L.groups[lo];
+      t_beg = G.task0;
+      t_end = lo + 1 < L.n_groups ? L.groups[lo + 1].task0 : L.n_tasks;
+    }
+    const unsigned t = task - t_beg;
+    const int qc = (int)(t / (unsigned)G.ntile), tile = (int)(t - (unsigned)qc * (unsigned)G.ntile);
+    const InstDesc& in = A.inst[G.inst];
+    const int sub = lane / G.tw, rank = tile * G.tw + lane - sub * G.tw;
+    bool on = sub < G.reps && rank < G.ne;
+    int e = on ? rank : 0;
+    if (G.perm_off >= 0) e = A.perm[G.perm_off + e];
+    // the emitter: cell, stream identity, weight
+    int c[3];
+    uint32_t id;
+    emitter_cell<DIM>(in, S, G.inst, G.kind, e, c, id);
+    double w;
+    const int kb = G.inst * A.nb + G.band;
+    if (G.kind == 0) {
+      w = A.coef[in.bc_off + (long long)G.band * in.ncells + e];
+      if (!ADJ) {
+        double Te = A.T[in.cell_off + e];
+        if (A.srcshift) Te += A.srcshift[in.cell_off + e];
+        w *= Te;
+      }
+    } else {
+      w = A.wcoef[(long long)kb * 6 + G.kind - 1];
+      if (!ADJ) w *= A.wallTf[in.bface_off + in.wface_off[G.kind - 1] + e];
+    }
+    on = on && (__double_as_longlong(w) << 1) != 0;  // +-0: nothing to trace
+    const int n0 = in.n[0], n1 = in.n[1], n2 = in.n[2];
+    const float vtm = A.vtm32[kb], va = vtm * TIE_LOG_ABS;
+    float ih[3], lo[3], hi[3];
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) {
+      ih[a] = __frcp_rn(in.hf[a]);
+      lo[a] = (float)-c[a];
+      hi[a] = (float)((a == 0 ? n0 : (a == 1 ? n1 : n2)) - c[a]);
+    }
+    const int cell0 = c[0] + n0 * (c[1] + n1 * c[2]);
+    const long long bcbase = in.bc_off + (long long)G.band * in.ncells, coff = in.cell_off;
+    const uint32_t inst_id = in.inst_id;
+    double acc = 0.0;
+    const int qbeg = qc * (L.qch * G.reps) + sub, qend = min(G.per, (qc + 1) * (L.qch * G.reps));
+    for (int q = on ? qbeg : qend; q < qend; q += G.reps) {
+      Stream st;
+      st.init(A.seed, inst_id, (uint32_t)G.band, A.epoch, id, (uint32_t)q);
+      float xi[3], s[3];
+      emit_segment<DIM>(st, G.kind, xi, s);
+      const float D = __fmul_rn(-__logf(word_uniform<float>(st.first)), vtm);
+      const float eD = fmaf(D, TIE_LOG_REL, va), rel = fmaf(D, LAND_REL, eD);
+      bool out = false, near = false;
+      int o[3] = {0, 0, 0};
+#pragma unroll
+      for (int a = 0; a < DIM; ++a) {
+        const float g = s[a] * ih[a];
+        const float X = fmaf(g, D, xi[a]), tol = fmaf(fabsf(g), rel, LAND_ABS);
+        out |= lo[a] - X > tol || X - hi[a] > tol;  // beyond a wall for the FP64 walk too
+        o[a] = floor_near(X, tol, near);
+      }
+      if (out) continue;
+      if (near) {
+        defer_particle(S, G.first + (unsigned)q * (unsigned)G.ne + (unsigned)rank, 0u);
+        continue;
+      }
+      const int cell = cell0 + o[0] + (DIM >= 2 ? n0 * o[1] : 0) + (DIM == 3 ? n0 * n1 * o[2] : 0);
+      if (ADJ) acc += L.lamVm[coff + cell];
+      else deposit<K32>(A, S, bcbase + cell, w);
+    }
+    if (ADJ) {
+      acc *= w;
+      if (G.kind == 0) {
+        if (acc != 0.0) atomicAdd(&A.adj_out[coff + e], acc);
+      } else {
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, d);
+        if (lane == 0 && acc != 0.0) atomicAdd(&A.adj_wall[in.wall_off + G.kind - 1], acc);
+      }
+    }
+  }
+}
+
+// Bands with null candidates: every lane follows the candidates of its own particle, and a warp
+// refills its idle lanes once LAND_REFILL of them are idle (particles q-major in the group's
+// visiting order, claimed in runs, as in sweep_staged_kernel).
+template <int DIM, bool ADJ, bool K32>
+__global__ void __launch_bounds__(LAND_NT) land_chain_kernel(SweepArgs A, StagedArgs S, LandArgs L) {
+  const int lane = threadIdx.x & 31;
+  const unsigned lt_mask = (1u << lane) - 1u, total = (unsigned)A.total_particles;
+  unsigned rbeg = 0, rend = 0, pid = 0;
+  bool alive = false, exhausted = false;
+  unsigned g_first = 1, g_end = 0, g_mag = 0;  // the lane's cached group
+  int g_ne = 1, g_perm = -1, kind = 0, band = 0, inst = 0, emitter = 0, acc_slot = 0, acc_inst = 0;
+  bool all_real = false;
+  long long bcbase = 0, coff = 0;
+  int n0 = 1, n1 = 1, n2 = 1, cell0 = 0;
+  float vtm = 0.f, D = 0.f, eD = 0.f;
+  float xi[3], g[3], lo[3], hi[3];
+  uint32_t ub = 0;
+  double w = 0.0, acc = 0.0;
+  Stream st;
+  auto flush_wall = [&] {
+    if (acc != 0.0) atomicAdd(&A.adj_wall[A.inst[acc_inst].wall_off + acc_slot], acc);
+    acc = 0.0;
+  };
+  for (;;) {
+    const unsigned dead = __ballot_sync(0xffffffffu, !alive);
+    if (!exhausted && (__popc(dead) >= LAND_REFILL)) {
+      if (rbeg == rend) {
+        unsigned long long got = 0;
+        if (lane == 0) got = atomicAdd(L.next, (unsigned long long)S.warp_grab);
+        got = __shfl_sync(0xffffffffu, got, 0);
+        if (got < total) {
+          rbeg = (unsigned)got;
+          rend = (unsigned)min(got + (unsigned long long)S.warp_grab, (unsigned long long)total);
+        } else {
+          exhausted = true;
+        }
+      }
+      const unsigned r = __popc(dead & lt_mask), take = min((unsigned)__popc(dead), rend - rbeg);
+      if (!alive && r < take) {
+        pid = rbeg + r;
+        if (pid < g_first || pid >= g_end) {
+          const int gi = find_group(A.groups, A.n_groups, (long long)pid);
+          const Group G = A.groups[gi];
+          g_first = (unsigned)G.first_particle;
+          g_end = (unsigned)(G.first_particle + (long long)G.n_emitters * G.per_emitter);
+          g_ne = G.n_emitters;
+          g_mag = S.group_mag[gi];
+          g_perm = G.perm_off;
+          kind = G.kind;
+          band = G.band;
+          inst = G.inst;
+          const InstDesc& in = A.inst[inst];
+          n0 = in.n[0];
+          n1 = in.n[1];
+          n2 = in.n[2];
+          bcbase = in.bc_off + (long long)band * in.ncells;
+          coff = in.cell_off;
+          vtm = A.vtm32[(long long)inst * A.nb + band];
+          all_real = A.all_real[(long long)inst * A.nb + band] != 0;
+        }
+        const InstDesc& in = A.inst[inst];
+        const unsigned local = pid - g_first;
+        const int q = (int)udiv(local, (unsigned)g_ne, g_mag);
+        int e = (int)(local - (unsigned)q * (unsigned)g_ne);
+        if (g_perm >= 0) e = A.perm[g_perm + e];
+        if (kind == 0) {
+          w = A.coef[bcbase + e];
+          if (!ADJ) {
+            double Te = A.T[coff + e];
+            if (A.srcshift) Te += A.srcshift[coff + e];
+            w *= Te;
+          }
+        } else {
+          w = A.wcoef[((long long)inst * A.nb + band) * 6 + kind - 1];
+          if (!ADJ) w *= A.wallTf[in.bface_off + in.wface_off[kind - 1] + e];
+          if (ADJ && (acc_slot != kind - 1 || acc_inst != inst)) {
+            flush_wall();
+            acc_slot = kind - 1;
+            acc_inst = inst;
+          }
+        }
+        if ((__double_as_longlong(w) << 1) != 0) {
+          int c[3];
+          uint32_t id;
+          float s[3];
+          emitter = e;
+          emitter_cell<DIM>(in, S, inst, kind, e, c, id);
+          st.init(A.seed, in.inst_id, (uint32_t)band, A.epoch, id, (uint32_t)q);
+          emit_segment<DIM>(st, kind, xi, s);
+#pragma unroll
+          for (int a = 0; a < DIM; ++a) {
+            g[a] = s[a] * __frcp_rn(in.hf[a]);
+            lo[a] = (float)-c[a];
+            hi[a] = (float)((a == 0 ? n0 : (a == 1 ? n1 : n2)) - c[a]);
+          }
+          cell0 = c[0] + n0 * (c[1] + n1 * c[2]);
+          ub = all_real ? 0u : st.even_word();
+          st.j += 2;
+          D = __fmul_rn(-__logf(word_uniform<float>(st.first)), vtm);
+          eD = fmaf(D, TIE_LOG_REL, vtm * TIE_LOG_ABS);
+          alive = true;
+        }
+      }
+      rbeg += take;
+    }
+    if (!__any_sync(0xffffffffu, alive)) {
+      if (exhausted) break;
+      continue;
+    }
+    if (alive) {
+#pragma unroll 1
+      for (int it = 0; it < S.walk_k; ++it) {
+        if (it > 0 && __popc(__activemask()) < WALK_MIN_LANES) break;
+        const float rel = fmaf(D, LAND_REL, eD);
+        bool out = false, in_dom = true, near = false;
+        int o[3] = {0, 0, 0};
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) {
+          const float X = fmaf(g[a], D, xi[a]), tol = fmaf(fabsf(g[a]), rel, LAND_ABS);
+          out |= lo[a] - X > tol || X - hi[a] > tol;
+          in_dom = in_dom && X - lo[a] > tol && hi[a] - X > tol && tol < 0.5f;
+          o[a] = floor_near(X, tol, near);
+        }
+        if (out) {  // absorbed by a wall
+          alive = false;
+          break;
+        }
+        // at the first wall within rounding, or a bound beyond the neighbouring cells
+        bool real = all_real, defer = !in_dom;
+        const int cell = cell0 + o[0] + (DIM >= 2 ? n0 * o[1] : 0) + (DIM == 3 ? n0 * n1 * o[2] : 0);
+        if (!defer) {
+          if (all_real) {
+            defer = near;
+          } else {
+            // rejected wherever it lies within the bound when the draw exceeds the largest ratio
+            // of the cell's neighbourhood; otherwise the cell and the ratio must be certain
+            const float ua = word_uniform<float>(ub);
+            if (ua - A.ratio_nb32[bcbase + cell] < TIE_ACC) {
+              const float ra = A.ratio32[bcbase + cell];
+              defer = near || fabsf(ua - ra) < TIE_ACC;
+              real = ua < ra;
+            }
+          }
+        }
+        if (defer) {
+          defer_particle(S, pid, 0u);
+          alive = false;
+          break;
+        }
+        if (real) {
+          if (ADJ) {
+            const double val = w * L.lamVm[coff + cell];
+            if (kind == 0) atomicAdd(&A.adj_out[coff + emitter], val);
+            else acc += val;
+          } else {
+            deposit<K32>(A, S, bcbase + cell, w);
+          }
+          alive = false;
+          break;
+        }
+        uint32_t uw;
+        st.next_pair(uw, ub);
+        const float ell = __fmul_rn(-__logf(word_uniform<float>(uw)), vtm);
+        D = __fadd_rn(D, ell);
+        eD = fmaf(D, TIE_SUM, fmaf(ell, TIE_LOG_REL, eD + vtm * TIE_LOG_ABS));
+      }
+    }
+  }
+  if (ADJ) flush_wall();
+}
+
+__global__ void lam_over_vm_kernel(long long n, const double* lam, const double* invVm, double* out) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+    out[i] = lam[i] * invVm[i];
+}
+
+template <int DIM, bool ADJ, bool K32>
+cudaError_t launch_dim(const Ctx* c, const SweepArgs& a, const StagedArgs& S, const LandArgs& L, cudaStream_t s) {
+  const void* f = c->all_real_all ? (const void*)land_kernel<DIM, ADJ, K32> : (const void*)land_chain_kernel<DIM, ADJ, K32>;
+  int nb = 0;
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f, LAND_NT, 0);
+  if (e != cudaSuccess) return e;
+  // warps beyond the work would only claim and leave
+  const long long warps = c->all_real_all ? (long long)L.n_tasks : (a.total_particles + S.warp_grab - 1) / S.warp_grab;
+  const long long want = (warps * 32 + LAND_NT - 1) / LAND_NT;
+  const int blocks = (int)std::max<long long>(1, std::min<long long>(want, (long long)c->sm_count * std::max(nb, 1)));
+  if (c->all_real_all) land_kernel<DIM, ADJ, K32><<<blocks, LAND_NT, 0, s>>>(a, S, L);
+  else land_chain_kernel<DIM, ADJ, K32><<<blocks, LAND_NT, 0, s>>>(a, S, L);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_land(const Ctx* c, const SweepArgs& a, bool adj, cudaStream_t s) {
+  StagedArgs S = {};
+  S.warp_grab = c->opt.warp_grab > 0 ? c->opt.warp_grab : 256;
+  S.walk_k = c->opt.walk_k > 0 ? c->opt.walk_k : 16;
+  S.group_mag = adj ? c->d_all_group_mag : c->d_group_mag;
+  S.mag_n0 = c->d_mag;
+  S.mag_n1 = c->d_mag + c->n_inst;
+  S.mag_wall = c->d_mag + 2 * c->n_inst;
+  S.defer = c->d_defer;
+  S.defer_n = c->d_defer_n;
+  S.defer_cap = c->defer_cap;
+  S.err = c->d_err;
+  const bool k32 = !adj && c->opt.tally == IUGKP_TALLY_STAGED_K32;
+  S.R32 = k32 ? c->d_R32 : nullptr;
+  LandArgs L;
+  L.groups = adj ? c->d_land_all : c->d_land_fwd;
+  L.n_groups = a.n_groups;
+  L.n_tasks = adj ? c->land_all_tasks : c->land_fwd_tasks;
+  L.qch = adj ? c->land_all_qch : c->land_fwd_qch;
+  L.next = reinterpret_cast<unsigned long long*>(c->d_defer_n + 2);
+  L.lamVm = c->d_work;
+  cudaError_t e = cudaMemsetAsync(c->d_defer_n, 0, 4 * sizeof(unsigned), s);  // queue length and task counter
+  if (e != cudaSuccess) return e;
+  const size_t bc = (size_t)c->nb * c->total_cells;
+  if (adj) {
+    // lambda / (V m), gathered by every particle: into the correction solve's scratch, free
+    // until the correction that follows on the same stream
+    lam_over_vm_kernel<<<(unsigned)std::min<long long>((c->total_cells + 255) / 256, 8ll * c->sm_count), 256, 0, s>>>(
+        c->total_cells, a.lambda, a.invVm, c->d_work);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    switch (c->dim) {
+      case 1: e = launch_dim<1, true, false>(c, a, S, L, s); break;
+      case 2: e = launch_dim<2, true, false>(c, a, S, L, s); break;
+      default: e = launch_dim<3, true, false>(c, a, S, L, s); break;
+    }
+    if (e != cudaSuccess) return e;
+    return launch_adjoint_replay(c, a, s);
+  }
+  if (k32) {
+    if ((e = cudaMemsetAsync(c->d_R32, 0, bc * sizeof(float2), s)) != cudaSuccess) return e;
+    switch (c->dim) {
+      case 1: e = launch_dim<1, false, true>(c, a, S, L, s); break;
+      case 2: e = launch_dim<2, false, true>(c, a, S, L, s); break;
+      default: e = launch_dim<3, false, true>(c, a, S, L, s); break;
+    }
+    if (e != cudaSuccess) return e;
+    if ((e = launch_k32_finalize(c, c->d_R32, a.R, (long long)bc, s)) != cudaSuccess) return e;
+  } else {
+    switch (c->dim) {
+      case 1: e = launch_dim<1, false, false>(c, a, S, L, s); break;
+      case 2: e = launch_dim<2, false, false>(c, a, S, L, s); break;
+      default: e = launch_dim<3, false, false>(c, a, S, L, s); break;
+    }
+    if (e != cudaSuccess) return e;
+  }
+  return launch_replay(c, a, S, s);  // the deferred particles, in FP64
+}
+
+// Tasks of the landing sweep over a group list: tiles of at most 32 emitters (equal widths;
+// narrow groups put several particles of an emitter side by side), qch particles per emitter and
+// task: at most LAND_QCH, fewer where that would leave warps without work.
+void land_tasks(const Ctx* c, const std::vector<Group>& groups, std::vector<LandGroup>& out, unsigned& n_tasks, int& qch) {
+  long long total = 0;
+  for (const Group& g : groups) total += (long long)g.n_emitters * g.per_emitter;
+  const long long warps = (long long)std::max(1, c->sm_count) * LAND_WARPS_PER_SM;
+  qch = (int)std::max<long long>(1, std::min<long long>(LAND_QCH, total / (32 * 4 * warps)));
+  long long t0 = 0;
+  out.clear();
+  for (const Group& g : groups) {
+    LandGroup l;
+    l.first = (unsigned)g.first_particle;
+    l.inst = g.inst;
+    l.band = g.band;
+    l.kind = g.kind;
+    l.ne = g.n_emitters;
+    l.per = g.per_emitter;
+    l.perm_off = g.perm_off;
+    l.ntile = (g.n_emitters + 31) / 32;
+    l.tw = (g.n_emitters + l.ntile - 1) / l.ntile;
+    l.reps = 32 / l.tw;
+    l.task0 = (unsigned)t0;
+    const long long run = (long long)qch * l.reps;
+    t0 += (long long)l.ntile * ((l.per + run - 1) / run);
+    out.push_back(l);
+  }
+  n_tasks = (unsigned)t0;
+}
+
+}  // namespace iugkp

@@ -73,4 +73,28 @@ struct StagedArgs {
 #endif
 };
 
+// Landing sweeps (land.cu).
+constexpr int LAND_NT = 256;          // threads per block
+constexpr int LAND_QCH = 16;          // particles per emitter and task at most
+constexpr int LAND_WARPS_PER_SM = 40; // resident warps the task size is chosen for
+constexpr int LAND_REFILL = 8;        // idle lanes that trigger a refill (null-candidate chains)
+
+// A group's tasks: tiles of tw emitters (reps particles of an emitter side by side where tw is
+// at most 16) x runs of qch * reps particles per emitter, tiles fastest; task0 is its first.
+struct LandGroup {
+  unsigned first;                 // first particle (forward or adjoint numbering)
+  int inst, band, kind, ne, per, perm_off;
+  int tw, ntile, reps;
+  unsigned task0;
+};
+
+struct LandArgs {
+  const LandGroup* groups;
+  int n_groups;
+  unsigned n_tasks;
+  int qch;
+  unsigned long long* next;       // next unclaimed task (or particle, where chains are followed)
+  const double* lamVm;            // adjoint: [cells] lambda / (V m)
+};
+
 }  // namespace iugkp

@@ -1,4 +1,4 @@
-// Fast forward sweep and adjoint re-trace: FP32 walk, persistent blocks (a pass-synchronous
+// Fast forward sweep: FP32 walk, persistent blocks (a pass-synchronous
 // kernel for 2D, a per-lane-refill kernel for every dimension), face tallies staged in
 // shared memory in fixed point. Same method and draws as the plain sweep
 // (arXiv 2506.09465 Sec. 3.1 steps (1)-(3), Sec. 3.2 null collisions); only the
@@ -35,6 +35,7 @@
 #include "device.cuh"
 #include "internal.h"
 #include "staged.h"
+#include "walk32.cuh"
 
 namespace iugkp {
 
@@ -99,29 +100,6 @@ __device__ __forceinline__ float axis_exit(int i, int s, int n, float t, float d
 
 __device__ __forceinline__ int clampi(int v, int n) { return min(max(v, 0), n - 1); }
 
-// ---- FP32 decisions checked against the FP64 walk ----
-// The FP32 walk and the FP64 walk follow each particle with the same draws, so their path
-// lengths differ by rounding only, and a decision taken in FP32 is the FP64 walk's unless the
-// FP32 value lies within a bound of the decision's boundary: a face (the count of faces before
-// a candidate along an axis, hence its cell), the first wall (a candidate or an absorption),
-// the acceptance ratio. A particle with such a decision is not tallied further: it goes to a
-// queue that the FP64 walk replays after the sweep (replay_kernel, adjoint_replay_kernel).
-// Path-length bounds, FP32 against FP64:
-//  * a face count's quotient u = (D - t) / d, times d: TIE_REL (D + d) + eD, TIE_REL covering
-//    the rounding of the direction (sqrtf, sincospif, products), cell size, first-face
-//    distance, quotient (__fdividef) and difference, about 2^-19.4 in all, taken as 2^-18;
-//    the wall distance tex likewise within TIE_REL tex;
-//  * eD bounds |D32 - D64|: per flight TIE_LOG_ABS v tau_maj + TIE_LOG_REL l for the fast
-//    logarithm, the FP32 v tau_maj and the product's rounding, plus TIE_SUM D for each
-//    addition to D. The logarithm's error over all 2^23 uniforms the walk draws is measured
-//    (walk_bounds_kernel) at about a third of its share of this allowance.
-// The acceptance ratio in FP32 is within 2^-24 of the FP64 ratio (both below 1).
-constexpr float TIE_REL = 0x1p-18f;
-constexpr float TIE_LOG_ABS = 0x1p-22f;
-constexpr float TIE_LOG_REL = 0x1p-20f;
-constexpr float TIE_SUM = 0x1p-23f;
-constexpr float TIE_ACC = 0x1p-24f;
-
 // Tie bits of one axis for the count n = faces_before(D, t, d): bit sh when D lies within the
 // bound (base = TIE_REL D + eD, plus TIE_REL d) below a face, so that the FP64 walk may count
 // one face more; bit sh + 1 when within it above one (one fewer). None when d = inf (NaN).
@@ -173,13 +151,6 @@ __device__ __forceinline__ bool all_reject(const float* ratio, int ncells, int c
     if (c < 0 || c >= ncells || !(u - ratio[c] >= TIE_ACC)) return false;
   }
   return true;
-}
-
-// Queues a particle for the FP64 replay: forward index and (candidates tallied << 1) | group.
-__device__ __forceinline__ void defer_particle(const StagedArgs& S, unsigned pid, unsigned meta) {
-  const unsigned i = atomicAdd(S.defer_n, 1u);
-  if (i < S.defer_cap) S.defer[i] = make_uint2(pid, meta);
-  else atomicOr(S.err, ERR_DEFER);
 }
 
 enum { CAND_NULL = 0, CAND_REAL = 1, CAND_DEFER = 2 };
@@ -277,13 +248,10 @@ struct EmitCache {
 
 // Emits forward particle pid into the lane state. Returns false for a zero-weight
 // particle (nothing to trace).
-// ADJ: the adjoint re-trace; w is then the particle's weight per unit emission
-// temperature (every emitter is traced) and `emitter` receives the cell (>= 0) or the
-// wall slot (-1 - wall) the particle's gather belongs to.
-template <int DIM, bool ADJ>
-__device__ __forceinline__ bool staged_emit(const SweepArgs& A, const StagedArgs& S, unsigned pid, bool useF,
-                                            double& w, int& band, PW& f, Stream& st, uint32_t& ub, EmitCache& ec,
-                                            const InstDesc& in, int k, int& emitter, bool two) {
+template <int DIM>
+__device__ __forceinline__ bool staged_emit(const SweepArgs& A, const StagedArgs& S, unsigned pid, double& w,
+                                            int& band, PW& f, Stream& st, uint32_t& ub, EmitCache& ec,
+                                            const InstDesc& in, int k, bool two) {
   if (pid < ec.g_first || pid >= ec.g_end) {
     const int gi = find_group(A.groups, A.n_groups, (long long)pid);
     const Group G = A.groups[gi];
@@ -312,13 +280,8 @@ __device__ __forceinline__ bool staged_emit(const SweepArgs& A, const StagedArgs
   const int kind = ec.g_kind;
   float xi0 = 0.5f, xi1 = 0.5f, xi2 = 0.5f, sx = 0.f, sy = 0.f, sz = 0.f;
   if (kind == 0) {
-    if (ADJ) {
-      w = A.coef[in.bc_off + (long long)b * in.ncells + e];
-    } else {
-      w = A.wemit[in.bc_off + (long long)b * in.ncells + e];  // from the w_max pre-pass
-      if ((__double_as_longlong(w) << 1) == 0) return false;   // +-0: nothing to trace
-    }
-    emitter = e;
+    w = A.wemit[in.bc_off + (long long)b * in.ncells + e];  // from the w_max pre-pass
+    if ((__double_as_longlong(w) << 1) == 0) return false;   // +-0: nothing to trace
     st.init(A.seed, in.inst_id, (uint32_t)b, A.epoch, (uint32_t)e, (uint32_t)q);
     if (DIM == 1) {
       f.i0 = e;
@@ -368,9 +331,8 @@ __device__ __forceinline__ bool staged_emit(const SweepArgs& A, const StagedArgs
       ec.w = A.wcoef[((long long)k * A.nb + b) * 6 + wl];  // per unit face temperature
       ec.e = -2;
     }
-    w = ADJ ? ec.w : ec.w * A.wallTf[in.bface_off + in.wface_off[wl] + e];
+    w = ec.w * A.wallTf[in.bface_off + in.wface_off[wl] + e];
     if (w == 0.0) return false;
-    emitter = -1 - wl;
     const int a = wl >> 1, side = wl & 1;
     // faces of wall a are enumerated over (o1, o2) = ((a+1)%3, (a+2)%3), o1 fastest
     const int no1 = a == 0 ? n1 : (a == 1 ? n2 : n0);
@@ -439,7 +401,7 @@ __device__ __forceinline__ bool staged_emit(const SweepArgs& A, const StagedArgs
     axis_init(sz, xi2, in.hf[2], f.t2, f.d2, f.s2);
     f.tex = fminf(f.tex, axis_exit(f.i2, f.s2, n2, f.t2, f.d2));
   }
-  if (!ADJ && DIM == 2 && two && f.d0 < f.d1) {
+  if (DIM == 2 && two && f.d0 < f.d1) {
     // y-group: its emission enters its own power balance (cell) or boundary flux (face)
     if (kind == 0) {
       atomicAdd(&S.DY[in.cell_off + e], -w);
@@ -462,25 +424,6 @@ __device__ __forceinline__ bool staged_emit(const SweepArgs& A, const StagedArgs
 // private ranges of the instance's particles and refill idle lanes together. Faces normal
 // to x go to a shared-memory copy of the instance's x-faces (when it fits), in units of
 // the instance's q; the block flushes it when it leaves the instance.
-// ADJ = true: the adjoint re-trace (see adjoint.cu for the map it transposes): no tallies;
-// a real collision gathers c_p lambda[stop] / (V m_stop) into the particle's emitter cell,
-// or into its wall, accumulated per lane while the lane stays on one wall group.
-// Compensated FP32 tally. The atomic returns the value it added to, so the exact rounding
-// error of the stored sum is known locally (Knuth's TwoSum, six FP32 operations); that error
-// and the low part of the FP64 addend go to the companion word. After n additions the pair
-// holds the sum to about n 2^-48 relative. (atom.add.f32 flushes subnormal results to zero:
-// an absolute error below 2^-126 per addition, far under the tally scale.)
-__device__ __forceinline__ void tally_k32(float2* p, double x) {
-  const float xh = __double2float_rn(x);
-  const float xl = __double2float_rn(x - (double)xh);
-  const float old = atomicAdd(&p->x, xh);
-  const float sum = __fadd_rn(old, xh);
-  const float bv = __fsub_rn(sum, old);
-  const float err = __fadd_rn(__fsub_rn(old, __fsub_rn(sum, bv)), __fsub_rn(xh, bv));
-  const float lo = __fadd_rn(err, xl);
-  if (lo != 0.f) atomicAdd(&p->y, lo);
-}
-
 // Instance holding entry j of a [band][cell] array: the last one whose bc_off is at or before j.
 __device__ __forceinline__ int bc_instance(const InstDesc* inst, int n_inst, long long j) {
   int lo = 0, hi = n_inst - 1;
@@ -514,7 +457,7 @@ __global__ void k32_finalize_kernel(const float2* src, double* dst, long long n,
   }
 }
 
-template <int DIM, bool ADJ, bool K32>
+template <int DIM, bool K32>
 __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A, StagedArgs S) {
   extern __shared__ unsigned win[];
   // cooperative tallies: per warp, each lane's particle parameters and the item list starts
@@ -526,7 +469,7 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
   for (int k = 0; k < CNT_N; ++k) cnt.v[k] = 0;
   const int lane = threadIdx.x & 31;
   const unsigned lt_mask = (1u << lane) - 1u;
-  const bool useF = !ADJ && A.F != nullptr;
+  const bool useF = A.F != nullptr;
   const int n_inst = S.n_inst;
   int start = 0;
   {
@@ -578,12 +521,9 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
     ec.g_first = 1;
     ec.g_end = 0;  // empty: forces a lookup on the first emission
     ec.e = -1;
-    int emitter = 0;        // adjoint: gather target of the lane's particle
-    int acc_slot = 0;       // adjoint: wall slot of the pending per-lane wall sum
-    double acc = 0.0;
     float eD = 0.f;         // bound of |D - D_fp64| of the lane's particle
     int kc = 0;             // its candidates tallied so far
-    unsigned pid = 0;       // its forward (or adjoint) index
+    unsigned pid = 0;       // its forward index
     for (;;) {
       // ---- refill idle lanes together ----
       const unsigned dead = __ballot_sync(0xffffffffu, !alive);
@@ -602,12 +542,7 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
         const unsigned rank = __popc(dead & lt_mask);
         const unsigned take = min((unsigned)__popc(dead), rend - rbeg);
         if (!alive && rank < take) {
-          alive = staged_emit<DIM, ADJ>(A, S, rbeg + rank, useF, w, band, f, st, ub, ec, in, k, emitter, two);
-          if (ADJ && alive && emitter < 0 && emitter != acc_slot) {
-            if (acc != 0.0) atomicAdd(&A.adj_wall[in.wall_off + (-1 - acc_slot)], acc);
-            acc = 0.0;
-            acc_slot = emitter;
-          }
+          alive = staged_emit<DIM>(A, S, rbeg + rank, w, band, f, st, ub, ec, in, k, two);
           if (alive) {
             cnt.v[CNT_FLIGHTS] += 1;
             // round(w / q) as the low word of w qinv + 1.5 2^52 (one FMA, |w qinv| <= 2^26)
@@ -678,21 +613,16 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
           ++kc;
           // W collects w here; the sweep scales it by tau_maj afterwards (scale_by_taumaj), and
           // a band whose every candidate is real takes W = tau_maj R there instead
-          if (!ADJ && K32 && S.W32 && !all_real) tally_k32(&S.W32[ci], w);
-          else if (!ADJ && !K32 && A.W && !all_real) atomicAdd(&A.W[ci], w);
+          if (K32 && S.W32 && !all_real) tally_k32(&S.W32[ci], w);
+          else if (!K32 && A.W && !all_real) atomicAdd(&A.W[ci], w);
           if (oc == CAND_REAL) {
             cnt.v[CNT_REAL] += 1;
-            if (ADJ) {
-              const long long gc = in.cell_off + cell;
-              const double val = w * A.lambda[gc] * A.invVm[gc];
-              if (emitter >= 0) atomicAdd(&A.adj_out[in.cell_off + emitter], val);
-              else acc += val;
-            } else if (K32) {
+            if (K32) {
               tally_k32(&S.R32[ci], w);
             } else {
               atomicAdd(&A.R[ci], w);
             }
-            if (!ADJ && two && f.d0 < f.d1) atomicAdd(&S.DY[in.cell_off + cell], w);
+            if (two && f.d0 < f.d1) atomicAdd(&S.DY[in.cell_off + cell], w);
             ended = true;
             break;
           }
@@ -705,7 +635,7 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
       }
       if (walking) {
         if (deferred) {
-          defer_particle(S, pid, ADJ ? 0u : (((unsigned)kc << 1) | ((two && f.d0 < f.d1) ? 1u : 0u)));
+          defer_particle(S, pid, ((unsigned)kc << 1) | ((two && f.d0 < f.d1) ? 1u : 0u));
           ended = false;
           alive = false;
         }
@@ -746,7 +676,7 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
               c2 = min(q, m2 - 1);
             }
           }
-          if (!ADJ && wall_exit && tie) {
+          if (wall_exit && tie) {
             defer_particle(S, pid, ((unsigned)kc << 1) | ((two && f.d0 < f.d1) ? 1u : 0u));
             alive = false;
           } else {
@@ -930,7 +860,7 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
       // ---- 3D: the warp tallies the x- and y-face items of the particles that ended in this
       // pass together (lists 2 lane and 2 lane + 1, concatenated in order and cut into 32
       // equal contiguous chunks, one per lane), with global atomics ----
-      if (DIM == 3 && !ADJ && useF) {
+      if (DIM == 3 && useF) {
         int incl = nx3 + ny3;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -1037,7 +967,6 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
         }
       }
     }
-    if (ADJ && acc != 0.0) atomicAdd(&A.adj_wall[in.wall_off + (-1 - acc_slot)], acc);
     __syncthreads();
     if (wlen) {
       const double qs = wmax / WIN_SCALE;
@@ -1119,11 +1048,11 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_sync_kernel(SweepArgs A, S
       int4 pa_own, pb_own;  // this lane's item parameters, stored once its list slot is known
       if ((unsigned)lane < take) {
         double w;
-        int band, emitter;
+        int band;
         PW f;
         Stream st;
         uint32_t ub;
-        if (staged_emit<2, false>(A, S, rbeg + lane, true, w, band, f, st, ub, ec, in, k, emitter, two)) {
+        if (staged_emit<2>(A, S, rbeg + lane, w, band, f, st, ub, ec, in, k, two)) {
           cnt.v[CNT_FLIGHTS] += 1;
           const int qw = __double2loint(fma(w, qinv, 0x1.8p52));
           const bool yg = two && f.d0 < f.d1;
@@ -1310,140 +1239,6 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_sync_kernel(SweepArgs A, S
         if (v) atomicAdd(&Fx[i], (double)v * qs);
       }
     }
-    __syncthreads();
-  }
-  flush_lcounts(cnt, A.counters);
-}
-
-// The adjoint re-trace of 2D contexts, pass by pass: every pass of a warp emits up to 32
-// particles (every emitter's, per unit emission temperature), follows each to its real
-// collision or wall, and gathers c_p lambda[stop] / (V m_stop) into the particle's emitter
-// cell (or its wall, summed per lane while the lane stays on one wall group). Same
-// particles and draws as the per-lane-refill re-trace of sweep_staged_kernel<DIM, true>.
-template <bool REAL>
-__global__ void __launch_bounds__(STAGED_NT, 1) adjoint_sync_kernel(SweepArgs A, StagedArgs S) {
-  __shared__ int s_inst;
-  LCounts cnt;
-#pragma unroll
-  for (int k = 0; k < CNT_N; ++k) cnt.v[k] = 0;
-  const int lane = threadIdx.x & 31;
-  const int n_inst = S.n_inst;
-  int start = 0;
-  {
-    const double pos = (blockIdx.x + 0.5) / gridDim.x * S.cost_total;
-    while (start + 1 < n_inst && S.cost_prefix[start + 1] <= pos) ++start;
-  }
-  for (int visit = 0; visit < n_inst; ++visit) {
-    const int k = (start + visit) % n_inst;
-    if (threadIdx.x == 0) s_inst = (*(volatile unsigned long long*)&S.inst_next[k] < (unsigned long long)S.inst_end[k]) ? k : -1;
-    __syncthreads();
-    if (s_inst < 0) {
-      __syncthreads();
-      continue;
-    }
-    const InstDesc& in = A.inst[k];
-    const int n0 = in.n[0], n1 = in.n[1];
-    const unsigned pend = (unsigned)S.inst_end[k];
-    unsigned rbeg = 0, rend = 0;  // this warp's private particle range
-    EmitCache ec;
-    ec.g_first = 1;
-    ec.g_end = 0;  // empty: forces a lookup on the first emission
-    ec.e = -1;
-    int acc_slot = 0;  // wall slot of the pending per-lane wall sum
-    double acc = 0.0;
-    for (;;) {
-      if (rbeg == rend) {  // private range used up: take the next one of the instance
-        unsigned long long got = 0;
-        if (lane == 0) got = atomicAdd(&S.inst_next[k], (unsigned long long)S.warp_grab);
-        got = __shfl_sync(0xffffffffu, got, 0);
-        if (got >= pend) break;
-        rbeg = (unsigned)got;
-        rend = (unsigned)min(got + (unsigned long long)S.warp_grab, (unsigned long long)pend);
-      }
-      const unsigned take = min(32u, rend - rbeg);
-      if ((unsigned)lane < take) {
-        double w;
-        int band, emitter;
-        PW f;
-        Stream st;
-        uint32_t ub;
-        if (staged_emit<2, true>(A, S, rbeg + lane, false, w, band, f, st, ub, ec, in, k, emitter, false)) {
-          if (emitter < 0 && emitter != acc_slot) {
-            if (acc != 0.0) atomicAdd(&A.adj_wall[in.wall_off + (-1 - acc_slot)], acc);
-            acc = 0.0;
-            acc_slot = emitter;
-          }
-          cnt.v[CNT_FLIGHTS] += 1;
-          const float vtm = A.vtm32[(long long)k * A.nb + band];
-          const bool all_real = REAL || A.all_real[(long long)k * A.nb + band] != 0;
-          const long long bcbase = in.bc_off + (long long)band * in.ncells;
-          // the forward sweep's decisions, with the same deferrals to the FP64 replay
-          const int m0 = faces_to_wall(f.i0, f.s0, n0), m1 = faces_to_wall(f.i1, f.s1, n1);
-          const float ea = vtm * TIE_LOG_ABS;
-          float eD = fmaf(f.D, TIE_LOG_REL, ea);
-          bool wall_exit = false, deferred = false;
-          int fb0 = 0, fb1 = 0;  // faces before the latest candidate, per axis
-#pragma unroll 1
-          for (;;) {
-            const float base = fmaf(TIE_REL, f.D, eD);
-            if (f.D - f.tex > base) {
-              cnt.v[CNT_WALL_EXITS] += 1;
-              wall_exit = true;
-              break;
-            }
-            if (f.tex - f.D <= fmaf(TIE_REL, f.tex, eD)) {
-              deferred = true;
-              break;
-            }
-            bool near = false;  // a count within the bound of a face, found with it for all-real bands
-            if (all_real) {
-              fb0 = count_near(f.D, f.t0, f.d0, base, near);
-              fb1 = count_near(f.D, f.t1, f.d1, base, near);
-            } else {
-              fb0 = faces_before(f.D, f.t0, f.d0);
-              fb1 = faces_before(f.D, f.t1, f.d1);
-            }
-            const int cell = clampi(f.i0 + f.s0 * fb0, n0) + n0 * clampi(f.i1 + f.s1 * fb1, n1);
-            const int oc = candidate_outcome<2>(A, bcbase, in.ncells, f, base, fb0, fb1, 0, cell, all_real, near, ub,
-                                                n0, n1, 1, n0, 0);
-            if (oc == CAND_DEFER) {
-              deferred = true;
-              break;
-            }
-            cnt.v[CNT_CANDIDATES] += 1;
-            if (oc == CAND_REAL) {
-              cnt.v[CNT_REAL] += 1;
-              const long long gc = in.cell_off + cell;
-              const double val = w * A.lambda[gc] * A.invVm[gc];
-              if (emitter >= 0) atomicAdd(&A.adj_out[in.cell_off + emitter], val);
-              else acc += val;
-              break;
-            }
-            uint32_t uw;
-            st.next_pair(uw, ub);
-            const float ell = __fmul_rn(-__logf(word_uniform<float>(uw)), vtm);
-            f.D = __fadd_rn(f.D, ell);
-            eD = fmaf(f.D, TIE_SUM, fmaf(ell, TIE_LOG_REL, eD + ea));
-          }
-          if (deferred) {
-            defer_particle(S, rbeg + lane, 0u);
-          } else {
-            // faces crossed, for the event counters (as in the forward sweep)
-            int c0, c1;
-            if (wall_exit) {
-              c0 = f.i2 == 0 ? m0 - 1 : min(faces_before(f.tex, f.t0, f.d0), m0 - 1);
-              c1 = f.i2 == 1 ? m1 - 1 : min(faces_before(f.tex, f.t1, f.d1), m1 - 1);
-            } else {
-              c0 = min(fb0, m0 - 1);
-              c1 = min(fb1, m1 - 1);
-            }
-            cnt.v[CNT_CROSSINGS] += c0 + c1;
-          }
-        }
-      }
-      rbeg += take;
-    }
-    if (acc != 0.0) atomicAdd(&A.adj_wall[in.wall_off + (-1 - acc_slot)], acc);
     __syncthreads();
   }
   flush_lcounts(cnt, A.counters);
@@ -1798,12 +1593,12 @@ cudaError_t launch_sweep_staged(const Ctx* c, const SweepArgs& a, cudaStream_t s
     if (a.F && (e = cudaMemsetAsync(c->d_F32, 0, (size_t)c->total_faces * sizeof(float2), s)) != cudaSuccess)
       return e;
     switch (c->dim) {
-      case 1: sweep_staged_kernel<1, false, true><<<blocks, STAGED_NT, smem, s>>>(a, S); break;
+      case 1: sweep_staged_kernel<1, true><<<blocks, STAGED_NT, smem, s>>>(a, S); break;
       case 2:
         if (sync) launch_sync<true>(c, a, S, blocks, smem, s);
-        else sweep_staged_kernel<2, false, true><<<blocks, STAGED_NT, smem, s>>>(a, S);
+        else sweep_staged_kernel<2, true><<<blocks, STAGED_NT, smem, s>>>(a, S);
         break;
-      default: sweep_staged_kernel<3, false, true><<<blocks, STAGED_NT, smem, s>>>(a, S); break;
+      default: sweep_staged_kernel<3, true><<<blocks, STAGED_NT, smem, s>>>(a, S); break;
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int fb = c->sm_count * 4;
@@ -1814,12 +1609,12 @@ cudaError_t launch_sweep_staged(const Ctx* c, const SweepArgs& a, cudaStream_t s
     if ((e = launch_replay(c, a, S, s)) != cudaSuccess) return e;
   } else {
     switch (c->dim) {
-      case 1: sweep_staged_kernel<1, false, false><<<blocks, STAGED_NT, smem, s>>>(a, S); break;
+      case 1: sweep_staged_kernel<1, false><<<blocks, STAGED_NT, smem, s>>>(a, S); break;
       case 2:
         if (sync) launch_sync<false>(c, a, S, blocks, smem, s);
-        else sweep_staged_kernel<2, false, false><<<blocks, STAGED_NT, smem, s>>>(a, S);
+        else sweep_staged_kernel<2, false><<<blocks, STAGED_NT, smem, s>>>(a, S);
         break;
-      default: sweep_staged_kernel<3, false, false><<<blocks, STAGED_NT, smem, s>>>(a, S); break;
+      default: sweep_staged_kernel<3, false><<<blocks, STAGED_NT, smem, s>>>(a, S); break;
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = launch_replay(c, a, S, s)) != cudaSuccess) return e;
@@ -1874,48 +1669,9 @@ cudaError_t launch_sweep_staged(const Ctx* c, const SweepArgs& a, cudaStream_t s
   return e;
 }
 
-// Adjoint re-trace with the staged kernel over every emitter (all groups).
-cudaError_t launch_adjoint_staged(const Ctx* c, const SweepArgs& a, cudaStream_t s) {
-  StagedArgs S;
-  S.n_inst = c->n_inst;
-  S.inst_next = c->d_inst_next;
-  S.inst_end = c->d_all_end;
-  S.cost_prefix = c->d_all_cost_prefix;
-  S.cost_total = c->all_cost_total;
-  S.window = c->d_window;
-  S.wmax = reinterpret_cast<const double*>(c->d_wmax);
-  S.warp_grab = c->opt.warp_grab > 0 ? c->opt.warp_grab : 256;
-  S.walk_k = c->opt.walk_k > 0 ? c->opt.walk_k : 16;
-  S.refill = c->opt.refill_lanes;
-  S.group_mag = c->d_all_group_mag;
-  S.mag_n0 = c->d_mag;
-  S.mag_n1 = c->d_mag + c->n_inst;
-  S.mag_wall = c->d_mag + 2 * c->n_inst;
-  S.defer = c->d_defer;
-  S.defer_n = c->d_defer_n;
-  S.defer_cap = c->defer_cap;
-  S.err = c->d_err;
-  cudaError_t e = cudaMemcpyAsync(c->d_inst_next, c->d_all_beg, c->n_inst * sizeof(long long),
-                                  cudaMemcpyDeviceToDevice, s);
-  if (e != cudaSuccess) return e;
-  if ((e = cudaMemsetAsync(c->d_defer_n, 0, sizeof(unsigned), s)) != cudaSuccess) return e;
-  S.R32 = S.W32 = S.F32 = nullptr;
-  S.DY = S.EY = S.GX = nullptr;
-  S.gx_stride = 0;
-  const int blocks = c->sm_count * c->adj_blocks_per_sm;
-  if (c->dim == 2 && (c->opt.refill_lanes == 0 || c->opt.refill_lanes == 32)) {
-    // pass-synchronous re-trace (refill only when all 32 lanes are idle)
-    if (c->all_real_all) adjoint_sync_kernel<true><<<blocks, STAGED_NT, 0, s>>>(a, S);
-    else adjoint_sync_kernel<false><<<blocks, STAGED_NT, 0, s>>>(a, S);
-  } else {
-    switch (c->dim) {
-      case 1: sweep_staged_kernel<1, true, false><<<blocks, STAGED_NT, 0, s>>>(a, S); break;
-      case 2: sweep_staged_kernel<2, true, false><<<blocks, STAGED_NT, 0, s>>>(a, S); break;
-      default: sweep_staged_kernel<3, true, false><<<blocks, STAGED_NT, 0, s>>>(a, S); break;
-    }
-  }
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  return launch_adjoint_replay(c, a, s);  // the deferred particles, in FP64
+cudaError_t launch_k32_finalize(const Ctx* c, const float2* src, double* dst, long long n, cudaStream_t s) {
+  k32_finalize_kernel<<<c->sm_count * 4, 256, 0, s>>>(src, dst, n, 0);
+  return cudaGetLastError();
 }
 
 // Measured accuracy of the FP32 operations the tie bounds rely on, over every uniform the
@@ -2015,9 +1771,9 @@ double walk_bound_fraction(const double* m) {
 cudaError_t configure_staged(Ctx* c) {
   cudaError_t e = cudaSuccess;
   const size_t smem = (size_t)c->staged_cap * sizeof(unsigned);
-  const void* fwd[6] = {(const void*)sweep_staged_kernel<1, false, false>, (const void*)sweep_staged_kernel<2, false, false>,
-                        (const void*)sweep_staged_kernel<3, false, false>, (const void*)sweep_staged_kernel<1, false, true>,
-                        (const void*)sweep_staged_kernel<2, false, true>, (const void*)sweep_staged_kernel<3, false, true>};
+  const void* fwd[6] = {(const void*)sweep_staged_kernel<1, false>, (const void*)sweep_staged_kernel<2, false>,
+                        (const void*)sweep_staged_kernel<3, false>, (const void*)sweep_staged_kernel<1, true>,
+                        (const void*)sweep_staged_kernel<2, true>, (const void*)sweep_staged_kernel<3, true>};
   for (const void* f : fwd)
     if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
   const void* syn[8] = {(const void*)sweep_sync_kernel<false, false, false>, (const void*)sweep_sync_kernel<true, false, false>,
@@ -2031,10 +1787,6 @@ cudaError_t configure_staged(Ctx* c) {
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nk, fwd[c->dim + 2], STAGED_NT, smem)) != cudaSuccess) return e;
   nb = std::min(nb, nk);  // one grid size for both tally modes
   c->staged_blocks_per_sm = nb > 0 ? nb : 1;
-  void* fa = c->dim == 1 ? (void*)sweep_staged_kernel<1, true, false>
-                         : (c->dim == 2 ? (void*)sweep_staged_kernel<2, true, false> : (void*)sweep_staged_kernel<3, true, false>);
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fa, STAGED_NT, 0)) != cudaSuccess) return e;
-  c->adj_blocks_per_sm = nb > 0 ? nb : 1;
   return cudaSuccess;
 }
 
