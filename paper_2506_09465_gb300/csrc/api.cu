@@ -136,7 +136,7 @@ void free_all(Ctx* c) {
                   c->d_all_group_mag, c->d_R32, c->d_W32, c->d_F32, c->d_m2, c->d_wallTf,
                   c->d_pslot_off, c->d_phome_off, c->d_pnband, c->d_pnwall, c->d_px, c->d_pband, c->d_phome,
                   c->d_pcount, c->d_pfcount, c->d_phome_w, c->d_wemit, c->d_DY, c->d_EY, c->d_GX, c->d_Fd,
-                  c->d_all_real, c->d_defer, c->d_defer_n, c->d_land_fwd, c->d_land_all};
+                  c->d_all_real, c->d_defer, c->d_defer_n, c->d_land_fwd, c->d_land_all, c->d_items, c->d_diff};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (c->h_pinned) cudaFreeHost(c->h_pinned);
@@ -793,6 +793,13 @@ iugkp_status iugkp_create_batch(int n, const iugkp_grid* g, const double* const*
       return bail(IUGKP_ECUDA);
     }
   }
+  if (c->opt.precision == IUGKP_TRACK_FP64) {
+    // faces whose row the FP32 filter of the FP64 sweep leaves open: a few in 10^5; room for one
+    // in every eight particles (beyond that they are found on the spot)
+    c->items_cap = (unsigned)std::min<long long>(c->total_particles / 8 + 65536, 1ll << 28);
+    if ((s = dalloc(c, &c->d_items, (size_t)(c->dim > 1 ? c->items_cap : 1))) != IUGKP_OK) return bail(s);
+    if (c->dim == 1 && (s = dalloc(c, &c->d_diff, (size_t)EXACT_DIFF_COPIES * (face_off + n))) != IUGKP_OK) return bail(s);
+  }
   if (c->dim == 2) {
     if ((s = dalloc(c, &c->d_DY, cell_off)) != IUGKP_OK) return bail(s);
     if ((s = dalloc(c, &c->d_EY, (size_t)c->total_bfaces)) != IUGKP_OK) return bail(s);
@@ -907,6 +914,23 @@ bool staged_path(const Ctx* c) {
   return c->opt.tally != IUGKP_TALLY_FP64 && c->opt.precision == IUGKP_TRACK_FP32 && c->fwd_particles < (1ll << 31);
 }
 
+// Every axis short enough for FP32 cell coordinates (and, in the faces' case, 32-bit indices).
+bool land_sizes(const Ctx* c) {
+  for (const InstDesc& in : c->h_inst) {
+    if (in.nfaces >= (1ll << 32)) return false;
+    for (int a = 0; a < in.dim; ++a)
+      if (in.n[a] >= (1 << 23)) return false;
+  }
+  return true;
+}
+
+// FP64 tracking by the filtered sweep (exact.cu): the default step budget or more (the plain
+// kernel counts every crossing against it), as all queue entries and indices are 32-bit.
+bool exact_path(const Ctx* c) {
+  return c->opt.precision == IUGKP_TRACK_FP64 && c->opt.step_budget >= EXACT_MIN_BUDGET &&
+         c->fwd_particles < (1ll << 31) && land_sizes(c);
+}
+
 // Buffers of the compensated FP32 tallies; allocated outside any stream capture.
 iugkp_status ensure_k32(Ctx* c) {
   if (c->d_R32) return IUGKP_OK;
@@ -932,7 +956,8 @@ iugkp_status sweep_async(Ctx* c, const double* T, unsigned epoch, double* R, dou
   unsigned long long* cnt = counters ? counters : c->d_counters;
   CK(cudaMemsetAsync(cnt, 0, CNT_N * sizeof(unsigned long long), s), "clear counters");
   CK(cudaMemsetAsync(c->d_work_counter, 0, sizeof(unsigned long long), s), "clear work counter");
-  if (staged && wall && !F) {  // the staged sweep derives wall tallies from the face tallies
+  const bool exact = !staged && exact_path(c);
+  if ((staged || exact) && wall && !F) {  // the wall tallies follow from the face tallies
     F = c->d_F;
     CK(cudaMemsetAsync(F, 0, c->total_faces * sizeof(double), s), "clear F");
   }
@@ -949,25 +974,19 @@ iugkp_status sweep_async(Ctx* c, const double* T, unsigned epoch, double* R, dou
   a.epoch = epoch;
   if (staged)
     CK(launch_sweep_staged(c, a, s), "staged sweep launch");
+  else if (exact)
+    CK(launch_exact(c, a, s), "filtered FP64 sweep launch");
   else
     CK(launch_sweep(c, a, s), "sweep launch");
   return IUGKP_OK;
 }
 
-// Every axis short enough for the landing sweeps' FP32 cell coordinates.
-bool land_sizes(const Ctx* c) {
-  for (const InstDesc& in : c->h_inst)
-    for (int a = 0; a < in.dim; ++a)
-      if (in.n[a] >= (1 << 23)) return false;
-  return true;
-}
-
 // A sweep of which only the real collisions are read (the macro update and the correction take
 // R alone): R into c->d_R, no W, no faces, no walls, no event counts.
 iugkp_status sweep_real_async(Ctx* c, const double* T, unsigned epoch, cudaStream_t s) {
-  if (!staged_path(c) || !land_sizes(c))
+  if (!(staged_path(c) && land_sizes(c)) && !exact_path(c))
     return sweep_async(c, T, epoch, c->d_R, nullptr, nullptr, nullptr, nullptr, s);
-  if (c->opt.tally == IUGKP_TALLY_STAGED_K32) {
+  if (c->opt.tally == IUGKP_TALLY_STAGED_K32) {  // FP32 tracking only
     if (!c->d_R32) return fail(c, IUGKP_EINVAL, "compensated tally buffers missing");
   } else {
     CK(cudaMemsetAsync(c->d_R, 0, (size_t)c->nb * c->total_cells * sizeof(double), s), "clear R");
@@ -1501,8 +1520,9 @@ namespace {
 // The adjoint re-trace: the landing kernels for the FP32 walk with staged tallies (the
 // fast path), else the plain one-thread-per-particle kernel.
 cudaError_t adjoint_sweep(Ctx* c, const SweepArgs& a, cudaStream_t s) {
-  if (c->opt.tally != IUGKP_TALLY_FP64 && c->opt.precision == IUGKP_TRACK_FP32 && c->total_particles < (1ll << 31) &&
-      land_sizes(c))
+  const bool filtered = c->opt.precision == IUGKP_TRACK_FP64 ? c->opt.step_budget >= EXACT_MIN_BUDGET
+                                                             : c->opt.tally != IUGKP_TALLY_FP64;
+  if (filtered && c->total_particles < (1ll << 31) && land_sizes(c))
     return launch_land(c, a, true, s);
   return launch_adjoint(c, a, s);
 }

@@ -189,8 +189,12 @@ struct Ctx {
   unsigned* d_all_group_mag = nullptr;  // [all groups] the same for the adjoint re-trace
   // particles the staged FP32 walk left to the FP64 replay (sweep and adjoint re-trace)
   uint2* d_defer = nullptr;
-  unsigned* d_defer_n = nullptr;     // [4] queue length, unused, 64-bit claim counter of the landing sweeps
+  unsigned* d_defer_n = nullptr;     // [4] queue length, queued faces (exact.cu), 64-bit claim counter (land.cu, exact.cu)
   unsigned defer_cap = 0;
+  // filtered FP64 sweep (exact.cu; contexts with FP64 tracking): queued faces, 1D face differences
+  uint2* d_items = nullptr;
+  unsigned items_cap = 0;
+  double* d_diff = nullptr;
   // landing sweeps (land.cu): tasks of the forward groups and of every group (adjoint)
   LandGroup* d_land_fwd = nullptr;
   LandGroup* d_land_all = nullptr;
@@ -226,6 +230,8 @@ cudaError_t launch_axpy_grad(const Ctx* c, const double* at, const double* g, do
 cudaError_t launch_sweep_staged(const Ctx* c, const SweepArgs& a, cudaStream_t s);
 cudaError_t configure_staged(Ctx* c);
 cudaError_t launch_k32_finalize(const Ctx* c, const float2* src, double* dst, long long n, cudaStream_t s);
+cudaError_t launch_exact(const Ctx* c, const SweepArgs& a, cudaStream_t s);
+cudaError_t launch_face_closure(const Ctx* c, const SweepArgs& a, cudaStream_t s);
 cudaError_t launch_land(const Ctx* c, const SweepArgs& a, bool adj, cudaStream_t s);
 void land_tasks(const Ctx* c, const std::vector<Group>& groups, std::vector<LandGroup>& out, unsigned& n_tasks, int& qch);
 cudaError_t launch_replay(const Ctx* c, const SweepArgs& a, const StagedArgs& S, cudaStream_t s);

@@ -79,6 +79,12 @@ constexpr int LAND_QCH = 16;          // particles per emitter and task at most
 constexpr int LAND_WARPS_PER_SM = 40; // resident warps the task size is chosen for
 constexpr int LAND_REFILL = 8;        // idle lanes that trigger a refill (null-candidate chains)
 
+// Filtered FP64 sweep (exact.cu): copies of the 1D face differences (by block), and the
+// candidates after which a particle goes to the replay, which counts its steps against the budget.
+constexpr int EXACT_DIFF_COPIES = 16;
+constexpr int EXACT_MAX_CANDIDATES = 1 << 20;
+constexpr long long EXACT_MIN_BUDGET = 1ll << 24;  // smaller step budgets take the plain kernel
+
 // A group's tasks: tiles of tw emitters (reps particles of an emitter side by side where tw is
 // at most 16) x runs of qch * reps particles per emitter, tiles fastest; task0 is its first.
 struct LandGroup {

@@ -83,9 +83,6 @@ __device__ __forceinline__ int ceil_count(float u) {
   return __float_as_int(__fadd_ru(fmaxf(u, 0.f), 8388608.f)) - 0x4B000000;
 }
 
-// i as a float for 0 <= i < 2^23, placed in the mantissa of 2^23 (no conversion instruction).
-__device__ __forceinline__ float small_int_float(int i) { return __int_as_float(0x4B000000 | i) - 8388608.f; }
-
 // Faces normal to one axis reached before path length L: #{k >= 0 : t + k d < L}.
 __device__ __forceinline__ int faces_before(float L, float t, float d) {
   return L > t ? ceil_count(__fdividef(L - t, d)) : 0;
@@ -1361,9 +1358,11 @@ __global__ void boundary_emission_kernel(const InstDesc* inst, int dim, const in
                                          const double* wallTf, double* F) {
   const int k = blockIdx.z, wl = blockIdx.y;
   const int a = wl >> 1, side = wl & 1;
-  if (dim >= 2 && a == dim - 1 && side == 1) return;
   const InstDesc& in = inst[k];
-  if (two_group(in, window, k)) return;  // added with the group balances
+  if (window) {  // null: every face was tallied, nothing is derived
+    if (dim >= 2 && a == dim - 1 && side == 1) return;
+    if (two_group(in, window, k)) return;  // added with the group balances
+  }
   const double u = wall_unit[k * 6 + wl];
   const double* tf = wallTf + in.bface_off + in.wface_off[wl];
   const int nf = wall_faces(in, a);
@@ -1667,6 +1666,23 @@ cudaError_t launch_sweep_staged(const Ctx* c, const SweepArgs& a, cudaStream_t s
     e = cudaGetLastError();
   }
   return e;
+}
+
+// What follows a sweep that tallied every face (exact.cu): W scaled, the walls' emission added to
+// their faces, the walls' absorbed power.
+cudaError_t launch_face_closure(const Ctx* c, const SweepArgs& a, cudaStream_t s) {
+  cudaError_t e = cudaSuccess;
+  if (a.W) {
+    scale_by_taumaj_kernel<<<c->sm_count * 4, 256, 0, s>>>(c->d_inst, c->n_inst, c->nb, c->d_taumaj, c->d_all_real,
+                                                          a.R, a.W, (long long)c->nb * c->total_cells);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  if (!a.F) return e;
+  boundary_emission_kernel<<<dim3(8, 2 * c->dim, c->n_inst), 256, 0, s>>>(c->d_inst, c->dim, nullptr, c->d_wall_unit,
+                                                                         c->d_wallTf, a.F);
+  if ((e = cudaGetLastError()) != cudaSuccess || !a.wall) return e;
+  wall_absorbed_kernel<<<dim3(2 * c->dim, c->n_inst), 256, 0, s>>>(c->d_inst, c->d_wall_unit, c->d_wallTf, a.F, a.wall);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_k32_finalize(const Ctx* c, const float2* src, double* dst, long long n, cudaStream_t s) {

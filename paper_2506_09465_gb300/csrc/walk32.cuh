@@ -10,6 +10,9 @@
 
 namespace iugkp {
 
+// i as a float for 0 <= i < 2^23, placed in the mantissa of 2^23 (no conversion instruction).
+__device__ __forceinline__ float small_int_float(int i) { return __int_as_float(0x4B000000 | i) - 8388608.f; }
+
 // ---- FP32 decisions checked against the FP64 walk ----
 // The FP32 walk and the FP64 walk follow each particle with the same draws, so their path
 // lengths differ by rounding only, and a decision taken in FP32 is the FP64 walk's unless the

@@ -57,9 +57,10 @@ def test_steady_loop_sweep_equals_the_full_sweep(shape, particles, tally):
 def test_adjoint_retrace_equals_the_plain_fp64_one(shape):
     ins = instances(shape)
     out = []
-    for opt in ({}, {"precision": 0, "tally": 0}):
+    for opt in ({}, {"precision": 0, "tally": 0}, {"precision": 0, "tally": 0, "step_budget": (1 << 24) - 1}):
         s = gpu_solver(ins, C2, V2, 300, 300, seed=9, newton=0, **opt)
         g = torch.as_tensor(np.random.default_rng(2).uniform(0.0, 1.0, s.total_cells), device="cuda")
         out.append(s.adjoint(g, 1e-9, 50000))  # no correction: thousands of iterations where cells are thick
-    for a, b in zip(*out):
-        assert float((a - b).abs().max()) <= 1e-11 * float(b.abs().max())
+    for got in out[:2]:  # FP32 and FP64 tracking; budgets below 2^24 take the plain kernel
+        for a, b in zip(got, out[2]):
+            assert float((a - b).abs().max()) <= 1e-11 * float(b.abs().max())
