@@ -135,7 +135,7 @@ void free_all(Ctx* c) {
                   c->d_group_mag, c->d_mag, c->d_wall_unit,
                   c->d_all_group_mag, c->d_R32, c->d_W32, c->d_F32, c->d_m2, c->d_wallTf,
                   c->d_pslot_off, c->d_phome_off, c->d_pnband, c->d_pnwall, c->d_px, c->d_pband, c->d_phome,
-                  c->d_pcount, c->d_pfcount, c->d_phome_w, c->d_wemit, c->d_DY, c->d_EY, c->d_GX, c->d_Fd,
+                  c->d_pcount, c->d_pfcount, c->d_phome_w, c->d_wemit, c->d_DY, c->d_EY, c->d_GX, c->d_Fx, c->d_Fi, c->d_ticket, c->d_wpart,
                   c->d_all_real, c->d_defer, c->d_defer_n, c->d_land_fwd, c->d_land_all, c->d_items, c->d_diff};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -294,11 +294,11 @@ iugkp_status rebuild_forward_groups(Ctx* c) {
   iugkp_status s = upload(c, &c->d_groups_fwd, c->h_groups_fwd);
   if (s != IUGKP_OK) return s;
   {
-    // w_max pre-pass: each group's blocks in proportion to its emitters, about two blocks per
+    // w_max pre-pass: each group's blocks in proportion to its emitters, about eight blocks per
     // SM in all, at least WMAX_MIN_CHUNK emitters per block
     long long total = 0;
     for (const Group& g : c->h_groups_fwd) total += g.n_emitters;
-    const long long nblk = 2 * (long long)std::max(1, c->sm_count);
+    const long long nblk = 8 * (long long)std::max(1, c->sm_count);
     const long long chunk = std::max<long long>(WMAX_MIN_CHUNK, (total + nblk - 1) / nblk);
     std::vector<int> bpre(1, 0);
     for (const Group& g : c->h_groups_fwd) bpre.push_back(bpre.back() + (int)((g.n_emitters + chunk - 1) / chunk));
@@ -306,6 +306,9 @@ iugkp_status rebuild_forward_groups(Ctx* c) {
     if (c->d_wmax_bpre) cudaFree(c->d_wmax_bpre);
     c->d_wmax_bpre = nullptr;
     if ((s = upload(c, &c->d_wmax_bpre, bpre)) != IUGKP_OK) return s;
+    if (c->d_wpart) cudaFree(c->d_wpart);
+    c->d_wpart = nullptr;
+    if ((s = dalloc(c, &c->d_wpart, (size_t)c->wmax_blocks)) != IUGKP_OK) return s;
   }
   // Staged sweep: each instance's forward particles are contiguous (groups are ordered
   // by instance); blocks start on instances in proportion to the estimated cost.
@@ -800,11 +803,20 @@ iugkp_status iugkp_create_batch(int n, const iugkp_grid* g, const double* const*
     if ((s = dalloc(c, &c->d_items, (size_t)(c->dim > 1 ? c->items_cap : 1))) != IUGKP_OK) return bail(s);
     if (c->dim == 1 && (s = dalloc(c, &c->d_diff, (size_t)EXACT_DIFF_COPIES * (face_off + n))) != IUGKP_OK) return bail(s);
   }
+  if (c->dim <= 2 && c->opt.precision == IUGKP_TRACK_FP32) {
+    if ((s = dalloc(c, &c->d_Fx, face_off)) != IUGKP_OK) return bail(s);
+    if ((s = dalloc(c, &c->d_Fi, face_off)) != IUGKP_OK) return bail(s);
+  }
+  if ((s = dalloc(c, &c->d_ticket, 1 + (size_t)n)) != IUGKP_OK) return bail(s);
+  if (cudaMemset(c->d_ticket, 0, (1 + (size_t)n) * sizeof(unsigned)) != cudaSuccess) {
+    cudaGetLastError();
+    fail(c, IUGKP_ECUDA, "clear of the block counters");
+    return bail(IUGKP_ECUDA);
+  }
   if (c->dim == 2) {
     if ((s = dalloc(c, &c->d_DY, cell_off)) != IUGKP_OK) return bail(s);
     if ((s = dalloc(c, &c->d_EY, (size_t)c->total_bfaces)) != IUGKP_OK) return bail(s);
     if ((s = dalloc(c, &c->d_GX, (size_t)GX_COPIES * c->total_bfaces)) != IUGKP_OK) return bail(s);
-    if ((s = dalloc(c, &c->d_Fd, face_off)) != IUGKP_OK) return bail(s);
   }
   if ((s = dalloc(c, &c->d_wall, c->total_walls)) != IUGKP_OK) return bail(s);
   if ((s = dalloc(c, &c->d_red, 1024)) != IUGKP_OK) return bail(s);
@@ -943,23 +955,19 @@ iugkp_status ensure_k32(Ctx* c) {
 
 iugkp_status sweep_async(Ctx* c, const double* T, unsigned epoch, double* R, double* W, double* F, double* wall,
                          unsigned long long* counters, cudaStream_t s) {
-  const size_t bc = (size_t)c->nb * c->total_cells;
-  const bool staged = staged_path(c);
-  const bool k32 = staged && c->opt.tally == IUGKP_TALLY_STAGED_K32;
-  if (k32 && !c->d_R32) return fail(c, IUGKP_EINVAL, "compensated tally buffers missing");
-  if (!k32) {  // the compensated mode writes R and W whole after the sweep
+  const bool staged = staged_path(c), exact = !staged && exact_path(c);
+  if (staged && c->opt.tally == IUGKP_TALLY_STAGED_K32 && !c->d_R32)
+    return fail(c, IUGKP_EINVAL, "compensated tally buffers missing");
+  unsigned long long* cnt = counters ? counters : c->d_counters;
+  if (staged || exact) {  // their first pass clears what they tally in
+    if (wall && !F) F = c->d_F;  // the wall tallies follow from the face tallies
+  } else {
+    const size_t bc = (size_t)c->nb * c->total_cells;
     CK(cudaMemsetAsync(R, 0, bc * sizeof(double), s), "clear R");
     if (W) CK(cudaMemsetAsync(W, 0, bc * sizeof(double), s), "clear W");
-  }
-  if (F) CK(cudaMemsetAsync(F, 0, c->total_faces * sizeof(double), s), "clear F");
-  if (wall) CK(cudaMemsetAsync(wall, 0, c->total_walls * sizeof(double), s), "clear wall");
-  unsigned long long* cnt = counters ? counters : c->d_counters;
-  CK(cudaMemsetAsync(cnt, 0, CNT_N * sizeof(unsigned long long), s), "clear counters");
-  CK(cudaMemsetAsync(c->d_work_counter, 0, sizeof(unsigned long long), s), "clear work counter");
-  const bool exact = !staged && exact_path(c);
-  if ((staged || exact) && wall && !F) {  // the wall tallies follow from the face tallies
-    F = c->d_F;
-    CK(cudaMemsetAsync(F, 0, c->total_faces * sizeof(double), s), "clear F");
+    if (F) CK(cudaMemsetAsync(F, 0, c->total_faces * sizeof(double), s), "clear F");
+    if (wall) CK(cudaMemsetAsync(wall, 0, c->total_walls * sizeof(double), s), "clear wall");
+    CK(cudaMemsetAsync(cnt, 0, CNT_N * sizeof(unsigned long long), s), "clear counters");
   }
   SweepArgs a = base_args(c);
   a.groups = c->d_groups_fwd;
@@ -988,8 +996,6 @@ iugkp_status sweep_real_async(Ctx* c, const double* T, unsigned epoch, cudaStrea
     return sweep_async(c, T, epoch, c->d_R, nullptr, nullptr, nullptr, nullptr, s);
   if (c->opt.tally == IUGKP_TALLY_STAGED_K32) {  // FP32 tracking only
     if (!c->d_R32) return fail(c, IUGKP_EINVAL, "compensated tally buffers missing");
-  } else {
-    CK(cudaMemsetAsync(c->d_R, 0, (size_t)c->nb * c->total_cells * sizeof(double), s), "clear R");
   }
   SweepArgs a = base_args(c);
   a.groups = c->d_groups_fwd;
@@ -1288,7 +1294,7 @@ iugkp_status iugkp_check_fp32_walk(double* out6) {
 namespace {
 
 // One IUGKP iteration cur -> nxt without host round trips: sweep, macro update, Newton
-// correction (CG status checked on the device), residual sums into res_dev[0..1]. The update
+// correction (CG status checked on the device), residual sums into res_dev[0..1] (if given). The update
 // reads R alone, so the sweep tallies nothing else but, on request, the faces (into c->d_F).
 iugkp_status iteration_async(Ctx* c, const double* cur, double* nxt, unsigned epoch, bool want_F, double* res_dev,
                              cudaStream_t s) {
@@ -1300,7 +1306,7 @@ iugkp_status iteration_async(Ctx* c, const double* cur, double* nxt, unsigned ep
     CK(launch_newton(c, cur, nxt, c->d_R, s), "newton");
     CK(launch_pcg_check(c, s), "pcg check");
   }
-  CK(launch_residual(c, cur, nxt, 0.0, res_dev, s), "residual");
+  if (res_dev) CK(launch_residual(c, cur, nxt, 0.0, res_dev, s), "residual");
   return IUGKP_OK;
 }
 
@@ -1502,7 +1508,7 @@ iugkp_status iugkp_average(iugkp_ctx* ctx, double* T_inout_dev, int n_steps, uns
   double* nxt = c->d_T2;
   for (int k = 0; k < n_steps; ++k) {
     // the solve's update with fresh draws: epoch_first + k
-    iugkp_status st = iteration_async(c, cur, nxt, epoch_first + (unsigned)k, F_mean_dev != nullptr, c->d_scalar + 4, s);
+    iugkp_status st = iteration_async(c, cur, nxt, epoch_first + (unsigned)k, F_mean_dev != nullptr, nullptr, s);
     if (st != IUGKP_OK) return st;
     CK(launch_welford(c, nxt, T_mean_dev, m2, c->total_cells, k + 1, s), "welford");
     if (F_mean_dev) CK(launch_welford(c, c->d_F, F_mean_dev, nullptr, c->total_faces, k + 1, s), "flux mean");
@@ -1517,13 +1523,16 @@ iugkp_status iugkp_average(iugkp_ctx* ctx, double* T_inout_dev, int n_steps, uns
 
 namespace {
 
-// The adjoint re-trace: the landing kernels for the FP32 walk with staged tallies (the
+// The adjoint re-trace into a.adj_out and a.adj_wall (cleared here): the landing kernels for the FP32 walk with staged tallies (the
 // fast path), else the plain one-thread-per-particle kernel.
 cudaError_t adjoint_sweep(Ctx* c, const SweepArgs& a, cudaStream_t s) {
   const bool filtered = c->opt.precision == IUGKP_TRACK_FP64 ? c->opt.step_budget >= EXACT_MIN_BUDGET
                                                              : c->opt.tally != IUGKP_TALLY_FP64;
   if (filtered && c->total_particles < (1ll << 31) && land_sizes(c))
     return launch_land(c, a, true, s);
+  cudaError_t e = cudaMemsetAsync(a.adj_out, 0, c->total_cells * sizeof(double), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(a.adj_wall, 0, c->total_walls * sizeof(double), s);
+  if (e != cudaSuccess) return e;
   return launch_adjoint(c, a, s);
 }
 
@@ -1548,12 +1557,9 @@ iugkp_status iugkp_adjoint(iugkp_ctx* ctx, const double* T_star_dev, const doubl
   double* lam = lambda_dev ? lambda_dev : half + nc;
   double* nxt = half + 2 * nc;
   CK(cudaMemsetAsync(lam, 0, nc * sizeof(double), s), "clear lambda");
-  // |g| max as the residual floor.
-  std::vector<double> hg(nc);
-  CK(cudaMemcpyAsync(hg.data(), g_dev, nc * sizeof(double), cudaMemcpyDeviceToHost, s), "g readback");
-  CK(cudaStreamSynchronize(s), "g sync");
+  // max |g| as the residual floor, read back with the first residual
+  CK(launch_absmax(c, g_dev, (long long)nc, c->d_scalar + 2, s), "largest g");
   double gmax = 0.0;
-  for (double x : hg) gmax = std::max(gmax, std::fabs(x));
   SweepArgs a = base_args(c);
   a.groups = c->d_groups_all;
   a.n_groups = (int)c->h_groups_all.size();
@@ -1566,25 +1572,29 @@ iugkp_status iugkp_adjoint(iugkp_ctx* ctx, const double* T_star_dev, const doubl
   int it = 0;
   while (it < max_iter) {
     a.lambda = lam;
-    CK(cudaMemsetAsync(at, 0, nc * sizeof(double), s), "clear");
-    CK(cudaMemsetAsync(grad_wall_dev, 0, c->total_walls * sizeof(double), s), "clear");
     CK(adjoint_sweep(c, a, s), "adjoint sweep");
     CK(launch_axpy_grad(c, at, g_dev, half, s), "adjoint axpy");
     if (c->opt.newton) {
       CK(launch_adjoint_correction(c, lam, half, nxt, s), "adjoint correction");
-      if ((st = pcg_status(c, s, nullptr)) != IUGKP_OK) return st;
     } else {
       CK(cudaMemcpyAsync(nxt, half, nc * sizeof(double), cudaMemcpyDeviceToDevice, s), "copy");
     }
-    if ((st = residual(c, lam, nxt, gmax, s, &res)) != IUGKP_OK) return st;
+    // one synchronisation per iteration: the residual sums, max |g| and the solver's status
+    CK(launch_residual(c, lam, nxt, 0.0, c->d_scalar, s), "residual");
+    CK(cudaMemcpyAsync(c->h_pinned, c->d_scalar, 3 * sizeof(double), cudaMemcpyDeviceToHost, s), "residual readback");
+    if (c->opt.newton) {
+      if ((st = pcg_status(c, s, nullptr)) != IUGKP_OK) return st;
+    } else {
+      CK(cudaStreamSynchronize(s), "residual sync");
+    }
+    gmax = c->h_pinned[2];
+    res = residual_from_sums(c, c->h_pinned, gmax);
     CK(cudaMemcpyAsync(lam, nxt, nc * sizeof(double), cudaMemcpyDeviceToDevice, s), "copy lambda");
     ++it;
     if (res <= tol) break;
   }
   // Gradients at the converged lambda: dJ/dQ = (A^T lambda) / m, dJ/dT_w = B_w^T lambda.
   a.lambda = lam;
-  CK(cudaMemsetAsync(at, 0, nc * sizeof(double), s), "clear");
-  CK(cudaMemsetAsync(grad_wall_dev, 0, c->total_walls * sizeof(double), s), "clear");
   CK(adjoint_sweep(c, a, s), "adjoint sweep");
   CK(launch_grad_source(c, at, grad_source_dev, s), "grad source");
   if ((st = check_device(c, s)) != IUGKP_OK) return st;

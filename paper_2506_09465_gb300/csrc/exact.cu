@@ -404,38 +404,6 @@ __global__ void __launch_bounds__(64) exact_replay_kernel(SweepArgs A, StagedArg
   }
 }
 
-// 1D faces from the differences: F[f] += the sum of the differences up to f, over the copies.
-// One block per instance; chunks of 1024 faces, prefix sums in a fixed order.
-__global__ void __launch_bounds__(1024) face_runs_kernel(const InstDesc* inst, const double* diff, long long stride,
-                                                         double* F) {
-  __shared__ double wsum[32];
-  const InstDesc& in = inst[blockIdx.x];
-  const double* d = diff + in.face_off + blockIdx.x;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double carry = 0.0;
-  for (int f0 = 0; f0 < (int)in.nfaces; f0 += 1024) {
-    const int f = f0 + threadIdx.x;
-    double v = 0.0;
-    if (f < (int)in.nfaces)
-      for (int c = 0; c < EXACT_DIFF_COPIES; ++c) v += d[c * stride + f];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const double t = __shfl_up_sync(0xffffffffu, v, o);
-      if (lane >= o) v += t;
-    }
-    if (lane == 31) wsum[warp] = v;
-    __syncthreads();
-    double before = carry, all = carry;
-    for (int w = 0; w < 32; ++w) {
-      if (w == warp) before = all;
-      all += wsum[w];
-    }
-    if (f < (int)in.nfaces) F[in.face_off + f] += before + v;
-    carry = all;
-    __syncthreads();
-  }
-}
-
 template <int DIM>
 cudaError_t launch_dim(const Ctx* c, const SweepArgs& a, const StagedArgs& S, const LandArgs& L, const ExactArgs& X,
                        cudaStream_t s) {
@@ -474,22 +442,28 @@ cudaError_t launch_exact(const Ctx* c, const SweepArgs& a, cudaStream_t s) {
   X.cap = c->items_cap;
   X.diff = c->d_diff;
   X.diff_stride = c->total_faces + c->n_inst;
-  cudaError_t e = cudaMemsetAsync(c->d_defer_n, 0, 4 * sizeof(unsigned), s);
+  PrologueArgs P = {};
+  auto clear = [&](void* p, size_t n) {
+    if (!p || !n) return;
+    P.clear[P.n_clear] = reinterpret_cast<unsigned long long*>(p);
+    P.words[P.n_clear++] = (long long)n;
+  };
+  clear(a.R, (size_t)c->nb * c->total_cells);
+  if (!c->all_real_all) clear(a.W, (size_t)c->nb * c->total_cells);  // else W = tau_maj R afterwards
+  clear(a.F, (size_t)c->total_faces);
+  clear(a.counters, CNT_N);
+  clear(c->d_defer_n, 2);
+  if (c->dim == 1 && a.F) clear(c->d_diff, (size_t)EXACT_DIFF_COPIES * X.diff_stride);
+  cudaError_t e = launch_prologue(c, a, P, s);
   if (e != cudaSuccess) return e;
-  if (c->dim == 1 && a.F &&
-      (e = cudaMemsetAsync(c->d_diff, 0, (size_t)EXACT_DIFF_COPIES * X.diff_stride * sizeof(double), s)) != cudaSuccess)
-    return e;
   switch (c->dim) {
     case 1: e = launch_dim<1>(c, a, S, L, X, s); break;
     case 2: e = launch_dim<2>(c, a, S, L, X, s); break;
     default: e = launch_dim<3>(c, a, S, L, X, s); break;
   }
   if (e != cudaSuccess) return e;
-  if (c->dim == 1 && a.F) {
-    face_runs_kernel<<<c->n_inst, 1024, 0, s>>>(c->d_inst, c->d_diff, X.diff_stride, a.F);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
-  return launch_face_closure(c, a, s);
+  // W scaled, the walls' emission added to their faces, the walls' absorbed power
+  return launch_close_tallied(c, a, c->dim == 1 && a.F ? c->d_diff : nullptr, X.diff_stride, s);
 }
 
 }  // namespace iugkp

@@ -108,7 +108,10 @@ struct Ctx {
   double* d_DY = nullptr;        // [cells]
   double* d_EY = nullptr;        // [total_bfaces]
   double* d_GX = nullptr;        // [GX_COPIES * total_bfaces]
-  double* d_Fd = nullptr;        // [total_faces] faces derived from the group balances
+  double* d_Fx = nullptr;        // [total_faces] 1D and 2D staged sweep: FP64 face sums (replayed particles)
+  long long* d_Fi = nullptr;     // [total_faces] ... and fixed-point face sums in units of q
+  unsigned* d_ticket = nullptr;  // [1 + n_inst] finished blocks of the passes around a trace (0 between launches)
+  unsigned long long* d_wpart = nullptr;  // [wmax_blocks] largest weight of each block of the pass before it
   bool any_two_group = false;    // some instance of the context uses the two-group tallies
   bool all_two_group = false;    // ... every instance does (no face follows from a column walk)
   bool sync_ok = false;          // 2D: the pass-synchronous staged kernel applies
@@ -226,12 +229,18 @@ cudaError_t launch_adjoint_correction(const Ctx* c, const double* lam, const dou
 cudaError_t launch_residual(const Ctx* c, const double* T0, const double* T1, double dT_ref, double* out_dev,
                             cudaStream_t s);
 cudaError_t launch_pcg_check(const Ctx* c, cudaStream_t s);
+cudaError_t launch_absmax(const Ctx* c, const double* x, long long n, double* out, cudaStream_t s);
 cudaError_t launch_axpy_grad(const Ctx* c, const double* at, const double* g, double* lam_half, cudaStream_t s);
 cudaError_t launch_sweep_staged(const Ctx* c, const SweepArgs& a, cudaStream_t s);
 cudaError_t configure_staged(Ctx* c);
 cudaError_t launch_k32_finalize(const Ctx* c, const float2* src, double* dst, long long n, cudaStream_t s);
 cudaError_t launch_exact(const Ctx* c, const SweepArgs& a, cudaStream_t s);
-cudaError_t launch_face_closure(const Ctx* c, const SweepArgs& a, cudaStream_t s);
+cudaError_t launch_prologue(const Ctx* c, const SweepArgs& a, const PrologueArgs& P, cudaStream_t s);
+cudaError_t launch_close_tallied(const Ctx* c, const SweepArgs& a, const double* diff, long long diff_stride,
+                                 cudaStream_t s);
+cudaError_t launch_close_1d(const Ctx* c, const SweepArgs& a, cudaStream_t s);
+cudaError_t launch_close_2d(const Ctx* c, const SweepArgs& a, cudaStream_t s);
+cudaError_t launch_close_3d(const Ctx* c, const SweepArgs& a, cudaStream_t s);
 cudaError_t launch_land(const Ctx* c, const SweepArgs& a, bool adj, cudaStream_t s);
 void land_tasks(const Ctx* c, const std::vector<Group>& groups, std::vector<LandGroup>& out, unsigned& n_tasks, int& qch);
 cudaError_t launch_replay(const Ctx* c, const SweepArgs& a, const StagedArgs& S, cudaStream_t s);

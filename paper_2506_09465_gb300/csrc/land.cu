@@ -303,9 +303,23 @@ cudaError_t launch_land(const Ctx* c, const SweepArgs& a, bool adj, cudaStream_t
   L.qch = adj ? c->land_all_qch : c->land_fwd_qch;
   L.next = reinterpret_cast<unsigned long long*>(c->d_defer_n + 2);
   L.lamVm = c->d_work;
-  cudaError_t e = cudaMemsetAsync(c->d_defer_n, 0, 4 * sizeof(unsigned), s);  // queue length and task counter
-  if (e != cudaSuccess) return e;
   const size_t bc = (size_t)c->nb * c->total_cells;
+  PrologueArgs P = {};
+  auto clear = [&](void* p, size_t n) {
+    P.clear[P.n_clear] = reinterpret_cast<unsigned long long*>(p);
+    P.words[P.n_clear++] = (long long)n;
+  };
+  clear(c->d_defer_n, 2);  // queue length and claim counter
+  if (adj) {
+    clear(a.adj_out, (size_t)c->total_cells);
+    clear(a.adj_wall, (size_t)c->total_walls);
+  } else if (k32) {
+    clear(c->d_R32, bc);
+  } else {
+    clear(a.R, bc);
+  }
+  cudaError_t e = launch_prologue(c, a, P, s);
+  if (e != cudaSuccess) return e;
   if (adj) {
     // lambda / (V m), gathered by every particle: into the correction solve's scratch, free
     // until the correction that follows on the same stream
@@ -321,7 +335,6 @@ cudaError_t launch_land(const Ctx* c, const SweepArgs& a, bool adj, cudaStream_t
     return launch_adjoint_replay(c, a, s);
   }
   if (k32) {
-    if ((e = cudaMemsetAsync(c->d_R32, 0, bc * sizeof(float2), s)) != cudaSuccess) return e;
     switch (c->dim) {
       case 1: e = launch_dim<1, false, true>(c, a, S, L, s); break;
       case 2: e = launch_dim<2, false, true>(c, a, S, L, s); break;

@@ -211,6 +211,21 @@ __global__ void __launch_bounds__(256) residual_stage2(const double* partial, do
   }
 }
 
+// Largest |x| (NaN left out) as the bit pattern of a non-negative double, max-reduced into *out.
+__global__ void __launch_bounds__(256) absmax_kernel(long long total, const double* x, unsigned long long* out) {
+  unsigned long long m = 0;
+  for (long long i = blockIdx.x * 256ll + threadIdx.x; i < total; i += (long long)gridDim.x * 256) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x[i]) & 0x7fffffffffffffffull;
+    if (b <= 0x7ff0000000000000ull && b > m) m = b;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long t = __shfl_down_sync(0xffffffffu, m, o);
+    m = t > m ? t : m;
+  }
+  if ((threadIdx.x & 31) == 0 && m) atomicMax(out, m);
+}
+
 static unsigned grid_for(const Ctx* c, long long n) {
   long long b = (n + 255) / 256;
   long long cap = (long long)c->sm_count * 8;
@@ -295,6 +310,13 @@ cudaError_t launch_welford(const Ctx* c, const double* x, double* mean, double* 
 
 cudaError_t launch_scale(const Ctx* c, double* x, long long n, double a, cudaStream_t s) {
   scale_kernel<<<grid_for(c, n), 256, 0, s>>>(n, x, a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_absmax(const Ctx* c, const double* x, long long n, double* out, cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(out, 0, sizeof(double), s);
+  if (e != cudaSuccess) return e;
+  absmax_kernel<<<grid_for(c, n), 256, 0, s>>>(n, x, reinterpret_cast<unsigned long long*>(out));
   return cudaGetLastError();
 }
 

@@ -16,9 +16,9 @@ constexpr int COOP3_BYTES = (STAGED_NT / 32) * COOP3_INT4_PER_WARP * 16;
 
 // Shared-memory x-face window: one 32-bit word per face holding the low word of a 64-bit
 // fixed-point sum in units of w_max 2^-26 (a contribution is below 2^26 units); words start
-// at 2^31, and a wrap of the word adds +-2^32 units (= 64 w_max) to the FP64 face at once.
+// at 2^31, and a wrap of the word adds +-2^32 units to the
+// face's 64-bit sum at once.
 constexpr double WIN_SCALE = 0x1p26;
-constexpr double WIN_CARRY = 0x1p6;             // 2^32 units in multiples of w_max
 constexpr unsigned WIN_BIAS = 0x80000000u;
 
 // Copies of the two-group exit tally GX (one per block, by block index modulo the count),
@@ -58,6 +58,7 @@ struct StagedArgs {
   double* GX;                     // [GX_COPIES][total_bfaces] exits of the x-group through the low
                                   // y-wall and of the y-group through the low x-wall (signed flux)
   long long gx_stride;            // total_bfaces: entries per copy of GX
+  long long* Fi;                  // [total_faces] fixed-point face sums in units of the instance's q
   // Particles whose FP32 walk lies within rounding of a decision of the FP64 walk are left
   // untallied and replayed by the FP64 walk after the sweep (replay_kernel): entry
   // {forward index, (candidates already tallied << 1) | y-group}.
@@ -71,6 +72,38 @@ struct StagedArgs {
     return GX + (long long)(blockIdx.x % (unsigned)GX_COPIES) * gx_stride;
   }
 #endif
+};
+
+// The pass before a trace (closing.cu).
+struct PrologueArgs {
+  int n_clear;
+  unsigned long long* clear[12];  // buffers to clear and their sizes in 8-byte words
+  long long words[12];
+  int n_inst;
+  unsigned long long* next;       // [n_inst] claim counters <- next_from, or null
+  const long long* next_from;
+  int wmax_blocks;                // blocks of the emitter weights (0: none)
+  const int* bpre;                // [groups + 1] first block of each group
+  unsigned long long* wpart;      // [wmax_blocks]
+  unsigned long long* wmax;       // [n_inst]
+  unsigned* ticket;               // 0 between launches
+};
+
+// The pass after a 2D staged trace (closing.cu).
+struct Close2D {
+  const int2* window;
+  const double* wmax;
+  const long long* Fi;
+  const double* Fx;
+  const double* bal;              // [cells] balances, or null (one band: formed on the spot)
+  const double* Vm;
+  const double* wall_unit;
+  const double* DY;
+  const double* EY;
+  const double* GX;
+  long long gx_stride;
+  unsigned* ticket;               // [n_inst], 0 between launches
+  int line_blocks;
 };
 
 // Landing sweeps (land.cu).

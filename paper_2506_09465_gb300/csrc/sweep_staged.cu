@@ -152,6 +152,11 @@ __device__ __forceinline__ bool all_reject(const float* ratio, int ncells, int c
 
 enum { CAND_NULL = 0, CAND_REAL = 1, CAND_DEFER = 2 };
 
+// Adds n units of q to the fixed-point sum of a face.
+__device__ __forceinline__ void add_units(long long* Fi, long long face, long long n) {
+  atomicAdd(reinterpret_cast<unsigned long long*>(&Fi[face]), (unsigned long long)n);
+}
+
 // Outcome of the candidate at path length f.D, whose face counts fb and cell the caller took
 // in FP32 (the first wall lies beyond it by more than the bound, so it is a candidate for the
 // FP64 walk too): CAND_NULL or CAND_REAL when the FP64 walk decides the same, CAND_DEFER
@@ -183,52 +188,6 @@ __device__ __forceinline__ int candidate_outcome(const SweepArgs& A, long long b
 }
 
 }  // namespace
-
-// The largest |weight| of each forward group's emitters, max-reduced into its instance's slot
-// (non-negative doubles order like their bit patterns). Group g has blocks [bpre[g],
-// bpre[g + 1]) of the grid, in proportion to its emitters (about two blocks per SM in all), so
-// the FP64 weight arithmetic is spread over the SMs in proportion to the work.
-__global__ void group_wmax_kernel(SweepArgs A, const int* bpre, unsigned long long* wmax_bits) {
-  __shared__ double sh[32];
-  int gi = 0;
-  {
-    int hi = A.n_groups - 1;  // the last group whose first block is at or before this one
-    while (gi < hi) {
-      const int mid = (gi + hi + 1) >> 1;
-      if (bpre[mid] <= (int)blockIdx.x) gi = mid;
-      else hi = mid - 1;
-    }
-  }
-  const Group G = A.groups[gi];
-  const int by = (int)blockIdx.x - bpre[gi], ny = bpre[gi + 1] - bpre[gi];
-  const InstDesc& in = A.inst[G.inst];
-  double m = 0.0;
-  if (G.kind == 0) {
-    const long long base = in.bc_off + (long long)G.band * in.ncells;
-    for (int e = by * blockDim.x + threadIdx.x; e < in.ncells; e += ny * blockDim.x) {
-      double Te = A.T[in.cell_off + e];
-      if (A.srcshift) Te += A.srcshift[in.cell_off + e];
-      const double w = A.coef[base + e] * Te;
-      A.wemit[base + e] = w;  // the weight of every particle of this emitter
-      m = fmax(m, fabs(w));
-    }
-  } else {
-    const int wl = G.kind - 1;
-    const double wc = A.wcoef[((long long)G.inst * A.nb + G.band) * 6 + wl];
-    const double* tf = A.wallTf + in.bface_off + in.wface_off[wl];
-    for (int j = by * blockDim.x + threadIdx.x; j < G.n_emitters; j += ny * blockDim.x)
-      m = fmax(m, fabs(wc * tf[j]));
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double r = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) r = fmax(r, sh[w]);
-    atomicMax(&wmax_bits[G.inst], (unsigned long long)__double_as_longlong(r));
-  }
-}
 
 // Emits particle pid (global forward index) into lane state. Returns false for a
 // zero-weight particle (nothing to trace).
@@ -421,30 +380,6 @@ __device__ __forceinline__ bool staged_emit(const SweepArgs& A, const StagedArgs
 // private ranges of the instance's particles and refill idle lanes together. Faces normal
 // to x go to a shared-memory copy of the instance's x-faces (when it fits), in units of
 // the instance's q; the block flushes it when it leaves the instance.
-// Instance holding entry j of a [band][cell] array: the last one whose bc_off is at or before j.
-__device__ __forceinline__ int bc_instance(const InstDesc* inst, int n_inst, long long j) {
-  int lo = 0, hi = n_inst - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (inst[mid].bc_off <= j) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
-}
-
-// The candidate estimator W = sum of w tau_maj over candidates (Sec. 3.2): the staged sweep
-// sums w per (band, cell) and multiplies by the instance's tau_maj of the band here; in a band
-// with tau = tau_maj in every cell every candidate is real, so there W = tau_maj R (the sweep
-// leaves W alone).
-__global__ void scale_by_taumaj_kernel(const InstDesc* inst, int n_inst, int nb, const double* taumaj,
-                                       const int* all_real, const double* R, double* W, long long total) {
-  for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < total; j += (long long)gridDim.x * blockDim.x) {
-    const int k = bc_instance(inst, n_inst, j);
-    const long long kb = (long long)k * nb + (j - inst[k].bc_off) / inst[k].ncells;
-    W[j] = (all_real[kb] ? R[j] : W[j]) * taumaj[kb];
-  }
-}
-
 // FP64 value of compensated tallies: dst = hi + lo (add = 0) or dst += hi + lo (add = 1).
 __global__ void k32_finalize_kernel(const float2* src, double* dst, long long n, int add) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -499,8 +434,7 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
     const bool two = DIM == 2 && useF && wbase == 0 && (long long)wlen == in.nfaces;
     for (unsigned i = threadIdx.x; i < wlen; i += STAGED_NT) win[i] = WIN_BIAS;
     __syncthreads();
-    const double wmax = S.wmax[k];
-    const double qinv = wmax > 0.0 ? WIN_SCALE / wmax : 0.0;
+    const double qinv = S.wmax[k] > 0.0 ? WIN_SCALE / S.wmax[k] : 0.0;
     const unsigned pend = (unsigned)S.inst_end[k];
     unsigned rbeg = 0, rend = 0;  // this warp's private particle range
     double w = 0.0;
@@ -691,9 +625,7 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
                 // exit through the low y-wall: the one face normal to y this group tallies
                 if (ex == 1 && f.s1 < 0) {
                   const int col = f.i0 + f.s0 * c0;
-                  if (two) atomicAdd(&S.gx()[in.bface_off + in.wface_off[2] + col], -w);
-                  else if (K32) tally_k32(&S.F32[face_off + fax1 + col], -w);
-                  else atomicAdd(&A.F[face_off + fax1 + col], -w);
+                  atomicAdd(&S.gx()[in.bface_off + in.wface_off[2] + col], -w);
                 }
                 kend = c0 + (ex == 0 ? 1 : 0);
                 const bool flat = !(f.d1 < INFINITY);
@@ -726,9 +658,7 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
               // faces normal to the last axis: only the low boundary is tallied (the rest
               // follow from conservation)
               if (DIM == 2 && ex == 1 && f.s1 < 0) {
-                const long long fi = face_off + fax1 + (f.i0 + f.s0 * c0);
-                if (K32) tally_k32(&S.F32[fi], -w);
-                else atomicAdd(&A.F[fi], -w);
+                atomicAdd(&S.gx()[in.bface_off + in.wface_off[2] + (f.i0 + f.s0 * c0)], -w);
               } else if (DIM == 3 && ex == 2 && f.s2 < 0) {
                 const long long fi = face_off + fax2 + (f.i0 + f.s0 * c0) + (long long)n0 * (f.i1 + f.s1 * c1);
                 if (K32) tally_k32(&S.F32[fi], -w);
@@ -847,7 +777,7 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
               // |q| <= 2^26, so the word can wrap only from within 2^26 of 0 / 2^32
               if (old + 0x04000000u < 0x08000000u) {
                 const int carry = ((int)q >> 31) + (old + q < old ? 1 : 0);
-                if (carry) atomicAdd(&A.F[face_off + face], (double)carry * S.wmax[k] * WIN_CARRY);
+                if (carry) add_units(S.Fi, face_off + face, (long long)carry << 32);
               }
             }
           }
@@ -916,7 +846,7 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
           const unsigned old = atomicAdd(&win[rel], qwx);
           if (old + 0x04000000u < 0x08000000u) {  // a wrap starts within 2^26 of 0 / 2^32
             const int carry = ((int)qwx >> 31) + (old + qwx < old ? 1 : 0);
-            if (carry) atomicAdd(&A.F[face_off + xface], (double)carry * S.wmax[k] * WIN_CARRY);
+            if (carry) add_units(S.Fi, face_off + xface, (long long)carry << 32);
           }
         };
         if (DIM == 2 && (two || wfull)) {
@@ -965,13 +895,9 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
       }
     }
     __syncthreads();
-    if (wlen) {
-      const double qs = wmax / WIN_SCALE;
-      double* Fx = A.F + face_off + wbase;  // x-faces come first
-      for (unsigned i = threadIdx.x; i < wlen; i += STAGED_NT) {
-        const int v = (int)(win[i] - WIN_BIAS);
-        if (v) atomicAdd(&Fx[i], (double)v * qs);
-      }
+    for (unsigned i = threadIdx.x; i < wlen; i += STAGED_NT) {  // x-faces come first
+      const int v = (int)(win[i] - WIN_BIAS);
+      if (v) add_units(S.Fi, face_off + wbase + i, v);
     }
     __syncthreads();
   }
@@ -1139,14 +1065,8 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_sync_kernel(SweepArgs A, S
             const float dp = yg ? f.d1 : f.d0, dq = yg ? f.d0 : f.d1;
             const int cp = yg ? c1 : c0, mq = yg ? m0 : m1, axp = yg ? 1 : 0;
             if (ex == 1 - axp && (yg ? f.s0 : f.s1) < 0) {  // exit through the low q-wall
-              if (two) {
-                const int j = yg ? in.wface_off[0] + f.i1 + f.s1 * c1 : in.wface_off[2] + f.i0 + f.s0 * c0;
-                atomicAdd(&S.gx()[in.bface_off + j], -w);
-              } else {
-                const int col = f.i0 + f.s0 * c0;
-                if (K32) tally_k32(&S.F32[face_off + fax1 + col], -w);
-                else atomicAdd(&A.F[face_off + fax1 + col], -w);
-              }
+              const int j = yg ? in.wface_off[0] + f.i1 + f.s1 * c1 : in.wface_off[2] + f.i0 + f.s0 * c0;
+              atomicAdd(&S.gx()[in.bface_off + j], -w);
             }
             nitem = cp + (ex == axp ? 1 : 0);
             const bool flat = !(dq < INFINITY);
@@ -1211,16 +1131,14 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_sync_kernel(SweepArgs A, S
             const unsigned q = (unsigned)pb.z;
             const unsigned rel = (unsigned)(face - wbase);
             if (PARTIAL && rel >= wlen) {  // outside the window: the same contribution, globally
-              const double val = (double)(int)q * (S.wmax[k] / WIN_SCALE);
-              if (K32) tally_k32(&S.F32[face_off + face], val);
-              else atomicAdd(&A.F[face_off + face], val);
+              add_units(S.Fi, face_off + face, (long long)(int)q);
               continue;
             }
             const unsigned old = atomicAdd(&win[rel], q);
             // |q| <= 2^26, so the word can wrap only from within 2^26 of 0 / 2^32
             if (old + 0x04000000u < 0x08000000u) {
               const int carry = ((int)q >> 31) + (old + q < old ? 1 : 0);
-              if (carry) atomicAdd(&A.F[face_off + face], (double)carry * S.wmax[k] * WIN_CARRY);
+              if (carry) add_units(S.Fi, face_off + face, (long long)carry << 32);
             }
           }
         }
@@ -1228,304 +1146,13 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_sync_kernel(SweepArgs A, S
       }
     }
     __syncthreads();
-    {
-      const double qs = S.wmax[k] / WIN_SCALE;
-      double* Fx = A.F + face_off + wbase;
-      for (unsigned i = threadIdx.x; i < wlen; i += STAGED_NT) {
-        const int v = (int)(win[i] - WIN_BIAS);
-        if (v) atomicAdd(&Fx[i], (double)v * qs);
-      }
+    for (unsigned i = threadIdx.x; i < wlen; i += STAGED_NT) {
+      const int v = (int)(win[i] - WIN_BIAS);
+      if (v) add_units(S.Fi, face_off + wbase + i, v);
     }
     __syncthreads();
   }
   flush_lcounts(cnt, A.counters);
-}
-
-// Absorbed minus emitted power of every cell, sum_b R_b - V m T_emit (T_emit = T + Q/m), in
-// one pass over the [band][cell] tallies (coalesced; the column walk below then reads one
-// value per cell instead of one per band).
-__global__ void cell_balance_kernel(const InstDesc* inst, int n_inst, int nb, long long total, const double* T,
-                                    const double* srcshift, const double* Vm, const double* R, double* out) {
-  for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < total; g += (long long)gridDim.x * blockDim.x) {
-    int k = 0;
-    while (k + 1 < n_inst && inst[k + 1].cell_off <= g) ++k;
-    const InstDesc& in = inst[k];
-    const long long c = g - in.cell_off;
-    double r = 0.0;
-    for (int b = 0; b < nb; ++b) r += R[in.bc_off + (long long)b * in.ncells + c];
-    double te = T[g];
-    if (srcshift) te += srcshift[g];
-    out[g] = r - Vm[g] * te;
-  }
-}
-
-// Faces normal to the last axis from per-cell conservation, one thread per column:
-// F[k+1] = F[k] + (net inflow through the other axes' faces of cell k) - (R_k - S_k),
-// S_k = V m T_emit (emitted thermal and source power; bal = R - S from cell_balance_kernel),
-// starting from the tallied low boundary face.
-template <int DIM>
-__device__ __forceinline__ double column_step(const InstDesc& in, const double* bal, const double* Fi, long long c) {
-  const int n0 = in.n[0], n1 = in.n[1];
-  const long long row = c / n0;  // x-face index of the cell's low face = c + row
-  double inflow = Fi[in.fax_off[0] + c + row] - Fi[in.fax_off[0] + c + row + 1];
-  if (DIM == 3) {
-    const int cz = (int)(c / ((long long)n0 * n1));
-    const long long fy = in.fax_off[1] + c + (long long)n0 * cz;
-    inflow += Fi[fy] - Fi[fy + n0];
-  }
-  return inflow - bal[in.cell_off + c];
-}
-
-// Block: 32 adjacent columns x DERIVE_SEG segments (one warp per segment, so loads are
-// coalesced across columns). Each thread sums its segment's increments, the segments'
-// offsets follow from a prefix over the block's shared sums, then each thread writes its
-// segment's running values.
-constexpr int DERIVE_SEG = 8;
-
-// A 2D instance whose faces all sit in the staged window uses the two-group tallies.
-__device__ __forceinline__ bool two_group(const InstDesc& in, const int2* window, int k) {
-  return in.dim == 2 && window[k].x == 0 && (long long)window[k].y == in.nfaces;
-}
-
-template <int DIM>
-__global__ void __launch_bounds__(32 * DERIVE_SEG) derive_last_axis_kernel(const InstDesc* inst, int n_inst,
-                                                                         const int2* window, const double* bal,
-                                                                         double* F) {
-  __shared__ double segsum[DERIVE_SEG][32];
-  const int k = blockIdx.y;
-  if (k >= n_inst) return;
-  const InstDesc& in = inst[k];
-  if (two_group(in, window, k)) return;
-  const int n0 = in.n[0], n1 = in.n[1], n2 = in.n[2];
-  const int nlast = DIM == 2 ? n1 : n2;
-  const int ncol = in.ncells / nlast;
-  double* Fi = F + in.face_off;
-  const int lane = threadIdx.x & 31, seg = threadIdx.x >> 5;
-  const int seglen = (nlast + DERIVE_SEG - 1) / DERIVE_SEG;
-  const int k0 = seg * seglen, k1 = min(nlast, k0 + seglen);
-  for (int cbase = blockIdx.x * 32; cbase < ncol; cbase += gridDim.x * 32) {
-    const int col = cbase + lane;
-    const bool ok = col < ncol;
-    const int ix = ok ? col % n0 : 0, iy = (ok && DIM == 3) ? col / n0 : 0;
-    const long long stride = DIM == 2 ? n0 : (long long)n0 * n1;
-    const long long base_cell = DIM == 2 ? ix : ix + (long long)n0 * iy;
-    double part = 0.0;
-    if (ok)
-      for (int kk = k0; kk < k1; ++kk) part += column_step<DIM>(in, bal, Fi, base_cell + kk * stride);
-    segsum[seg][lane] = part;
-    __syncthreads();
-    if (ok) {
-      // low boundary face of this column, then the segments below this one
-      const long long f0 = DIM == 2 ? in.fax_off[1] + ix : in.fax_off[2] + ix + (long long)n0 * iy;
-      double acc = Fi[f0];
-      for (int sg = 0; sg < seg; ++sg) acc += segsum[sg][lane];
-      for (int kk = k0; kk < k1; ++kk) {
-        const long long c = base_cell + kk * stride;
-        acc += column_step<DIM>(in, bal, Fi, c);
-        const long long fn = DIM == 2 ? in.fax_off[1] + c + n0 : in.fax_off[2] + c + (long long)n0 * n1;
-        Fi[fn] = acc;
-      }
-    }
-    __syncthreads();
-  }
-  (void)n2;
-}
-
-// Faces of wall w = 2a + side of an instance, enumerated as j1 + n(o1) j2 (o1 = (a+1)%3,
-// o2 = (a+2)%3); returns the face index within the instance.
-__device__ __forceinline__ long long wall_face(const InstDesc& in, int a, int side, int j) {
-  const int n0 = in.n[0], n1 = in.n[1], n2 = in.n[2];
-  if (a == 0) {
-    const int j1 = j % n1, j2 = j / n1;
-    return in.fax_off[0] + (side ? n0 : 0) + (long long)(n0 + 1) * (j1 + (long long)n1 * j2);
-  }
-  if (a == 1) {
-    const int j1 = j % n2, j2 = j / n2;
-    return in.fax_off[1] + j2 + (long long)n0 * ((side ? n1 : 0) + (long long)(n1 + 1) * j1);
-  }
-  const int j1 = j % n0, j2 = j / n0;
-  return in.fax_off[2] + j1 + (long long)n0 * (j2 + (long long)n1 * (side ? n2 : 0));
-}
-
-__device__ __forceinline__ int wall_faces(const InstDesc& in, int a) {
-  return in.n[(a + 1) % 3] * in.n[(a + 2) % 3];
-}
-
-// Power entering through every boundary face from its wall's emission (N_w particles of
-// weight C_b v_b A T_w / (4 N_w) per face and band), except on the high side of the
-// derived axis (that axis is rebuilt from conservation). Grid: (faces, walls, instances).
-__global__ void boundary_emission_kernel(const InstDesc* inst, int dim, const int2* window, const double* wall_unit,
-                                         const double* wallTf, double* F) {
-  const int k = blockIdx.z, wl = blockIdx.y;
-  const int a = wl >> 1, side = wl & 1;
-  const InstDesc& in = inst[k];
-  if (window) {  // null: every face was tallied, nothing is derived
-    if (dim >= 2 && a == dim - 1 && side == 1) return;
-    if (two_group(in, window, k)) return;  // added with the group balances
-  }
-  const double u = wall_unit[k * 6 + wl];
-  const double* tf = wallTf + in.bface_off + in.wface_off[wl];
-  const int nf = wall_faces(in, a);
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < nf; j += gridDim.x * blockDim.x) {
-    const double e = u * tf[j];
-    if (e != 0.0) F[in.face_off + wall_face(in, a, side, j)] += side ? -e : e;
-  }
-}
-
-// Two-group instances (2D): the faces each group did not tally follow from that group's
-// power balance in every cell. x-group, column i, faces normal to y from the bottom up:
-//   G[j+1] = G[j] + (X[i,j] - X[i+1,j]) - ((R - S)_c - D_y,c),
-// starting from the x-group's net flux through the bottom face (its exits there plus its
-// share of the wall's emission, the whole emission minus the y-group's); X are the x-group's
-// tallied faces plus its share of the emission on the x-walls. y-group, row j, faces
-// normal to x from the left:
-//   H[i+1] = H[i] + (Y[i,j] - Y[i,j+1]) - D_y,c,
-// starting from its exits through the left wall and its emission there; Y are its tallied
-// faces plus its emission on the y-walls. One warp per line, prefix sums over chunks of 32
-// cells in a fixed order; results go to Fd (F is only read).
-__global__ void __launch_bounds__(256) derive_two_group_kernel(const InstDesc* inst, int nb, const int2* window,
-                                                               const double* T, const double* srcshift,
-                                                               const double* Vm, const double* R,
-                                                               const double* wall_unit, const double* wallTf,
-                                                               const double* DY, const double* EY, const double* GX,
-                                                               long long gx_stride, const double* F, double* Fd) {
-  const int k = blockIdx.y;
-  const InstDesc& in = inst[k];
-  if (!two_group(in, window, k)) return;
-  const int n0 = in.n[0], n1 = in.n[1];
-  const int line = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (line >= n0 + n1) return;
-  const double* Fi = F + in.face_off;
-  double* Fo = Fd + in.face_off;
-  const long long fax1 = in.fax_off[1];
-  const double* ey = EY + in.bface_off;
-  // the exit tally of boundary face j, summed over the copies of GX
-  auto gx = [&](long long j) {
-    double t = 0.0;
-    for (int r = 0; r < GX_COPIES; ++r) t += GX[r * gx_stride + in.bface_off + j];
-    return t;
-  };
-  const double* tf = wallTf + in.bface_off;
-  const double* dy = DY + in.cell_off;
-  // signed flux of the whole emission of wall wl through its face j
-  auto etot = [&](int wl, int j) {
-    const double e = wall_unit[k * 6 + wl] * tf[in.wface_off[wl] + j];
-    return (wl & 1) ? -e : e;
-  };
-  if (line < n0) {
-    const int i = line;
-    double acc = gx(in.wface_off[2] + i) + etot(2, i) - ey[in.wface_off[2] + i];
-    if (lane == 0) Fo[fax1 + i] = acc;
-    for (int j0 = 0; j0 < n1; j0 += 32) {
-      const int j = j0 + lane;
-      double v = 0.0;
-      if (j < n1) {
-        const long long c = i + (long long)n0 * j;
-        const long long fl = c + j;  // x-face (i, j)
-        double left = Fi[fl], right = Fi[fl + 1];
-        if (i == 0) left += etot(0, j) - ey[in.wface_off[0] + j];
-        if (i == n0 - 1) right += etot(1, j) - ey[in.wface_off[1] + j];
-        double rr = 0.0;
-        for (int b = 0; b < nb; ++b) rr += R[in.bc_off + (long long)b * in.ncells + c];
-        double te = T[in.cell_off + c];
-        if (srcshift) te += srcshift[in.cell_off + c];
-        v = (left - right) - (rr - Vm[in.cell_off + c] * te - dy[c]);
-      }
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const double t = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += t;
-      }
-      if (j < n1) Fo[fax1 + i + (long long)n0 * (j + 1)] = acc + v;
-      acc += __shfl_sync(0xffffffffu, v, 31);
-    }
-  } else {
-    const int j = line - n0;
-    double acc = gx(in.wface_off[0] + j) + ey[in.wface_off[0] + j];
-    if (lane == 0) Fo[(long long)(n0 + 1) * j] = acc;
-    for (int ib = 0; ib < n0; ib += 32) {
-      const int i = ib + lane;
-      double v = 0.0;
-      if (i < n0) {
-        const long long c = i + (long long)n0 * j;
-        double bot = Fi[fax1 + c], top = Fi[fax1 + c + n0];
-        if (j == 0) bot += ey[in.wface_off[2] + i];
-        if (j == n1 - 1) top += ey[in.wface_off[3] + i];
-        v = (bot - top) - dy[c];
-      }
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const double t = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += t;
-      }
-      if (i < n0) Fo[(long long)(n0 + 1) * j + i + 1] = acc + v;
-      acc += __shfl_sync(0xffffffffu, v, 31);
-    }
-  }
-}
-
-// Two-group instances: every face = its tallied group's sum + the other group's derived
-// flux + the tallied group's share of the wall emission on boundary faces.
-__global__ void assemble_two_group_kernel(const InstDesc* inst, const int2* window, const double* wall_unit,
-                                          const double* wallTf, const double* EY, const double* Fd, double* F) {
-  const int k = blockIdx.y;
-  const InstDesc& in = inst[k];
-  if (!two_group(in, window, k)) return;
-  const int n0 = in.n[0], n1 = in.n[1];
-  const long long X = in.fax_off[1];
-  const double* ey = EY + in.bface_off;
-  const double* tf = wallTf + in.bface_off;
-  for (long long f = blockIdx.x * (long long)blockDim.x + threadIdx.x; f < in.nfaces;
-       f += (long long)gridDim.x * blockDim.x) {
-    double add = Fd[in.face_off + f];
-    if (f < X) {
-      const int i = (int)(f % (n0 + 1)), j = (int)(f / (n0 + 1));
-      if (i == 0) add += wall_unit[k * 6 + 0] * tf[in.wface_off[0] + j] - ey[in.wface_off[0] + j];
-      if (i == n0) add += -wall_unit[k * 6 + 1] * tf[in.wface_off[1] + j] - ey[in.wface_off[1] + j];
-    } else {
-      const long long g = f - X;
-      const int i = (int)(g % n0), jf = (int)(g / n0);
-      if (jf == 0) add += ey[in.wface_off[2] + i];
-      if (jf == n1) add += ey[in.wface_off[3] + i];
-    }
-    F[in.face_off + f] += add;
-  }
-}
-
-// Absorbed power of each wall = its emission + the outward net flux through its faces.
-// One block per (wall, instance); fixed-order reduction.
-__global__ void __launch_bounds__(256) wall_absorbed_kernel(const InstDesc* inst, const double* wall_unit,
-                                                            const double* wallTf, const double* F, double* wall) {
-  __shared__ double sh[8], shT[8];
-  const int k = blockIdx.y, wl = blockIdx.x;
-  const int a = wl >> 1, side = wl & 1;
-  const InstDesc& in = inst[k];
-  const int nf = wall_faces(in, a);
-  const double* tf = wallTf + in.bface_off + in.wface_off[wl];
-  double sum = 0.0, tsum = 0.0;
-  for (int j = threadIdx.x; j < nf; j += 256) {
-    sum += F[in.face_off + wall_face(in, a, side, j)];
-    tsum += tf[j];
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    sum += __shfl_down_sync(0xffffffffu, sum, o);
-    tsum += __shfl_down_sync(0xffffffffu, tsum, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    sh[threadIdx.x >> 5] = sum;
-    shT[threadIdx.x >> 5] = tsum;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0, ts = 0.0;
-    for (int w = 0; w < 8; ++w) {
-      t += sh[w];
-      ts += shT[w];
-    }
-    const double emitted = wall_unit[k * 6 + wl] * ts;  // sum over faces of their emission
-    wall[in.wall_off + wl] = emitted + (side ? t : -t);
-  }
 }
 
 template <bool K32>
@@ -1539,8 +1166,13 @@ void launch_sync(const Ctx* c, const SweepArgs& a, const StagedArgs& S, int bloc
   }
 }
 
-cudaError_t launch_sweep_staged(const Ctx* c, const SweepArgs& a, cudaStream_t s) {
-  StagedArgs S;
+cudaError_t launch_sweep_staged(const Ctx* c, const SweepArgs& a_in, cudaStream_t s) {
+  // 1D and 2D: the trace's fixed-point face sums go to Fi, the FP64 ones to Fx, and the closing
+  // pass writes every face of the caller's F from them; 3D tallies in the caller's F directly
+  SweepArgs a = a_in;
+  const bool fixed = a_in.F && c->dim <= 2;
+  if (fixed) a.F = c->d_Fx;
+  StagedArgs S = {};
   S.n_inst = c->n_inst;
   S.inst_next = c->d_inst_next;
   S.inst_end = c->d_inst_end;
@@ -1559,38 +1191,57 @@ cudaError_t launch_sweep_staged(const Ctx* c, const SweepArgs& a, cudaStream_t s
   S.defer_n = c->d_defer_n;
   S.defer_cap = c->defer_cap;
   S.err = c->d_err;
-  cudaError_t e = cudaMemcpyAsync(c->d_inst_next, c->d_inst_beg, c->n_inst * sizeof(long long),
-                                  cudaMemcpyDeviceToDevice, s);
-  if (e != cudaSuccess) return e;
-  if ((e = cudaMemsetAsync(c->d_wmax, 0, c->n_inst * sizeof(double), s)) != cudaSuccess) return e;
-  if ((e = cudaMemsetAsync(c->d_defer_n, 0, sizeof(unsigned), s)) != cudaSuccess) return e;
-  group_wmax_kernel<<<c->wmax_blocks, 256, 0, s>>>(a, c->d_wmax_bpre, c->d_wmax);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  const size_t smem = (size_t)c->staged_cap * sizeof(unsigned);
-  const int blocks = c->sm_count * c->staged_blocks_per_sm;
-  const bool two = a.F && c->dim == 2 && c->any_two_group;
   S.DY = c->d_DY;
   S.EY = c->d_EY;
   S.GX = c->d_GX;
   S.gx_stride = c->total_bfaces;
-  if (two) {
-    if ((e = cudaMemsetAsync(c->d_DY, 0, (size_t)c->total_cells * sizeof(double), s)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(c->d_EY, 0, (size_t)c->total_bfaces * sizeof(double), s)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(c->d_GX, 0, (size_t)GX_COPIES * c->total_bfaces * sizeof(double), s)) != cudaSuccess) return e;
-  }
+  S.Fi = c->d_Fi;
   const bool k32 = c->opt.tally == IUGKP_TALLY_STAGED_K32;
-  // pass-synchronous schedule: refill only when all 32 lanes are idle (the default where it
-  // applies)
-  const bool sync = c->sync_ok && a.F && (c->opt.refill_lanes == 0 || c->opt.refill_lanes == 32);
+  const size_t bc = (size_t)c->nb * c->total_cells;
   S.R32 = k32 ? c->d_R32 : nullptr;
   S.W32 = k32 && a.W ? c->d_W32 : nullptr;
   S.F32 = k32 && a.F ? c->d_F32 : nullptr;
+  PrologueArgs P = {};
+  auto clear = [&](void* p, size_t n) {
+    if (!p || !n) return;
+    P.clear[P.n_clear] = reinterpret_cast<unsigned long long*>(p);
+    P.words[P.n_clear++] = (long long)n;
+  };
   if (k32) {
-    const size_t bc = (size_t)c->nb * c->total_cells;
-    if ((e = cudaMemsetAsync(c->d_R32, 0, bc * sizeof(float2), s)) != cudaSuccess) return e;
-    if (a.W && (e = cudaMemsetAsync(c->d_W32, 0, bc * sizeof(float2), s)) != cudaSuccess) return e;
-    if (a.F && (e = cudaMemsetAsync(c->d_F32, 0, (size_t)c->total_faces * sizeof(float2), s)) != cudaSuccess)
-      return e;
+    clear(S.R32, bc);
+    clear(S.W32, bc);
+    clear(S.F32, (size_t)c->total_faces);
+  } else {
+    clear(a.R, bc);
+    if (!c->all_real_all) clear(a.W, bc);  // else W = tau_maj R afterwards
+  }
+  if (a.F) clear(a.F, (size_t)c->total_faces);
+  if (fixed) clear(c->d_Fi, (size_t)c->total_faces);
+  if (a.F && c->dim == 2) {
+    clear(c->d_GX, (size_t)GX_COPIES * c->total_bfaces);
+    if (c->any_two_group) {
+      clear(c->d_DY, (size_t)c->total_cells);
+      clear(c->d_EY, (size_t)c->total_bfaces);
+    }
+  }
+  clear(a.counters, CNT_N);
+  clear(c->d_defer_n, 2);
+  P.n_inst = c->n_inst;
+  P.next = c->d_inst_next;
+  P.next_from = c->d_inst_beg;
+  P.wmax_blocks = c->wmax_blocks;
+  P.bpre = c->d_wmax_bpre;
+  P.wpart = c->d_wpart;
+  P.wmax = c->d_wmax;
+  P.ticket = c->d_ticket;
+  cudaError_t e = launch_prologue(c, a, P, s);
+  if (e != cudaSuccess) return e;
+  const size_t smem = (size_t)c->staged_cap * sizeof(unsigned);
+  const int blocks = c->sm_count * c->staged_blocks_per_sm;
+  // pass-synchronous schedule: refill only when all 32 lanes are idle (the default where it
+  // applies)
+  const bool sync = c->sync_ok && a.F && (c->opt.refill_lanes == 0 || c->opt.refill_lanes == 32);
+  if (k32) {
     switch (c->dim) {
       case 1: sweep_staged_kernel<1, true><<<blocks, STAGED_NT, smem, s>>>(a, S); break;
       case 2:
@@ -1603,9 +1254,8 @@ cudaError_t launch_sweep_staged(const Ctx* c, const SweepArgs& a, cudaStream_t s
     const int fb = c->sm_count * 4;
     k32_finalize_kernel<<<fb, 256, 0, s>>>(c->d_R32, a.R, (long long)bc, 0);
     if (a.W) k32_finalize_kernel<<<fb, 256, 0, s>>>(c->d_W32, a.W, (long long)bc, 0);
-    if (a.F) k32_finalize_kernel<<<fb, 256, 0, s>>>(c->d_F32, a.F, c->total_faces, 1);
+    if (a.F && (c->dim == 3 || !sync)) k32_finalize_kernel<<<fb, 256, 0, s>>>(c->d_F32, a.F, c->total_faces, 1);
     // the deferred particles add to the FP64 outputs (after the finalize, which overwrites R and W)
-    if ((e = launch_replay(c, a, S, s)) != cudaSuccess) return e;
   } else {
     switch (c->dim) {
       case 1: sweep_staged_kernel<1, false><<<blocks, STAGED_NT, smem, s>>>(a, S); break;
@@ -1615,74 +1265,12 @@ cudaError_t launch_sweep_staged(const Ctx* c, const SweepArgs& a, cudaStream_t s
         break;
       default: sweep_staged_kernel<3, false><<<blocks, STAGED_NT, smem, s>>>(a, S); break;
     }
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = launch_replay(c, a, S, s)) != cudaSuccess) return e;
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if (a.W) {
-    scale_by_taumaj_kernel<<<c->sm_count * 4, 256, 0, s>>>(c->d_inst, c->n_inst, c->nb, c->d_taumaj, c->d_all_real,
-                                                          a.R, a.W, (long long)c->nb * c->total_cells);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
-  if (a.F) {
-    boundary_emission_kernel<<<dim3(8, 2 * c->dim, c->n_inst), 256, 0, s>>>(c->d_inst, c->dim, c->d_window,
-                                                                           c->d_wall_unit, c->d_wallTf, a.F);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
-  if (a.F && c->dim >= 2 && !c->all_two_group) {
-    // one block per 32 columns of the largest instance (columns of the last axis)
-    long long maxcol = 0;
-    for (const InstDesc& in : c->h_inst) maxcol = std::max<long long>(maxcol, in.ncells / (c->dim == 2 ? in.n[1] : in.n[2]));
-    dim3 grid((unsigned)std::min<long long>((maxcol + 31) / 32, 4096), (unsigned)c->n_inst);
-    // absorbed minus emitted power per cell, into the correction solve's scratch (free until
-    // the Newton step, which runs after the sweep on the same stream)
-    cell_balance_kernel<<<c->sm_count * 4, 256, 0, s>>>(c->d_inst, c->n_inst, c->nb, c->total_cells, a.T, a.srcshift,
-                                                        c->d_Vm, a.R, c->d_work);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if (c->dim == 2)
-      derive_last_axis_kernel<2><<<grid, 32 * DERIVE_SEG, 0, s>>>(c->d_inst, c->n_inst, c->d_window, c->d_work, a.F);
-    else
-      derive_last_axis_kernel<3><<<grid, 32 * DERIVE_SEG, 0, s>>>(c->d_inst, c->n_inst, c->d_window, c->d_work, a.F);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  if (two) {
-    long long lines = 0, faces = 0;
-    for (const InstDesc& in : c->h_inst) {
-      lines = std::max<long long>(lines, in.n[0] + in.n[1]);
-      faces = std::max<long long>(faces, in.nfaces);
-    }
-    derive_two_group_kernel<<<dim3((unsigned)((lines + 7) / 8), (unsigned)c->n_inst), 256, 0, s>>>(
-        c->d_inst, c->nb, c->d_window, a.T, a.srcshift, c->d_Vm, a.R, c->d_wall_unit, c->d_wallTf, c->d_DY, c->d_EY,
-        c->d_GX, c->total_bfaces, a.F, c->d_Fd);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    assemble_two_group_kernel<<<dim3((unsigned)std::min<long long>((faces + 255) / 256, 1024), (unsigned)c->n_inst), 256,
-                                0, s>>>(c->d_inst, c->d_window, c->d_wall_unit, c->d_wallTf, c->d_EY, c->d_Fd, a.F);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
-  if (a.F && a.wall) {
-    wall_absorbed_kernel<<<dim3(2 * c->dim, c->n_inst), 256, 0, s>>>(c->d_inst, c->d_wall_unit, c->d_wallTf, a.F,
-                                                                    a.wall);
-    e = cudaGetLastError();
-  }
-  return e;
-}
-
-// What follows a sweep that tallied every face (exact.cu): W scaled, the walls' emission added to
-// their faces, the walls' absorbed power.
-cudaError_t launch_face_closure(const Ctx* c, const SweepArgs& a, cudaStream_t s) {
-  cudaError_t e = cudaSuccess;
-  if (a.W) {
-    scale_by_taumaj_kernel<<<c->sm_count * 4, 256, 0, s>>>(c->d_inst, c->n_inst, c->nb, c->d_taumaj, c->d_all_real,
-                                                          a.R, a.W, (long long)c->nb * c->total_cells);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
-  if (!a.F) return e;
-  boundary_emission_kernel<<<dim3(8, 2 * c->dim, c->n_inst), 256, 0, s>>>(c->d_inst, c->dim, nullptr, c->d_wall_unit,
-                                                                         c->d_wallTf, a.F);
-  if ((e = cudaGetLastError()) != cudaSuccess || !a.wall) return e;
-  wall_absorbed_kernel<<<dim3(2 * c->dim, c->n_inst), 256, 0, s>>>(c->d_inst, c->d_wall_unit, c->d_wallTf, a.F, a.wall);
-  return cudaGetLastError();
+  if ((e = launch_replay(c, a, S, s)) != cudaSuccess) return e;
+  if (c->dim == 3) return launch_close_3d(c, a_in, s);
+  if (c->dim == 2) return launch_close_2d(c, a_in, s);
+  return launch_close_1d(c, a_in, s);
 }
 
 cudaError_t launch_k32_finalize(const Ctx* c, const float2* src, double* dst, long long n, cudaStream_t s) {

@@ -113,15 +113,19 @@ class Solver:
     def zeros(self, n, dtype=torch.float64):
         return torch.zeros(n, dtype=dtype, device=self.device)
 
+    def empty(self, n, dtype=torch.float64):
+        """An output that a call writes whole."""
+        return torch.empty(n, dtype=dtype, device=self.device)
+
     # -- calls -------------------------------------------------------------------
     def sweep(self, T: torch.Tensor, epoch: int = 0, want_W=True, want_F=True, want_wall=True, stream=None):
         """One sweep from the cell temperatures T (device FP64). Returns dict of R, W, F, wall,
         counters (flights, candidates, real, crossings, wall exits, dropped)."""
-        R = self.zeros(self.nb * self.total_cells)
-        W = self.zeros(self.nb * self.total_cells) if want_W else None
-        F = self.zeros(self.total_faces) if want_F else None
-        wall = self.zeros(self.total_walls) if want_wall else None
-        cnt = torch.zeros(6, dtype=torch.int64, device=self.device)
+        R = self.empty(self.nb * self.total_cells)
+        W = self.empty(self.nb * self.total_cells) if want_W else None
+        F = self.empty(self.total_faces) if want_F else None
+        wall = self.empty(self.total_walls) if want_wall else None
+        cnt = torch.empty(6, dtype=torch.int64, device=self.device)
         st = self.lib.iugkp_sweep(self.ctx, _dptr(T), epoch, _dptr(R), _dptr(W), _dptr(F), _dptr(wall), _dptr(cnt),
                                   _stream_ptr(stream))
         L.check(st, self.ctx)
@@ -133,8 +137,8 @@ class Solver:
         L.check(st, self.ctx)
 
     def macro(self, R, W=None, stream=None):
-        T_half = self.zeros(self.total_cells)
-        T_E = self.zeros(self.total_cells) if W is not None else None
+        T_half = self.empty(self.total_cells)
+        T_E = self.empty(self.total_cells) if W is not None else None
         L.check(self.lib.iugkp_macro(self.ctx, _dptr(R), _dptr(W), _dptr(T_half), _dptr(T_E), _stream_ptr(stream)),
                 self.ctx)
         return T_half, T_E
@@ -156,9 +160,9 @@ class Solver:
         return T, it.value, res.value
 
     def adjoint(self, g, tol=1e-10, max_iter=500, stream=None):
-        gs = self.zeros(self.total_cells)
-        gw = self.zeros(self.total_walls)
-        lam = self.zeros(self.total_cells)
+        gs = self.empty(self.total_cells)
+        gw = self.empty(self.total_walls)
+        lam = self.empty(self.total_cells)
         L.check(self.lib.iugkp_adjoint(self.ctx, None, _dptr(g), tol, max_iter, _dptr(gs), _dptr(gw), _dptr(lam),
                                        _stream_ptr(stream)), self.ctx)
         return gs, gw, lam
@@ -166,9 +170,9 @@ class Solver:
     def average(self, T, n_steps, epoch_first, want_var=True, want_F=False, stream=None):
         """Statistical averaging after convergence (iugkp_average): n_steps fresh-draw
         iterations from T (updated in place to the last iterate); returns (mean, var, F_mean)."""
-        mean = self.zeros(self.total_cells)
-        var = self.zeros(self.total_cells) if want_var else None
-        Fm = self.zeros(self.total_faces) if want_F else None
+        mean = self.empty(self.total_cells)
+        var = self.empty(self.total_cells) if want_var else None
+        Fm = self.empty(self.total_faces) if want_F else None
         L.check(self.lib.iugkp_average(self.ctx, _dptr(T), int(n_steps), int(epoch_first), _dptr(mean), _dptr(var),
                                        _dptr(Fm), _stream_ptr(stream)), self.ctx)
         return mean, var, Fm
@@ -180,10 +184,10 @@ class Solver:
     def persistent_step(self, T, iteration, stream=None):
         """One iteration of the persistent population (iugkp_persistent_step): returns
         dict(R, W, wall, counters, slots)."""
-        R = self.zeros(self.nb * self.total_cells)
-        W = self.zeros(self.nb * self.total_cells)
-        wall = self.zeros(self.total_walls)
-        cnt = torch.zeros(6, dtype=torch.int64, device=self.device)
+        R = self.empty(self.nb * self.total_cells)
+        W = self.empty(self.nb * self.total_cells)
+        wall = self.empty(self.total_walls)
+        cnt = torch.empty(6, dtype=torch.int64, device=self.device)
         n = ctypes.c_longlong(0)
         L.check(self.lib.iugkp_persistent_step(self.ctx, _dptr(T), int(iteration), _dptr(R), _dptr(W), _dptr(wall),
                                                _dptr(cnt), ctypes.byref(n), _stream_ptr(stream)), self.ctx)
