@@ -69,13 +69,24 @@ __global__ void __launch_bounds__(256) prologue_kernel(SweepArgs A, PrologueArgs
     double* out = A.wemit + in.bc_off + (long long)G.band * in.ncells;
     const double* T = A.T + in.cell_off;
     const double* sft = A.srcshift ? A.srcshift + in.cell_off : nullptr;
-#pragma unroll 4
-    for (int e = by * 256 + threadIdx.x; e < in.ncells; e += ny * 256) {
-      double Te = T[e];
-      if (sft) Te += sft[e];
-      const double w = coef[e] * Te;
-      out[e] = w;  // the weight of every particle of this emitter
-      take(w);
+    const int ncells = in.ncells, hop = ny * 256;
+    for (int e0 = by * 256 + threadIdx.x; e0 < ncells; e0 += 4 * hop) {
+      double t[4], c[4], d[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {  // the loads of four emitters in flight
+        const int e = e0 + u * hop;
+        t[u] = e < ncells ? __ldg(&T[e]) : 0.0;
+        c[u] = e < ncells ? __ldg(&coef[e]) : 0.0;
+        d[u] = sft && e < ncells ? __ldg(&sft[e]) : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int e = e0 + u * hop;
+        if (e >= ncells) break;
+        const double w = c[u] * (sft ? t[u] + d[u] : t[u]);
+        out[e] = w;  // the weight of every particle of this emitter
+        take(w);
+      }
     }
   } else {
     const int wl = G.kind - 1;
@@ -102,9 +113,14 @@ __global__ void __launch_bounds__(256) prologue_kernel(SweepArgs A, PrologueArgs
   for (int k = threadIdx.x; k < P.n_inst; k += 256) P.wmax[k] = 0ull;
   if (threadIdx.x == 0) *P.ticket = 0u;
   __syncthreads();
-  for (int g = threadIdx.x; g < A.n_groups; g += 256) {
-    unsigned long long v = 0;
-    for (int b = P.bpre[g]; b < P.bpre[g + 1]; ++b) v = max(v, __ldcg(&P.wpart[b]));
+  for (int b = threadIdx.x; b < P.wmax_blocks; b += 256) {
+    int g = 0, hi = A.n_groups - 1;
+    while (g < hi) {
+      const int mid = (g + hi + 1) >> 1;
+      if (P.bpre[mid] <= b) g = mid;
+      else hi = mid - 1;
+    }
+    const unsigned long long v = __ldcg(&P.wpart[b]);
     if (v) atomicMax(&P.wmax[A.groups[g].inst], v);
   }
 }
@@ -118,14 +134,20 @@ __device__ __forceinline__ void finish_cell(const SweepArgs& A, int n_inst, cons
   const InstDesc& in = A.inst[k];
   const long long j0 = in.bc_off + (g - in.cell_off);
   double r = 0.0;
-#pragma unroll 4
-  for (int b = 0; b < A.nb; ++b) {
-    const long long j = j0 + (long long)b * in.ncells;
-    const double x = A.R[j];
-    r += x;
-    if (A.W) {
-      const int kb = k * A.nb + b;
-      A.W[j] = (A.all_real[kb] ? x : A.W[j]) * A.taumaj[kb];
+  for (int b0 = 0; b0 < A.nb; b0 += 8) {
+    double x[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)  // the loads of eight bands in flight
+      x[u] = b0 + u < A.nb ? __ldg(&A.R[j0 + (long long)(b0 + u) * in.ncells]) : 0.0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      if (b0 + u >= A.nb) break;
+      r += x[u];
+      if (A.W) {
+        const long long j = j0 + (long long)(b0 + u) * in.ncells;
+        const int kb = k * A.nb + b0 + u;
+        A.W[j] = (__ldg(&A.all_real[kb]) ? x[u] : A.W[j]) * __ldg(&A.taumaj[kb]);
+      }
     }
   }
   if (bal) {
@@ -136,7 +158,7 @@ __device__ __forceinline__ void finish_cell(const SweepArgs& A, int n_inst, cons
 }
 
 __device__ __forceinline__ void scale_entry(const SweepArgs& A, int k, long long j) {
-  const int kb = k * A.nb + (int)((j - A.inst[k].bc_off) / A.inst[k].ncells);
+  const int kb = A.nb == 1 ? k : k * A.nb + (int)((j - A.inst[k].bc_off) / A.inst[k].ncells);
   A.W[j] = (A.all_real[kb] ? A.R[j] : A.W[j]) * A.taumaj[kb];
 }
 
@@ -484,7 +506,32 @@ __global__ void __launch_bounds__(256) close_2d_kernel(SweepArgs A, Close2D C) {
   if (!last) return;
   __threadfence();
   if (threadIdx.x == 0) C.ticket[k] = 0u;
-  for (int wl = 0; wl < 4; ++wl) wall_block(A, C.wall_unit, k, wl, false, true);
+  // absorbed power of each wall, one warp per wall: its emission plus the outward net flux
+  const int wl = threadIdx.x >> 5;
+  if (wl >= 4) return;
+  const int a = wl >> 1, side = wl & 1, nf = a == 0 ? n1 : n0;
+  double sum = 0.0, tsum = 0.0;
+  for (int j0 = lane; j0 < nf; j0 += 128) {
+    double v[4], t[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {  // the loads of four faces in flight
+      const int j = j0 + 32 * u;
+      const long long f = a == 0 ? (side ? n0 : 0) + (long long)(n0 + 1) * j : fax1 + j + (long long)n0 * (side ? n1 : 0);
+      v[u] = j < nf ? __ldcg(&F[f]) : 0.0;
+      t[u] = j < nf ? tf[in.wface_off[wl] + j] : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      sum += v[u];
+      tsum += t[u];
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    sum += __shfl_down_sync(0xffffffffu, sum, o);
+    tsum += __shfl_down_sync(0xffffffffu, tsum, o);
+  }
+  if (lane == 0) A.wall[in.wall_off + wl] = C.wall_unit[k * 6 + wl] * tsum + (side ? sum : -sum);
 }
 
 }  // namespace

@@ -90,8 +90,6 @@ __device__ __forceinline__ double shfl_d(double x, int src) {
 // an exit through the low wall of an untallied axis goes to that wall's face (one-group
 // instances) or to the group's exit tally GX (two-group). Emission needs nothing: the staged
 // sweep and its post-passes account for it.
-constexpr unsigned REPLAY_PER_WARP = 32;  // queue entries per warp and round
-
 template <int DIM>
 __global__ void __launch_bounds__(256) replay_kernel(SweepArgs A, StagedArgs S) {
   Counts cnt;
@@ -100,16 +98,19 @@ __global__ void __launch_bounds__(256) replay_kernel(SweepArgs A, StagedArgs S) 
   const int lane = threadIdx.x & 31;
   const unsigned n = min(*S.defer_n, S.defer_cap);
   // Warp j of block b is warp a = j G + b (G blocks: warp j of every block comes before warp
-  // j + 1 of any), and warp a takes entries E a .. E a + E - 1 (E = REPLAY_PER_WARP; then E (a
-  // + W) .., W warps in the grid). The queue is short: numbered b 8 + j, the warps that got
-  // work were all in the first few blocks, on a few SMs (measured: the busiest SM active 3.6
-  // times as long as the average); this way the first warps to get work are the first warp of
-  // every block.
+  // j + 1 of any), and warp a takes entries E a .. E a + E - 1 (then E (a + W) .., W warps in the
+  // grid). The queue is short: numbered b 8 + j, the warps that got work were all in the first
+  // few blocks, on a few SMs (measured: the busiest SM active 3.6 times as long as the average);
+  // this way the first warps to get work are the first warp of every block. E, at most 32, is
+  // what spreads the queue over G / 2 warps (four per SM): a warp's particles share its FP64
+  // instructions, but their faces are tallied one particle after the other, so a queue of a few
+  // hundred is done sooner with one or two particles per warp.
   const unsigned W = gridDim.x * blockDim.x >> 5;
   const unsigned wid = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  const unsigned half = max(1u, gridDim.x >> 1), E = min(32u, max(1u, (n + half - 1) / half));
   // all lanes of a warp run the same rounds (the face items are tallied by the whole warp)
-  for (unsigned i0 = REPLAY_PER_WARP * wid; i0 < n; i0 += REPLAY_PER_WARP * W) {
-    const unsigned i = lane < (int)REPLAY_PER_WARP ? i0 + lane : n;
+  for (unsigned i0 = E * wid; i0 < n; i0 += E * W) {
+    const unsigned i = lane < (int)E ? i0 + lane : n;
     // the lane's particle, kept for the face items
     int kinst = 0, ex = 0, tall = 0;  // instance, exit axis (-1: real collision), tallied axes (bits)
     double w = 0.0;
