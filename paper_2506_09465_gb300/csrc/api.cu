@@ -136,7 +136,8 @@ void free_all(Ctx* c) {
                   c->d_all_group_mag, c->d_R32, c->d_W32, c->d_F32, c->d_m2, c->d_wallTf,
                   c->d_pslot_off, c->d_phome_off, c->d_pnband, c->d_pnwall, c->d_px, c->d_pband, c->d_phome,
                   c->d_pcount, c->d_pfcount, c->d_phome_w, c->d_wemit, c->d_DY, c->d_EY, c->d_GX, c->d_Fx, c->d_Fi, c->d_ticket, c->d_wpart,
-                  c->d_all_real, c->d_defer, c->d_defer_n, c->d_land_fwd, c->d_land_all, c->d_items, c->d_diff};
+                  c->d_all_real, c->d_defer, c->d_defer_n, c->d_land_fwd, c->d_land_all, c->d_items, c->d_diff, c->d_sync_groups, c->d_sync_beg,
+                  c->d_sync_end};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (c->h_pinned) cudaFreeHost(c->h_pinned);
@@ -263,6 +264,31 @@ void broadcast_wall_T(Ctx* c) {
     }
 }
 
+// Tasks of the pass-synchronous 2D sweep over the forward groups, for the options' warp_grab.
+iugkp_status build_sync_tasks(Ctx* c) {
+  if (c->dim != 2) return IUGKP_OK;
+  const int grab = c->opt.warp_grab > 0 ? c->opt.warp_grab : 256;
+  std::vector<LandGroup> lg;
+  land_tasks(c, c->h_groups_fwd, lg, c->sync_tasks, c->sync_qch, std::max(1, grab / 32), STAGED_NT / 32);
+  if (c->fwd_particles == 0) c->sync_tasks = 0;
+  std::vector<long long> beg(c->n_inst, 0);
+  std::vector<unsigned> end(c->n_inst, 0);
+  for (size_t g = 0; g < lg.size() && c->sync_tasks; ++g) {  // groups are ordered by instance
+    if (g == 0 || lg[g].inst != lg[g - 1].inst) beg[lg[g].inst] = lg[g].task0;
+    end[lg[g].inst] = g + 1 < lg.size() ? lg[g + 1].task0 : c->sync_tasks;
+  }
+  void* olds[] = {c->d_sync_groups, c->d_sync_beg, c->d_sync_end};
+  for (void* p : olds)
+    if (p) cudaFree(p);
+  c->d_sync_groups = nullptr;
+  c->d_sync_beg = nullptr;
+  c->d_sync_end = nullptr;
+  iugkp_status s;
+  if ((s = upload(c, &c->d_sync_groups, lg)) != IUGKP_OK) return s;
+  if ((s = upload(c, &c->d_sync_beg, beg)) != IUGKP_OK) return s;
+  return upload(c, &c->d_sync_end, end);
+}
+
 // Forward groups leave out walls whose faces are all at zero temperature (their
 // particles weigh zero).
 iugkp_status rebuild_forward_groups(Ctx* c) {
@@ -350,9 +376,10 @@ iugkp_status rebuild_forward_groups(Ctx* c) {
   c->d_group_mag = nullptr;
   if ((s = upload(c, &c->d_group_mag, gmag)) != IUGKP_OK) return s;
   std::vector<LandGroup> lg;
-  land_tasks(c, c->h_groups_fwd, lg, c->land_fwd_tasks, c->land_fwd_qch);
+  land_tasks(c, c->h_groups_fwd, lg, c->land_fwd_tasks, c->land_fwd_qch, LAND_QCH, LAND_WARPS_PER_SM);
   if (c->fwd_particles == 0) c->land_fwd_tasks = 0;  // the all-zero placeholder group
   if ((s = upload(c, &c->d_land_fwd, lg)) != IUGKP_OK) return s;
+  if ((s = build_sync_tasks(c)) != IUGKP_OK) return s;
   if ((s = upload(c, &c->d_inst_beg, beg)) != IUGKP_OK) return s;
   if ((s = upload(c, &c->d_inst_end, end)) != IUGKP_OK) return s;
   if ((s = upload(c, &c->d_cost_prefix, prefix)) != IUGKP_OK) return s;
@@ -754,7 +781,7 @@ iugkp_status iugkp_create_batch(int n, const iugkp_grid* g, const double* const*
     for (const Group& g : c->h_groups_all) gmag.push_back(div_magic(g.n_emitters));
     UP(c->d_all_group_mag, gmag);
     std::vector<LandGroup> lg;
-    land_tasks(c, c->h_groups_all, lg, c->land_all_tasks, c->land_all_qch);
+    land_tasks(c, c->h_groups_all, lg, c->land_all_tasks, c->land_all_qch, LAND_QCH, LAND_WARPS_PER_SM);
     UP(c->d_land_all, lg);
   }
   {
@@ -1216,9 +1243,11 @@ iugkp_status iugkp_autotune(iugkp_ctx* ctx, const double* T_dev, unsigned epoch,
     int keep = *knobs[kdx];
     for (int j = 0; j < counts[kdx]; ++j) {
       *knobs[kdx] = values[kdx][j];
+      if (kdx == 1 && (st = build_sync_tasks(c)) != IUGKP_OK) return st;
       double t = 0.0;
       if ((st = time_sweep(&t)) != IUGKP_OK) {
         *knobs[kdx] = keep;
+        if (kdx == 1) build_sync_tasks(c);
         return st;
       }
       if (t < best) {
@@ -1227,6 +1256,7 @@ iugkp_status iugkp_autotune(iugkp_ctx* ctx, const double* T_dev, unsigned epoch,
       }
     }
     *knobs[kdx] = keep;
+    if (kdx == 1 && (st = build_sync_tasks(c)) != IUGKP_OK) return st;
   }
   if ((st = check_device(c, s)) != IUGKP_OK) return st;
   if (out) {

@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(EXACT_NT) exact_kernel(SweepArgs A, StagedArgs
     task = __shfl_sync(0xffffffffu, task, 0);
     if (task >= L.n_tasks) break;
     tg.find(L, task);
-    const LandGroup& G = tg.G;
+    const LandGroup& G = L.groups[tg.gi];
     const unsigned t = task - tg.t_beg;
     const int qc = (int)(t / (unsigned)G.ntile), tile = (int)(t - (unsigned)qc * (unsigned)G.ntile);
     const InstDesc& in = A.inst[G.inst];

@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(LAND_NT) land_kernel(SweepArgs A, StagedArgs S
     task = __shfl_sync(0xffffffffu, task, 0);
     if (task >= L.n_tasks) return;
     tg.find(L, task);
-    const LandGroup& G = tg.G;
+    const LandGroup& G = L.groups[tg.gi];
     const unsigned t = task - tg.t_beg;
     const int qc = (int)(t / (unsigned)G.ntile), tile = (int)(t - (unsigned)qc * (unsigned)G.ntile);
     const InstDesc& in = A.inst[G.inst];
@@ -353,14 +353,15 @@ cudaError_t launch_land(const Ctx* c, const SweepArgs& a, bool adj, cudaStream_t
   return launch_replay(c, a, S, s);  // the deferred particles, in FP64
 }
 
-// Tasks of the landing sweep over a group list: tiles of at most 32 emitters (equal widths;
+// Tasks of a sweep over a group list: tiles of at most 32 emitters (equal widths;
 // narrow groups put several particles of an emitter side by side), qch particles per emitter and
-// task: at most LAND_QCH, fewer where that would leave warps without work.
-void land_tasks(const Ctx* c, const std::vector<Group>& groups, std::vector<LandGroup>& out, unsigned& n_tasks, int& qch) {
+// task: at most qch_max, fewer where that would leave warps without work.
+void land_tasks(const Ctx* c, const std::vector<Group>& groups, std::vector<LandGroup>& out, unsigned& n_tasks, int& qch,
+                int qch_max, int warps_per_sm) {
   long long total = 0;
   for (const Group& g : groups) total += (long long)g.n_emitters * g.per_emitter;
-  const long long warps = (long long)std::max(1, c->sm_count) * LAND_WARPS_PER_SM;
-  qch = (int)std::max<long long>(1, std::min<long long>(LAND_QCH, total / (32 * 4 * warps)));
+  const long long warps = (long long)std::max(1, c->sm_count) * warps_per_sm;
+  qch = (int)std::max<long long>(1, std::min<long long>(qch_max, total / (32 * 4 * warps)));
   long long t0 = 0;
   out.clear();
   for (const Group& g : groups) {

@@ -197,7 +197,7 @@ struct LaneEmitter {
 // The group of a claimed task, kept until a task of another group comes.
 struct TaskGroup {
   unsigned t_beg = 1, t_end = 0;  // tasks of the cached group
-  LandGroup G;
+  int gi = 0;
   __device__ __forceinline__ void find(const LandArgs& L, unsigned task) {
     if (task >= t_beg && task < t_end) return;
     int lo = 0, hi = L.n_groups - 1;
@@ -206,8 +206,8 @@ struct TaskGroup {
       if (L.groups[mid].task0 <= task) lo = mid;
       else hi = mid - 1;
     }
-    G = L.groups[lo];
-    t_beg = G.task0;
+    gi = lo;
+    t_beg = L.groups[lo].task0;
     t_end = lo + 1 < L.n_groups ? L.groups[lo + 1].task0 : L.n_tasks;
   }
 };

@@ -136,4 +136,10 @@ struct LandArgs {
   const double* lamVm;            // adjoint: [cells] lambda / (V m)
 };
 
+// Tasks of the pass-synchronous 2D sweep: those of an instance are contiguous.
+struct SyncArgs {
+  LandArgs L;
+  const unsigned* task_end;       // [n_inst]
+};
+
 }  // namespace iugkp

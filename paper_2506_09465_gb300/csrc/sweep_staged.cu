@@ -34,6 +34,7 @@
 
 #include "device.cuh"
 #include "internal.h"
+#include "landing.cuh"
 #include "staged.h"
 #include "walk32.cuh"
 
@@ -915,7 +916,7 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
 // instance's x-faces exceed the window (a centred run of them sits there); the faces outside
 // take global atomics of the same fixed-point contribution.
 template <bool K32, bool REAL, bool PARTIAL>
-__global__ void __launch_bounds__(STAGED_NT, 1) sweep_sync_kernel(SweepArgs A, StagedArgs S) {
+__global__ void __launch_bounds__(STAGED_NT, 1) sweep_sync_kernel(SweepArgs A, StagedArgs S, SyncArgs Y) {
   extern __shared__ unsigned win[];
   __shared__ int4 s_par[STAGED_NT / 32][64];
   __shared__ int s_lst[STAGED_NT / 32][33];
@@ -932,9 +933,11 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_sync_kernel(SweepArgs A, S
   }
   int4* par = s_par[threadIdx.x >> 5];
   int* lst = s_lst[threadIdx.x >> 5];
+  TaskGroup tg;
   for (int visit = 0; visit < n_inst; ++visit) {
     const int k = (start + visit) % n_inst;
-    if (threadIdx.x == 0) s_inst = (*(volatile unsigned long long*)&S.inst_next[k] < (unsigned long long)S.inst_end[k]) ? k : -1;
+    const unsigned task_end = Y.task_end[k];
+    if (threadIdx.x == 0) s_inst = (*(volatile unsigned long long*)&S.inst_next[k] < (unsigned long long)task_end) ? k : -1;
     __syncthreads();
     if (s_inst < 0) {
       __syncthreads();
@@ -951,42 +954,80 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_sync_kernel(SweepArgs A, S
     for (unsigned i = threadIdx.x; i < wlen; i += STAGED_NT) win[i] = WIN_BIAS;
     __syncthreads();
     const double qinv = S.wmax[k] > 0.0 ? WIN_SCALE / S.wmax[k] : 0.0;
-    const unsigned pend = (unsigned)S.inst_end[k];
-    unsigned rbeg = 0, rend = 0;  // this warp's private particle range
-    EmitCache ec;
-    ec.g_first = 1;
-    ec.g_end = 0;  // empty: forces a lookup on the first emission
-    ec.e = -1;
+    const float h0 = in.hf[0], h1 = in.hf[1];
+    const uint32_t inst_id = in.inst_id;
+    const int ncells = in.ncells;
+    const long long coff = in.cell_off;
+    double* const gx = S.gx() + in.bface_off;
     for (;;) {
-      if (rbeg == rend) {  // private range used up: take the next one of the instance
-        unsigned long long got = 0;
-        if (lane == 0) got = atomicAdd(&S.inst_next[k], (unsigned long long)S.warp_grab);
-        got = __shfl_sync(0xffffffffu, got, 0);
-        if (got >= pend) break;
-        rbeg = (unsigned)got;
-        rend = (unsigned)min(got + (unsigned long long)S.warp_grab, (unsigned long long)pend);
+      // the next task of the instance: a tile of emitters (one or more lanes each) x a run of
+      // particle numbers; the lanes keep their emitters for the run
+      unsigned long long got = 0;
+      if (lane == 0) got = atomicAdd(&S.inst_next[k], 1ull);
+      got = __shfl_sync(0xffffffffu, got, 0);
+      if (got >= task_end) break;
+      tg.find(Y.L, (unsigned)got);
+      const LandGroup& G = Y.L.groups[tg.gi];
+      const unsigned tk = (unsigned)got - tg.t_beg;
+      const int qc = (int)(tk / (unsigned)G.ntile), tile = (int)(tk - (unsigned)qc * (unsigned)G.ntile);
+      const int kind = G.kind, band = G.band;
+      const int sub = lane / G.tw, rank = tile * G.tw + lane - sub * G.tw;
+      int e = sub < G.reps && rank < G.ne ? rank : 0;
+      if (G.perm_off >= 0) e = A.perm[G.perm_off + e];
+      int c[3];
+      uint32_t id;
+      emitter_cell<2>(in, S, k, kind, e, c, id);
+      const long long bcbase = in.bc_off + (long long)band * ncells;
+      double w;
+      if (kind == 0) {
+        w = A.wemit[bcbase + e];  // from the pass before the trace
+      } else {
+        w = A.wcoef[(long long)(k * A.nb + band) * 6 + kind - 1] * A.wallTf[in.bface_off + in.wface_off[kind - 1] + e];
       }
-      const unsigned take = min(32u, rend - rbeg);
-      int nitem = 0;
-      int4 pa_own, pb_own;  // this lane's item parameters, stored once its list slot is known
-      if ((unsigned)lane < take) {
-        double w;
-        int band;
-        PW f;
-        Stream st;
-        uint32_t ub;
-        if (staged_emit<2>(A, S, rbeg + lane, w, band, f, st, ub, ec, in, k, two)) {
-          cnt.v[CNT_FLIGHTS] += 1;
-          const int qw = __double2loint(fma(w, qinv, 0x1.8p52));
+      // +-0: nothing to trace
+      const bool on = sub < G.reps && rank < G.ne && (__double_as_longlong(w) << 1) != 0;
+      const int qw = __double2loint(fma(w, qinv, 0x1.8p52));
+      const float vtm = A.vtm32[k * A.nb + band];
+      const bool all_real = REAL || A.all_real[k * A.nb + band] != 0;
+      const float ea = vtm * TIE_LOG_ABS;
+      const int qbeg = qc * (Y.L.qch * G.reps) + sub, qend = min(G.per, (qc + 1) * (Y.L.qch * G.reps));
+      int n_yg = 0;  // the lane's y-group flights of this task: their emission enters its own balance
+      for (int pass = 0; pass < Y.L.qch; ++pass) {
+        const int q = qbeg + pass * G.reps;
+        const bool act = on && q < qend;
+        if (!__any_sync(0xffffffffu, act)) break;
+        int nitem = 0;
+        int4 pa_own, pb_own;  // this lane's item parameters, stored once its list slot is known
+        if (act) {
+          PW f;
+          Stream st;
+          uint32_t ub;
+          st.init(A.seed, inst_id, (uint32_t)band, A.epoch, id, (uint32_t)q);
+          {
+            float xi[3], s[3];
+            emit_segment<2>(st, kind, xi, s);
+            f.i0 = c[0];
+            f.i1 = c[1];
+            axis_init(s[0], xi[0], h0, f.t0, f.d0, f.s0);
+            f.tex = axis_exit(f.i0, f.s0, n0, f.t0, f.d0);
+            axis_init(s[1], xi[1], h1, f.t1, f.d1, f.s1);
+            const float e1 = axis_exit(f.i1, f.s1, n1, f.t1, f.d1);
+            f.i2 = e1 < f.tex ? 1 : 0;  // the axis of the wall the segment reaches (x on ties)
+            f.tex = fminf(f.tex, e1);
+          }
           const bool yg = two && f.d0 < f.d1;
+          n_yg += yg ? 1 : 0;
+          // the first candidate: its path word from block 0's unused bits; its acceptance word
+          // only where some cell of the band may reject (else the particle ends at its first
+          // candidate, so no later draw is taken)
+          ub = all_real ? 0u : st.even_word();
+          st.j += 2;
+          f.D = __fmul_rn(-__logf(word_uniform<float>(st.first)), vtm);
+          cnt.v[CNT_FLIGHTS] += 1;
           const unsigned qwx = (unsigned)((yg ? f.s1 : f.s0) > 0 ? qw : -qw);
-          const float vtm = A.vtm32[(long long)k * A.nb + band];
-          const bool all_real = REAL || A.all_real[(long long)k * A.nb + band] != 0;
-          const long long bcbase = in.bc_off + (long long)band * in.ncells;
           // candidates (Sec. 3.2) until the particle collides for real or reaches a wall; a
           // decision within rounding of the FP64 walk's defers the particle to the FP64 replay
           const int m0 = faces_to_wall(f.i0, f.s0, n0), m1 = faces_to_wall(f.i1, f.s1, n1);
-          const float ea = vtm * TIE_LOG_ABS;
           float eD = fmaf(f.D, TIE_LOG_REL, ea);  // bound of |D - D_fp64|
           bool wall_exit = false, deferred = false;
           int fb0 = 0, fb1 = 0;  // faces before the latest candidate, per axis
@@ -1012,7 +1053,7 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_sync_kernel(SweepArgs A, S
             }
             const int cell = clampi(f.i0 + f.s0 * fb0, n0) + n0 * clampi(f.i1 + f.s1 * fb1, n1);
             const long long ci = bcbase + cell;
-            const int oc = candidate_outcome<2>(A, bcbase, in.ncells, f, base, fb0, fb1, 0, cell, all_real, near, ub,
+            const int oc = candidate_outcome<2>(A, bcbase, ncells, f, base, fb0, fb1, 0, cell, all_real, near, ub,
                                                 n0, n1, 1, n0, 0);
             if (oc == CAND_DEFER) {
               deferred = true;
@@ -1028,7 +1069,7 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_sync_kernel(SweepArgs A, S
               cnt.v[CNT_REAL] += 1;
               if (K32) tally_k32(&S.R32[ci], w);
               else atomicAdd(&A.R[ci], w);
-              if (yg) atomicAdd(&S.DY[in.cell_off + cell], w);
+              if (yg) atomicAdd(&S.DY[coff + cell], w);
               break;
             }
             uint32_t uw;
@@ -1055,7 +1096,7 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_sync_kernel(SweepArgs A, S
             c1 = min(fb1, m1 - 1);
           }
           if (deferred) {
-            defer_particle(S, rbeg + lane, ((unsigned)kc << 1) | (yg ? 1u : 0u));
+            defer_particle(S, G.first + (unsigned)q * (unsigned)G.ne + (unsigned)rank, ((unsigned)kc << 1) | (yg ? 1u : 0u));
           } else {
             if (wall_exit) cnt.v[CNT_WALL_EXITS] += 1;
             cnt.v[CNT_CROSSINGS] += c0 + c1;
@@ -1066,7 +1107,7 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_sync_kernel(SweepArgs A, S
             const int cp = yg ? c1 : c0, mq = yg ? m0 : m1, axp = yg ? 1 : 0;
             if (ex == 1 - axp && (yg ? f.s0 : f.s1) < 0) {  // exit through the low q-wall
               const int j = yg ? in.wface_off[0] + f.i1 + f.s1 * c1 : in.wface_off[2] + f.i0 + f.s0 * c0;
-              atomicAdd(&S.gx()[in.bface_off + j], -w);
+              atomicAdd(&gx[j], -w);
             }
             nitem = cp + (ex == axp ? 1 : 0);
             const bool flat = !(dq < INFINITY);
@@ -1081,8 +1122,6 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_sync_kernel(SweepArgs A, S
             pb_own = make_int4(__float_as_int(u0), __float_as_int(r), (int)qwx, 0);
           }
         }
-      }
-      rbeg += take;
       // ---- the pass's face items: each lane's list is cut into segments of SEG items, the
       // segments are numbered in lane order and dealt to the lanes round-robin, 32 to a
       // round; a lane runs SEG steps of its segment with its list's parameters (no per-item
@@ -1144,6 +1183,15 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_sync_kernel(SweepArgs A, S
         }
         __syncwarp();
       }
+      }
+      if (n_yg > 0) {
+        if (kind == 0) {
+          atomicAdd(&S.DY[coff + e], -(double)n_yg * w);
+        } else {
+          const int wl = kind - 1;
+          atomicAdd(&S.EY[in.bface_off + in.wface_off[wl] + e], (double)n_yg * ((wl & 1) ? -w : w));
+        }
+      }
     }
     __syncthreads();
     for (unsigned i = threadIdx.x; i < wlen; i += STAGED_NT) {
@@ -1157,12 +1205,20 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_sync_kernel(SweepArgs A, S
 
 template <bool K32>
 void launch_sync(const Ctx* c, const SweepArgs& a, const StagedArgs& S, int blocks, size_t smem, cudaStream_t s) {
+  SyncArgs Y;
+  Y.L.groups = c->d_sync_groups;
+  Y.L.n_groups = a.n_groups;
+  Y.L.n_tasks = c->sync_tasks;
+  Y.L.qch = c->sync_qch;
+  Y.L.next = nullptr;
+  Y.L.lamVm = nullptr;
+  Y.task_end = c->d_sync_end;
   if (c->all_real_all) {
-    if (c->sync_partial) sweep_sync_kernel<K32, true, true><<<blocks, STAGED_NT, smem, s>>>(a, S);
-    else sweep_sync_kernel<K32, true, false><<<blocks, STAGED_NT, smem, s>>>(a, S);
+    if (c->sync_partial) sweep_sync_kernel<K32, true, true><<<blocks, STAGED_NT, smem, s>>>(a, S, Y);
+    else sweep_sync_kernel<K32, true, false><<<blocks, STAGED_NT, smem, s>>>(a, S, Y);
   } else {
-    if (c->sync_partial) sweep_sync_kernel<K32, false, true><<<blocks, STAGED_NT, smem, s>>>(a, S);
-    else sweep_sync_kernel<K32, false, false><<<blocks, STAGED_NT, smem, s>>>(a, S);
+    if (c->sync_partial) sweep_sync_kernel<K32, false, true><<<blocks, STAGED_NT, smem, s>>>(a, S, Y);
+    else sweep_sync_kernel<K32, false, false><<<blocks, STAGED_NT, smem, s>>>(a, S, Y);
   }
 }
 
@@ -1201,6 +1257,9 @@ cudaError_t launch_sweep_staged(const Ctx* c, const SweepArgs& a_in, cudaStream_
   S.R32 = k32 ? c->d_R32 : nullptr;
   S.W32 = k32 && a.W ? c->d_W32 : nullptr;
   S.F32 = k32 && a.F ? c->d_F32 : nullptr;
+  // pass-synchronous schedule: refill only when all 32 lanes are idle (the default where it
+  // applies)
+  const bool sync = c->sync_ok && a.F && (c->opt.refill_lanes == 0 || c->opt.refill_lanes == 32);
   PrologueArgs P = {};
   auto clear = [&](void* p, size_t n) {
     if (!p || !n) return;
@@ -1228,7 +1287,7 @@ cudaError_t launch_sweep_staged(const Ctx* c, const SweepArgs& a_in, cudaStream_
   clear(c->d_defer_n, 2);
   P.n_inst = c->n_inst;
   P.next = c->d_inst_next;
-  P.next_from = c->d_inst_beg;
+  P.next_from = sync ? c->d_sync_beg : c->d_inst_beg;
   P.wmax_blocks = c->wmax_blocks;
   P.bpre = c->d_wmax_bpre;
   P.wpart = c->d_wpart;
@@ -1238,9 +1297,6 @@ cudaError_t launch_sweep_staged(const Ctx* c, const SweepArgs& a_in, cudaStream_
   if (e != cudaSuccess) return e;
   const size_t smem = (size_t)c->staged_cap * sizeof(unsigned);
   const int blocks = c->sm_count * c->staged_blocks_per_sm;
-  // pass-synchronous schedule: refill only when all 32 lanes are idle (the default where it
-  // applies)
-  const bool sync = c->sync_ok && a.F && (c->opt.refill_lanes == 0 || c->opt.refill_lanes == 32);
   if (k32) {
     switch (c->dim) {
       case 1: sweep_staged_kernel<1, true><<<blocks, STAGED_NT, smem, s>>>(a, S); break;
