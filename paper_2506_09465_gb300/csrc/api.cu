@@ -1475,9 +1475,9 @@ iugkp_status iugkp_persistent_reset(iugkp_ctx* ctx, void* cuda_stream) {
     if ((st = upload(c, &c->d_pnband, c->h_nband)) != IUGKP_OK) return st;
     if ((st = upload(c, &c->d_pnwall, c->h_nwall)) != IUGKP_OK) return st;
     if ((st = dalloc(c, &c->d_px, (size_t)7 * c->pers_n)) != IUGKP_OK) return st;
-    if ((st = dalloc(c, &c->d_pband, (size_t)c->pers_n)) != IUGKP_OK) return st;
+    if ((st = dalloc(c, &c->d_pband, c->nb > 1 ? (size_t)c->pers_n : 1)) != IUGKP_OK) return st;
     if ((st = dalloc(c, &c->d_phome, (size_t)c->pers_n)) != IUGKP_OK) return st;
-    if ((st = dalloc(c, &c->d_pcount, (size_t)2 * c->pers_homes)) != IUGKP_OK) return st;
+    if ((st = dalloc(c, &c->d_pcount, (size_t)2 * ((c->pers_homes + 1) & ~1ll))) != IUGKP_OK) return st;
     if ((st = dalloc(c, &c->d_pfcount, (size_t)2 * PERS_FACE_REPLICAS * pers_face_homes(c))) != IUGKP_OK) return st;
     if ((st = dalloc(c, &c->d_phome_w, (size_t)c->pers_homes)) != IUGKP_OK) return st;
   }
@@ -1496,20 +1496,9 @@ iugkp_status iugkp_persistent_step(iugkp_ctx* ctx, const double* T_dev, unsigned
   if (!T_dev || !R_dev) return fail(c, IUGKP_EINVAL, "T_dev and R_dev are required");
   if (!c->d_px) return fail(c, IUGKP_EINVAL, "call iugkp_persistent_reset first");
   cudaStream_t s = (cudaStream_t)cuda_stream;
-  const size_t bc = (size_t)c->nb * c->total_cells;
   double* W = W_dev ? W_dev : c->d_W;
   double* wall = wall_dev ? wall_dev : c->d_wall;
   unsigned long long* cnt = counters_dev ? counters_dev : c->d_counters;
-  CK(cudaMemsetAsync(R_dev, 0, bc * sizeof(double), s), "clear R");
-  CK(cudaMemsetAsync(W, 0, bc * sizeof(double), s), "clear W");
-  CK(cudaMemsetAsync(wall, 0, (size_t)c->total_walls * sizeof(double), s), "clear wall");
-  CK(cudaMemsetAsync(cnt, 0, CNT_N * sizeof(unsigned long long), s), "clear counters");
-  {
-    const size_t fr = (size_t)PERS_FACE_REPLICAS * pers_face_homes(c);
-    CK(cudaMemsetAsync(c->d_pfcount + (c->pers_parity ? 0 : fr), 0, fr * sizeof(unsigned), s), "clear face counts");
-  }
-  CK(cudaMemsetAsync(c->d_pcount + (c->pers_parity ? 0 : c->pers_homes), 0, (size_t)c->pers_homes * sizeof(unsigned), s),
-     "clear counts");
   CK(launch_persistent_step(c, T_dev, iteration, R_dev, W, wall, cnt, s), "persistent step");
   c->pers_parity ^= 1;
   if (slots_out) *slots_out = c->pers_n;

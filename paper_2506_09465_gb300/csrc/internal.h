@@ -158,9 +158,9 @@ struct Ctx {
   double* d_px = nullptr;         // [7 * pers_n] doubles: x, y, z, s_x, s_y, s_z (FP64, or FP32 packed
                                   // at the start), then w at 6 * pers_n
   double* d_phome_w = nullptr;    // [pers_homes] power per re-emitted particle of each home
-  int* d_pband = nullptr;
+  int* d_pband = nullptr;         // band of each slot (several bands only)
   int* d_phome = nullptr;
-  unsigned* d_pcount = nullptr;   // [2 * pers_homes] (cell homes; the entries of face homes stay 0)
+  unsigned* d_pcount = nullptr;   // two halves of pers_homes, each padded to 8 bytes (the entries of face homes stay 0)
   unsigned* d_pfcount = nullptr;  // [2 * PERS_FACE_REPLICAS * face homes] face-home counts, replicated
   double* h_pinned = nullptr;    // [8 + n_inst] host readback
   // multigrid preconditioner of the Newton correction (mg_setup.cu, mgpcg.cu)

@@ -132,6 +132,13 @@ __device__ __forceinline__ Real quot(Real a, Real b) { return a / b; }
 template <>
 __device__ __forceinline__ float quot<float>(float a, float b) { return __fdividef(a, b); }
 
+// Products and sums whose rounding is fixed, however the code around them is arranged: a position
+// is a rounded product, and a step along the direction adds to it with one rounding.
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+
 // Wall power: each thread sums its absorptions per wall of the instance it is in (one FP64
 // add per absorption); a warp adds its sums, grouped by wall, to the block's shared copy when
 // the instance of one of its lanes changes and at the end, and the block adds its copy to
@@ -216,15 +223,21 @@ __global__ void __launch_bounds__(PERS_NT, 4) persistent_step_kernel(PArgs A) {
     }
     if (i >= ns) continue;
     const InstDesc& in = INS[k];
-    const int b = __ldcs(A.band + i);
+    const int b = A.nb == 1 ? 0 : __ldcs(A.band + i);
     const unsigned hw = __ldcs(A.home + i);
-    Real x[3], s[3];
+    // a due slot is re-emitted whole: its position, direction and weight are neither read nor,
+    // when it ended due, written
+    const bool was_due = (hw & DUE_BIT) != 0u;
+    Real x[3] = {(Real)0, (Real)0, (Real)0}, s[3] = {(Real)0, (Real)0, (Real)0};
+    double w = 0.0;
+    if (!was_due) {
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      x[a] = a < DIM ? __ldcs(px + a * ns + i) : (Real)0;
-      s[a] = a < DIM ? __ldcs(px + (3 + a) * ns + i) : (Real)0;
+      for (int a = 0; a < DIM; ++a) {
+        x[a] = __ldcs(px + a * ns + i);
+        s[a] = __ldcs(px + (3 + a) * ns + i);
+      }
+      w = __ldcs(A.pw + i);
     }
-    double w = __ldcs(A.pw + i);
     int h = (int)(hw & ~DUE_BIT);
     const int n0 = in.n[0], n1 = in.n[1];
     if (k * A.nb + b != kb) {
@@ -238,82 +251,78 @@ __global__ void __launch_bounds__(PERS_NT, 4) persistent_step_kernel(PArgs A) {
     }
     Stream st;  // block 0 is computed by the emission, or else by the flight's draw
     st.init_lazy(A.seed, in.inst_id, (uint32_t)b, A.it, 0x80000000u, (uint32_t)(i - k_beg));
-    if (hw & DUE_BIT) {
+    if (was_due) {
       w = A.home_w[hbase + h];
       st.load_block(0);
-      if (h < in.ncells) {
-        // re-emission in the cell of the real collision (Sec. 3.2 step (2))
+      // re-emission from the cell of the real collision (Sec. 3.2 step (2)) or from the boundary
+      // face that absorbed it (black wall). A warp mixes both, so the draws, square roots and the
+      // sine and cosine are shared; the two differ in the words they take and where the
+      // components go.
+      const bool cell = h < in.ncells;
+      const uint32_t wx = st.buf.x, wy = st.buf.y, wz = st.buf.z, ww = st.buf.w;
+      // word of mu (cell) or of the normal component (wall), word of phi
+      uint32_t um = DIM == 1 ? (cell ? wy : wx) : (DIM == 2 ? (cell ? wz : wy) : (cell ? ww : wz));
+      uint32_t up = DIM == 2 ? (cell ? ww : wz) : ww;
+      if (DIM == 3 && cell) {
+        st.load_block(1);
+        up = st.buf.x;
+      }
+      const Real u_m = word_uniform<Real>(um);
+      const Real mu = (Real)2 * u_m - (Real)1;
+      Real sp = (Real)0, cp = (Real)0, sn = (Real)0;
+      if (DIM >= 2) {
+        const Real v_cell = fma_rn(-mu, mu, (Real)1), v_wall = (Real)1 - u_m;
+        sn = sqrt(cell ? v_cell : v_wall);
+        RealTraits<Real>::sincos2pi(word_uniform<Real>(up), &sp, &cp);
+      }
+      if (cell) {
         const unsigned r0 = udiv((unsigned)h, (unsigned)n0, A.mag[k]);
         const unsigned r1 = DIM == 3 ? udiv(r0, (unsigned)n1, A.mag[A.n_inst + k]) : 0u;
         const int ci[3] = {h - (int)r0 * n0, (int)(r0 - r1 * (unsigned)n1), (int)r1};
         const Real hx = cell_h<Real>(in, 0), hy = cell_h<Real>(in, 1), hz = cell_h<Real>(in, 2);
-        Real u_mu, u_phi = (Real)0.5;
-        if (DIM == 1) {
-          x[0] = (int_to_real<Real>(ci[0]) + word_uniform<Real>(st.buf.x)) * hx;
-          u_mu = word_uniform<Real>(st.buf.y);
-        } else if (DIM == 2) {
-          x[0] = (int_to_real<Real>(ci[0]) + word_uniform<Real>(st.buf.x)) * hx;
-          x[1] = (int_to_real<Real>(ci[1]) + word_uniform<Real>(st.buf.y)) * hy;
-          u_mu = word_uniform<Real>(st.buf.z);
-          u_phi = word_uniform<Real>(st.buf.w);
-        } else {
-          x[0] = (int_to_real<Real>(ci[0]) + word_uniform<Real>(st.buf.x)) * hx;
-          x[1] = (int_to_real<Real>(ci[1]) + word_uniform<Real>(st.buf.y)) * hy;
-          x[2] = (int_to_real<Real>(ci[2]) + word_uniform<Real>(st.buf.z)) * hz;
-          u_mu = word_uniform<Real>(st.buf.w);
-          st.load_block(1);
-          u_phi = word_uniform<Real>(st.buf.x);
-        }
-        const Real mu = (Real)2 * u_mu - (Real)1;
+        x[0] = mul_rn(int_to_real<Real>(ci[0]) + word_uniform<Real>(wx), hx);
+        if (DIM >= 2) x[1] = mul_rn(int_to_real<Real>(ci[1]) + word_uniform<Real>(wy), hy);
+        if (DIM == 3) x[2] = mul_rn(int_to_real<Real>(ci[2]) + word_uniform<Real>(wz), hz);
         s[0] = mu;
         if (DIM >= 2) {
-          const Real sn = sqrt((Real)1 - mu * mu);
-          Real sp, cp;
-          RealTraits<Real>::sincos2pi(u_phi, &sp, &cp);
           s[1] = sn * cp;
           s[2] = sn * sp;
         }
         st.j = thermal_uniforms(DIM);
       } else {
-        // re-emission from the boundary face that absorbed it (black wall)
         const int bf = h - in.ncells;
         int wl = 0;
-        while (wl + 1 < 2 * DIM && bf >= in.wface_off[wl + 1]) ++wl;
+#pragma unroll
+        for (int q = 1; q < 2 * DIM; ++q) wl += bf >= in.wface_off[q] ? 1 : 0;
         const int a = wl >> 1, side = wl & 1, o1 = (a + 1) % 3, o2 = (a + 2) % 3;
         const int j = bf - in.wface_off[wl];
-        const int no1 = in.n[o1];
-        const int jq = (int)udiv((unsigned)j, (unsigned)no1, A.mag[2 * A.n_inst + 3 * k + a]);
-        int f[3] = {0, 0, 0};
-        put(f, a, side ? in.n[a] : 0);
-        put(f, o1, j - jq * no1);
-        put(f, o2, jq);
-        Real u_n, u_phi = (Real)0.5;
+        const Real mn = sqrt(u_m);
+        const Real nrm = side ? -mn : mn;
         if (DIM == 1) {
-          u_n = word_uniform<Real>(st.buf.x);
+          x[0] = mul_rn(int_to_real<Real>(side ? n0 : 0), cell_h<Real>(in, 0));
+          s[0] = nrm;
         } else if (DIM == 2) {
-          const int t = (o1 < 2) ? o1 : o2;
-          put(x, t, (int_to_real<Real>(pick(f, t)) + word_uniform<Real>(st.buf.x)) * cell_h<Real>(in, t));
-          u_n = word_uniform<Real>(st.buf.y);
-          u_phi = word_uniform<Real>(st.buf.z);
+          // the faces of a wall run along the other axis
+          const Real tang = mul_rn(int_to_real<Real>(j) + word_uniform<Real>(wx), a == 0 ? cell_h<Real>(in, 1) : cell_h<Real>(in, 0));
+          const Real edge = mul_rn(int_to_real<Real>(side ? (a == 0 ? n0 : n1) : 0), a == 0 ? cell_h<Real>(in, 0) : cell_h<Real>(in, 1));
+          x[0] = a == 0 ? edge : tang;
+          x[1] = a == 0 ? tang : edge;
+          s[0] = a == 0 ? nrm : sn * sp;
+          s[1] = a == 0 ? sn * cp : nrm;
         } else {
+          const int no1 = in.n[o1];
+          const int jq = (int)udiv((unsigned)j, (unsigned)no1, A.mag[2 * A.n_inst + 3 * k + a]);
+          int f[3] = {0, 0, 0};
+          put(f, a, side ? in.n[a] : 0);
+          put(f, o1, j - jq * no1);
+          put(f, o2, jq);
           const int t0 = o1 < o2 ? o1 : o2, t1 = o1 < o2 ? o2 : o1;
-          put(x, t0, (int_to_real<Real>(pick(f, t0)) + word_uniform<Real>(st.buf.x)) * cell_h<Real>(in, t0));
-          put(x, t1, (int_to_real<Real>(pick(f, t1)) + word_uniform<Real>(st.buf.y)) * cell_h<Real>(in, t1));
-          u_n = word_uniform<Real>(st.buf.z);
-          u_phi = word_uniform<Real>(st.buf.w);
-        }
-        put(x, a, int_to_real<Real>(pick(f, a)) * cell_h<Real>(in, a));
-        const Real mn = sqrt(u_n);
-        put(s, a, side ? -mn : mn);
-        if (DIM >= 2) {
-          const Real stn = sqrt((Real)1 - u_n);
-          Real sp, cp;
-          RealTraits<Real>::sincos2pi(u_phi, &sp, &cp);
-          put(s, o1, stn * cp);
-          put(s, o2, stn * sp);
-        } else {
-          put(s, o1, (Real)0);
-          put(s, o2, (Real)0);
+          put(x, t0, mul_rn(int_to_real<Real>(pick(f, t0)) + word_uniform<Real>(wx), cell_h<Real>(in, t0)));
+          put(x, t1, mul_rn(int_to_real<Real>(pick(f, t1)) + word_uniform<Real>(wy), cell_h<Real>(in, t1)));
+          put(x, a, mul_rn(int_to_real<Real>(pick(f, a)), cell_h<Real>(in, a)));
+          put(s, a, nrm);
+          put(s, o1, sn * cp);
+          put(s, o2, sn * sp);
         }
         st.j = wall_uniforms(DIM);
       }
@@ -342,8 +351,8 @@ __global__ void __launch_bounds__(PERS_NT, 4) persistent_step_kernel(PArgs A) {
       wacc[wl * PERS_NT + threadIdx.x] += w;
       const int a = wl >> 1, o1 = (a + 1) % 3, o2 = (a + 2) % 3;
       int j1 = 0, j2 = 0;
-      if (o1 < DIM) j1 = min(floor_nonneg<Real>(quot<Real>(pick(x, o1) + tw * pick(s, o1), cell_h<Real>(in, o1))), in.n[o1] - 1);
-      if (o2 < DIM) j2 = min(floor_nonneg<Real>(quot<Real>(pick(x, o2) + tw * pick(s, o2), cell_h<Real>(in, o2))), in.n[o2] - 1);
+      if (o1 < DIM) j1 = min(floor_nonneg<Real>(quot<Real>(fma_rn(tw, pick(s, o1), pick(x, o1)), cell_h<Real>(in, o1))), in.n[o1] - 1);
+      if (o2 < DIM) j2 = min(floor_nonneg<Real>(quot<Real>(fma_rn(tw, pick(s, o2), pick(x, o2)), cell_h<Real>(in, o2))), in.n[o2] - 1);
       const int bf = in.wface_off[wl] + j2 * in.n[o1] + j1;
       h = in.ncells + bf;
       atomicAdd(&A.f_new[(long long)lane * A.n_fhomes + fbase + bf], 1u);
@@ -351,7 +360,7 @@ __global__ void __launch_bounds__(PERS_NT, 4) persistent_step_kernel(PArgs A) {
       int ci[3] = {0, 0, 0};
 #pragma unroll
       for (int a = 0; a < DIM; ++a) {
-        x[a] += ell * s[a];
+        x[a] = fma_rn(ell, s[a], x[a]);
         ci[a] = min(floor_nonneg<Real>(quot<Real>(x[a], cell_h<Real>(in, a))), in.n[a] - 1);
       }
       const int c = ci[0] + n0 * (ci[1] + n1 * ci[2]);
@@ -371,12 +380,14 @@ __global__ void __launch_bounds__(PERS_NT, 4) persistent_step_kernel(PArgs A) {
         due = 0u;  // step (6): same direction and weight, a new path next iteration
       }
     }
+    if (!due) {
 #pragma unroll
-    for (int a = 0; a < DIM; ++a) {
-      __stcs(px + a * ns + i, x[a]);
-      __stcs(px + (3 + a) * ns + i, s[a]);
+      for (int a = 0; a < DIM; ++a) {
+        __stcs(px + a * ns + i, x[a]);
+        if (was_due) __stcs(px + (3 + a) * ns + i, s[a]);
+      }
+      if (was_due) __stcs(A.pw + i, w);
     }
-    __stcs(A.pw + i, w);
     __stcs(A.home + i, (unsigned)h | due);
   }
   flush_wall_sums<NW>(wacc, k_acc, wall_shared, swall, A.wall, lane);
@@ -409,12 +420,16 @@ __global__ void persistent_finish_W_kernel(const InstDesc* inst, int n_inst, int
 
 // Power per particle re-emitted from each (band, home) this iteration: the home's power
 // (C_b T_emit V / tau_b for a cell, C_b v_b T_face A / 4 for a boundary face) over the
-// particles that ended there in the previous iteration (0 where none did).
+// particles that ended there in the previous iteration (0 where none did). The step's outputs and
+// the counts it makes are cleared in the same launch (P).
 __global__ void persistent_home_power_kernel(const InstDesc* inst, int n_inst, int nb, const long long* home_off,
                                              const long long* nband, const long long* nwall, const double* T,
                                              const double* srcshift, const double* coef, const double* wcoef,
                                              const double* wallTf, const unsigned* n_prev, const unsigned* f_prev,
-                                             long long n_fhomes, double* home_w, long long n_homes) {
+                                             long long n_fhomes, double* home_w, long long n_homes, PrologueArgs P) {
+  for (int q = 0; q < P.n_clear; ++q)
+    for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < P.words[q]; j += (long long)gridDim.x * blockDim.x)
+      P.clear[q][j] = 0ull;
   for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n_homes;
        j += (long long)gridDim.x * blockDim.x) {
     int k = 0;
@@ -479,8 +494,9 @@ cudaError_t launch_persistent_step(const Ctx* c, const double* T, unsigned it, d
   a.home_w = c->d_phome_w;
   a.band = c->d_pband;
   a.home = reinterpret_cast<unsigned*>(c->d_phome);
-  a.n_prev = c->d_pcount + (c->pers_parity ? c->pers_homes : 0);
-  a.n_new = c->d_pcount + (c->pers_parity ? 0 : c->pers_homes);
+  const long long half = (c->pers_homes + 1) & ~1ll;  // each half of d_pcount is padded to 8 bytes
+  a.n_prev = c->d_pcount + (c->pers_parity ? half : 0);
+  a.n_new = c->d_pcount + (c->pers_parity ? 0 : half);
   a.n_fhomes = c->pers_homes - (long long)c->nb * c->total_cells;
   const long long fr = (long long)PERS_FACE_REPLICAS * a.n_fhomes;
   const unsigned* f_prev = c->d_pfcount + (c->pers_parity ? fr : 0);
@@ -493,10 +509,22 @@ cudaError_t launch_persistent_step(const Ctx* c, const double* T, unsigned it, d
   a.it = it;
   a.n_slots = c->pers_n;
   {
+    PrologueArgs P = {};
+    auto clear = [&](void* p, size_t words) {
+      P.clear[P.n_clear] = reinterpret_cast<unsigned long long*>(p);
+      P.words[P.n_clear++] = (long long)words;
+    };
+    const size_t bc = (size_t)c->nb * c->total_cells;
+    clear(R, bc);
+    if (!c->all_real_all) clear(W, bc);  // else W = tau_maj R afterwards
+    clear(wall, (size_t)c->total_walls);
+    clear(counters, CNT_N);
+    clear(a.f_new, (size_t)(fr / 2));        // 32 copies: an even number of words
+    clear(a.n_new, (size_t)((c->pers_homes + 1) / 2));  // the halves are padded to 8 bytes
     const unsigned hb = (unsigned)std::min<long long>((c->pers_homes + 255) / 256 + 1, (long long)c->sm_count * 16);
     persistent_home_power_kernel<<<hb, 256, 0, s>>>(c->d_inst, c->n_inst, c->nb, c->d_phome_off, c->d_pnband,
                                                     c->d_pnwall, T, c->d_srcshift, c->d_coef, c->d_wcoef, c->d_wallTf,
-                                                    a.n_prev, f_prev, a.n_fhomes, c->d_phome_w, c->pers_homes);
+                                                    a.n_prev, f_prev, a.n_fhomes, c->d_phome_w, c->pers_homes, P);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
@@ -528,29 +556,37 @@ namespace {
 // every home counted with its own number of slots.
 __global__ void persistent_init_kernel(const InstDesc* inst, int n_inst, int nb, const long long* slot_off,
                                        const long long* home_off, const long long* nband, const long long* nwall,
-                                       long long n_slots, long long n_homes, double* state, int* band, unsigned* home,
+                                       long long n_slots, long long n_homes, int* band, unsigned* home,
                                        unsigned* count_prev, unsigned* fcount_prev) {
   const long long stride = (long long)gridDim.x * blockDim.x;
+  // a thread's slots only grow, so its instance, band and run of equal homes only move on (slots
+  // and homes are below 2^31: 32-bit divisions)
+  int k = -1, b = 0;
+  bool walls = false;
+  long long inst_end = 0, run_beg = 0, run_end = 0;
+  unsigned homes = 1;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n_slots; i += stride) {
-    int k = 0;
-    while (k + 1 < n_inst && slot_off[k + 1] <= i) ++k;
-    const InstDesc& in = inst[k];
-    long long r = i - slot_off[k];
-    int b = 0, h = 0;
-    long long thermal = 0;
-    for (int bb = 0; bb < nb; ++bb) thermal += nband[(long long)k * nb + bb] * in.ncells;
-    if (r < thermal) {
-      while (r >= nband[(long long)k * nb + b] * in.ncells) r -= nband[(long long)k * nb + b] * in.ncells, ++b;
-      h = (int)(r % in.ncells);
-    } else {
-      r -= thermal;
-      const long long nbf = (home_off[k + 1] - home_off[k]) / nb - in.ncells;
-      while (r >= nwall[b] * nbf) r -= nwall[b] * nbf, ++b;
-      h = in.ncells + (int)(r % nbf);
+    while (i >= run_end) {
+      if (i >= inst_end) {  // the next instance's first run: band 0 of its cells
+        ++k;
+        run_beg = inst_end;
+        inst_end = slot_off[k + 1];
+        b = 0;
+        walls = false;
+      } else {
+        run_beg = run_end;
+        if (++b == nb) {
+          b = 0;
+          walls = true;
+        }
+      }
+      const long long nbf = (home_off[k + 1] - home_off[k]) / nb - inst[k].ncells;
+      homes = (unsigned)(walls ? nbf : inst[k].ncells);
+      run_end = run_beg + (walls ? nwall[b] : nband[(long long)k * nb + b]) * homes;
     }
-    band[i] = b;
-    home[i] = (unsigned)h | DUE_BIT;
-    for (int q = 0; q < 7; ++q) state[q * n_slots + i] = 0.0;
+    const unsigned h = (unsigned)(i - run_beg) % homes + (walls ? (unsigned)inst[k].ncells : 0u);
+    if (nb > 1) band[i] = b;
+    home[i] = h | DUE_BIT;  // due: position, direction and weight come with the emission
   }
   for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n_homes; j += stride) {
     int k = 0;
@@ -571,7 +607,7 @@ __global__ void persistent_init_kernel(const InstDesc* inst, int n_inst, int nb,
 cudaError_t launch_persistent_init(Ctx* c, cudaStream_t s) {
   const unsigned blocks = (unsigned)std::min<long long>((c->pers_n + 255) / 256 + 1, (long long)c->sm_count * 16);
   persistent_init_kernel<<<blocks, 256, 0, s>>>(c->d_inst, c->n_inst, c->nb, c->d_pslot_off, c->d_phome_off, c->d_pnband,
-                                                c->d_pnwall, c->pers_n, c->pers_homes, c->d_px, c->d_pband,
+                                                c->d_pnwall, c->pers_n, c->pers_homes, c->d_pband,
                                                 reinterpret_cast<unsigned*>(c->d_phome), c->d_pcount, c->d_pfcount);
   return cudaGetLastError();
 }
