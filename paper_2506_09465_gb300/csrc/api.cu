@@ -264,12 +264,13 @@ void broadcast_wall_T(Ctx* c) {
     }
 }
 
-// Tasks of the pass-synchronous 2D sweep over the forward groups, for the options' warp_grab.
+// Tasks, band by band, of the pass-synchronous 2D sweep (for the options' warp_grab) and of the
+// filtered FP64 sweep over the forward groups.
 iugkp_status build_sync_tasks(Ctx* c) {
-  if (c->dim != 2) return IUGKP_OK;
+  if (c->dim != 2 && c->opt.precision != IUGKP_TRACK_FP64) return IUGKP_OK;
   const int grab = c->opt.warp_grab > 0 ? c->opt.warp_grab : 256;
   std::vector<LandGroup> lg;
-  land_tasks(c, c->h_groups_fwd, lg, c->sync_tasks, c->sync_qch, std::max(1, grab / 32), STAGED_NT / 32);
+  land_tasks(c, c->h_groups_fwd, lg, c->sync_tasks, c->sync_qch, std::max(1, grab / 32), STAGED_NT / 32, false);
   if (c->fwd_particles == 0) c->sync_tasks = 0;
   std::vector<long long> beg(c->n_inst, 0);
   std::vector<unsigned> end(c->n_inst, 0);
@@ -376,7 +377,7 @@ iugkp_status rebuild_forward_groups(Ctx* c) {
   c->d_group_mag = nullptr;
   if ((s = upload(c, &c->d_group_mag, gmag)) != IUGKP_OK) return s;
   std::vector<LandGroup> lg;
-  land_tasks(c, c->h_groups_fwd, lg, c->land_fwd_tasks, c->land_fwd_qch, LAND_QCH, LAND_WARPS_PER_SM);
+  land_tasks(c, c->h_groups_fwd, lg, c->land_fwd_tasks, c->land_fwd_qch, LAND_QCH, LAND_WARPS_PER_SM, true);
   if (c->fwd_particles == 0) c->land_fwd_tasks = 0;  // the all-zero placeholder group
   if ((s = upload(c, &c->d_land_fwd, lg)) != IUGKP_OK) return s;
   if ((s = build_sync_tasks(c)) != IUGKP_OK) return s;
@@ -781,7 +782,7 @@ iugkp_status iugkp_create_batch(int n, const iugkp_grid* g, const double* const*
     for (const Group& g : c->h_groups_all) gmag.push_back(div_magic(g.n_emitters));
     UP(c->d_all_group_mag, gmag);
     std::vector<LandGroup> lg;
-    land_tasks(c, c->h_groups_all, lg, c->land_all_tasks, c->land_all_qch, LAND_QCH, LAND_WARPS_PER_SM);
+    land_tasks(c, c->h_groups_all, lg, c->land_all_tasks, c->land_all_qch, LAND_QCH, LAND_WARPS_PER_SM, true);
     UP(c->d_land_all, lg);
   }
   {

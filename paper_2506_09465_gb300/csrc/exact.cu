@@ -431,10 +431,10 @@ cudaError_t launch_exact(const Ctx* c, const SweepArgs& a, cudaStream_t s) {
   S.defer_cap = c->defer_cap;
   S.err = c->d_err;
   LandArgs L = {};
-  L.groups = c->d_land_fwd;
+  L.groups = c->d_sync_groups;
   L.n_groups = a.n_groups;
-  L.n_tasks = c->land_fwd_tasks;
-  L.qch = c->land_fwd_qch;
+  L.n_tasks = c->sync_tasks;
+  L.qch = c->sync_qch;
   L.next = reinterpret_cast<unsigned long long*>(c->d_defer_n + 2);
   ExactArgs X = {};
   X.items = c->d_items;

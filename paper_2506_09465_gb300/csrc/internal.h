@@ -194,8 +194,8 @@ struct Ctx {
   uint2* d_defer = nullptr;
   unsigned* d_defer_n = nullptr;     // [4] queue length, queued faces (exact.cu), 64-bit claim counter (land.cu, exact.cu)
   unsigned defer_cap = 0;
-  // tasks of the pass-synchronous 2D sweep (as many particles per emitter and task as warp_grab
-  // allows): the groups', and each instance's range
+  // tasks of the pass-synchronous 2D sweep and of the filtered FP64 sweep (as many particles per
+  // emitter and task as warp_grab allows): the groups', and each instance's range
   LandGroup* d_sync_groups = nullptr;
   long long* d_sync_beg = nullptr;
   unsigned* d_sync_end = nullptr;
@@ -250,7 +250,7 @@ cudaError_t launch_close_2d(const Ctx* c, const SweepArgs& a, cudaStream_t s);
 cudaError_t launch_close_3d(const Ctx* c, const SweepArgs& a, cudaStream_t s);
 cudaError_t launch_land(const Ctx* c, const SweepArgs& a, bool adj, cudaStream_t s);
 void land_tasks(const Ctx* c, const std::vector<Group>& groups, std::vector<LandGroup>& out, unsigned& n_tasks, int& qch,
-                int qch_max, int warps_per_sm);
+                int qch_max, int warps_per_sm, bool join);
 cudaError_t launch_replay(const Ctx* c, const SweepArgs& a, const StagedArgs& S, cudaStream_t s);
 cudaError_t launch_adjoint_replay(const Ctx* c, const SweepArgs& a, cudaStream_t s);
 cudaError_t launch_walk_bounds(unsigned long long* out, cudaStream_t s);

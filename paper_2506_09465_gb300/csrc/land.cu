@@ -25,10 +25,11 @@ __device__ __forceinline__ void deposit(const SweepArgs& A, const StagedArgs& S,
 }
 
 // Bands whose every candidate is real: one candidate per particle, no chain. A lane keeps its
-// emitter for qch particles in a row, so the cell coordinates, the weight, the first Philox
-// rounds (the counter's emitter word does not change) and, in the adjoint, the gathered sum stay
-// in registers; the lanes of a warp hold neighbouring emitters. Tasks (a tile of emitters x a
-// run of particle numbers) are claimed one at a time by each warp.
+// emitter for qch particles in a row (over its bands in turn: with tens of bands an emitter has
+// only a few particles in each), so the cell coordinates, the weight, the first Philox rounds (the
+// counter's emitter word does not change) and, in the adjoint, the gathered sum stay in registers;
+// the lanes of a warp hold neighbouring emitters. Tasks (a tile of emitters x a run of particle
+// numbers) are claimed one at a time by each warp.
 template <int DIM, bool ADJ, bool K32>
 __global__ void __launch_bounds__(LAND_NT) land_kernel(SweepArgs A, StagedArgs S, LandArgs L) {
   const int lane = threadIdx.x & 31;
@@ -39,51 +40,68 @@ __global__ void __launch_bounds__(LAND_NT) land_kernel(SweepArgs A, StagedArgs S
     task = __shfl_sync(0xffffffffu, task, 0);
     if (task >= L.n_tasks) return;
     tg.find(L, task);
-    const LandGroup& G = L.groups[tg.gi];
+    int gi = tg.gi;
     const unsigned t = task - tg.t_beg;
-    const int qc = (int)(t / (unsigned)G.ntile), tile = (int)(t - (unsigned)qc * (unsigned)G.ntile);
-    const InstDesc& in = A.inst[G.inst];
+    const int ntile = L.groups[gi].ntile, reps = L.groups[gi].reps, kind = L.groups[gi].kind;
+    const int qc = (int)(t / (unsigned)ntile), tile = (int)(t - (unsigned)qc * (unsigned)ntile);
+    int pass = qc * L.qch;
+    const int pass_end = pass + L.qch;
+    // the chain's first band with passes left
+    while (L.groups[gi].next >= 0 && L.groups[L.groups[gi].next].pass0 <= pass) gi = L.groups[gi].next;
+    const InstDesc& in = A.inst[L.groups[gi].inst];
     LaneEmitter<DIM> em;
-    em.template init<ADJ>(A, S, G, in, tile, lane);
+    em.template init<ADJ>(A, S, L.groups[gi], in, tile, lane);
     const int n0 = in.n[0], n1 = in.n[1];
-    const float vtm = A.vtm32[G.inst * A.nb + G.band], va = vtm * TIE_LOG_ABS;
-    const long long bcbase = in.bc_off + (long long)G.band * in.ncells, coff = in.cell_off;
+    const long long coff = in.cell_off;
     const uint32_t inst_id = in.inst_id;
-    double acc = 0.0;
-    const int qbeg = qc * (L.qch * G.reps) + em.sub, qend = min(G.per, (qc + 1) * (L.qch * G.reps));
-    for (int q = em.on ? qbeg : qend; q < qend; q += G.reps) {
-      Stream st;
-      st.init(A.seed, inst_id, (uint32_t)G.band, A.epoch, em.id, (uint32_t)q);
-      float xi[3], s[3];
-      emit_segment<DIM>(st, G.kind, xi, s);
-      const float D = __fmul_rn(-__logf(word_uniform<float>(st.first)), vtm);
-      const float eD = fmaf(D, TIE_LOG_REL, va), rel = fmaf(D, LAND_REL, eD);
-      bool out = false, near = false;
-      int o[3] = {0, 0, 0};
+    double gather = 0.0;
+    for (;;) {
+      const LandGroup& G = L.groups[gi];
+      const int band = G.band, per = G.per, next = G.next;
+      const unsigned first = G.first;
+      const float vtm = A.vtm32[G.inst * A.nb + band], va = vtm * TIE_LOG_ABS;
+      const long long bcbase = in.bc_off + (long long)band * in.ncells;
+      const int band_end = next >= 0 ? min(pass_end, L.groups[next].pass0) : pass_end;
+      double acc = 0.0;
+      const int qend = em.on ? min(per, (band_end - G.pass0) * reps) : 0;
+      for (int q = (pass - G.pass0) * reps + em.sub; q < qend; q += reps) {
+        Stream st;
+        st.init(A.seed, inst_id, (uint32_t)band, A.epoch, em.id, (uint32_t)q);
+        float xi[3], s[3];
+        emit_segment<DIM>(st, kind, xi, s);
+        const float D = __fmul_rn(-__logf(word_uniform<float>(st.first)), vtm);
+        const float eD = fmaf(D, TIE_LOG_REL, va), rel = fmaf(D, LAND_REL, eD);
+        bool out = false, near = false;
+        int o[3] = {0, 0, 0};
 #pragma unroll
-      for (int a = 0; a < DIM; ++a) {
-        const float g = s[a] * em.ih[a];
-        const float X = fmaf(g, D, xi[a]), tol = fmaf(fabsf(g), rel, LAND_ABS);
-        out |= em.lo[a] - X > tol || X - em.hi[a] > tol;  // beyond a wall for the FP64 walk too
-        o[a] = floor_near(X, tol, near);
+        for (int a = 0; a < DIM; ++a) {
+          const float g = s[a] * em.ih[a];
+          const float X = fmaf(g, D, xi[a]), tol = fmaf(fabsf(g), rel, LAND_ABS);
+          out |= em.lo[a] - X > tol || X - em.hi[a] > tol;  // beyond a wall for the FP64 walk too
+          o[a] = floor_near(X, tol, near);
+        }
+        if (out) continue;
+        if (near) {
+          defer_particle(S, first + (unsigned)q * (unsigned)L.groups[gi].ne + (unsigned)em.rank, 0u);
+          continue;
+        }
+        const int cell = em.cell0 + o[0] + (DIM >= 2 ? n0 * o[1] : 0) + (DIM == 3 ? n0 * n1 * o[2] : 0);
+        if (ADJ) acc += L.lamVm[coff + cell];
+        else deposit<K32>(A, S, bcbase + cell, em.w);
       }
-      if (out) continue;
-      if (near) {
-        defer_particle(S, G.first + (unsigned)q * (unsigned)G.ne + (unsigned)em.rank, 0u);
-        continue;
-      }
-      const int cell = em.cell0 + o[0] + (DIM >= 2 ? n0 * o[1] : 0) + (DIM == 3 ? n0 * n1 * o[2] : 0);
-      if (ADJ) acc += L.lamVm[coff + cell];
-      else deposit<K32>(A, S, bcbase + cell, em.w);
+      if (ADJ && em.on) gather = fma(acc, em.w, gather);
+      pass = band_end;
+      if (next < 0 || pass >= pass_end) break;
+      gi = next;
+      em.template weight<ADJ>(A, L.groups[gi], in);
     }
     if (ADJ) {
-      acc *= em.w;
-      if (G.kind == 0) {
-        if (acc != 0.0) atomicAdd(&A.adj_out[coff + em.e], acc);
+      if (kind == 0) {
+        if (gather != 0.0) atomicAdd(&A.adj_out[coff + em.e], gather);
       } else {
 #pragma unroll
-        for (int d = 16; d > 0; d >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, d);
-        if (lane == 0 && acc != 0.0) atomicAdd(&A.adj_wall[in.wall_off + G.kind - 1], acc);
+        for (int d = 16; d > 0; d >>= 1) gather += __shfl_down_sync(0xffffffffu, gather, d);
+        if (lane == 0 && gather != 0.0) atomicAdd(&A.adj_wall[in.wall_off + kind - 1], gather);
       }
     }
   }
@@ -356,13 +374,15 @@ cudaError_t launch_land(const Ctx* c, const SweepArgs& a, bool adj, cudaStream_t
 // Tasks of a sweep over a group list: tiles of at most 32 emitters (equal widths;
 // narrow groups put several particles of an emitter side by side), qch particles per emitter and
 // task: at most qch_max, fewer where that would leave warps without work.
+// join: the groups of one instance and kind over its bands form a chain whose passes are numbered
+// through (where all of them visit their emitters in emitter order); only a chain's first group
+// has tasks then.
 void land_tasks(const Ctx* c, const std::vector<Group>& groups, std::vector<LandGroup>& out, unsigned& n_tasks, int& qch,
-                int qch_max, int warps_per_sm) {
+                int qch_max, int warps_per_sm, bool join) {
   long long total = 0;
   for (const Group& g : groups) total += (long long)g.n_emitters * g.per_emitter;
   const long long warps = (long long)std::max(1, c->sm_count) * warps_per_sm;
   qch = (int)std::max<long long>(1, std::min<long long>(qch_max, total / (32 * 4 * warps)));
-  long long t0 = 0;
   out.clear();
   for (const Group& g : groups) {
     LandGroup l;
@@ -376,10 +396,41 @@ void land_tasks(const Ctx* c, const std::vector<Group>& groups, std::vector<Land
     l.ntile = (g.n_emitters + 31) / 32;
     l.tw = (g.n_emitters + l.ntile - 1) / l.ntile;
     l.reps = 32 / l.tw;
-    l.task0 = (unsigned)t0;
-    const long long run = (long long)qch * l.reps;
-    t0 += (long long)l.ntile * ((l.per + run - 1) / run);
+    l.next = -1;
+    l.pass0 = 0;
     out.push_back(l);
+  }
+  std::vector<long long> passes(out.size());
+  std::vector<char> joined(out.size(), 0);
+  for (size_t g = 0; g < out.size(); ++g) passes[g] = (out[g].per + out[g].reps - 1) / out[g].reps;
+  if (join) {
+    for (size_t g0 = 0; g0 < out.size();) {  // one instance at a time
+      size_t g1 = g0;
+      while (g1 < out.size() && out[g1].inst == out[g0].inst) ++g1;
+      std::vector<int> last(7, -1);
+      std::vector<size_t> head(7, 0);
+      for (size_t g = g0; g < g1; ++g) {
+        const int k = out[g].kind;
+        if (out[g].perm_off >= 0) continue;
+        if (last[k] >= 0) {
+          out[last[k]].next = (int)g;
+          out[g].pass0 = (int)passes[head[k]];
+          passes[head[k]] += passes[g];
+          joined[g] = 1;
+        } else {
+          head[k] = g;
+        }
+        last[k] = (int)g;
+      }
+      g0 = g1;
+    }
+  }
+  // a chained group gets no tasks (the search for a task's group takes the last group that starts at
+  // or before it: never one whose start is the next head's)
+  long long t0 = 0;
+  for (size_t g = 0; g < out.size(); ++g) {
+    out[g].task0 = (unsigned)t0;
+    if (!joined[g]) t0 += (long long)out[g].ntile * ((passes[g] + qch - 1) / qch);
   }
   n_tasks = (unsigned)t0;
 }

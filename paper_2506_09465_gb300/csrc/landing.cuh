@@ -159,18 +159,12 @@ struct LaneEmitter {
   int rank, e, sub, cell0;
   uint32_t id;
   double w;
-  bool on;
+  bool has, on;
   float ih[3], lo[3], hi[3];
   int c[3];
+  // The emitter's weight in the group's band.
   template <bool ADJ>
-  __device__ __forceinline__ void init(const SweepArgs& A, const StagedArgs& S, const LandGroup& G, const InstDesc& in,
-                                       int tile, int lane) {
-    sub = lane / G.tw;
-    rank = tile * G.tw + lane - sub * G.tw;
-    on = sub < G.reps && rank < G.ne;
-    e = on ? rank : 0;
-    if (G.perm_off >= 0) e = A.perm[G.perm_off + e];
-    emitter_cell<DIM>(in, S, G.inst, G.kind, e, c, id);
+  __device__ __forceinline__ void weight(const SweepArgs& A, const LandGroup& G, const InstDesc& in) {
     if (G.kind == 0) {
       w = A.coef[in.bc_off + (long long)G.band * in.ncells + e];
       if (!ADJ) {
@@ -182,7 +176,18 @@ struct LaneEmitter {
       w = A.wcoef[(long long)(G.inst * A.nb + G.band) * 6 + G.kind - 1];
       if (!ADJ) w *= A.wallTf[in.bface_off + in.wface_off[G.kind - 1] + e];
     }
-    on = on && (__double_as_longlong(w) << 1) != 0;  // +-0: nothing to trace
+    on = has && (__double_as_longlong(w) << 1) != 0;  // +-0: nothing to trace
+  }
+  template <bool ADJ>
+  __device__ __forceinline__ void init(const SweepArgs& A, const StagedArgs& S, const LandGroup& G, const InstDesc& in,
+                                       int tile, int lane) {
+    sub = lane / G.tw;
+    rank = tile * G.tw + lane - sub * G.tw;
+    has = sub < G.reps && rank < G.ne;
+    e = has ? rank : 0;
+    if (G.perm_off >= 0) e = A.perm[G.perm_off + e];
+    emitter_cell<DIM>(in, S, G.inst, G.kind, e, c, id);
+    weight<ADJ>(A, G, in);
     const int n0 = in.n[0], n1 = in.n[1], n2 = in.n[2];
 #pragma unroll
     for (int a = 0; a < DIM; ++a) {

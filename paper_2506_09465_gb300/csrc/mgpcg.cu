@@ -357,83 +357,100 @@ __device__ void vcycle(const MGArgs& A, const InstMG& m, cg::cluster_group& cl, 
 // barrier. The solve runs inside FP64 iterative refinement: the solution is accumulated in
 // FP64 and its residual S - A X is formed with the FP64 operator, until it meets rtol.
 
-// Tiles of the dense products: FDT_BM rows x FDT_BN columns of the output per tile (each of
-// the 512 threads 4 rows x 4 columns, from one float4 of each operand per term), FDT_BK terms
-// per stage; the next stage's operands are loaded into registers while the current stage is
-// multiplied from shared memory. Shared rows are padded by 4 words (16-byte aligned float4
+// Tiles of the dense products: BM rows x FDT_BN columns of the output per tile (each of the 512
+// threads BM / 16 rows x 4 columns, from one vector of each operand per term), FDT_BK terms per
+// stage; the next stage's operands are loaded into registers while the current stage is
+// multiplied from shared memory. BM is 32 where a CTA's rows fit (axes up to 256 cells: with 64
+// more than half of the products of a 192-cell axis were of padding), else 64; an output's terms
+// are summed in the same order either way. Shared rows are padded by 4 words (16-byte aligned
 // reads, at most 2-way conflicts on the transposing stores).
-constexpr int FDT_BM = 64, FDT_BN = 128, FDT_BK = 16;
-constexpr int FDT_AS = FDT_BM + 4, FDT_BS = FDT_BN + 4;
+constexpr int FDT_BM_MAX = 64, FDT_BN = 128, FDT_BK = 16;
+constexpr int FDT_AS = FDT_BM_MAX + 4, FDT_BS = FDT_BN + 4;
 
 // out(j, i) for rows j in [j0, j1) and columns i < N of sum over k < K of L(j, k) R(k, i).
 // L_KC: L is contiguous along k (else along j); R_IC: R is contiguous along i (else along
 // k); the tile loads run along the contiguous index.
-template <int NT, bool L_KC, bool R_IC, class FL, class FR, class FE>
+template <int NT, int BM, bool L_KC, bool R_IC, class FL, class FR, class FE>
 __device__ __forceinline__ void tile_product(int j0, int j1, int N, int K, FL L, FR R, FE out, float* As,
                                              float* Bs) {
-  static_assert(NT == 512, "4 x 4 outputs per thread: 512 threads = 16 x 32 groups");
-  constexpr int NA = FDT_BK * FDT_BM / NT, NB = FDT_BK * FDT_BN / NT;  // loads per thread and stage
+  static_assert(NT == 512 && (BM == 32 || BM == 64), "512 threads = 16 x 32 groups of BM / 16 x 4 outputs");
+  constexpr int NR = BM / 16;
+  constexpr int NA = FDT_BK * BM / NT, NB = FDT_BK * FDT_BN / NT;  // loads per thread and stage
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  for (int jt = j0; jt < j1; jt += FDT_BM) {
+  for (int jt = j0; jt < j1; jt += BM) {
     for (int it = 0; it < N; it += FDT_BN) {
-      float acc[4][4];
+      float acc[NR][4];
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
+      for (int r = 0; r < NR; ++r)
 #pragma unroll
         for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
-      float ra[NA], rb[NB];
-      auto load = [&](int kt) {
+      // two register sets: a stage's operands are loaded two stages before they are multiplied (an
+      // L2 round trip is longer than one stage's products)
+      float ra[2][NA], rb[2][NB];
+      auto load = [&](int kt, float(&a)[NA], float(&b)[NB]) {
 #pragma unroll
         for (int q = 0; q < NA; ++q) {
           const int e = threadIdx.x + q * NT;
-          const int kk = L_KC ? e % FDT_BK : e / FDT_BM, jj = L_KC ? e / FDT_BK : e % FDT_BM;
-          ra[q] = (jt + jj < j1 && kt + kk < K) ? L(jt + jj, kt + kk) : 0.f;
+          const int kk = L_KC ? e % FDT_BK : e / BM, jj = L_KC ? e / FDT_BK : e % BM;
+          a[q] = (jt + jj < j1 && kt + kk < K) ? L(jt + jj, kt + kk) : 0.f;
         }
 #pragma unroll
         for (int q = 0; q < NB; ++q) {
           const int e = threadIdx.x + q * NT;
           const int kk = R_IC ? e / FDT_BN : e % FDT_BK, ii = R_IC ? e % FDT_BN : e / FDT_BK;
-          rb[q] = (kt + kk < K && it + ii < N) ? R(kt + kk, it + ii) : 0.f;
+          b[q] = (kt + kk < K && it + ii < N) ? R(kt + kk, it + ii) : 0.f;
         }
       };
-      auto store = [&](int buf) {
+      auto store = [&](int buf, const float(&a)[NA], const float(&b)[NB]) {
 #pragma unroll
         for (int q = 0; q < NA; ++q) {
           const int e = threadIdx.x + q * NT;
-          const int kk = L_KC ? e % FDT_BK : e / FDT_BM, jj = L_KC ? e / FDT_BK : e % FDT_BM;
-          As[(buf * FDT_BK + kk) * FDT_AS + jj] = ra[q];
+          const int kk = L_KC ? e % FDT_BK : e / BM, jj = L_KC ? e / FDT_BK : e % BM;
+          As[(buf * FDT_BK + kk) * FDT_AS + jj] = a[q];
         }
 #pragma unroll
         for (int q = 0; q < NB; ++q) {
           const int e = threadIdx.x + q * NT;
           const int kk = R_IC ? e / FDT_BN : e % FDT_BK, ii = R_IC ? e % FDT_BN : e / FDT_BK;
-          Bs[(buf * FDT_BK + kk) * FDT_BS + ii] = rb[q];
+          Bs[(buf * FDT_BK + kk) * FDT_BS + ii] = b[q];
         }
       };
-      load(0);
-      store(0);
-      __syncthreads();
-      int buf = 0;
-      for (int kt = 0; kt < K; kt += FDT_BK) {
-        const bool more = kt + FDT_BK < K;
-        if (more) load(kt + FDT_BK);
+      // one stage: multiply buffer `buf`, load the stage after next into the set it came from, store
+      // the next stage's set into the other buffer
+      auto stage = [&](int kt, int buf, float(&a_far)[NA], float(&b_far)[NB], const float(&a_next)[NA],
+                       const float(&b_next)[NB]) {
+        if (kt + 2 * FDT_BK < K) load(kt + 2 * FDT_BK, a_far, b_far);
 #pragma unroll
         for (int k = 0; k < FDT_BK; ++k) {
-          const float4 a = *reinterpret_cast<const float4*>(&As[(buf * FDT_BK + k) * FDT_AS + 4 * ty]);
+          float av[NR];
+          if constexpr (NR == 4) {
+            const float4 a = *reinterpret_cast<const float4*>(&As[(buf * FDT_BK + k) * FDT_AS + 4 * ty]);
+            av[0] = a.x, av[1] = a.y, av[2] = a.z, av[3] = a.w;
+          } else {
+            const float2 a = *reinterpret_cast<const float2*>(&As[(buf * FDT_BK + k) * FDT_AS + 2 * ty]);
+            av[0] = a.x, av[1] = a.y;
+          }
           const float4 b = *reinterpret_cast<const float4*>(&Bs[(buf * FDT_BK + k) * FDT_BS + 4 * tx]);
-          const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+          const float bv[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
-          for (int r = 0; r < 4; ++r)
+          for (int r = 0; r < NR; ++r)
 #pragma unroll
             for (int c = 0; c < 4; ++c) acc[r][c] = fmaf(av[r], bv[c], acc[r][c]);
         }
-        if (more) store(buf ^ 1);
+        if (kt + FDT_BK < K) store(buf ^ 1, a_next, b_next);
         __syncthreads();
-        buf ^= 1;
+      };
+      load(0, ra[0], rb[0]);
+      if (FDT_BK < K) load(FDT_BK, ra[1], rb[1]);
+      store(0, ra[0], rb[0]);
+      __syncthreads();
+      for (int kt = 0; kt < K; kt += 2 * FDT_BK) {
+        stage(kt, 0, ra[0], rb[0], ra[1], rb[1]);
+        if (kt + FDT_BK < K) stage(kt + FDT_BK, 1, ra[1], rb[1], ra[0], rb[0]);
       }
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int j = jt + 4 * ty + r;
+      for (int r = 0; r < NR; ++r) {
+        const int j = jt + NR * ty + r;
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
           const int i = it + 4 * tx + c;
@@ -446,9 +463,9 @@ __device__ __forceinline__ void tile_product(int j0, int j1, int N, int K, FL L,
 
 // Solves the instance's correction by fast diagonalization with FP64 refinement (at most
 // MG32_PASSES_FD passes); returns the passes taken, or -1 if rtol was not met.
-template <int NT, int CS>
+template <int NT, int CS, int BM>
 __device__ int fd_solve(const MGArgs& A, const InstMG& m, cg::cluster_group& cl, int rank, ClusterRed<NT, CS>& red,
-                        double* sh) {
+                        double* sh, float* As, float* Bs) {
   const int nx = m.fnx, ny = m.fny;
   const long long off = m.cell_off, n = m.nc[0];
   const long long sy = m.n[0][0];
@@ -461,8 +478,6 @@ __device__ int fd_solve(const MGArgs& A, const InstMG& m, cg::cluster_group& cl,
   float* Sf = A.lt + m.off[0];  // scaled residual (FP32)
   float* T1 = A.lb + m.off[0];  // Qy^T S, then Qy T2
   float* T2 = A.lx + m.off[0];  // (Qy^T S Qx) ./ (ly + lx)
-  __shared__ __align__(16) float As[2 * FDT_BK * FDT_AS];
-  __shared__ __align__(16) float Bs[2 * FDT_BK * FDT_BS];
   double v[4];
   v[0] = 0.0;
   for (long long c = lo + threadIdx.x; c < hi; c += NT) {
@@ -481,23 +496,23 @@ __device__ int fd_solve(const MGArgs& A, const InstMG& m, cg::cluster_group& cl,
     for (long long c = lo + threadIdx.x; c < hi; c += NT) Sf[c] = (float)(__ldcg(&A.Z[off + c]) * sc);
     cl.sync();
     // T1 = Qy^T S (rows j of this CTA), then T2 = T1 Qx ./ (ly_j + lx_i) (same rows)
-    tile_product<NT, false, true>(
+    tile_product<NT, BM, false, true>(
         j0, j1, nx, ny, [&](int j, int k) { return __ldg(&Qy[(long long)k * ny + j]); },
         [&](int k, int i) { return __ldcg(&Sf[(long long)k * nx + i]); },
         [&](int j, int i, float x) { T1[(long long)j * nx + i] = x; }, As, Bs);
     __syncthreads();
-    tile_product<NT, true, true>(
+    tile_product<NT, BM, true, true>(
         j0, j1, nx, nx, [&](int j, int k) { return __ldcg(&T1[(long long)j * nx + k]); },
         [&](int k, int i) { return __ldg(&Qx[(long long)k * nx + i]); },
         [&](int j, int i, float x) { T2[(long long)j * nx + i] = x / (ly[j] + lx[i]); }, As, Bs);
     cl.sync();
     // T1 = Qy T2, then the correction T1 Qx^T added to the FP64 solution (scaled back)
-    tile_product<NT, true, true>(
+    tile_product<NT, BM, true, true>(
         j0, j1, nx, ny, [&](int j, int k) { return __ldg(&Qy[(long long)j * ny + k]); },
         [&](int k, int i) { return __ldcg(&T2[(long long)k * nx + i]); },
         [&](int j, int i, float x) { T1[(long long)j * nx + i] = x; }, As, Bs);
     __syncthreads();
-    tile_product<NT, true, false>(
+    tile_product<NT, BM, true, false>(
         j0, j1, nx, nx, [&](int j, int k) { return __ldcg(&T1[(long long)j * nx + k]); },
         [&](int k, int i) { return __ldg(&Qx[(long long)i * nx + k]); },
         [&](int j, int i, float x) { A.X[off + (long long)j * nx + i] += (double)x * rn; }, As, Bs);
@@ -699,8 +714,11 @@ __global__ void __launch_bounds__(NT) mgpcg_kernel(MGArgs A) {
   const long long sy = m.n[0][0], sz = (long long)m.n[0][0] * m.n[0][1];
   ClusterRed<NT, CS> red{slot, 0};
   if (m.direct) {
-    const int passes = m.direct == 2 ? fd_solve_small<NT, CS>(A, m, cl, rank, red, sh, mg_smem)
-                                     : fd_solve<NT, CS>(A, m, cl, rank, red, sh);
+    __shared__ __align__(16) float As[2 * FDT_BK * FDT_AS];
+    __shared__ __align__(16) float Bs[2 * FDT_BK * FDT_BS];
+    const int passes = m.direct == 2       ? fd_solve_small<NT, CS>(A, m, cl, rank, red, sh, mg_smem)
+                       : m.fny <= 32 * CS ? fd_solve<NT, CS, 32>(A, m, cl, rank, red, sh, As, Bs)
+                                          : fd_solve<NT, CS, 64>(A, m, cl, rank, red, sh, As, Bs);
     if (rank == 0 && threadIdx.x == 0) A.iters_out[k] = passes;
     cl.sync();  // no CTA leaves while another may still read its shared memory
     return;
@@ -871,8 +889,11 @@ __global__ void __launch_bounds__(NT, 1) mgpcg32_kernel(MGArgs A, float* V32) {
   const float *dg = A.ldiag + m.off[0], *cx = A.lcx + m.off[0], *cy = A.lcy + m.off[0], *cz = A.lcz + m.off[0];
   ClusterRed<NT, CS> red{slot, 0};
   if (m.direct) {
-    const int passes = m.direct == 2 ? fd_solve_small<NT, CS>(A, m, cl, rank, red, sh, mg_smem)
-                                     : fd_solve<NT, CS>(A, m, cl, rank, red, sh);
+    __shared__ __align__(16) float As[2 * FDT_BK * FDT_AS];
+    __shared__ __align__(16) float Bs[2 * FDT_BK * FDT_BS];
+    const int passes = m.direct == 2       ? fd_solve_small<NT, CS>(A, m, cl, rank, red, sh, mg_smem)
+                       : m.fny <= 32 * CS ? fd_solve<NT, CS, 32>(A, m, cl, rank, red, sh, As, Bs)
+                                          : fd_solve<NT, CS, 64>(A, m, cl, rank, red, sh, As, Bs);
     if (rank == 0 && threadIdx.x == 0) A.iters_out[k] = passes;
     cl.sync();  // no CTA leaves while another may still read its shared memory
     return;

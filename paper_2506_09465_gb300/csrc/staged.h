@@ -125,6 +125,8 @@ struct LandGroup {
   int inst, band, kind, ne, per, perm_off;
   int tw, ntile, reps;
   unsigned task0;
+  int next;                       // group of the next band of the same emitters, or -1 (land_tasks)
+  int pass0;                      // passes of the bands before this one in such a chain
 };
 
 struct LandArgs {
