@@ -130,14 +130,16 @@ void free_all(Ctx* c) {
                   c->d_theta, c->d_theta_m, c->d_diag, c->d_cx, c->d_cy, c->d_cz, c->d_pcg, c->d_work, c->d_T2,
                   c->d_R, c->d_W, c->d_F, c->d_wall, c->d_red, c->d_counters, c->d_work_counter, c->d_err,
                   c->d_pcg_iters, c->d_scalar, c->d_adj, c->d_mg, c->d_mg_diag, c->d_mg_dinv, c->d_mg_cx,
-                  c->d_mg_cy, c->d_mg_cz, c->d_mg_cinv, c->d_mg_b, c->d_mg_x, c->d_mg_t, c->d_mg_r, c->d_fd_q, c->d_fd_lam,
+                  c->d_mg_cy, c->d_mg_cz, c->d_mg_cinv, c->d_mg_b, c->d_mg_x, c->d_mg_t, c->d_fd_q, c->d_fd_lam,
                   c->d_inst_beg, c->d_inst_end, c->d_inst_next, c->d_cost_prefix, c->d_window, c->d_wmax,
                   c->d_group_mag, c->d_mag, c->d_wall_unit,
                   c->d_all_group_mag, c->d_R32, c->d_W32, c->d_F32, c->d_m2, c->d_wallTf,
                   c->d_pslot_off, c->d_phome_off, c->d_pnband, c->d_pnwall, c->d_px, c->d_pband, c->d_phome,
                   c->d_pcount, c->d_pfcount, c->d_phome_w, c->d_wemit, c->d_DY, c->d_EY, c->d_GX, c->d_Fx, c->d_Fi, c->d_ticket, c->d_wpart,
                   c->d_all_real, c->d_defer, c->d_defer_n, c->d_land_fwd, c->d_land_all, c->d_items, c->d_diff, c->d_sync_groups, c->d_sync_beg,
-                  c->d_sync_end};
+                  c->d_sync_end, c->team_plan[0].d_teams, c->team_plan[0].d_order, c->team_plan[0].d_block_team,
+                  c->team_plan[0].d_bar, c->team_plan[0].d_slots, c->team_plan[1].d_teams, c->team_plan[1].d_order,
+                  c->team_plan[1].d_block_team, c->team_plan[1].d_bar, c->team_plan[1].d_slots};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (c->h_pinned) cudaFreeHost(c->h_pinned);
@@ -1593,11 +1595,10 @@ iugkp_status iugkp_adjoint(iugkp_ctx* ctx, const double* T_star_dev, const doubl
   while (it < max_iter) {
     a.lambda = lam;
     CK(adjoint_sweep(c, a, s), "adjoint sweep");
-    CK(launch_axpy_grad(c, at, g_dev, half, s), "adjoint axpy");
     if (c->opt.newton) {
-      CK(launch_adjoint_correction(c, lam, half, nxt, s), "adjoint correction");
+      CK(launch_adjoint_correction(c, at, g_dev, lam, half, nxt, s), "adjoint correction");
     } else {
-      CK(cudaMemcpyAsync(nxt, half, nc * sizeof(double), cudaMemcpyDeviceToDevice, s), "copy");
+      CK(launch_axpy_grad(c, at, g_dev, nxt, s), "adjoint axpy");
     }
     // one synchronisation per iteration: the residual sums, max |g| and the solver's status
     CK(launch_residual(c, lam, nxt, 0.0, c->d_scalar, s), "residual");

@@ -25,6 +25,17 @@ constexpr int PERS_FACE_REPLICAS = 32;
 
 struct InstMG;
 
+// Blocks of a correction kernel, dealt to teams that take an instance each (mgpcg.cu).
+struct TeamPlan {
+  int blocks = 0;                // 0: no instance of this kind
+  size_t smem = 0;               // dynamic shared memory per block
+  void* d_teams = nullptr;
+  int* d_order = nullptr;
+  int* d_block_team = nullptr;
+  unsigned* d_bar = nullptr;     // barrier words (0 between launches)
+  double* d_slots = nullptr;     // partial sums of the blocks
+};
+
 // Arguments of the forward and adjoint sweep kernels (all device pointers).
 struct SweepArgs {
   const InstDesc* inst;
@@ -165,7 +176,7 @@ struct Ctx {
   double* h_pinned = nullptr;    // [8 + n_inst] host readback
   // multigrid preconditioner of the Newton correction (mg_setup.cu, mgpcg.cu)
   struct InstMG* d_mg = nullptr;
-  size_t mg_smem_bytes = 0;      // dynamic shared memory of the PCG kernel (CTA 0's coarse levels)
+  TeamPlan team_plan[2];         // multigrid CG, fast diagonalization
   float* d_mg_diag = nullptr;
   float* d_mg_dinv = nullptr;
   float* d_mg_cx = nullptr;
@@ -175,7 +186,6 @@ struct Ctx {
   float* d_mg_b = nullptr;
   float* d_mg_x = nullptr;
   float* d_mg_t = nullptr;
-  float* d_mg_r = nullptr;
   float* d_fd_q = nullptr;       // fast diagonalization: eigenvector matrices (FP32)
   float* d_fd_lam = nullptr;     // ... and eigenvalues
   long long mg_level_cells = 0;
@@ -231,8 +241,8 @@ cudaError_t launch_sweep(const Ctx* c, const SweepArgs& a, cudaStream_t s);
 cudaError_t launch_adjoint(const Ctx* c, const SweepArgs& a, cudaStream_t s);
 cudaError_t launch_macro(const Ctx* c, const double* R, const double* W, double* T_half, double* T_E, cudaStream_t s);
 cudaError_t launch_newton(const Ctx* c, const double* T_n, double* T_half, const double* R, cudaStream_t s);
-cudaError_t launch_adjoint_correction(const Ctx* c, const double* lam, const double* half, double* out,
-                                      cudaStream_t s);
+cudaError_t launch_adjoint_correction(const Ctx* c, const double* at, const double* g, const double* lam, double* half,
+                                      double* out, cudaStream_t s);
 cudaError_t launch_residual(const Ctx* c, const double* T0, const double* T1, double dT_ref, double* out_dev,
                             cudaStream_t s);
 cudaError_t launch_pcg_check(const Ctx* c, cudaStream_t s);
@@ -256,11 +266,7 @@ cudaError_t launch_adjoint_replay(const Ctx* c, const SweepArgs& a, cudaStream_t
 cudaError_t launch_walk_bounds(unsigned long long* out, cudaStream_t s);
 double walk_bound_fraction(const double* measured);
 cudaError_t measure_atomic_rate(int sm_count, double* out_rate);
-cudaError_t launch_mgpcg(const Ctx* c, const double* rhs, cudaStream_t s);
-size_t mg_solo_smem_bytes(const std::vector<InstMG>& h_mg);
-cudaError_t configure_mgpcg(Ctx* c, size_t smem);
-size_t fd_small_smem_bytes();  // dynamic shared memory of the in-shared-memory fast diagonalization
-int fd_small_max_n();          // its largest axis size
+cudaError_t configure_mgpcg(Ctx* c, const std::vector<InstMG>& h_mg);
 iugkp_status build_multigrid(Ctx* c, const std::vector<double>& diag, const std::vector<double>& cx,
                              const std::vector<double>& cy, const std::vector<double>& cz,
                              const std::vector<double>& kap, double cvsum);

@@ -212,15 +212,19 @@ iugkp_status build_multigrid(Ctx* c, const std::vector<double>& diag, const std:
       if (nx <= FD_MAX_N && ny <= FD_MAX_N &&
           separable_parts(in, kap.data() + in.cell_off, cvsum, diag.data() + in.cell_off, cx.data() + in.cell_off,
                           cy.data() + in.cell_off, part)) {
-        // 2: every operand in shared memory (small axes), 1: tiles through L2
-        m.direct = (nx <= fd_small_max_n() && ny <= fd_small_max_n()) ? 2 : 1;
+        m.direct = 1;
         m.fnx = nx;
         m.fny = ny;
         std::vector<double> lam, Q;
         tridiag_eigen(part[0][0], part[0][1], lam, Q);
+        while (fq.size() % 4) fq.push_back(0.f);  // 16-byte rows of chunks (fd_solve)
         m.qx_off = (long long)fq.size();
         m.lx_off = (long long)flam.size();
         for (double x : Q) fq.push_back((float)x);
+        while (fq.size() % 4) fq.push_back(0.f);
+        m.qxt_off = (long long)fq.size();
+        for (int i = 0; i < nx; ++i)
+          for (int j = 0; j < nx; ++j) fq.push_back((float)Q[(size_t)j * nx + i]);
         for (double x : lam) flam.push_back((float)x);
         tridiag_eigen(part[1][0], part[1][1], lam, Q);
         m.qy_off = (long long)fq.size();
@@ -265,7 +269,7 @@ iugkp_status build_multigrid(Ctx* c, const std::vector<double>& diag, const std:
       for (int a = 0; a < 3; ++a) m.n[l][a] = lv[l].n[a];
       m.nc[l] = lv[l].nc;
       m.off[l] = level_off;
-      level_off += lv[l].nc;
+      level_off += (lv[l].nc + 3) & ~3ll;  // every level starts on 16 bytes
       for (long long i = 0; i < lv[l].nc; ++i) {
         ldiag.push_back((float)lv[l].diag[i]);
         ldinv.push_back((float)(1.0 / lv[l].diag[i]));
@@ -273,6 +277,7 @@ iugkp_status build_multigrid(Ctx* c, const std::vector<double>& diag, const std:
         lcy.push_back((float)lv[l].c[1][i]);
         lcz.push_back((float)lv[l].c[2][i]);
       }
+      for (std::vector<float>* p : {&ldiag, &ldinv, &lcx, &lcy, &lcz}) p->resize((size_t)level_off, 0.f);
     }
     // Dense coarsest matrix and its inverse.
     const Level& cl = lv.back();
@@ -321,11 +326,7 @@ iugkp_status build_multigrid(Ctx* c, const std::vector<double>& diag, const std:
   if ((s = up(&c->d_mg_b, zeros)) != IUGKP_OK) return s;
   if ((s = up(&c->d_mg_x, zeros)) != IUGKP_OK) return s;
   if ((s = up(&c->d_mg_t, zeros)) != IUGKP_OK) return s;
-  if ((s = up(&c->d_mg_r, zeros)) != IUGKP_OK) return s;
-  size_t smem = mg_solo_smem_bytes(mgs);
-  for (const InstMG& m : mgs)
-    if (m.direct == 2) smem = std::max(smem, fd_small_smem_bytes());
-  const cudaError_t e = configure_mgpcg(c, smem);
+  const cudaError_t e = configure_mgpcg(c, mgs);
   if (e != cudaSuccess) return fail(c, IUGKP_ECUDA, std::string("multigrid kernel set-up: ") + cudaGetErrorString(e));
   return IUGKP_OK;
 }
