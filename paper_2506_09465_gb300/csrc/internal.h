@@ -250,6 +250,8 @@ cudaError_t launch_absmax(const Ctx* c, const double* x, long long n, double* ou
 cudaError_t launch_axpy_grad(const Ctx* c, const double* at, const double* g, double* lam_half, cudaStream_t s);
 cudaError_t launch_sweep_staged(const Ctx* c, const SweepArgs& a, cudaStream_t s);
 cudaError_t configure_staged(Ctx* c);
+cudaError_t configure_chain();
+cudaError_t launch_chain(const Ctx* c, const SweepArgs& a, const StagedArgs& S, bool k32, cudaStream_t s);
 cudaError_t launch_k32_finalize(const Ctx* c, const float2* src, double* dst, long long n, cudaStream_t s);
 cudaError_t launch_exact(const Ctx* c, const SweepArgs& a, cudaStream_t s);
 cudaError_t launch_prologue(const Ctx* c, const SweepArgs& a, const PrologueArgs& P, cudaStream_t s);

@@ -4,15 +4,13 @@
 namespace iugkp {
 
 constexpr int STAGED_NT = 1024;                 // threads per persistent block
-constexpr int WALK_MIN_LANES = 8;               // 3D per-lane walk: fewest lanes worth a step
+constexpr int WALK_MIN_LANES = 8;               // landing chains: fewest lanes worth a step
 
-// 3D face tallies: the warp tallies the items of the particles that ended together; per warp a
-// table of 64 item lists (the x- and y-faces of each lane's particle, 3 int4 of parameters
-// each) and their 65 start offsets, in the dynamic shared memory (3D instances keep no face
-// window there).
-constexpr int COOP3_LISTS = 64;
-constexpr int COOP3_INT4_PER_WARP = COOP3_LISTS * 3 + 17;  // parameters, then the starts (65 ints)
-constexpr int COOP3_BYTES = (STAGED_NT / 32) * COOP3_INT4_PER_WARP * 16;
+// 3D sweep (sweep_chain.cu): threads of a block (five warps per scheduler: with four 17.3 ms, five
+// 15.4 ms, six 17.7 ms on four boxes up to 64^3), and the idle lanes that trigger a refill (2 to 4:
+// the same, 8: 3 % more).
+constexpr int CHAIN_NT = 640;
+constexpr int CHAIN_REFILL = 4;
 
 // Shared-memory x-face window: one 32-bit word per face holding the low word of a 64-bit
 // fixed-point sum in units of w_max 2^-26 (a contribution is below 2^26 units); words start

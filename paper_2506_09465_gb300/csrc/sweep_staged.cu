@@ -1,5 +1,5 @@
-// Fast forward sweep: FP32 walk, persistent blocks (a pass-synchronous
-// kernel for 2D, a per-lane-refill kernel for every dimension), face tallies staged in
+// Fast forward sweep in 1D and 2D (3D: sweep_chain.cu): FP32 walk, persistent blocks (a
+// pass-synchronous kernel for 2D, a per-lane-refill kernel for both), face tallies staged in
 // shared memory in fixed point. Same method and draws as the plain sweep
 // (arXiv 2506.09465 Sec. 3.1 steps (1)-(3), Sec. 3.2 null collisions); only the
 // arithmetic precision of the walk and the way tallies are accumulated differ.
@@ -11,18 +11,17 @@
 //    (native shared-memory atomics, about five times the rate of 64-bit ones) whose rare
 //    wrap-arounds add +-2^32 q to the FP64 face at once, flushed to the FP64 array when the
 //    block leaves the instance; x-faces outside the window take global atomics;
-//  * faces normal to the last axis (y in 2D, z in 3D) are not tallied, except on the low
+//  * faces normal to y in 2D are not tallied, except on the low
 //    boundary: every particle conserves power, so in every cell the net inflow equals the
 //    absorbed minus emitted power, and the last-axis faces follow exactly by a prefix sum
 //    along each column (derive_last_axis_kernel);
-//  * in 3D the y-faces are tallied with global FP64 atomics;
 //  * 2D instances whose faces all fit the window use two-group tallies instead: a particle
 //    tallies only the faces normal to the axis it crosses less often, and each group's
 //    other faces follow from that group's own per-cell balance (derive_two_group_kernel,
 //    assemble_two_group_kernel);
 //  * a warp tallies the face items of the particles that ended together: in the
 //    pass-synchronous kernel each lane takes segments of 8 items of one list, dealt
-//    round-robin; in the per-lane-refill kernel each lane takes one contiguous chunk of the
+//    round-robin; in the 2D per-lane-refill kernel each lane takes one contiguous chunk of the
 //    concatenated item lists;
 //  * nothing is tallied per particle for the walls: the power a wall emits enters through
 //    its faces deterministically (N particles of known weight per face), and the power it
@@ -35,160 +34,11 @@
 #include "device.cuh"
 #include "internal.h"
 #include "landing.cuh"
+#include "segment.cuh"
 #include "staged.h"
 #include "walk32.cuh"
 
 namespace iugkp {
-
-namespace {
-
-struct LCounts {
-  unsigned v[CNT_N];  // per thread and launch: far below 2^32
-};
-
-__device__ __forceinline__ void flush_lcounts(LCounts& c, unsigned long long* out) {
-  if (!out) return;
-#pragma unroll
-  for (int k = 0; k < CNT_N; ++k) {
-    unsigned long long x = c.v[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-    if ((threadIdx.x & 31) == 0 && x) atomicAdd(&out[k], x);
-  }
-}
-
-// Register-resident path state. The direction does not change at null collisions, so the
-// path from emission to the end (real collision or wall) is one straight segment: i_a is
-// the emission cell, t_a the path length at which the first face normal to axis a is
-// reached, d_a the path length per cell along a (+inf when s_a = 0), so the k-th face along
-// a is reached at t_a + k d_a. D: path length of the current candidate collision;
-// tex: path length at which the segment leaves the domain.
-struct PW {
-  int i0, i1, i2;
-  int s0, s1, s2;
-  float t0, t1, t2;
-  float d0, d1, d2;
-  float D, tex;
-};
-
-__device__ __forceinline__ void axis_init(float s, float xi, float h, float& t, float& d, int& st) {
-  const float as = fabsf(s);
-  st = s > 0.f ? 1 : -1;
-  d = __fdividef(h, as);  // +inf when s = 0
-  t = (s > 0.f ? 1.f - xi : xi) * d;
-}
-
-// ceil(max(u, 0)) for u < 2^23 without a float-to-integer conversion: adding 2^23 with
-// rounding upwards lands on 2^23 + ceil(u), whose bits minus those of 2^23 are the count.
-__device__ __forceinline__ int ceil_count(float u) {
-  return __float_as_int(__fadd_ru(fmaxf(u, 0.f), 8388608.f)) - 0x4B000000;
-}
-
-// Faces normal to one axis reached before path length L: #{k >= 0 : t + k d < L}.
-__device__ __forceinline__ int faces_before(float L, float t, float d) {
-  return L > t ? ceil_count(__fdividef(L - t, d)) : 0;
-}
-
-// Faces up to and including the wall along one axis, and the path length of the wall face.
-__device__ __forceinline__ int faces_to_wall(int i, int s, int n) { return s > 0 ? n - i : i + 1; }
-__device__ __forceinline__ float axis_exit(int i, int s, int n, float t, float d) {
-  const int m = faces_to_wall(i, s, n);
-  return m > 1 ? fmaf(small_int_float(m - 1), d, t) : t;
-}
-
-__device__ __forceinline__ int clampi(int v, int n) { return min(max(v, 0), n - 1); }
-
-// Tie bits of one axis for the count n = faces_before(D, t, d): bit sh when D lies within the
-// bound (base = TIE_REL D + eD, plus TIE_REL d) below a face, so that the FP64 walk may count
-// one face more; bit sh + 1 when within it above one (one fewer). None when d = inf (NaN).
-__device__ __forceinline__ unsigned tie_bits(float D, float t, float d, float base, int n, int sh) {
-  const float u = __fdividef(D - t, d);
-  const float fr = small_int_float(n) - u;  // up to the next face, in cells: [0, 1]
-  const float tol = fmaf(TIE_REL, d, base);
-  if (fr * d <= tol) return 1u << sh;
-  if ((1.f - fr) * d <= tol && n > 0) return 2u << sh;
-  return 0u;
-}
-
-// faces_before, and in `near` whether D lies within the bound of a face of this axis (either
-// side; the direction is not needed when every candidate is real).
-__device__ __forceinline__ int count_near(float D, float t, float d, float base, bool& near) {
-  const float u = __fdividef(D - t, d);
-  const float c = __fadd_ru(fmaxf(u, 0.f), 8388608.f);  // 2^23 + ceil(max(u, 0))
-  const float fr = (c - 8388608.f) - u;
-  near |= fminf(fr, 1.f - fr) * d <= fmaf(TIE_REL, d, base);
-  return __float_as_int(c) - 0x4B000000;
-}
-
-// Axis a's bit of `hit` when the count one more than n reaches the wall (m faces to it).
-__device__ __forceinline__ unsigned tie_hits_wall(unsigned tie, int a, int n, int m) {
-  return ((tie >> (2 * a)) & 1u) && n + 1 >= m ? 1u << (2 * a) : 0u;
-}
-
-// A candidate flagged near faces (tie, two bits per axis) may lie, in the FP64 walk, in a cell
-// across the flagged faces. True when every such cell rejects it by more than the ratio's
-// rounding: the FP64 walk then goes on identically, and only the cell of this candidate's W
-// may differ. False when an alternative lies beyond a wall (hit) or any cell may accept.
-// st_a: the cell index step of one more face along axis a (s_a times the axis stride).
-__device__ __forceinline__ bool all_reject(const float* ratio, int ncells, int cell, unsigned tie, unsigned hit, int st0,
-                                           int st1, int st2, float u) {
-  if (tie & hit) return false;
-#pragma unroll 1
-  for (unsigned k = 0; k < 8u; ++k) {
-    int c = cell;
-    bool ok = true;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      if (!((k >> a) & 1u)) continue;
-      const unsigned t = (tie >> (2 * a)) & 3u;
-      const int st = a == 0 ? st0 : (a == 1 ? st1 : st2);
-      ok = ok && t != 0u;
-      c += t == 1u ? st : -st;
-    }
-    if (!ok) continue;
-    if (c < 0 || c >= ncells || !(u - ratio[c] >= TIE_ACC)) return false;
-  }
-  return true;
-}
-
-enum { CAND_NULL = 0, CAND_REAL = 1, CAND_DEFER = 2 };
-
-// Adds n units of q to the fixed-point sum of a face.
-__device__ __forceinline__ void add_units(long long* Fi, long long face, long long n) {
-  atomicAdd(reinterpret_cast<unsigned long long*>(&Fi[face]), (unsigned long long)n);
-}
-
-// Outcome of the candidate at path length f.D, whose face counts fb and cell the caller took
-// in FP32 (the first wall lies beyond it by more than the bound, so it is a candidate for the
-// FP64 walk too): CAND_NULL or CAND_REAL when the FP64 walk decides the same, CAND_DEFER
-// otherwise. A candidate whose acceptance draw exceeds the largest ratio of its cell's
-// neighbourhood (by more than the ratio's rounding) is rejected wherever it lies, and needs no
-// face test; its W may sit in the neighbouring cell. ub: the acceptance word; sy, sz: cell
-// index steps along y and z.
-// all_real: every candidate of the band is real, and near tells whether a count lies within
-// the bound of a face (count_near); otherwise the tie bits are found here when needed.
-template <int DIM>
-__device__ __forceinline__ int candidate_outcome(const SweepArgs& A, long long bcbase, int ncells, const PW& f,
-                                                 float base, int fb0, int fb1, int fb2, int cell, bool all_real,
-                                                 bool near, uint32_t ub, int n0, int n1, int n2, int sy, int sz) {
-  if (all_real) return near ? CAND_DEFER : CAND_REAL;
-  const float ua = word_uniform<float>(ub);
-  if (ua - A.ratio_nb32[bcbase + cell] >= TIE_ACC) return CAND_NULL;
-  unsigned tie = tie_bits(f.D, f.t0, f.d0, base, fb0, 0);
-  if (DIM >= 2) tie |= tie_bits(f.D, f.t1, f.d1, base, fb1, 2);
-  if (DIM == 3) tie |= tie_bits(f.D, f.t2, f.d2, base, fb2, 4);
-  const float ra = A.ratio32[bcbase + cell];
-  if (tie) {
-    unsigned hit = tie_hits_wall(tie, 0, fb0, faces_to_wall(f.i0, f.s0, n0));
-    if (DIM >= 2) hit |= tie_hits_wall(tie, 1, fb1, faces_to_wall(f.i1, f.s1, n1));
-    if (DIM == 3) hit |= tie_hits_wall(tie, 2, fb2, faces_to_wall(f.i2, f.s2, n2));
-    if (!all_reject(A.ratio32 + bcbase, ncells, cell, tie, hit, f.s0, f.s1 * sy, f.s2 * sz, ua)) return CAND_DEFER;
-  }
-  if (fabsf(ua - ra) < TIE_ACC) return CAND_DEFER;
-  return ua < ra ? CAND_REAL : CAND_NULL;
-}
-
-}  // namespace
 
 // Emits particle pid (global forward index) into lane state. Returns false for a
 // zero-weight particle (nothing to trace).
@@ -247,30 +97,18 @@ __device__ __forceinline__ bool staged_emit(const SweepArgs& A, const StagedArgs
     } else {
       const int r = (int)udiv((unsigned)e, (unsigned)n0, S.mag_n0[k]);
       f.i0 = e - r * n0;
-      if (DIM == 2) {
-        f.i1 = r;
-        f.i2 = 0;
-      } else {
-        f.i2 = (int)udiv((unsigned)r, (unsigned)n1, S.mag_n1[k]);
-        f.i1 = r - f.i2 * n1;
-      }
+      f.i1 = r;
+      f.i2 = 0;
     }
     float u_mu, u_phi = 0.5f;
     if (DIM == 1) {
       xi0 = word_uniform<float>(st.buf.x);
       u_mu = word_uniform<float>(st.buf.y);
-    } else if (DIM == 2) {
+    } else {
       xi0 = word_uniform<float>(st.buf.x);
       xi1 = word_uniform<float>(st.buf.y);
       u_mu = word_uniform<float>(st.buf.z);
       u_phi = word_uniform<float>(st.buf.w);
-    } else {
-      xi0 = word_uniform<float>(st.buf.x);
-      xi1 = word_uniform<float>(st.buf.y);
-      xi2 = word_uniform<float>(st.buf.z);
-      u_mu = word_uniform<float>(st.buf.w);
-      st.load_block(1);
-      u_phi = word_uniform<float>(st.buf.x);
     }
     const float mu = 2.f * u_mu - 1.f;
     sx = mu;
@@ -317,15 +155,10 @@ __device__ __forceinline__ bool staged_emit(const SweepArgs& A, const StagedArgs
     float t0 = 0.5f, t1 = 0.5f;  // tangential fractions, in axis order
     if (DIM == 1) {
       u_n = word_uniform<float>(st.buf.x);
-    } else if (DIM == 2) {
+    } else {
       t0 = word_uniform<float>(st.buf.x);
       u_n = word_uniform<float>(st.buf.y);
       u_phi = word_uniform<float>(st.buf.z);
-    } else {
-      t0 = word_uniform<float>(st.buf.x);
-      t1 = word_uniform<float>(st.buf.y);
-      u_n = word_uniform<float>(st.buf.z);
-      u_phi = word_uniform<float>(st.buf.w);
     }
     const float mn = sqrtf(u_n);
     const float sn = DIM >= 2 ? sqrtf(1.f - u_n) : 0.f;
@@ -350,13 +183,9 @@ __device__ __forceinline__ bool staged_emit(const SweepArgs& A, const StagedArgs
   if (DIM >= 2) {
     axis_init(sy, xi1, in.hf[1], f.t1, f.d1, f.s1);
     const float e1 = axis_exit(f.i1, f.s1, n1, f.t1, f.d1);
-    // 2D: the axis of the wall the segment reaches (x on ties), kept in the unused i2
-    if (DIM == 2) f.i2 = e1 < f.tex ? 1 : 0;
+    // the axis of the wall the segment reaches (x on ties), kept in the unused i2
+    f.i2 = e1 < f.tex ? 1 : 0;
     f.tex = fminf(f.tex, e1);
-  }
-  if (DIM >= 3) {
-    axis_init(sz, xi2, in.hf[2], f.t2, f.d2, f.s2);
-    f.tex = fminf(f.tex, axis_exit(f.i2, f.s2, n2, f.t2, f.d2));
   }
   if (DIM == 2 && two && f.d0 < f.d1) {
     // y-group: its emission enters its own power balance (cell) or boundary flux (face)
@@ -497,19 +326,14 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
       // ---- candidates (Sec. 3.2): up to walk_k per lane. The candidate lies at path length D
       // of the straight segment; its cell follows from the faces before D on each axis.
       // W tally, then acceptance with probability tau_maj / tau(x); a rejected candidate
-      // draws the next flight length and the particle goes on in the same direction. In 3D
-      // the walk stops early once fewer than WALK_MIN_LANES lanes are still walking: the lanes
-      // whose particles ended get their items tallied and are refilled sooner, and the others go
-      // on in the next pass (16-box batch at refill 4, walk_k 8: 75.9 -> 74.6 ms) ----
+      // draws the next flight length and the particle goes on in the same direction ----
       int nitem = 0;  // cooperative tallies: face items of the lane's particle ended in this pass
-      int nx3 = 0, ny3 = 0;  // 3D: x- and y-face items of the lane's particle ended in this pass
       bool ended = false, wall_exit = false, deferred = false;
       const bool walking = alive && !tally;
       const bool all_real = A.all_real[(long long)k * A.nb + band] != 0;
       if (walking) {
 #pragma unroll 1
         for (int it = 0; it < S.walk_k; ++it) {
-          if (DIM == 3 && it > 0 && __popc(__activemask()) < WALK_MIN_LANES) break;
           // a decision within rounding of the FP64 walk's defers the particle to the FP64 replay
           const float base = fmaf(TIE_REL, f.D, eD);
           if (f.D - f.tex > base) {  // the segment reaches a wall first: absorbed there
@@ -521,21 +345,18 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
             break;
           }
           bool near = false;  // a count within the bound of a face, found with it for all-real bands
-          int fb0, fb1 = 0, fb2 = 0;
+          int fb0, fb1 = 0;
           if (all_real) {
             fb0 = count_near(f.D, f.t0, f.d0, base, near);
             if (DIM >= 2) fb1 = count_near(f.D, f.t1, f.d1, base, near);
-            if (DIM == 3) fb2 = count_near(f.D, f.t2, f.d2, base, near);
           } else {
             fb0 = faces_before(f.D, f.t0, f.d0);
             if (DIM >= 2) fb1 = faces_before(f.D, f.t1, f.d1);
-            if (DIM == 3) fb2 = faces_before(f.D, f.t2, f.d2);
           }
           int cell = clampi(f.i0 + f.s0 * fb0, n0);
           if (DIM >= 2) cell += sy_cell * clampi(f.i1 + f.s1 * fb1, n1);
-          if (DIM == 3) cell += sz_cell * clampi(f.i2 + f.s2 * fb2, n2);
           const long long ci = bcbase + cell;
-          const int oc = candidate_outcome<DIM>(A, bcbase, ncells, f, base, fb0, fb1, fb2, cell, all_real, near, ub,
+          const int oc = candidate_outcome<DIM>(A, bcbase, ncells, f, base, fb0, fb1, 0, cell, all_real, near, ub,
                                                 n0, n1, n2, sy_cell, sz_cell);
           if (oc == CAND_DEFER) {
             ended = deferred = true;
@@ -579,15 +400,14 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
           if (wall_exit) {
             const float e0 = axis_exit(f.i0, f.s0, n0, f.t0, f.d0);
             const float e1 = DIM >= 2 ? axis_exit(f.i1, f.s1, n1, f.t1, f.d1) : INFINITY;
-            const float e2 = DIM == 3 ? axis_exit(f.i2, f.s2, n2, f.t2, f.d2) : INFINITY;
-            ex = (e0 <= e1 && e0 <= e2) ? 0 : (e1 <= e2 ? 1 : 2);
+            ex = e0 <= e1 ? 0 : 1;
           }
           // at a wall, the faces of the other axes crossed before it: a count within rounding
           // of the FP64 walk's (the segment leaves near a cell corner) defers the particle
           bool tie = false;
           const float bx = TIE_REL * f.tex;
           const int m0 = faces_to_wall(f.i0, f.s0, n0);
-          int c0 = m0 - 1, c1 = 0, c2 = 0, m1 = 1;
+          int c0 = m0 - 1, c1 = 0, m1 = 1;
           if (ex != 0) {
             const int q = count_near(L, f.t0, f.d0, bx, tie);
             c0 = min(q, m0 - 1);
@@ -600,20 +420,12 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
               c1 = min(q, m1 - 1);
             }
           }
-          if (DIM == 3) {
-            const int m2 = faces_to_wall(f.i2, f.s2, n2);
-            c2 = m2 - 1;
-            if (ex != 2) {
-              const int q = count_near(L, f.t2, f.d2, bx, tie);
-              c2 = min(q, m2 - 1);
-            }
-          }
           if (wall_exit && tie) {
             defer_particle(S, pid, ((unsigned)kc << 1) | ((two && f.d0 < f.d1) ? 1u : 0u));
             alive = false;
           } else {
             if (wall_exit) cnt.v[CNT_WALL_EXITS] += 1;
-            cnt.v[CNT_CROSSINGS] += c0 + c1 + c2;
+            cnt.v[CNT_CROSSINGS] += c0 + c1;
             if (DIM == 2 && (two || wfull)) {
               // Face items k = 0 .. kend-1 along the tallied axis p (the other axis: q). Item k
               // is the face index a0 + k sp + sq min(ceil(u0 + k r), lim): the k-th face normal
@@ -660,54 +472,11 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
               // follow from conservation)
               if (DIM == 2 && ex == 1 && f.s1 < 0) {
                 atomicAdd(&S.gx()[in.bface_off + in.wface_off[2] + (f.i0 + f.s0 * c0)], -w);
-              } else if (DIM == 3 && ex == 2 && f.s2 < 0) {
-                const long long fi = face_off + fax2 + (f.i0 + f.s0 * c0) + (long long)n0 * (f.i1 + f.s1 * c1);
-                if (K32) tally_k32(&S.F32[fi], -w);
-                else atomicAdd(&A.F[fi], -w);
               }
-              if (DIM == 3) {
-                // Two item lists, tallied below by the whole warp: the x-faces crossed (the wall
-                // face too when the particle leaves through x) and the y-faces. Item k of the list
-                // along axis p is the face a0 + k sp + sq1 min(ceil(u1 + k r1), lim1) + sq2
-                // min(ceil(u2 + k r2), lim2): the k-th face normal to p, in the cell row and
-                // layer given by the faces of the other two axes crossed before it (ceil((t_p +
-                // k d_p - t_q) / d_q) = ceil(u + k r), u = (t_p - t_q) / d_q, r = d_p / d_q).
-                int4* tab = reinterpret_cast<int4*>(win) + (threadIdx.x >> 5) * COOP3_INT4_PER_WARP + 6 * lane;
-                auto ur = [](float tp, float dp, float tq, float dq, float& u, float& r) {
-                  const bool flat = !(dq < INFINITY);
-                  u = flat ? -1.f : __fdividef(tp - tq, dq);
-                  r = flat ? 0.f : __fdividef(dp, dq);
-                };
-                float u1, r1, u2, r2;
-                nx3 = c0 + (ex == 0 ? 1 : 0);
-                ny3 = c1 + (ex == 1 ? 1 : 0);
-                ur(f.t0, f.d0, f.t1, f.d1, u1, r1);
-                ur(f.t0, f.d0, f.t2, f.d2, u2, r2);
-                double ws = f.s0 > 0 ? w : -w;
-                tab[0] = make_int4((f.s0 > 0 ? f.i0 + 1 : f.i0) + sy_xf * f.i1 + sz_xf * f.i2, f.s0, f.s1 * sy_xf,
-                                   faces_to_wall(f.i1, f.s1, n1) - 1);
-                tab[1] = make_int4(f.s2 * sz_xf, faces_to_wall(f.i2, f.s2, n2) - 1, __float_as_int(u1),
-                                   __float_as_int(r1));
-                tab[2] = make_int4(__float_as_int(u2), __float_as_int(r2), __double2loint(ws), __double2hiint(ws));
-                ur(f.t1, f.d1, f.t0, f.d0, u1, r1);
-                ur(f.t1, f.d1, f.t2, f.d2, u2, r2);
-                ws = f.s1 > 0 ? w : -w;
-                const int sz_yf = n0 * (n1 + 1);  // y-face index step along z
-                tab[3] = make_int4((int)fax1 + f.i0 + n0 * (f.s1 > 0 ? f.i1 + 1 : f.i1) + sz_yf * f.i2, f.s1 * n0, f.s0,
-                                   m0 - 1);
-                tab[4] = make_int4(f.s2 * sz_yf, faces_to_wall(f.i2, f.s2, n2) - 1, __float_as_int(u1),
-                                   __float_as_int(r1));
-                tab[5] = make_int4(__float_as_int(u2), __float_as_int(r2), __double2loint(ws), __double2hiint(ws));
-                alive = false;
-              } else {
-              // x-faces crossed (the wall face too when the particle leaves through x),
-              // then in 3D the y-faces
+              // x-faces crossed (the wall face too when the particle leaves through x)
               kcur = 0;
               kend = c0 + (ex == 0 ? 1 : 0);
-              if (DIM == 3) {
-                f.tex = small_int_float(kend);  // first y-face item
-                kend += c1 + (ex == 1 ? 1 : 0);
-              } else if (DIM == 2) {
+              if (DIM == 2) {
                 // rows of the x-face crossings, incrementally: faces normal to y before the
                 // k-th x-face = ceil(u0 + k r), u0 = (t0 - t1) / d1, r = d0 / d1
                 const bool flat = !(f.d1 < INFINITY);
@@ -717,7 +486,6 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
               }
               tally = kend > 0;
               alive = tally;
-              }
             } else {
               alive = false;
             }
@@ -785,57 +553,6 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
           __syncwarp();
         }
       }
-      // ---- 3D: the warp tallies the x- and y-face items of the particles that ended in this
-      // pass together (lists 2 lane and 2 lane + 1, concatenated in order and cut into 32
-      // equal contiguous chunks, one per lane), with global atomics ----
-      if (DIM == 3 && useF) {
-        int incl = nx3 + ny3;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int t = __shfl_up_sync(0xffffffffu, incl, o);
-          if (lane >= o) incl += t;
-        }
-        const int total = __shfl_sync(0xffffffffu, incl, 31);
-        if (total > 0) {
-          const int4* tab = reinterpret_cast<const int4*>(win) + (threadIdx.x >> 5) * COOP3_INT4_PER_WARP;
-          int* lst = reinterpret_cast<int*>(reinterpret_cast<int4*>(win) + (threadIdx.x >> 5) * COOP3_INT4_PER_WARP +
-                                            3 * COOP3_LISTS);
-          const int excl = incl - nx3 - ny3;
-          lst[2 * lane] = excl;
-          lst[2 * lane + 1] = excl + nx3;
-          if (lane == 31) lst[COOP3_LISTS] = total;
-          __syncwarp();
-          const int k0 = (lane * total) >> 5, k1 = ((lane + 1) * total) >> 5;
-          if (k0 < k1) {
-            int l = 0;  // the last list starting at or before k0
-#pragma unroll
-            for (int st = 32; st > 0; st >>= 1)
-              if (lst[l + st] <= k0) l += st;
-            int lend = lst[l + 1];
-            int4 pa = tab[3 * l], pb = tab[3 * l + 1], pc = tab[3 * l + 2];
-#pragma unroll 1
-            for (int kk = k0; kk < k1; ++kk) {
-              if (kk >= lend) {  // the next non-empty list
-                do {
-                  ++l;
-                  lend = lst[l + 1];
-                } while (lend <= kk);
-                pa = tab[3 * l];
-                pb = tab[3 * l + 1];
-                pc = tab[3 * l + 2];
-              }
-              const float fk = small_int_float(kk - lst[l]);
-              const int face = pa.x + (kk - lst[l]) * pa.y +
-                               pa.z * min(ceil_count(fmaf(fk, __int_as_float(pb.w), __int_as_float(pb.z))), pa.w) +
-                               pb.x * min(ceil_count(fmaf(fk, __int_as_float(pc.y), __int_as_float(pc.x))), pb.y);
-              const double val = __hiloint2double(pc.w, pc.z);
-              if (K32) tally_k32(&S.F32[face_off + face], val);
-              else atomicAdd(&A.F[face_off + face], val);
-            }
-          }
-          __syncwarp();
-        }
-      }
       // ---- face tallies of ended particles: up to walk_k per lane ----
       if (tally) {
         const int kstop = min(kend, kcur + S.walk_k);
@@ -862,26 +579,9 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
         } else {
 #pragma unroll 1
           for (; kcur < kstop; ++kcur, fk += 1.f) {
-            if (DIM == 3 && fk >= f.tex) {
-              // y-face item: the (kcur - kx)-th face normal to y along the segment
-              const float fm = fk - f.tex;  // exact: both are small integers
-              const int mm = ceil_count(fm);
-              const float tm = fmaf(fm, f.d1, f.t1);
-              const int col = clampi(f.i0 + f.s0 * faces_before(tm, f.t0, f.d0), n0);
-              const int lay = clampi(f.i2 + f.s2 * faces_before(tm, f.t2, f.d2), n2);
-              const int jf = f.s1 > 0 ? f.i1 + 1 + mm : f.i1 - mm;
-              const long long fi = face_off + fax1 + col + (long long)n0 * (jf + (long long)(n1 + 1) * lay);
-              if (K32) tally_k32(&S.F32[fi], f.s1 > 0 ? w : -w);
-              else atomicAdd(&A.F[fi], f.s1 > 0 ? w : -w);
-              continue;
-            }
             int xface = f.s0 > 0 ? f.i0 + 1 + kcur : f.i0 - kcur;
             if (DIM == 2) {
               xface += sy_xf * (f.i1 + f.s1 * min(ceil_count(fmaf(fk, f.tex, f.D)), f.i2));
-            } else if (DIM == 3) {
-              const float tk = fmaf(fk, f.d0, f.t0);
-              xface += sy_xf * clampi(f.i1 + f.s1 * faces_before(tk, f.t1, f.d1), n1) +
-                       sz_xf * clampi(f.i2 + f.s2 * faces_before(tk, f.t2, f.d2), n2);
             }
             const unsigned rel = (unsigned)(xface - wbase);
             if (rel < wlen) window_add(xface, rel);
@@ -1304,7 +1004,7 @@ cudaError_t launch_sweep_staged(const Ctx* c, const SweepArgs& a_in, cudaStream_
         if (sync) launch_sync<true>(c, a, S, blocks, smem, s);
         else sweep_staged_kernel<2, true><<<blocks, STAGED_NT, smem, s>>>(a, S);
         break;
-      default: sweep_staged_kernel<3, true><<<blocks, STAGED_NT, smem, s>>>(a, S); break;
+      default: launch_chain(c, a, S, true, s); break;
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int fb = c->sm_count * 4;
@@ -1319,7 +1019,7 @@ cudaError_t launch_sweep_staged(const Ctx* c, const SweepArgs& a_in, cudaStream_
         if (sync) launch_sync<false>(c, a, S, blocks, smem, s);
         else sweep_staged_kernel<2, false><<<blocks, STAGED_NT, smem, s>>>(a, S);
         break;
-      default: sweep_staged_kernel<3, false><<<blocks, STAGED_NT, smem, s>>>(a, S); break;
+      default: launch_chain(c, a, S, false, s); break;
     }
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -1430,10 +1130,10 @@ double walk_bound_fraction(const double* m) {
 
 cudaError_t configure_staged(Ctx* c) {
   cudaError_t e = cudaSuccess;
+  if (c->dim == 3) return configure_chain();
   const size_t smem = (size_t)c->staged_cap * sizeof(unsigned);
-  const void* fwd[6] = {(const void*)sweep_staged_kernel<1, false>, (const void*)sweep_staged_kernel<2, false>,
-                        (const void*)sweep_staged_kernel<3, false>, (const void*)sweep_staged_kernel<1, true>,
-                        (const void*)sweep_staged_kernel<2, true>, (const void*)sweep_staged_kernel<3, true>};
+  const void* fwd[4] = {(const void*)sweep_staged_kernel<1, false>, (const void*)sweep_staged_kernel<2, false>,
+                        (const void*)sweep_staged_kernel<1, true>, (const void*)sweep_staged_kernel<2, true>};
   for (const void* f : fwd)
     if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
   const void* syn[8] = {(const void*)sweep_sync_kernel<false, false, false>, (const void*)sweep_sync_kernel<true, false, false>,
@@ -1444,7 +1144,7 @@ cudaError_t configure_staged(Ctx* c) {
     if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
   int nb = 0, nk = 0;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fwd[c->dim - 1], STAGED_NT, smem)) != cudaSuccess) return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nk, fwd[c->dim + 2], STAGED_NT, smem)) != cudaSuccess) return e;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nk, fwd[c->dim + 1], STAGED_NT, smem)) != cudaSuccess) return e;
   nb = std::min(nb, nk);  // one grid size for both tally modes
   c->staged_blocks_per_sm = nb > 0 ? nb : 1;
   return cudaSuccess;
