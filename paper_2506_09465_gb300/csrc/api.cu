@@ -137,9 +137,7 @@ void free_all(Ctx* c) {
                   c->d_pslot_off, c->d_phome_off, c->d_pnband, c->d_pnwall, c->d_px, c->d_pband, c->d_phome,
                   c->d_pcount, c->d_pfcount, c->d_phome_w, c->d_wemit, c->d_DY, c->d_EY, c->d_GX, c->d_Fx, c->d_Fi, c->d_ticket, c->d_wpart,
                   c->d_all_real, c->d_defer, c->d_defer_n, c->d_land_fwd, c->d_land_all, c->d_items, c->d_diff, c->d_sync_groups, c->d_sync_beg,
-                  c->d_sync_end, c->team_plan[0].d_teams, c->team_plan[0].d_order, c->team_plan[0].d_block_team,
-                  c->team_plan[0].d_bar, c->team_plan[0].d_slots, c->team_plan[1].d_teams, c->team_plan[1].d_order,
-                  c->team_plan[1].d_block_team, c->team_plan[1].d_bar, c->team_plan[1].d_slots};
+                  c->d_sync_end, c->team_plan[0].d_buf, c->team_plan[1].d_buf};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (c->h_pinned) cudaFreeHost(c->h_pinned);

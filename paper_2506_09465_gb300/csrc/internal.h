@@ -28,7 +28,9 @@ struct InstMG;
 // Blocks of a correction kernel, dealt to teams that take an instance each (mgpcg.cu).
 struct TeamPlan {
   int blocks = 0;                // 0: no instance of this kind
+  int threads = 0;               // per block
   size_t smem = 0;               // dynamic shared memory per block
+  char* d_buf = nullptr;         // the arrays below
   void* d_teams = nullptr;
   int* d_order = nullptr;
   int* d_block_team = nullptr;

@@ -8,7 +8,7 @@
 // memory (L2) between team barriers, and reduce dot products in a fixed rank order (every block
 // gets the same value, so all take the same branch). With one 8-block cluster per instance
 // the largest of four boxes (64^3, 64 cells per thread and phase) set the time on 8 of 152 SMs:
-// 5.5 ms per solve of 11 CG steps, now 1.3 ms (latency of L2 round trips and of the barriers, one
+// 5.5 ms per solve of 11 CG steps, now 1.4 ms (latency of L2 round trips and of the barriers, one
 // instruction in six cycles issued; the loads of two cells in flight at once cost 8 % in index
 // arithmetic).
 // The V-cycle: damped Jacobi smoothing (two sweeps before and two after), restriction by summing
@@ -18,6 +18,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstring>
 
 #include "internal.h"
 #include "mg.h"
@@ -26,6 +27,7 @@ namespace iugkp {
 
 constexpr int MG32_PASSES_FD = 6;  // refinement passes of the fast diagonalization solve at most
 constexpr int MG_NT = 1024;        // threads per block, multigrid CG
+constexpr int MG_SMALL_NT = 512;   // ... where every instance is small: fewer warps per barrier
 constexpr int FD_NT = 512;         // ... fast diagonalization
 // Polls of a team barrier (an L2 round trip each) before a block gives up: a second or so.
 constexpr unsigned TEAM_SPIN_LIMIT = 1u << 21;
@@ -102,6 +104,7 @@ struct Team {
   bool dead;         // a barrier was given up (the same for all threads of the block)
   static constexpr bool solo = false;
   __device__ static float ld(const float* p) { return __ldcg(p); }
+  __device__ __forceinline__ int stride() const { return (int)blockDim.x; }
   // What the team's blocks wrote before it is visible to all of them after it.
   __device__ __forceinline__ void sync() {
     __shared__ int s_open;
@@ -131,7 +134,7 @@ struct Team {
     hi = min(nc, lo + chunk);
   }
   // Sums NV values over the whole team in a fixed order; also a barrier.
-  template <int NT, int NV>
+  template <int NV>
   __device__ __forceinline__ void sum(double (&v)[NV], double* sh) {
     static_assert(NV <= 2, "two values at most");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -145,7 +148,7 @@ struct Team {
     __syncthreads();
     double* mine = slots + (size_t)buf * size * 2;
     if (warp < NV) {
-      double x = lane < NT / 32 ? sh[warp * 32 + lane] : 0.0;
+      double x = lane < (int)(blockDim.x >> 5) ? sh[warp * 32 + lane] : 0.0;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
       if (lane == 0) mine[rank * 2 + warp] = x;
@@ -171,30 +174,37 @@ struct Team {
 // in FP64. A team's blocks take whole units, so that a sum does not depend on how many blocks share
 // the instance. The products are formed in parallel over units and steps and pass through shared
 // memory to the warp that adds a unit's.
-constexpr int MG_RANKS = 8, MG_WARPS = 16, MG_UNITS = MG_RANKS * MG_WARPS;
+constexpr int MG_RANKS = 8, MG_WARPS = 16;
 constexpr int MG_STAGE = 128;  // unit steps staged at a time
 
+__host__ __device__ __forceinline__ int range_units_log(long long chunk) {
+  int l = 0;
+  while ((32 << l) < chunk && (1 << l) < MG_WARPS) ++l;
+  return l;
+}
+
 struct Units {
-  int n, chunk, steps;  // cells, cells of a range, steps of a unit
-  int u0, u1;           // this block's units
+  int n, chunk, steps, lw;  // cells, cells of a range, steps of a unit, 2^lw units of a range (all that have cells)
+  int u0, u1;               // this block's units
   __device__ __forceinline__ Units(int cells, const Team& tm) {
     n = cells;
     chunk = (cells + MG_RANKS - 1) / MG_RANKS;
     steps = (chunk + 32 * MG_WARPS - 1) / (32 * MG_WARPS);
-    const int per = (MG_UNITS + tm.size - 1) / tm.size;
-    u0 = min(MG_UNITS, tm.rank * per);
-    u1 = min(MG_UNITS, u0 + per);
+    lw = range_units_log(chunk);
+    const int all = MG_RANKS << lw, per = (all + tm.size - 1) / tm.size;
+    u0 = min(all, tm.rank * per);
+    u1 = min(all, u0 + per);
   }
   // Cell of a lane at a unit's step, or -1.
   __device__ __forceinline__ int cell(int unit, int step) const {
-    const int r = unit / MG_WARPS, o = (unit - r * MG_WARPS) * 32 + (threadIdx.x & 31) + step * (32 * MG_WARPS);
+    const int r = unit >> lw, o = (unit - (r << lw)) * 32 + (threadIdx.x & 31) + step * (32 * MG_WARPS);
     const int i = r * chunk + o;
     return o < chunk && i < n ? i : -1;
   }
   template <class F>
   __device__ __forceinline__ void each(F f) const {
     const int total = (u1 - u0) * steps;
-    for (int e = threadIdx.x >> 5; e < total; e += MG_NT / 32) {
+    for (int e = threadIdx.x >> 5; e < total; e += (int)(blockDim.x >> 5)) {
       const int q = e / steps, i = cell(u0 + q, e - q * steps);
       if (i >= 0) f(i);
     }
@@ -204,17 +214,15 @@ struct Units {
   template <int NS, int NV, unsigned A, unsigned B, class F>
   __device__ __forceinline__ void dot(F f, float (*stage)[NS * 32], double (&out)[NV]) const {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int sg = min(steps, MG_STAGE), ug = min(MG_NT / 32, MG_STAGE / sg);  // steps, units staged at a time
+    const int sg = min(steps, MG_STAGE), ug = MG_STAGE / sg;  // steps, units staged at a time (steps over MG_STAGE: one)
 #pragma unroll
     for (int v = 0; v < NV; ++v) out[v] = 0.0;
+    float acc[NV];
     for (int ub = u0; ub < u1; ub += ug) {
       const int nu = min(ug, u1 - ub);
-      float acc[NV];
-#pragma unroll
-      for (int v = 0; v < NV; ++v) acc[v] = 0.f;
       for (int sb = 0; sb < steps; sb += sg) {
         const int ns = min(sg, steps - sb), total = nu * ns;
-        for (int e = warp; e < total; e += MG_NT / 32) {
+        for (int e = warp; e < total; e += (int)(blockDim.x >> 5)) {
           const int q = e / ns, i = cell(ub + q, sb + e - q * ns);
           float x[NS];
 #pragma unroll
@@ -224,20 +232,24 @@ struct Units {
           for (int t = 0; t < NS; ++t) stage[e][t * 32 + lane] = x[t];
         }
         __syncthreads();
-        if (warp < nu) {
+        for (int u = warp; u < nu; u += (int)(blockDim.x >> 5)) {
+          if (sb == 0) {
+#pragma unroll
+            for (int v = 0; v < NV; ++v) acc[v] = 0.f;
+          }
 #pragma unroll 4
           for (int st = 0; st < ns; ++st) {
-            const float* x = stage[warp * ns + st];
+            const float* x = stage[u * ns + st];
 #pragma unroll
             for (int v = 0; v < NV; ++v)
               acc[v] = fmaf(x[((A >> (4 * v)) & 15u) * 32 + lane], x[((B >> (4 * v)) & 15u) * 32 + lane], acc[v]);
           }
+          if (sb + ns == steps) {
+#pragma unroll
+            for (int v = 0; v < NV; ++v) out[v] += (double)acc[v];
+          }
         }
         __syncthreads();
-      }
-      if (warp < nu) {
-#pragma unroll
-        for (int v = 0; v < NV; ++v) out[v] += (double)acc[v];
       }
     }
   }
@@ -247,9 +259,11 @@ struct Units {
 // memory: the work is small and every phase waits for the previous one, so the barriers and
 // L2 round trips are what they would cost on the team.
 struct SoloTeam {
+  int nt;  // threads: as many as the level has cells, whole warps (a barrier of 32 warps costs more than one of a few)
   static constexpr bool solo = true;
   __device__ static float ld(const float* p) { return *p; }
-  __device__ __forceinline__ void sync() const { __syncthreads(); }
+  __device__ __forceinline__ int stride() const { return nt; }
+  __device__ __forceinline__ void sync() const { asm volatile("bar.sync 1, %0;" ::"r"(nt) : "memory"); }
   __device__ __forceinline__ void range(int nc, int& lo, int& hi) const {
     lo = 0;
     hi = nc;
@@ -257,6 +271,7 @@ struct SoloTeam {
 };
 
 constexpr long long MG_SOLO_CELLS = 4096;
+constexpr long long MG_SMALL_CELLS = 1024;  // instances up to here take one block
 
 // out[i] = f(i) for every cell of a level that falls on this block: the finest level by units (its
 // vectors are the CG's), the others in contiguous ranges.
@@ -270,7 +285,7 @@ __device__ __forceinline__ void level_each(const TM& tm, int l, int nc, float* o
   }
   int lo, hi;
   tm.range(nc, lo, hi);
-  for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) out[i] = f(i);
+  for (int i = lo + threadIdx.x; i < hi; i += tm.stride()) out[i] = f(i);
 }
 
 __device__ __forceinline__ void level_coords(const int* n, int i, int& x, int& y, int& z) {
@@ -367,7 +382,7 @@ __device__ void vdown(const MGArgs& A, const InstMG& m, int l, const LevelView& 
   int clo, chi;
   tm.range(ncc, clo, chi);
   auto at = [&](int j) { return TM::ld(&v.x[j]); };
-  for (int I = clo + threadIdx.x; I < chi; I += blockDim.x) {
+  for (int I = clo + threadIdx.x; I < chi; I += tm.stride()) {
     int X0, Y0, Z0;
     level_coords(nC, I, X0, Y0, Z0);
     float sum = 0.f;
@@ -393,7 +408,7 @@ __device__ void vcoarsest(const MGArgs& A, const InstMG& m, const LevelView& v, 
   int lo, hi;
   tm.range(nc, lo, hi);
   const float* inv = A.cinv + m.cinv_off;
-  for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) {
+  for (int i = lo + threadIdx.x; i < hi; i += tm.stride()) {
     float sum = 0.f;
     for (int j = 0; j < nc; ++j) sum += inv[i * nc + j] * TM::ld(&v.b[j]);
     v.x[i] = sum;
@@ -437,23 +452,24 @@ __host__ __device__ __forceinline__ int solo_level(const InstMG& m) {
 // level's right-hand side into its shared memory, runs the rest of the cycle there, and writes
 // the level's correction back for the team.
 __device__ void vcycle(const MGArgs& A, const InstMG& m, Team& tm, float* smem) {
-  SoloTeam solo;
   const int L = m.levels;
   const int ls = solo_level(m);
+  SoloTeam solo;
+  solo.nt = min((int)blockDim.x, ((int)m.nc[ls] + 31) & ~31);
   for (int l = 0; l < ls; ++l) vdown(A, m, l, global_view(A, m, l), global_view(A, m, l + 1), tm);
-  if (tm.rank == 0) {
+  if (tm.rank == 0 && (int)threadIdx.x < solo.nt) {
     const LevelView top = solo_view(A, m, ls, ls, smem);
     const float* gb = A.lb + m.off[ls];
-    for (int i = threadIdx.x; i < m.nc[ls]; i += blockDim.x) top.b[i] = __ldcg(&gb[i]);
-    __syncthreads();
+    for (int i = threadIdx.x; i < m.nc[ls]; i += solo.nt) top.b[i] = __ldcg(&gb[i]);
+    solo.sync();
     for (int l = ls; l < L - 1; ++l) vdown(A, m, l, solo_view(A, m, l, ls, smem), solo_view(A, m, l + 1, ls, smem), solo);
     vcoarsest(A, m, solo_view(A, m, L - 1, ls, smem), solo);
     for (int l = L - 2; l >= ls; --l) {
       vup(A, m, l, solo_view(A, m, l, ls, smem), solo_view(A, m, l + 1, ls, smem), solo);
-      __syncthreads();
+      solo.sync();
     }
     float* gx = A.lx + m.off[ls];
-    for (int i = threadIdx.x; i < m.nc[ls]; i += blockDim.x) gx[i] = top.x[i];
+    for (int i = threadIdx.x; i < m.nc[ls]; i += solo.nt) gx[i] = top.x[i];
   }
   tm.sync();
   for (int l = ls - 1; l >= 0; --l) {
@@ -647,7 +663,7 @@ __device__ int fd_solve(const MGArgs& A, int k, const InstMG& m, Team& tm, doubl
     A.Z[off + c] = b;  // FP64 residual
     v[0] += b * b;
   }
-  tm.sum<FD_NT, 1>(v, sh);
+  tm.sum<1>(v, sh);
   const double bb = v[0], tol2 = A.rtol * A.rtol * bb;
   int passes = bb == 0.0 ? 0 : -1;
   double rr = bb;
@@ -682,7 +698,7 @@ __device__ int fd_solve(const MGArgs& A, int k, const InstMG& m, Team& tm, doubl
       A.Z[off + c] = r;
       v[0] += r * r;
     }
-    tm.sum<FD_NT, 1>(v, sh);  // also orders the residual's writes before the next pass
+    tm.sum<1>(v, sh);  // also orders the residual's writes before the next pass
     rr = v[0];
     if (rr <= tol2) passes = pass;
   }
@@ -758,7 +774,7 @@ __global__ void __launch_bounds__(MG_NT, 1) mgpcg_kernel(MGArgs A) {
       b32[i] = (float)bi;
       v[0] += bi * bi;
     });
-    tm.sum<MG_NT, 1>(v, sh);
+    tm.sum<1>(v, sh);
     const double bb = v[0];
     int it = 0;
     bool done = bb == 0.0;
@@ -771,7 +787,7 @@ __global__ void __launch_bounds__(MG_NT, 1) mgpcg_kernel(MGArgs A) {
         A.P[off + i] = zi;
         v[0] += A.Rr[off + i] * zi;
       });
-      tm.sum<MG_NT, 1>(v, sh);  // also orders the P writes before the first product
+      tm.sum<1>(v, sh);  // also orders the P writes before the first product
       double rz = v[0];
       while (it < A.maxit && !tm.dead) {
         ++it;
@@ -781,7 +797,7 @@ __global__ void __launch_bounds__(MG_NT, 1) mgpcg_kernel(MGArgs A) {
           A.Q[off + i] = q;
           v[0] += __ldcg(&A.P[off + i]) * q;
         });
-        tm.sum<MG_NT, 1>(v, sh);
+        tm.sum<1>(v, sh);
         const double alpha = rz / v[0];
         v[0] = 0.0;
         un.each([&](int i) {
@@ -792,7 +808,7 @@ __global__ void __launch_bounds__(MG_NT, 1) mgpcg_kernel(MGArgs A) {
           b32[i] = (float)ri;
           v[0] += ri * ri;
         });
-        tm.sum<MG_NT, 1>(v, sh);
+        tm.sum<1>(v, sh);
         if (v[0] <= tol2) {
           done = true;
           break;
@@ -806,7 +822,7 @@ __global__ void __launch_bounds__(MG_NT, 1) mgpcg_kernel(MGArgs A) {
           w[0] += A.Rr[off + i] * zi;
           w[1] += A.Q[off + i] * zi;
         });
-        tm.sum<MG_NT, 2>(w, sh);
+        tm.sum<2>(w, sh);
         const double beta = -alpha * w[1] / rz;
         rz = w[0];
         un.each([&](int i) { A.P[off + i] = (double)x32[i] + beta * A.P[off + i]; });
@@ -863,7 +879,7 @@ __global__ void __launch_bounds__(MG_NT, 1) mgpcg32_kernel(MGArgs A, float* V32)
       A.Z[off + i] = bi;
       v[0] += bi * bi;
     });
-    tm.sum<MG_NT, 1>(v, sh);
+    tm.sum<1>(v, sh);
     const double bb = v[0];
     const double tol2 = A.rtol * A.rtol * bb;
     double rr = bb;  // FP64 squared norm of the FP64 residual
@@ -889,7 +905,7 @@ __global__ void __launch_bounds__(MG_NT, 1) mgpcg32_kernel(MGArgs A, float* V32)
             x[1] = zi;
           },
           st2, v);
-      tm.sum<MG_NT, 1>(v, sh);  // also orders the P writes before the first product
+      tm.sum<1>(v, sh);  // also orders the P writes before the first product
       double rz = v[0];
       while (it < A.maxit && !tm.dead) {
         ++it;
@@ -902,7 +918,7 @@ __global__ void __launch_bounds__(MG_NT, 1) mgpcg32_kernel(MGArgs A, float* V32)
               x[1] = q;
             },
             st2, v);
-        tm.sum<MG_NT, 1>(v, sh);
+        tm.sum<1>(v, sh);
         const double alpha = rz / v[0];
         const float af = (float)alpha;
         un.dot<1, 1, 0, 0>(
@@ -913,7 +929,7 @@ __global__ void __launch_bounds__(MG_NT, 1) mgpcg32_kernel(MGArgs A, float* V32)
               x[0] = ri;
             },
             st1, v);
-        tm.sum<MG_NT, 1>(v, sh);  // also orders the residual's writes before the V-cycle
+        tm.sum<1>(v, sh);  // also orders the residual's writes before the V-cycle
         if (v[0] <= in2) break;
         vcycle(A, m, tm, mg_smem);
         // flexible (Polak-Ribiere) beta, as in the FP64 kernel
@@ -925,7 +941,7 @@ __global__ void __launch_bounds__(MG_NT, 1) mgpcg32_kernel(MGArgs A, float* V32)
               x[2] = __ldcg(&Z[i]);
             },
             st3, w);
-        tm.sum<MG_NT, 2>(w, sh);
+        tm.sum<2>(w, sh);
         const double beta = -alpha * w[1] / rz;
         rz = w[0];
         const float bf = (float)beta;
@@ -941,7 +957,7 @@ __global__ void __launch_bounds__(MG_NT, 1) mgpcg32_kernel(MGArgs A, float* V32)
         A.Z[off + i] = r;
         v[0] += r * r;
       });
-      tm.sum<MG_NT, 1>(v, sh);  // also orders the residual's writes before the next pass
+      tm.sum<1>(v, sh);  // also orders the residual's writes before the next pass
       rr = v[0];
       done = rr <= tol2;
     }
@@ -1020,11 +1036,14 @@ cudaError_t configure_mgpcg(Ctx* c, const std::vector<InstMG>& h_mg) {
         cost.push_back((double)m.fnx * (m.fnx + m.fny));
         smem = std::max(smem, fd_smem_floats(std::max(m.fnx, m.fny)) * sizeof(float));
       } else {
-        // parts: units, by their steps; no more blocks than give every warp a step
+        // parts: units, by their steps; no more blocks than give every warp a step, and one for
+        // small instances (a 400-cell film: 697 us on four blocks of 1024 threads, 446 on one of 512)
         const long long chunk = (m.nc[0] + MG_RANKS - 1) / MG_RANKS, steps = (chunk + 32 * MG_WARPS - 1) / (32 * MG_WARPS);
-        const int most = (int)std::min<long long>(MG_UNITS, MG_UNITS * steps / (MG_NT / 32));
+        const long long units = (long long)MG_RANKS << range_units_log(chunk);
+        const int most =
+            m.nc[0] <= MG_SMALL_CELLS ? 1 : (int)std::max<long long>(1, std::min(units, units * steps / (MG_NT / 32)));
         parts.push_back(most);
-        cost.push_back((double)steps * MG_UNITS / most);
+        cost.push_back((double)steps * units / most);
         size_t cells = 0;
         for (int l = solo_level(m); l < m.levels; ++l) cells += (size_t)m.nc[l];
         smem = std::max(std::max(smem, 3 * cells * sizeof(float)), (size_t)MG_STAGE * 96 * sizeof(float));
@@ -1032,6 +1051,9 @@ cudaError_t configure_mgpcg(Ctx* c, const std::vector<InstMG>& h_mg) {
     }
     p.blocks = 0;
     p.smem = smem;
+    p.threads = kind ? FD_NT : MG_NT;
+    if (kind == 0 && std::all_of(which.begin(), which.end(), [&](int k) { return h_mg[k].nc[0] <= MG_SMALL_CELLS; }))
+      p.threads = MG_SMALL_NT;
     if (which.empty()) continue;
     const void* f[2] = {kind ? (const void*)fd_kernel : (const void*)mgpcg_kernel,
                         kind ? (const void*)fd_kernel : (const void*)mgpcg32_kernel};
@@ -1046,16 +1068,20 @@ cudaError_t configure_mgpcg(Ctx* c, const std::vector<InstMG>& h_mg) {
     std::vector<int> order, block_team;
     plan_teams(which, cost, parts, c->sm_count, teams, order, block_team);
     p.blocks = (int)block_team.size();
-    auto up = [&](void** d, const void* h, size_t bytes) {
-      cudaError_t ue = cudaMalloc(d, bytes);
-      if (ue != cudaSuccess) return ue;
-      return h ? cudaMemcpy(*d, h, bytes, cudaMemcpyHostToDevice) : cudaMemset(*d, 0, bytes);
-    };
-    if ((e = up(&p.d_teams, teams.data(), teams.size() * sizeof(TeamDesc))) != cudaSuccess) return e;
-    if ((e = up((void**)&p.d_order, order.data(), order.size() * sizeof(int))) != cudaSuccess) return e;
-    if ((e = up((void**)&p.d_block_team, block_team.data(), block_team.size() * sizeof(int))) != cudaSuccess) return e;
-    if ((e = up((void**)&p.d_bar, nullptr, 2 * teams.size() * sizeof(unsigned))) != cudaSuccess) return e;
-    if ((e = up((void**)&p.d_slots, nullptr, 4 * block_team.size() * sizeof(double))) != cudaSuccess) return e;
+    // one buffer: partial sums and barrier words (zero), then the plan
+    const size_t at_bar = 4 * block_team.size() * sizeof(double), at_teams = at_bar + 2 * teams.size() * sizeof(unsigned),
+                 at_order = at_teams + teams.size() * sizeof(TeamDesc), at_block = at_order + order.size() * sizeof(int);
+    std::vector<char> h(at_block + block_team.size() * sizeof(int), 0);
+    std::memcpy(h.data() + at_teams, teams.data(), teams.size() * sizeof(TeamDesc));
+    std::memcpy(h.data() + at_order, order.data(), order.size() * sizeof(int));
+    std::memcpy(h.data() + at_block, block_team.data(), block_team.size() * sizeof(int));
+    if ((e = cudaMalloc((void**)&p.d_buf, h.size())) != cudaSuccess) return e;
+    if ((e = cudaMemcpy(p.d_buf, h.data(), h.size(), cudaMemcpyHostToDevice)) != cudaSuccess) return e;
+    p.d_slots = reinterpret_cast<double*>(p.d_buf);
+    p.d_bar = reinterpret_cast<unsigned*>(p.d_buf + at_bar);
+    p.d_teams = p.d_buf + at_teams;
+    p.d_order = reinterpret_cast<int*>(p.d_buf + at_order);
+    p.d_block_team = reinterpret_cast<int*>(p.d_buf + at_block);
   }
   return cudaSuccess;
 }
@@ -1103,7 +1129,7 @@ static cudaError_t launch_correction(const Ctx* c, const CorrectionIO& io, cudaS
     a.slots = p.d_slots;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(p.blocks, 1, 1);
-    cfg.blockDim = dim3(kind ? FD_NT : MG_NT, 1, 1);
+    cfg.blockDim = dim3(p.threads, 1, 1);
     cfg.dynamicSmemBytes = p.smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
