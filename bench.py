@@ -27,7 +27,7 @@ KNS = (0.01, 0.1, 1.0, 10.0)
 # From one ncu capture of the current sweep kernel on this workload (the command and the
 # figures are in profiles/sweep_cavity128_4kn.md); retaken whenever the kernel changes.
 SWEEP_DRAM_BYTES = 2.81e6  # dram__bytes_read.sum + dram__bytes_write.sum per launch
-SWEEP_ISSUE_UTIL = 0.808   # smsp__issue_active of the same launch
+SWEEP_ISSUE_UTIL = 0.831   # smsp__issue_active of the same launch
 NGRID = 128
 NPART = 1024
 
@@ -438,8 +438,8 @@ def newton_step_time(lib, L, solver, T, T_half, R, stream, sp, flush, reps):
     """The correction solve alone (Newton right-hand side, solve, update) on the fields of one
     iteration, timed with CUDA events on the launching stream. The bench instances have uniform
     kappa, so the solve is the fast diagonalization (four dense FP32 products per refinement
-    pass, 4 nx ny (nx + ny) flops per instance, and one FP64 residual pass); it runs on one
-    8-CTA cluster per instance and is bound by the latency of its cluster barriers, so the
+    pass, 4 nx ny (nx + ny) flops per instance, and one FP64 residual pass); its blocks are dealt
+    to the instances and it is bound by the latency of their barriers and L2 reads, so the
     achieved rates are small by nature."""
     import ctypes
     import torch
@@ -462,7 +462,7 @@ def newton_step_time(lib, L, solver, T, T_half, R, stream, sp, flush, reps):
     flops = sum(4.0 * g.n[0] * g.n[1] * (g.n[0] + g.n[1]) for g in solver.grids) * its
     return {"ms": t, "method": "fast diagonalization (separable operator), FP64 refinement", "passes": its,
             "flops": flops, "achieved_tflops": flops / (t * 1e-3) / 1e12,
-            "note": "one 8-CTA cluster per instance; latency-bound (cluster barriers)"}
+            "note": "one team of blocks per instance; latency-bound (barriers, L2 reads)"}
 
 
 def slab_config(WL, make_solver):
@@ -839,11 +839,9 @@ def run_ours(args):
             "speedup_vs_plain_fp64_sweep": (sweep_counts[3] / sw_s) / plain["sweep_crossings_per_s"] if plain else None,
             "e2e": {"value": e2e_value, "unit": "cell-crossings/s", "h2d_bytes_per_step": nc * 8,
                     "d2h_bytes_per_step": nc * 8},
-            # per step: group_wmax, sweep, FP64 replay, scale_by_taumaj, boundary_emission,
-            # derive_two_group, assemble_two_group, wall_absorbed, macro, newton_rhs, correction
-            # solve, add_scaled, residual (2 kernels), plus three finalize passes (R, W, F) with
-            # compensated FP32 tallies
-            "gpu_launches": args.steps * (14 + (3 if tuned.get("tally") == 2 else 0)),
+            # per step: prologue, sweep, FP64 replay, closing pass, macro, correction solve,
+            # residual (2 kernels), plus two finalize passes (R, W) with compensated FP32 tallies
+            "gpu_launches": args.steps * (8 + (2 if tuned.get("tally") == 2 else 0)),
             "roofline": {"bound": "alu", "achieved": achieved / 1e12, "peak": peak_ops / 1e12,
                          "unit": "Tops/s (FP32+INT32 lane ops)", "frac": achieved / peak_ops,
                          # DRAM bytes (read + write) of one launch of this sweep kernel on this
