@@ -10,6 +10,7 @@
 #include <string>
 #include <vector>
 
+#include "fp32_range.h"
 #include "internal.h"
 
 using namespace iugkp;
@@ -743,7 +744,13 @@ iugkp_status iugkp_create_batch(int n, const iugkp_grid* g, const double* const*
   {
     std::vector<float> vtm((size_t)n * nb);
     for (int k = 0; k < n; ++k)
-      for (int bb = 0; bb < nb; ++bb) vtm[(size_t)k * nb + bb] = (float)(c->h_v[bb] * taumaj[(size_t)k * nb + bb]);
+      for (int bb = 0; bb < nb; ++bb) {
+        const double free_path = c->h_v[bb] * taumaj[(size_t)k * nb + bb];
+        vtm[(size_t)k * nb + bb] = (float)free_path;
+        c->fp32_lengths = c->fp32_lengths && fp32_length(free_path);
+      }
+    for (const InstDesc& in : c->h_inst)
+      for (int a = 0; a < dim; ++a) c->fp32_lengths = c->fp32_lengths && fp32_length(in.h[a]);
     UP(c->d_vtm32, vtm);
   }
   UP(c->d_v, c->h_v);
@@ -963,12 +970,17 @@ bool land_sizes(const Ctx* c) {
   return true;
 }
 
-// FP64 tracking by the filtered sweep (exact.cu): the default step budget or more (the plain
-// kernel counts every crossing against it), as all queue entries and indices are 32-bit.
-bool exact_path(const Ctx* c) {
-  return c->opt.precision == IUGKP_TRACK_FP64 && c->opt.step_budget >= EXACT_MIN_BUDGET &&
-         c->fwd_particles < (1ll << 31) && land_sizes(c);
+// FP64 tracking whose decisions may be filtered in FP32 (exact.cu, land.cu): the default step budget
+// or more (the plain kernel counts every crossing against it), and cell sizes and mean free paths
+// well inside FP32 (fp32_range.h; the plain kernel takes any). With FP32 tracking lengths beyond
+// FP32 leave particles to the FP64 replay instead.
+bool filtered_fp64(const Ctx* c) {
+  if (c->opt.precision != IUGKP_TRACK_FP64 || c->opt.step_budget < EXACT_MIN_BUDGET || !land_sizes(c)) return false;
+  return c->fp32_lengths;
 }
+
+// FP64 tracking by the filtered sweep (exact.cu): all queue entries and indices are 32-bit.
+bool exact_path(const Ctx* c) { return filtered_fp64(c) && c->fwd_particles < (1ll << 31); }
 
 // Buffers of the compensated FP32 tallies; allocated outside any stream capture.
 iugkp_status ensure_k32(Ctx* c) {
@@ -1542,12 +1554,13 @@ iugkp_status iugkp_average(iugkp_ctx* ctx, double* T_inout_dev, int n_steps, uns
 
 namespace {
 
-// The adjoint re-trace into a.adj_out and a.adj_wall (cleared here): the landing kernels for the FP32 walk with staged tallies (the
-// fast path), else the plain one-thread-per-particle kernel.
+// The adjoint re-trace into a.adj_out and a.adj_wall (cleared here): the landing kernels for the FP32
+// walk with staged tallies and for the filtered FP64 walk, else the plain one-thread-per-particle
+// kernel.
 cudaError_t adjoint_sweep(Ctx* c, const SweepArgs& a, cudaStream_t s) {
-  const bool filtered = c->opt.precision == IUGKP_TRACK_FP64 ? c->opt.step_budget >= EXACT_MIN_BUDGET
-                                                             : c->opt.tally != IUGKP_TALLY_FP64;
-  if (filtered && c->total_particles < (1ll << 31) && land_sizes(c))
+  const bool filtered = c->opt.precision == IUGKP_TRACK_FP64 ? filtered_fp64(c)
+                                                             : c->opt.tally != IUGKP_TALLY_FP64 && land_sizes(c);
+  if (filtered && c->total_particles < (1ll << 31))
     return launch_land(c, a, true, s);
   cudaError_t e = cudaMemsetAsync(a.adj_out, 0, c->total_cells * sizeof(double), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(a.adj_wall, 0, c->total_walls * sizeof(double), s);

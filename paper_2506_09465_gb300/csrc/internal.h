@@ -125,6 +125,7 @@ struct Ctx {
   long long* d_Fi = nullptr;     // [total_faces] ... and fixed-point face sums in units of q
   unsigned* d_ticket = nullptr;  // [1 + n_inst] finished blocks of the passes around a trace (0 between launches)
   unsigned long long* d_wpart = nullptr;  // [wmax_blocks] largest weight of each block of the pass before it
+  bool fp32_lengths = true;      // every cell size and mean free path well inside FP32 (fp32_range.h)
   bool any_two_group = false;    // some instance of the context uses the two-group tallies
   bool all_two_group = false;    // ... every instance does (no face follows from a column walk)
   bool sync_ok = false;          // 2D: the pass-synchronous staged kernel applies

@@ -20,6 +20,7 @@
 #include <cuda_runtime.h>
 
 #include "device.cuh"
+#include "fp32_range.h"
 #include "staged.h"
 #include "walk32.cuh"
 
@@ -30,11 +31,12 @@ constexpr float LAND_ABS = 0x1p-22f;
 constexpr float FLOOR_MAGIC = 12582912.f;  // 1.5 2^23: a round-down add leaves floor(X) in the low bits, |X| < 2^22
 
 // Position of a candidate along one axis: its cell offset and whether it lies within tol of a
-// face (either side).
+// face (either side). Where v tau_maj overflows FP32, X and tol are infinite and the offset is
+// no cell's: near then (face_near).
 __device__ __forceinline__ int floor_near(float X, float tol, bool& near) {
   const float Y = __fadd_rd(X, FLOOR_MAGIC);
   const float fr = X - (Y - FLOOR_MAGIC);
-  near |= fminf(fr, 1.f - fr) <= tol;
+  near |= face_near(fr, 1.f - fr, tol);
   return __float_as_int(Y) - 0x4B400000;
 }
 
