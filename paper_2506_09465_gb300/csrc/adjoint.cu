@@ -140,50 +140,50 @@ struct AdjointGather {
   }
 };
 
-// FP64 re-trace (analytic along the straight segment, replay.cuh) of the particles the staged
-// adjoint re-trace deferred; the forward sweep defers the same particles. One thread per
-// entry; entry x: the staged index, particle q of emitter e taken q-major within its group.
+// FP64 re-trace (analytic along the straight segment, replay.cuh) of one particle that the landing
+// re-trace left undecided; the forward sweep leaves the same particles. pid: the staged index, particle
+// q of emitter e taken q-major within its group.
 template <int DIM>
-__global__ void __launch_bounds__(128) adjoint_replay_kernel(SweepArgs A, const uint2* defer, const unsigned* defer_n,
-                                                             unsigned defer_cap) {
-  const unsigned n = min(*defer_n, defer_cap);
+__device__ __forceinline__ void adjoint_replay(const SweepArgs& A, unsigned pid) {
+  const Group G = A.groups[find_group(A.groups, A.n_groups, (long long)pid)];
+  const InstDesc& in = A.inst[G.inst];
+  const unsigned local = pid - (unsigned)G.first_particle;
+  const int q = (int)(local / (unsigned)G.n_emitters);
+  int e0 = (int)(local - (unsigned)q * (unsigned)G.n_emitters);
+  if (G.perm_off >= 0) e0 = A.perm[G.perm_off + e0];  // the staged visiting order
+  Walk<double, DIM> wk;
+  Stream st;
+  double coefp;
+  int e;
+  adjoint_emit<double, DIM>(A, G.first_particle + (long long)e0 * G.per_emitter + q, G, wk, st, coefp, e);
+  Seg64<DIM> sg;
+  sg.init(wk, in);
+  AdjointGather pol{A, in, coefp, 0.0};
+  int fb[DIM];
+  const int res = replay_candidates<DIM>(A, in, G.inst, G.band, wk, sg, st, fb, pol);
+  if (res < 0) atomicOr(A.err, ERR_BUDGET);
+  if (res <= 0) return;  // dropped, or absorbed by a wall: no gather
+  if (G.kind == 0) atomicAdd(&A.adj_out[in.cell_off + e], pol.val);
+  else atomicAdd(&A.adj_wall[in.wall_off + G.kind - 1], pol.val);
+}
+
+// The particles of the queue, one thread each, then those beyond it.
+template <int DIM>
+__global__ void __launch_bounds__(128) adjoint_replay_kernel(SweepArgs A, StagedArgs S) {
+  const unsigned n = min(*S.defer_n, S.defer_cap);
   // warp j of every block numbered before warp j + 1 of any, 32 entries each (as in
   // replay_kernel): the short queue's work is spread over the SMs
   const unsigned wid = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
-  for (unsigned i = 32u * wid + (threadIdx.x & 31); i < n; i += gridDim.x * blockDim.x) {
-    const unsigned pid = defer[i].x;
-    const Group G = A.groups[find_group(A.groups, A.n_groups, (long long)pid)];
-    const InstDesc& in = A.inst[G.inst];
-    const unsigned local = pid - (unsigned)G.first_particle;
-    const int q = (int)(local / (unsigned)G.n_emitters);
-    int e0 = (int)(local - (unsigned)q * (unsigned)G.n_emitters);
-    if (G.perm_off >= 0) e0 = A.perm[G.perm_off + e0];  // the staged visiting order
-    Walk<double, DIM> wk;
-    Stream st;
-    double coefp;
-    int e;
-    adjoint_emit<double, DIM>(A, G.first_particle + (long long)e0 * G.per_emitter + q, G, wk, st, coefp, e);
-    Seg64<DIM> sg;
-    sg.init(wk, in);
-    AdjointGather pol{A, in, coefp, 0.0};
-    int fb[DIM];
-    const int res = replay_candidates<DIM>(A, in, G.inst, G.band, wk, sg, st, fb, pol);
-    if (res < 0) {
-      atomicOr(A.err, ERR_BUDGET);
-      continue;
-    }
-    if (res == 0) continue;  // absorbed by a wall: no gather
-    if (G.kind == 0) atomicAdd(&A.adj_out[in.cell_off + e], pol.val);
-    else atomicAdd(&A.adj_wall[in.wall_off + G.kind - 1], pol.val);
-  }
+  for (unsigned i = 32u * wid + (threadIdx.x & 31); i < n; i += gridDim.x * blockDim.x) adjoint_replay<DIM>(A, S.defer[i].x);
+  for_overflow(S, [&](unsigned pid) { adjoint_replay<DIM>(A, pid); });
 }
 
-cudaError_t launch_adjoint_replay(const Ctx* c, const SweepArgs& a, cudaStream_t s) {
+cudaError_t launch_adjoint_replay(const Ctx* c, const SweepArgs& a, const StagedArgs& S, cudaStream_t s) {
   const int blocks = c->sm_count * 4;
   switch (c->dim) {
-    case 1: adjoint_replay_kernel<1><<<blocks, 128, 0, s>>>(a, c->d_defer, c->d_defer_n, c->defer_cap); break;
-    case 2: adjoint_replay_kernel<2><<<blocks, 128, 0, s>>>(a, c->d_defer, c->d_defer_n, c->defer_cap); break;
-    default: adjoint_replay_kernel<3><<<blocks, 128, 0, s>>>(a, c->d_defer, c->d_defer_n, c->defer_cap); break;
+    case 1: adjoint_replay_kernel<1><<<blocks, 128, 0, s>>>(a, S); break;
+    case 2: adjoint_replay_kernel<2><<<blocks, 128, 0, s>>>(a, S); break;
+    default: adjoint_replay_kernel<3><<<blocks, 128, 0, s>>>(a, S); break;
   }
   return cudaGetLastError();
 }

@@ -207,6 +207,7 @@ struct Ctx {
   uint2* d_defer = nullptr;
   unsigned* d_defer_n = nullptr;     // [4] queue length, queued faces (exact.cu), 64-bit claim counter (land.cu, exact.cu)
   unsigned defer_cap = 0;
+  unsigned* d_over = nullptr;        // [particles / 32] landing sweeps: particles beyond the queue (0 between launches)
   // tasks of the pass-synchronous 2D sweep and of the filtered FP64 sweep (as many particles per
   // emitter and task as warp_grab allows): the groups', and each instance's range
   LandGroup* d_sync_groups = nullptr;
@@ -267,7 +268,7 @@ cudaError_t launch_land(const Ctx* c, const SweepArgs& a, bool adj, cudaStream_t
 void land_tasks(const Ctx* c, const std::vector<Group>& groups, std::vector<LandGroup>& out, unsigned& n_tasks, int& qch,
                 int qch_max, int warps_per_sm, bool join);
 cudaError_t launch_replay(const Ctx* c, const SweepArgs& a, const StagedArgs& S, cudaStream_t s);
-cudaError_t launch_adjoint_replay(const Ctx* c, const SweepArgs& a, cudaStream_t s);
+cudaError_t launch_adjoint_replay(const Ctx* c, const SweepArgs& a, const StagedArgs& S, cudaStream_t s);
 cudaError_t launch_walk_bounds(unsigned long long* out, cudaStream_t s);
 double walk_bound_fraction(const double* measured);
 cudaError_t measure_atomic_rate(int sm_count, double* out_rate);

@@ -24,6 +24,17 @@ __device__ __forceinline__ void deposit(const SweepArgs& A, const StagedArgs& S,
   else atomicAdd(&A.R[j], w);
 }
 
+// Leaves a particle to the FP64 replay. The bound grows with the distance in cells: flights of some
+// 10^4 cells leave more particles undecided (5 % of a film of 10^5 cells at Kn 1) than the queue
+// holds (one in 32 and 65,536), and the plain FP64 kernel has no such limit; those beyond it are
+// marked in a bitmap that the replay goes through. (Following them on the spot takes 120 registers
+// in place of 64.)
+__device__ __forceinline__ void land_defer(const StagedArgs& S, unsigned pid) {
+  const unsigned i = atomicAdd(S.defer_n, 1u);
+  if (i < S.defer_cap) S.defer[i] = make_uint2(pid, 0u);
+  else atomicOr(&S.over[pid >> 5], 1u << (pid & 31u));
+}
+
 // Bands whose every candidate is real: one candidate per particle, no chain. A lane keeps its
 // emitter for qch particles in a row (over its bands in turn: with tens of bands an emitter has
 // only a few particles in each), so the cell coordinates, the weight, the first Philox rounds (the
@@ -82,7 +93,7 @@ __global__ void __launch_bounds__(LAND_NT) land_kernel(SweepArgs A, StagedArgs S
         }
         if (out) continue;
         if (near) {
-          defer_particle(S, first + (unsigned)q * (unsigned)L.groups[gi].ne + (unsigned)em.rank, 0u);
+          land_defer(S, first + (unsigned)q * (unsigned)L.groups[gi].ne + (unsigned)em.rank);
           continue;
         }
         const int cell = em.cell0 + o[0] + (DIM >= 2 ? n0 * o[1] : 0) + (DIM == 3 ? n0 * n1 * o[2] : 0);
@@ -252,7 +263,7 @@ __global__ void __launch_bounds__(LAND_NT) land_chain_kernel(SweepArgs A, Staged
           }
         }
         if (defer) {
-          defer_particle(S, pid, 0u);
+          land_defer(S, pid);
           alive = false;
           break;
         }
@@ -311,6 +322,8 @@ cudaError_t launch_land(const Ctx* c, const SweepArgs& a, bool adj, cudaStream_t
   S.defer = c->d_defer;
   S.defer_n = c->d_defer_n;
   S.defer_cap = c->defer_cap;
+  S.over = c->d_over;
+  S.over_words = (unsigned)((a.total_particles + 31) / 32);
   S.err = c->d_err;
   const bool k32 = !adj && c->opt.tally == IUGKP_TALLY_STAGED_K32;
   S.R32 = k32 ? c->d_R32 : nullptr;
@@ -350,7 +363,7 @@ cudaError_t launch_land(const Ctx* c, const SweepArgs& a, bool adj, cudaStream_t
       default: e = launch_dim<3, true, false>(c, a, S, L, s); break;
     }
     if (e != cudaSuccess) return e;
-    return launch_adjoint_replay(c, a, s);
+    return launch_adjoint_replay(c, a, S, s);
   }
   if (k32) {
     switch (c->dim) {

@@ -8,6 +8,7 @@
 
 #include "device.cuh"
 #include "internal.h"
+#include "staged.h"
 
 namespace iugkp {
 
@@ -86,6 +87,18 @@ __device__ __forceinline__ int replay_candidates(const SweepArgs& A, const InstD
     }
     st.next_pair(ua, ub);
     D += path64(ua, vb, tm);
+  }
+}
+
+// Calls f(particle) for the particles of a landing sweep that its queue could not hold, and clears
+// them; one word of the bitmap per thread. The whole grid calls it.
+template <class F>
+__device__ __forceinline__ void for_overflow(const StagedArgs& S, F f) {
+  if (!S.over || *S.defer_n <= S.defer_cap) return;
+  for (unsigned w = blockIdx.x * blockDim.x + threadIdx.x; w < S.over_words; w += gridDim.x * blockDim.x) {
+    unsigned bits = S.over[w];
+    if (bits) S.over[w] = 0u;
+    for (; bits; bits &= bits - 1u) f(32u * w + (unsigned)__ffs(bits) - 1u);
   }
 }
 

@@ -64,6 +64,10 @@ struct StagedArgs {
   unsigned* defer_n;              // entries pushed by this sweep (beyond defer_cap: overflow)
   unsigned defer_cap;
   int* err;                       // device error word (ERR_DEFER on overflow)
+  // Landing sweeps only (else null): bitmap of the particles beyond the queue, zero between launches
+  // (the replay clears what it takes).
+  unsigned* over;                 // [over_words]
+  unsigned over_words;
 #ifdef __CUDACC__
   // this block's copy of GX
   __device__ __forceinline__ double* gx() const {

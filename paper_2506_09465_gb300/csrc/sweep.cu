@@ -82,6 +82,27 @@ __device__ __forceinline__ double shfl_d(double x, int src) {
                           __shfl_sync(0xffffffffu, __double2loint(x), src));
 }
 
+// The real collision of a landing sweep's particle (forward index pid, nothing tallied yet) in FP64.
+template <int DIM>
+__device__ __noinline__ void replay_real(const SweepArgs& A, const StagedArgs& S, unsigned pid) {
+  Counts cnt;  // a landing sweep's event counts are not read
+  const Group G = A.groups[find_group(A.groups, A.n_groups, (long long)pid)];
+  const InstDesc& in = A.inst[G.inst];
+  const unsigned local = pid - (unsigned)G.first_particle;
+  const int q = (int)(local / (unsigned)G.n_emitters);
+  int e = (int)(local - (unsigned)q * (unsigned)G.n_emitters);
+  if (G.perm_off >= 0) e = A.perm[G.perm_off + e];  // the staged visiting order
+  int gj, fb[DIM];
+  double w;
+  Walk<double, DIM> wk;
+  Stream st;
+  if (!emit_particle<double, DIM, false>(A, G.first_particle + (long long)e * G.per_emitter + q, gj, w, wk, st)) return;
+  Seg64<DIM> sg;
+  sg.init(wk, in);
+  ReplayDeposits pol{A, S, in, w, 0, false, false, cnt};
+  if (replay_candidates<DIM>(A, in, G.inst, G.band, wk, sg, st, fb, pol) < 0) atomicOr(A.err, ERR_BUDGET);
+}
+
 // One thread per queue entry follows the particle's candidates in FP64 and makes its deposit
 // tallies; then the warp tallies the face items of its particles together, one particle at a
 // time (its segment broadcast from its lane), the lanes taking successive items. Faces
@@ -91,7 +112,8 @@ __device__ __forceinline__ double shfl_d(double x, int src) {
 // instances) or to the group's exit tally GX (two-group). Emission needs nothing: the staged
 // sweep and its post-passes account for it.
 template <int DIM>
-__global__ void __launch_bounds__(256) replay_kernel(SweepArgs A, StagedArgs S) {
+__global__ void __launch_bounds__(256)
+    replay_kernel(const __grid_constant__ SweepArgs A, const __grid_constant__ StagedArgs S) {
   Counts cnt;
 #pragma unroll
   for (int k = 0; k < CNT_N; ++k) cnt.v[k] = 0;
@@ -222,6 +244,7 @@ __global__ void __launch_bounds__(256) replay_kernel(SweepArgs A, StagedArgs S) 
     }
     (void)ex;
   }
+  for_overflow(S, [&](unsigned pid) { replay_real<DIM>(A, S, pid); });
   flush_counts(cnt, A.counters);
 }
 
