@@ -227,6 +227,10 @@ __global__ void __launch_bounds__(LAND_NT) land_chain_kernel(SweepArgs A, Staged
       if (exhausted) break;
       continue;
     }
+    if (alive && st.j >= L.max_j) {  // FP64 tracking: the replay keeps the step budget
+      land_defer(S, pid);
+      alive = false;
+    }
     if (alive) {
 #pragma unroll 1
       for (int it = 0; it < S.walk_k; ++it) {
@@ -334,6 +338,8 @@ cudaError_t launch_land(const Ctx* c, const SweepArgs& a, bool adj, cudaStream_t
   L.qch = adj ? c->land_all_qch : c->land_fwd_qch;
   L.next = reinterpret_cast<unsigned long long*>(c->d_defer_n + 2);
   L.lamVm = c->d_work;
+  // two uniforms per candidate; FP32 tracking follows a chain to its end, as its full sweep does
+  L.max_j = c->opt.precision == IUGKP_TRACK_FP64 ? 2u * EXACT_MAX_CANDIDATES : 0xffffffffu;
   const size_t bc = (size_t)c->nb * c->total_cells;
   PrologueArgs P = {};
   auto clear = [&](void* p, size_t n) {

@@ -115,7 +115,8 @@ constexpr int LAND_WARPS_PER_SM = 40; // resident warps the task size is chosen 
 constexpr int LAND_REFILL = 8;        // idle lanes that trigger a refill (null-candidate chains)
 
 // Filtered FP64 sweep (exact.cu): copies of the 1D face differences (by block), and the
-// candidates after which a particle goes to the replay, which counts its steps against the budget.
+// candidates after which a particle (there and in a landing sweep with FP64 tracking) goes to the
+// replay, which keeps the step budget.
 constexpr int EXACT_DIFF_COPIES = 16;
 constexpr int EXACT_MAX_CANDIDATES = 1 << 20;
 constexpr long long EXACT_MIN_BUDGET = 1ll << 24;  // smaller step budgets take the plain kernel
@@ -138,6 +139,7 @@ struct LandArgs {
   int qch;
   unsigned long long* next;       // next unclaimed task (or particle, where chains are followed)
   const double* lamVm;            // adjoint: [cells] lambda / (V m)
+  unsigned max_j;                 // chains: uniforms after which a particle goes to the replay
 };
 
 // Tasks of the pass-synchronous 2D sweep: those of an instance are contiguous.

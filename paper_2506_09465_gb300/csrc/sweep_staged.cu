@@ -916,6 +916,7 @@ void launch_sync(const Ctx* c, const SweepArgs& a, const StagedArgs& S, int bloc
   Y.L.qch = c->sync_qch;
   Y.L.next = nullptr;
   Y.L.lamVm = nullptr;
+  Y.L.max_j = 0;
   Y.task_end = c->d_sync_end;
   if (c->all_real_all) {
     if (c->sync_partial) sweep_sync_kernel<K32, true, true><<<blocks, STAGED_NT, smem, s>>>(a, S, Y);
