@@ -137,7 +137,7 @@ void free_all(Ctx* c) {
                   c->d_all_group_mag, c->d_R32, c->d_W32, c->d_F32, c->d_m2, c->d_wallTf,
                   c->d_pslot_off, c->d_phome_off, c->d_pnband, c->d_pnwall, c->d_px, c->d_pband, c->d_phome,
                   c->d_pcount, c->d_pfcount, c->d_phome_w, c->d_wemit, c->d_DY, c->d_EY, c->d_GX, c->d_Fx, c->d_Fi, c->d_ticket, c->d_wpart,
-                  c->d_all_real, c->d_defer, c->d_defer_n, c->d_over, c->d_land_fwd, c->d_land_all, c->d_items, c->d_diff, c->d_sync_groups, c->d_sync_beg,
+                  c->d_all_real, c->d_defer, c->d_defer_n, c->d_over, c->d_land_fwd, c->d_land_all, c->d_items, c->d_nodes, c->d_sync_groups, c->d_sync_beg,
                   c->d_sync_end, c->team_plan[0].d_buf, c->team_plan[1].d_buf};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -839,7 +839,10 @@ iugkp_status iugkp_create_batch(int n, const iugkp_grid* g, const double* const*
     // in every eight particles (beyond that they are found on the spot)
     c->items_cap = (unsigned)std::min<long long>(c->total_particles / 8 + 65536, 1ll << 28);
     if ((s = dalloc(c, &c->d_items, (size_t)(c->dim > 1 ? c->items_cap : 1))) != IUGKP_OK) return bail(s);
-    if (c->dim == 1 && (s = dalloc(c, &c->d_diff, (size_t)EXACT_DIFF_COPIES * (face_off + n))) != IUGKP_OK) return bail(s);
+    if (c->dim == 1) {  // few faces: copies of their trees, by block, against atomics on the same address
+      c->node_copies = (int)std::max<long long>(1, std::min<long long>(EXACT_NODE_COPIES, EXACT_NODE_FACES / face_off));
+      if ((s = dalloc(c, &c->d_nodes, (size_t)c->node_copies * 2 * face_off)) != IUGKP_OK) return bail(s);
+    }
   }
   if (c->dim <= 2 && c->opt.precision == IUGKP_TRACK_FP32) {
     if ((s = dalloc(c, &c->d_Fx, face_off)) != IUGKP_OK) return bail(s);

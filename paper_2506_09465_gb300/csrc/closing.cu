@@ -184,8 +184,9 @@ __device__ __forceinline__ int wall_faces(const InstDesc& in, int a) {
 
 // One block: the power entering through the faces of wall wl of instance k (N_w particles of
 // weight C_b v_b A T_w / (4 N_w) per face and band) added to F when `emit`, and the wall's
-// absorbed power, its emission plus the outward net flux through its faces (fixed-order
-// reduction), when wall is given.
+// absorbed power (fixed-order reduction) when `absorbed`: the sum of its faces as tallied, before
+// the emission enters them; or, where the emission is in them already, that emission plus the
+// outward net flux (a difference, to the rounding of the emission).
 __device__ void wall_block(const SweepArgs& A, const double* wall_unit, int k, int wl, bool emit, bool absorbed) {
   __shared__ double sh[8], shT[8];
   const int a = wl >> 1, side = wl & 1;
@@ -196,12 +197,12 @@ __device__ void wall_block(const SweepArgs& A, const double* wall_unit, int k, i
   double sum = 0.0, tsum = 0.0;
   for (int j = threadIdx.x; j < nf; j += blockDim.x) {
     const long long f = in.face_off + wall_face(in, a, side, j);
-    double v = __ldcg(&A.F[f]);
+    const double v = __ldcg(&A.F[f]);
+    sum += v;
     if (emit) {
       const double e = u * tf[j];
-      if (e != 0.0) A.F[f] = v = v + (side ? -e : e);
+      if (e != 0.0) A.F[f] = v + (side ? -e : e);
     }
-    sum += v;
     tsum += tf[j];
   }
   if (!absorbed) return;
@@ -222,69 +223,80 @@ __device__ void wall_block(const SweepArgs& A, const double* wall_unit, int k, i
       t += sh[w];
       ts += shT[w];
     }
-    A.wall[in.wall_off + wl] = u * ts + (side ? t : -t);
+    A.wall[in.wall_off + wl] = (emit ? 0.0 : u * ts) + (side ? t : -t);
   }
 }
 
-// 1D faces from the differences of runs (exact.cu): F[f] += the sum of the differences up to f, over
-// the copies; chunks of 256 faces, prefix sums in a fixed order.
-__device__ void face_runs(const InstDesc& in, int k, const double* diff, long long stride, double* F) {
-  __shared__ double wsum[8];
-  const double* d = diff + in.face_off + k;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double carry = 0.0;
-  for (int f0 = 0; f0 < (int)in.nfaces; f0 += 256) {
-    const int f = f0 + threadIdx.x;
-    double v = 0.0;
-    if (f < (int)in.nfaces)
-#pragma unroll
-      for (int c = 0; c < EXACT_DIFF_COPIES; ++c) v += d[c * stride + f];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const double t = __shfl_up_sync(0xffffffffu, v, o);
-      if (lane >= o) v += t;
-    }
-    if (lane == 31) wsum[warp] = v;
-    __syncthreads();
-    double before = carry, all = carry;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) {
-      if (w == warp) before = all;
-      all += wsum[w];
-    }
-    if (f < (int)in.nfaces) F[in.face_off + f] += before + v;
-    carry = all;
-    __syncthreads();
-  }
-}
-
-// After a trace that tallied every face (1D, and the filtered FP64 sweep): blocks [0, roles) take
-// the walls (one wall each; in 1D one instance each, after its faces: the runs of the FP64 sweep,
-// or the fixed-point sums Fi and FP64 sums Fx of the staged one), the others scale W.
+// After a trace that tallied every face (the staged sweep in 1D, the filtered FP64 sweep in 2D and 3D):
+// blocks [0, roles) take the walls (one wall each; in 1D one instance each, after its faces are formed
+// from the fixed-point sums Fi and the FP64 sums Fx), the others scale W.
 __global__ void __launch_bounds__(256) close_tallied_kernel(SweepArgs A, int n_inst, const double* wall_unit,
-                                                            const double* diff, long long diff_stride, const long long* Fi,
-                                                            const double* Fx, const double* wmax, long long total_bc,
-                                                            int roles) {
+                                                            const long long* Fi, const double* Fx, const double* wmax,
+                                                            long long total_bc, int roles) {
   if ((int)blockIdx.x < roles) {
     if (A.dim == 1) {
       const int k = blockIdx.x;
-      if (Fi) {
-        const InstDesc& in = A.inst[k];
-        const double qs = wmax[k] / WIN_SCALE;
-        for (long long f = in.face_off + threadIdx.x; f < in.face_off + in.nfaces; f += 256)
-          A.F[f] = Fi[f] ? fma((double)Fi[f], qs, Fx[f]) : Fx[f];
-        __threadfence_block();
-        __syncthreads();
-      }
-      if (diff) {
-        face_runs(A.inst[k], k, diff, diff_stride, A.F);
-        __threadfence_block();
-        __syncthreads();
-      }
+      const InstDesc& in = A.inst[k];
+      const double qs = wmax[k] / WIN_SCALE;
+      for (long long f = in.face_off + threadIdx.x; f < in.face_off + in.nfaces; f += 256)
+        A.F[f] = Fi[f] ? fma((double)Fi[f], qs, Fx[f]) : Fx[f];
+      __threadfence_block();
+      __syncthreads();
       for (int wl = 0; wl < 2; ++wl) wall_block(A, wall_unit, k, wl, true, A.wall != nullptr);
     } else {
       const int k = blockIdx.x / (2 * A.dim);
       wall_block(A, wall_unit, k, blockIdx.x - k * 2 * A.dim, true, A.wall != nullptr);
+    }
+    return;
+  }
+  if (!A.W) return;
+  const long long step = (long long)(gridDim.x - roles) * blockDim.x;
+  for (long long j = ((long long)blockIdx.x - roles) * blockDim.x + threadIdx.x; j < total_bc; j += step)
+    scale_entry(A, bc_instance(A.inst, n_inst, j), j);
+}
+
+// After the filtered FP64 sweep in 1D: blocks [0, roles) add to every face (which holds the replayed
+// particles' crossings) the nodes above its leaf, over the copies; a boundary face is its wall's
+// absorbed power then, and the wall's emission enters it. The others scale W.
+__global__ void __launch_bounds__(256) close_runs_kernel(SweepArgs A, int n_inst, const double* wall_unit, const double* node,
+                                                         long long stride, int copies, long long total_faces,
+                                                         long long total_bc, int roles) {
+  if ((int)blockIdx.x < roles) {
+    // eight lanes per face, lane q on the tree's levels q, q + 8, .. above the leaf: one or two L2
+    // round trips in a row, not one per level (51 faces: 6 us less)
+    const int q = threadIdx.x & 7;
+    for (long long g0 = blockIdx.x * 32ll; g0 < total_faces; g0 += roles * 32ll) {
+      const long long g = g0 + (threadIdx.x >> 3);
+      const bool ok = g < total_faces;
+      int k = 0;
+      for (int hi = n_inst - 1; k < hi;) {  // the last instance whose faces start at or before g
+        const int mid = (k + hi + 1) >> 1;
+        if (A.inst[mid].face_off <= g) k = mid;
+        else hi = mid - 1;
+      }
+      const InstDesc& in = A.inst[k];
+      const int n = (int)in.nfaces, f = (int)(g - in.face_off);
+      const double* t = node + 2 * in.face_off;
+      double v = 0.0;
+      for (unsigned i = ok ? (unsigned)(f + n) >> q : 0u; i; i >>= 8) {
+        double x[EXACT_NODE_COPIES];
+#pragma unroll
+        for (int c = 0; c < EXACT_NODE_COPIES; ++c)  // the loads of all copies in flight
+          x[c] = c < copies ? __ldcg(&t[c * stride + i]) : 0.0;
+#pragma unroll
+        for (int c = 0; c < EXACT_NODE_COPIES; ++c) v += x[c];
+      }
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (!ok || q != 0) continue;
+      v += A.F[g];
+      const int wl = f == 0 ? 0 : (f == n - 1 ? 1 : -1);
+      if (wl >= 0) {
+        if (A.wall) A.wall[in.wall_off + wl] = wl ? v : 0.0 - v;
+        const double e = wall_unit[k * 6 + wl] * A.wallTf[in.bface_off + in.wface_off[wl]];
+        if (e != 0.0) v += wl ? -e : e;
+      }
+      A.F[g] = v;
     }
     return;
   }
@@ -549,14 +561,18 @@ static unsigned cell_blocks(const Ctx* c, long long n) {
   return (unsigned)std::max<long long>(1, std::min<long long>((n + 255) / 256, 8ll * c->sm_count));
 }
 
-cudaError_t launch_close_tallied(const Ctx* c, const SweepArgs& a, const double* diff, long long diff_stride,
-                                 cudaStream_t s) {
+cudaError_t launch_close_tallied(const Ctx* c, const SweepArgs& a, cudaStream_t s) {
   const long long bc = (long long)c->nb * c->total_cells;
-  const int roles = a.F ? (c->dim == 1 ? c->n_inst : 2 * c->dim * c->n_inst) : 0;
   const unsigned extra = a.W ? cell_blocks(c, bc) : 0;
+  if (c->dim == 1 && a.F) {
+    const int roles = (int)cell_blocks(c, 8 * c->total_faces);
+    close_runs_kernel<<<roles + extra, 256, 0, s>>>(a, c->n_inst, c->d_wall_unit, c->d_nodes, 2 * c->total_faces,
+                                                    c->node_copies, c->total_faces, bc, roles);
+    return cudaGetLastError();
+  }
+  const int roles = a.F ? 2 * c->dim * c->n_inst : 0;
   if (roles + extra == 0) return cudaSuccess;
-  close_tallied_kernel<<<roles + extra, 256, 0, s>>>(a, c->n_inst, c->d_wall_unit, diff, diff_stride, nullptr, nullptr,
-                                                       nullptr, bc, roles);
+  close_tallied_kernel<<<roles + extra, 256, 0, s>>>(a, c->n_inst, c->d_wall_unit, nullptr, nullptr, nullptr, bc, roles);
   return cudaGetLastError();
 }
 
@@ -565,8 +581,8 @@ cudaError_t launch_close_1d(const Ctx* c, const SweepArgs& a, cudaStream_t s) {
   const int roles = a.F ? c->n_inst : 0;
   const unsigned extra = a.W ? cell_blocks(c, bc) : 0;
   if (roles + extra == 0) return cudaSuccess;
-  close_tallied_kernel<<<roles + extra, 256, 0, s>>>(a, c->n_inst, c->d_wall_unit, nullptr, 0, a.F ? c->d_Fi : nullptr,
-                                                     c->d_Fx, reinterpret_cast<const double*>(c->d_wmax), bc, roles);
+  close_tallied_kernel<<<roles + extra, 256, 0, s>>>(a, c->n_inst, c->d_wall_unit, c->d_Fi, c->d_Fx,
+                                                     reinterpret_cast<const double*>(c->d_wmax), bc, roles);
   return cudaGetLastError();
 }
 

@@ -15,13 +15,16 @@
 //    other axis q (rho_q = g_q / |g_a|, delta_a the distance to the first face in cells); the
 //    floor of that is the face's row. A warp deals its particles' faces to its lanes in segments.
 //    A row within the bound of a cell edge is queued and found in FP64.
-//  * In 1D the faces a particle crosses are one run: its weight is added where the run begins and
-//    subtracted after its end, and the faces are the prefix sums (a slab of 50 cells has all of
-//    its crossings on 51 addresses, whose FP64 atomics serialise at the L2).
+//  * In 1D the faces a particle crosses are one run (a slab of 50 cells has all of its crossings on
+//    51 addresses, whose FP64 atomics serialise at the L2): its weight is added to the O(log faces)
+//    nodes of a binary tree over the faces whose leaves make up the run, and a face is the sum over
+//    its leaf and the nodes above it. Nothing is subtracted, so a face keeps the digits that its own
+//    crossings have, deep in a thick film too, and an infinite or NaN weight stays with the faces it
+//    crosses (differences at the ends of the runs and prefix sums kept neither).
 //  * Candidates and exits within the bound of a face, a wall, a corner or the acceptance ratio
 //    leave the particle to the FP64 replay.
-//  * Power entering through the walls and absorbed by them follows from the faces
-//    (boundary_emission_kernel, wall_absorbed_kernel).
+//  * What a wall absorbs is the sum of its faces as tallied; the power it emits is added to them
+//    afterwards (closing.cu).
 //
 // Bounds, in units of 2^-23 relative: g 3.5 (landing.cuh); the wall distance W_a / |g_a|: g, one
 // rounding of W and the quotient's 2 ulp, 6 in all; rho 9 and rho (k + delta) 10.5. EXIT_REL and
@@ -51,9 +54,19 @@ struct ExactArgs {
   uint2* items;          // queued faces: {forward index, axis << 30 | k}
   unsigned* n_items;
   unsigned cap;
-  double* diff;          // 1D: [DIFF_COPIES][faces + 1 per instance] differences of the face tallies
-  long long diff_stride;
+  double* node;          // 1D: [copies][2 faces per instance] nodes of the trees over the faces
+  long long node_stride;
+  int copies;
 };
+
+// Adds w to the run of faces [a, b) of a tree over n faces (leaves at n .. 2 n - 1, the node above i
+// at i / 2: the bottom-up tree, which needs no power of two).
+__device__ __forceinline__ void add_run(double* node, int n, int a, int b, double w) {
+  for (unsigned l = (unsigned)(a + n), r = (unsigned)(b + n); l < r; l >>= 1, r >>= 1) {
+    if (l & 1u) atomicAdd(&node[l++], w);
+    if (r & 1u) atomicAdd(&node[--r], w);
+  }
+}
 
 // Emitter-major index of the particle with forward index pid (q-major in its group's visiting order).
 __device__ __forceinline__ long long emitter_major(const SweepArgs& A, unsigned pid) {
@@ -232,8 +245,7 @@ __global__ void __launch_bounds__(EXACT_NT) exact_kernel(SweepArgs A, StagedArgs
     const long long bcbase = in.bc_off + (long long)G.band * in.ncells;
     const uint32_t inst_id = in.inst_id;
     double* F = A.F ? A.F + in.face_off : nullptr;
-    double* diff = DIM == 1 && A.F ? X.diff + (blockIdx.x % EXACT_DIFF_COPIES) * X.diff_stride + in.face_off + G.inst : nullptr;
-    double run_start = 0.0;  // 1D: weight added where the runs of the lane's particles begin
+    double* node = DIM == 1 && A.F ? X.node + (blockIdx.x % (unsigned)X.copies) * X.node_stride + 2 * in.face_off : nullptr;
     const int qbeg = qc * (L.qch * G.reps) + em.sub, qend = min(G.per, (qc + 1) * (L.qch * G.reps));
     for (int j = 0; j < L.qch; ++j) {
       const int q = qbeg + j * G.reps;
@@ -335,9 +347,9 @@ __global__ void __launch_bounds__(EXACT_NT) exact_kernel(SweepArgs A, StagedArgs
             n_cross += c;
             items[a] = c + (a == p ? 1 : 0);
           }
-          if (DIM == 1 && diff && items[0] > 0) {
-            run_start += em.w;
-            atomicAdd(&diff[em.c[0] + 1 + (g[0] > 0.f ? items[0] : -items[0])], -em.w);
+          if (DIM == 1 && node && items[0] > 0) {
+            if (g[0] > 0.f) add_run(node, n0 + 1, em.c[0] + 1, em.c[0] + 1 + items[0], em.w);
+            else add_run(node, n0 + 1, em.c[0] + 1 - items[0], em.c[0] + 1, -em.w);
           }
         }
       }
@@ -366,7 +378,6 @@ __global__ void __launch_bounds__(EXACT_NT) exact_kernel(SweepArgs A, StagedArgs
         }
       }
     }
-    if (DIM == 1 && run_start != 0.0) atomicAdd(&diff[em.c[0] + 1], run_start);
   }
   unsigned long long v[5] = {n_fl, n_cand, n_real, n_cross, n_exit};
   const int slot[5] = {CNT_FLIGHTS, CNT_CANDIDATES, CNT_REAL, CNT_CROSSINGS, CNT_WALL_EXITS};
@@ -440,8 +451,9 @@ cudaError_t launch_exact(const Ctx* c, const SweepArgs& a, cudaStream_t s) {
   X.items = c->d_items;
   X.n_items = c->d_defer_n + 1;
   X.cap = c->items_cap;
-  X.diff = c->d_diff;
-  X.diff_stride = c->total_faces + c->n_inst;
+  X.node = c->d_nodes;
+  X.node_stride = 2 * c->total_faces;
+  X.copies = c->node_copies;
   PrologueArgs P = {};
   auto clear = [&](void* p, size_t n) {
     if (!p || !n) return;
@@ -453,7 +465,7 @@ cudaError_t launch_exact(const Ctx* c, const SweepArgs& a, cudaStream_t s) {
   clear(a.F, (size_t)c->total_faces);
   clear(a.counters, CNT_N);
   clear(c->d_defer_n, 2);
-  if (c->dim == 1 && a.F) clear(c->d_diff, (size_t)EXACT_DIFF_COPIES * X.diff_stride);
+  if (c->dim == 1 && a.F) clear(c->d_nodes, (size_t)X.copies * X.node_stride);
   cudaError_t e = launch_prologue(c, a, P, s);
   if (e != cudaSuccess) return e;
   switch (c->dim) {
@@ -462,8 +474,8 @@ cudaError_t launch_exact(const Ctx* c, const SweepArgs& a, cudaStream_t s) {
     default: e = launch_dim<3>(c, a, S, L, X, s); break;
   }
   if (e != cudaSuccess) return e;
-  // W scaled, the walls' emission added to their faces, the walls' absorbed power
-  return launch_close_tallied(c, a, c->dim == 1 && a.F ? c->d_diff : nullptr, X.diff_stride, s);
+  // W scaled, the walls' absorbed power, the walls' emission added to their faces
+  return launch_close_tallied(c, a, s);
 }
 
 }  // namespace iugkp

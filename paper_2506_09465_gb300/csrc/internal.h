@@ -215,10 +215,11 @@ struct Ctx {
   unsigned* d_sync_end = nullptr;
   unsigned sync_tasks = 0;
   int sync_qch = 1;
-  // filtered FP64 sweep (exact.cu; contexts with FP64 tracking): queued faces, 1D face differences
+  // filtered FP64 sweep (exact.cu; contexts with FP64 tracking): queued faces, 1D trees over the faces
   uint2* d_items = nullptr;
   unsigned items_cap = 0;
-  double* d_diff = nullptr;
+  double* d_nodes = nullptr;     // [node_copies][2 faces per instance]
+  int node_copies = 1;
   // landing sweeps (land.cu): tasks of the forward groups and of every group (adjoint)
   LandGroup* d_land_fwd = nullptr;
   LandGroup* d_land_all = nullptr;
@@ -259,8 +260,7 @@ cudaError_t launch_chain(const Ctx* c, const SweepArgs& a, const StagedArgs& S, 
 cudaError_t launch_k32_finalize(const Ctx* c, const float2* src, double* dst, long long n, cudaStream_t s);
 cudaError_t launch_exact(const Ctx* c, const SweepArgs& a, cudaStream_t s);
 cudaError_t launch_prologue(const Ctx* c, const SweepArgs& a, const PrologueArgs& P, cudaStream_t s);
-cudaError_t launch_close_tallied(const Ctx* c, const SweepArgs& a, const double* diff, long long diff_stride,
-                                 cudaStream_t s);
+cudaError_t launch_close_tallied(const Ctx* c, const SweepArgs& a, cudaStream_t s);
 cudaError_t launch_close_1d(const Ctx* c, const SweepArgs& a, cudaStream_t s);
 cudaError_t launch_close_2d(const Ctx* c, const SweepArgs& a, cudaStream_t s);
 cudaError_t launch_close_3d(const Ctx* c, const SweepArgs& a, cudaStream_t s);

@@ -114,10 +114,12 @@ constexpr int LAND_QCH = 16;          // particles per emitter and task at most
 constexpr int LAND_WARPS_PER_SM = 40; // resident warps the task size is chosen for
 constexpr int LAND_REFILL = 8;        // idle lanes that trigger a refill (null-candidate chains)
 
-// Filtered FP64 sweep (exact.cu): copies of the 1D face differences (by block), and the
+// Filtered FP64 sweep (exact.cu): copies of the 1D trees over the faces at most, and the faces of all of
+// them together (beyond, addresses are seldom the same); the
 // candidates after which a particle (there and in a landing sweep with FP64 tracking) goes to the
 // replay, which keeps the step budget.
-constexpr int EXACT_DIFF_COPIES = 16;
+constexpr int EXACT_NODE_COPIES = 16;
+constexpr long long EXACT_NODE_FACES = 1 << 15;
 constexpr int EXACT_MAX_CANDIDATES = 1 << 20;
 constexpr long long EXACT_MIN_BUDGET = 1ll << 24;  // smaller step budgets take the plain kernel
 
