@@ -254,8 +254,11 @@ cudaError_t launch_pcg_check(const Ctx* c, cudaStream_t s);
 cudaError_t launch_absmax(const Ctx* c, const double* x, long long n, double* out, cudaStream_t s);
 cudaError_t launch_axpy_grad(const Ctx* c, const double* at, const double* g, double* lam_half, cudaStream_t s);
 cudaError_t launch_sweep_staged(const Ctx* c, const SweepArgs& a, cudaStream_t s);
+// Allows a kernel all the dynamic shared memory a block may have. The limit belongs to the kernel, not
+// to a context: every context sets the same value, so that none lowers it for another that is alive.
+cudaError_t allow_shared(const void* kernel, size_t optin);
 cudaError_t configure_staged(Ctx* c);
-cudaError_t configure_chain();
+cudaError_t configure_chain(const Ctx* c);
 cudaError_t launch_chain(const Ctx* c, const SweepArgs& a, const StagedArgs& S, bool k32, cudaStream_t s);
 cudaError_t launch_k32_finalize(const Ctx* c, const float2* src, double* dst, long long n, cudaStream_t s);
 cudaError_t launch_exact(const Ctx* c, const SweepArgs& a, cudaStream_t s);

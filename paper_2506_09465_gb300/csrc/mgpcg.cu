@@ -1059,7 +1059,7 @@ cudaError_t configure_mgpcg(Ctx* c, const std::vector<InstMG>& h_mg) {
                         kind ? (const void*)fd_kernel : (const void*)mgpcg32_kernel};
     cudaError_t e;
     for (const void* q : f) {
-      if ((e = cudaFuncSetAttribute(q, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+      if ((e = allow_shared(q, c->smem_optin)) != cudaSuccess) return e;
       int nb = 0;
       if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, q, kind ? FD_NT : MG_NT, smem)) != cudaSuccess) return e;
       if (nb < 1) return cudaErrorLaunchOutOfResources;

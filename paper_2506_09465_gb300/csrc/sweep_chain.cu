@@ -518,11 +518,9 @@ __global__ void __launch_bounds__(CHAIN_NT, 1) sweep_chain_kernel(SweepArgs A, S
 
 constexpr size_t CHAIN_SMEM = sizeof(ChainLists) * (CHAIN_NT / 32);
 
-cudaError_t configure_chain() {
-  const cudaError_t e =
-      cudaFuncSetAttribute(sweep_chain_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CHAIN_SMEM);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(sweep_chain_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CHAIN_SMEM);
+cudaError_t configure_chain(const Ctx* c) {
+  const cudaError_t e = allow_shared((const void*)sweep_chain_kernel<false>, c->smem_optin);
+  return e != cudaSuccess ? e : allow_shared((const void*)sweep_chain_kernel<true>, c->smem_optin);
 }
 
 cudaError_t launch_chain(const Ctx* c, const SweepArgs& a, const StagedArgs& S, bool k32, cudaStream_t s) {

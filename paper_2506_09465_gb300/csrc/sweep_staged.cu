@@ -1133,20 +1133,27 @@ double walk_bound_fraction(const double* m) {
   return (Et + Ed + m[4] * ulp + ulp) / (double)TIE_REL;
 }
 
+cudaError_t allow_shared(const void* kernel, size_t optin) {
+  cudaFuncAttributes at;
+  const cudaError_t e = cudaFuncGetAttributes(&at, kernel);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(optin - at.sharedSizeBytes));
+}
+
 cudaError_t configure_staged(Ctx* c) {
   cudaError_t e = cudaSuccess;
-  if (c->dim == 3) return configure_chain();
+  if (c->dim == 3) return configure_chain(c);
   const size_t smem = (size_t)c->staged_cap * sizeof(unsigned);
   const void* fwd[4] = {(const void*)sweep_staged_kernel<1, false>, (const void*)sweep_staged_kernel<2, false>,
                         (const void*)sweep_staged_kernel<1, true>, (const void*)sweep_staged_kernel<2, true>};
   for (const void* f : fwd)
-    if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+    if ((e = allow_shared(f, c->smem_optin)) != cudaSuccess) return e;
   const void* syn[8] = {(const void*)sweep_sync_kernel<false, false, false>, (const void*)sweep_sync_kernel<true, false, false>,
                         (const void*)sweep_sync_kernel<false, true, false>, (const void*)sweep_sync_kernel<true, true, false>,
                         (const void*)sweep_sync_kernel<false, false, true>, (const void*)sweep_sync_kernel<true, false, true>,
                         (const void*)sweep_sync_kernel<false, true, true>, (const void*)sweep_sync_kernel<true, true, true>};
   for (const void* f : syn)
-    if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+    if ((e = allow_shared(f, c->smem_optin)) != cudaSuccess) return e;
   int nb = 0, nk = 0;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fwd[c->dim - 1], STAGED_NT, smem)) != cudaSuccess) return e;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nk, fwd[c->dim + 1], STAGED_NT, smem)) != cudaSuccess) return e;
