@@ -29,6 +29,7 @@ struct InstMG;
 struct TeamPlan {
   int blocks = 0;                // 0: no instance of this kind
   int threads = 0;               // per block
+  bool cluster = false;          // every team is one thread-block cluster
   size_t smem = 0;               // dynamic shared memory per block
   char* d_buf = nullptr;         // the arrays below
   void* d_teams = nullptr;

@@ -2,9 +2,10 @@
 // finite-volume diffusion operator, FP64 iterates and residual, preconditioned by one
 // aggregation-multigrid V-cycle in FP32; separable operators by fast diagonalization.
 //
-// One team of thread blocks per instance, one block per SM, all of them resident together (a
-// cooperative launch): the SMs are dealt to the instances by their cost (plan_teams). A team's
-// blocks split each level's cells in contiguous ranges, exchange neighbour values through global
+// One team of thread blocks per instance, one block per SM. Small instances: a team is one thread-block
+// cluster (ClusterTeam). Larger or many ones: all blocks resident together (a cooperative launch: it
+// starts once a block fits on each SM it needs), the SMs dealt to the instances by their cost
+// (plan_teams). A team's blocks split each level's cells in contiguous ranges, exchange neighbour values through global
 // memory (L2) between team barriers, and reduce dot products in a fixed rank order (every block
 // gets the same value, so all take the same branch). With one 8-block cluster per instance
 // the largest of four boxes (64^3, 64 cells per thread and phase) set the time on 8 of 152 SMs:
@@ -15,6 +16,7 @@
 // the children (P^T), Galerkin coarse operators P^T A P built on the host, prolongation by
 // injection scaled by alpha (the usual over-correction of piecewise-constant
 // aggregation), dense inverse on the coarsest level. It is symmetric, so CG stays CG.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -28,6 +30,7 @@ namespace iugkp {
 constexpr int MG32_PASSES_FD = 6;  // refinement passes of the fast diagonalization solve at most
 constexpr int MG_NT = 1024;        // threads per block, multigrid CG
 constexpr int MG_SMALL_NT = 512;   // ... where every instance is small: fewer warps per barrier
+constexpr int MG_CLUSTER = 8;      // blocks of a cluster team
 constexpr int FD_NT = 512;         // ... fast diagonalization
 // Polls of a team barrier (an L2 round trip each) before a block gives up: a second or so.
 constexpr unsigned TEAM_SPIN_LIMIT = 1u << 21;
@@ -103,6 +106,7 @@ struct Team {
   int buf;
   bool dead;         // a barrier was given up (the same for all threads of the block)
   static constexpr bool solo = false;
+  static constexpr long long solo_cells = 4096;  // levels up to here are the first block's alone
   __device__ static float ld(const float* p) { return __ldcg(p); }
   __device__ __forceinline__ int stride() const { return (int)blockDim.x; }
   // What the team's blocks wrote before it is visible to all of them after it.
@@ -168,6 +172,55 @@ struct Team {
   }
 };
 
+// The same for a team that is one thread-block cluster (MG_CLUSTER blocks, started together by the
+// hardware, so the launch needs nothing else of the device): the cluster's own barrier, which costs a
+// third of a round trip through L2, and partial sums read from the blocks' shared memory.
+struct ClusterTeam {
+  int rank, size;
+  double* slots;  // this block's shared memory: [2][2]
+  int buf;
+  static constexpr bool dead = false, solo = false;
+  static constexpr long long solo_cells = 1024;
+  __device__ static float ld(const float* p) { return __ldcg(p); }
+  __device__ __forceinline__ int stride() const { return (int)blockDim.x; }
+  __device__ __forceinline__ void sync() { cooperative_groups::this_cluster().sync(); }
+  __device__ __forceinline__ void range(int nc, int& lo, int& hi) const {
+    const int chunk = (nc + size - 1) / size;
+    lo = min(nc, rank * chunk);
+    hi = min(nc, lo + chunk);
+  }
+  template <int NV>
+  __device__ __forceinline__ void sum(double (&v)[NV], double* sh) {
+    static_assert(NV <= 2, "two values at most");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      double x = v[k];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+      if (lane == 0) sh[k * 32 + warp] = x;
+    }
+    __syncthreads();
+    if (warp < NV) {
+      double x = lane < (int)(blockDim.x >> 5) ? sh[warp * 32 + lane] : 0.0;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+      if (lane == 0) slots[buf * 2 + warp] = x;
+    }
+    sync();
+    if (warp < NV) {
+      double x = lane < size ? *cooperative_groups::this_cluster().map_shared_rank(slots + buf * 2 + warp, lane) : 0.0;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+      if (lane == 0) sh[64 + warp] = x;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < NV; ++k) v[k] = sh[64 + k];
+    buf ^= 1;  // a slot is written again only after the next sum's barrier
+  }
+};
+
 // The finest level's cells and the order of its FP32 sums. The cells are cut into MG_RANKS equal
 // ranges; unit (r, w) has the cells of range r whose offset modulo 32 MG_WARPS falls on 32 w .. 32 w
 // + 31, one per lane, in steps: a lane's products are added in FP32 over the steps, the lanes' sums
@@ -186,7 +239,8 @@ __host__ __device__ __forceinline__ int range_units_log(long long chunk) {
 struct Units {
   int n, chunk, steps, lw;  // cells, cells of a range, steps of a unit, 2^lw units of a range (all that have cells)
   int u0, u1;               // this block's units
-  __device__ __forceinline__ Units(int cells, const Team& tm) {
+  template <class TM>
+  __device__ __forceinline__ Units(int cells, const TM& tm) {
     n = cells;
     chunk = (cells + MG_RANKS - 1) / MG_RANKS;
     steps = (chunk + 32 * MG_WARPS - 1) / (32 * MG_WARPS);
@@ -255,7 +309,7 @@ struct Units {
   }
 };
 
-// Levels of at most MG_SOLO_CELLS cells go to the team's first block, their vectors in its shared
+// Levels of at most TM::solo_cells cells go to the team's first block, their vectors in its shared
 // memory: the work is small and every phase waits for the previous one, so the barriers and
 // L2 round trips are what they would cost on the team.
 struct SoloTeam {
@@ -270,8 +324,14 @@ struct SoloTeam {
   }
 };
 
-constexpr long long MG_SOLO_CELLS = 4096;
-constexpr long long MG_SMALL_CELLS = 1024;  // instances up to here take one block
+constexpr long long MG_SMALL_CELLS = 1024;  // instances up to here take one block of a team launch
+// Contexts whose largest instance lies in this range take one cluster per instance, as long as all
+// clusters run at once. Teams of four to eight blocks spend their time in L2 barriers there, or leave the
+// finest level to one block. us per solve (rtol 1e-3), teams / one cluster each: a 400-cell film
+// 313 / 290, 1000 cells 683 / 574, 4000 cells 1854 / 1276; a 64 x 64 square 400 / 265, 120 x 120 569 /
+// 474; a 16^3 box 316 / 212, 26^3 497 / 462. Outside it: 120 cells (one block) 188 / 191, 160 x 160 at
+// rtol 1e-8 1150 / 1199, 32^3 485 / 523.
+constexpr long long MG_CLUSTER_FROM = 256, MG_CLUSTER_CELLS = 18000;
 
 // out[i] = f(i) for every cell of a level that falls on this block: the finest level by units (its
 // vectors are the CG's), the others in contiguous ranges.
@@ -441,9 +501,9 @@ __device__ void vup(const MGArgs& A, const InstMG& m, int l, const LevelView& v,
 }
 
 // First level of an instance that the first block handles alone (the coarsest at the latest).
-__host__ __device__ __forceinline__ int solo_level(const InstMG& m) {
+__host__ __device__ __forceinline__ int solo_level(const InstMG& m, long long solo_cells) {
   int ls = 0;
-  while (ls < m.levels - 1 && m.nc[ls] > MG_SOLO_CELLS) ++ls;
+  while (ls < m.levels - 1 && m.nc[ls] > solo_cells) ++ls;
   return ls;
 }
 
@@ -451,9 +511,10 @@ __host__ __device__ __forceinline__ int solo_level(const InstMG& m) {
 // next one orders lx. The team shares the levels above solo_level; the first block copies that
 // level's right-hand side into its shared memory, runs the rest of the cycle there, and writes
 // the level's correction back for the team.
-__device__ void vcycle(const MGArgs& A, const InstMG& m, Team& tm, float* smem) {
+template <class TM>
+__device__ void vcycle(const MGArgs& A, const InstMG& m, TM& tm, float* smem) {
   const int L = m.levels;
-  const int ls = solo_level(m);
+  const int ls = solo_level(m, TM::solo_cells);
   SoloTeam solo;
   solo.nt = min((int)blockDim.x, ((int)m.nc[ls] + 31) & ~31);
   for (int l = 0; l < ls; ++l) vdown(A, m, l, global_view(A, m, l), global_view(A, m, l + 1), tm);
@@ -722,6 +783,19 @@ __device__ __forceinline__ Team block_team(const MGArgs& A, TeamDesc& d) {
   return tm;
 }
 
+__device__ __forceinline__ ClusterTeam block_cluster(const MGArgs& A, TeamDesc& d, double* slots) {
+  d = A.teams[A.block_team[blockIdx.x]];
+  ClusterTeam tm;
+  tm.rank = (int)blockIdx.x - d.first_block;
+  tm.size = d.size;
+  tm.slots = slots;
+  tm.buf = 0;
+  return tm;
+}
+
+// No block leaves while another may read its shared memory.
+__device__ __forceinline__ void leave_team(ClusterTeam& tm) { tm.sync(); }
+
 // The last block of a team to leave sets its barrier back for the next launch.
 __device__ __forceinline__ void leave_team(Team& tm) {
   if (tm.size == 1) return;
@@ -753,11 +827,8 @@ __global__ void __launch_bounds__(FD_NT, 1) fd_kernel(MGArgs A) {
 }
 
 // FP64 iterates, for tolerances near FP32's rounding.
-__global__ void __launch_bounds__(MG_NT, 1) mgpcg_kernel(MGArgs A) {
-  __shared__ double sh[66];
-  extern __shared__ float mg_smem[];  // the first block: the levels it handles alone
-  TeamDesc d;
-  Team tm = block_team(A, d);
+template <class TM>
+__device__ __forceinline__ void mgpcg(const MGArgs& A, TM& tm, const TeamDesc& d, double* sh, float* mg_smem) {
   for (int iq = d.inst_beg; iq < d.inst_end; ++iq) {
     const int k = A.order[iq];
     const InstMG& m = A.mg[k];
@@ -849,14 +920,11 @@ __global__ void __launch_bounds__(MG_NT, 1) mgpcg_kernel(MGArgs A) {
 // iterate are the CG's residual and preconditioned residual themselves.
 constexpr int MG32_PASSES = 4;
 
-__global__ void __launch_bounds__(MG_NT, 1) mgpcg32_kernel(MGArgs A, float* V32) {
-  __shared__ double sh[66];
-  extern __shared__ float mg_smem[];  // staged products, or the levels the first block handles alone
+template <class TM>
+__device__ __forceinline__ void mgpcg32(const MGArgs& A, float* V32, TM& tm, const TeamDesc& d, double* sh, float* mg_smem) {
   auto* st1 = reinterpret_cast<float(*)[32]>(mg_smem);
   auto* st2 = reinterpret_cast<float(*)[64]>(mg_smem);
   auto* st3 = reinterpret_cast<float(*)[96]>(mg_smem);
-  TeamDesc d;
-  Team tm = block_team(A, d);
   for (int iq = d.inst_beg; iq < d.inst_end; ++iq) {
     const int k = A.order[iq];
     const InstMG& m = A.mg[k];
@@ -968,6 +1036,36 @@ __global__ void __launch_bounds__(MG_NT, 1) mgpcg32_kernel(MGArgs A, float* V32)
   leave_team(tm);
 }
 
+// Shared memory: the levels the first block handles alone, or staged products.
+__global__ void __launch_bounds__(MG_NT, 1) mgpcg_kernel(MGArgs A) {
+  __shared__ double sh[66];
+  extern __shared__ float mg_smem[];
+  TeamDesc d;
+  Team tm = block_team(A, d);
+  mgpcg(A, tm, d, sh, mg_smem);
+}
+__global__ void __launch_bounds__(MG_NT, 1) mgpcg32_kernel(MGArgs A, float* V32) {
+  __shared__ double sh[66];
+  extern __shared__ float mg_smem[];
+  TeamDesc d;
+  Team tm = block_team(A, d);
+  mgpcg32(A, V32, tm, d, sh, mg_smem);
+}
+__global__ void __launch_bounds__(MG_SMALL_NT, 1) mgpcg_cluster_kernel(MGArgs A) {
+  __shared__ double sh[66], slots[4];
+  extern __shared__ float mg_smem[];
+  TeamDesc d;
+  ClusterTeam tm = block_cluster(A, d, slots);
+  mgpcg(A, tm, d, sh, mg_smem);
+}
+__global__ void __launch_bounds__(MG_SMALL_NT, 1) mgpcg32_cluster_kernel(MGArgs A, float* V32) {
+  __shared__ double sh[66], slots[4];
+  extern __shared__ float mg_smem[];
+  TeamDesc d;
+  ClusterTeam tm = block_cluster(A, d, slots);
+  mgpcg32(A, V32, tm, d, sh, mg_smem);
+}
+
 // Tolerances from here up run the FP32 iterates.
 constexpr double MG32_MIN_RTOL = 1e-5;
 
@@ -1019,6 +1117,30 @@ static void plan_teams(const std::vector<int>& which, const std::vector<double>&
   }
 }
 
+// Cluster teams that run at once on an otherwise idle device (0 where a cluster does not fit).
+static cudaError_t cluster_teams(const Ctx* c, size_t smem, int* most) {
+  const void* f[2] = {(const void*)mgpcg_cluster_kernel, (const void*)mgpcg32_cluster_kernel};
+  *most = 0;
+  for (int i = 0; i < 2; ++i) {
+    cudaError_t e = allow_shared(f[i], c->smem_optin);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(MG_CLUSTER, 1, 1);
+    cfg.blockDim = dim3(MG_SMALL_NT, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = MG_CLUSTER;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if ((e = cudaOccupancyMaxActiveClusters(&n, f[i], &cfg)) != cudaSuccess) return e;
+    *most = i == 0 ? n : std::min(*most, n);
+  }
+  return cudaSuccess;
+}
+
 // Uploads the team plans of the two kernels (separable operators, the others) and sets the
 // kernels' shared memory.
 cudaError_t configure_mgpcg(Ctx* c, const std::vector<InstMG>& h_mg) {
@@ -1037,7 +1159,7 @@ cudaError_t configure_mgpcg(Ctx* c, const std::vector<InstMG>& h_mg) {
         smem = std::max(smem, fd_smem_floats(std::max(m.fnx, m.fny)) * sizeof(float));
       } else {
         // parts: units, by their steps; no more blocks than give every warp a step, and one for
-        // small instances (a 400-cell film: 697 us on four blocks of 1024 threads, 446 on one of 512)
+        // small instances
         const long long chunk = (m.nc[0] + MG_RANKS - 1) / MG_RANKS, steps = (chunk + 32 * MG_WARPS - 1) / (32 * MG_WARPS);
         const long long units = (long long)MG_RANKS << range_units_log(chunk);
         const int most =
@@ -1045,19 +1167,26 @@ cudaError_t configure_mgpcg(Ctx* c, const std::vector<InstMG>& h_mg) {
         parts.push_back(most);
         cost.push_back((double)steps * units / most);
         size_t cells = 0;
-        for (int l = solo_level(m); l < m.levels; ++l) cells += (size_t)m.nc[l];
+        for (int l = solo_level(m, Team::solo_cells); l < m.levels; ++l) cells += (size_t)m.nc[l];
         smem = std::max(std::max(smem, 3 * cells * sizeof(float)), (size_t)MG_STAGE * 96 * sizeof(float));
       }
     }
     p.blocks = 0;
     p.smem = smem;
     p.threads = kind ? FD_NT : MG_NT;
-    if (kind == 0 && std::all_of(which.begin(), which.end(), [&](int k) { return h_mg[k].nc[0] <= MG_SMALL_CELLS; }))
-      p.threads = MG_SMALL_NT;
+    p.cluster = false;
     if (which.empty()) continue;
+    cudaError_t e;
+    long long largest = 0;
+    for (int k : which) largest = std::max<long long>(largest, h_mg[k].nc[0]);
+    if (kind == 0 && largest > MG_CLUSTER_FROM && largest <= MG_CLUSTER_CELLS) {
+      int most = 0;
+      if ((e = cluster_teams(c, smem, &most)) != cudaSuccess) return e;
+      p.cluster = (int)which.size() <= most;
+    }
+    if (kind == 0 && (p.cluster || largest <= MG_SMALL_CELLS)) p.threads = MG_SMALL_NT;
     const void* f[2] = {kind ? (const void*)fd_kernel : (const void*)mgpcg_kernel,
                         kind ? (const void*)fd_kernel : (const void*)mgpcg32_kernel};
-    cudaError_t e;
     for (const void* q : f) {
       if ((e = allow_shared(q, c->smem_optin)) != cudaSuccess) return e;
       int nb = 0;
@@ -1066,7 +1195,15 @@ cudaError_t configure_mgpcg(Ctx* c, const std::vector<InstMG>& h_mg) {
     }
     std::vector<TeamDesc> teams;
     std::vector<int> order, block_team;
-    plan_teams(which, cost, parts, c->sm_count, teams, order, block_team);
+    if (p.cluster) {
+      order = which;
+      for (int i = 0; i < (int)which.size(); ++i) {
+        teams.push_back({MG_CLUSTER * i, MG_CLUSTER, i, i + 1});
+        block_team.insert(block_team.end(), MG_CLUSTER, i);
+      }
+    } else {
+      plan_teams(which, cost, parts, c->sm_count, teams, order, block_team);
+    }
     p.blocks = (int)block_team.size();
     // one buffer: partial sums and barrier words (zero), then the plan
     const size_t at_bar = 4 * block_team.size() * sizeof(double), at_teams = at_bar + 2 * teams.size() * sizeof(unsigned),
@@ -1133,8 +1270,14 @@ static cudaError_t launch_correction(const Ctx* c, const CorrectionIO& io, cudaS
     cfg.dynamicSmemBytes = p.smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;  // the blocks of a team wait for one another
-    attr[0].val.cooperative = 1;
+    if (p.cluster) {
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = MG_CLUSTER;
+      attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    } else {
+      attr[0].id = cudaLaunchAttributeCooperative;  // the blocks of a team wait for one another
+      attr[0].val.cooperative = 1;
+    }
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     cudaError_t e;
@@ -1144,9 +1287,9 @@ static cudaError_t launch_correction(const Ctx* c, const CorrectionIO& io, cudaS
       // FP32 x, p, q in the space of the FP64 r and p (2 n doubles = 4 n floats >= 3 n floats);
       // the FP64 residual of the refinement in that of z
       float* v32 = reinterpret_cast<float*>(c->d_pcg + c->total_cells);
-      e = cudaLaunchKernelEx(&cfg, mgpcg32_kernel, a, v32);
+      e = cudaLaunchKernelEx(&cfg, p.cluster ? mgpcg32_cluster_kernel : mgpcg32_kernel, a, v32);
     } else {
-      e = cudaLaunchKernelEx(&cfg, mgpcg_kernel, a);
+      e = cudaLaunchKernelEx(&cfg, p.cluster ? mgpcg_cluster_kernel : mgpcg_kernel, a);
     }
     if (e != cudaSuccess) return e;
   }
