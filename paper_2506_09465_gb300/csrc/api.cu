@@ -10,6 +10,7 @@
 #include <string>
 #include <vector>
 
+#include "error_word.h"
 #include "fp32_range.h"
 #include "internal.h"
 
@@ -951,16 +952,12 @@ iugkp_status check_device(Ctx* c, cudaStream_t s) {
   int* h = reinterpret_cast<int*>(c->h_pinned + 15);
   CK(cudaMemcpyAsync(h, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, s), "error readback");
   CK(cudaStreamSynchronize(s), "stream synchronise");
-  int e = *h;
-  if (e) {
-    CK(cudaMemsetAsync(c->d_err, 0, sizeof(int), s), "error reset");
-    if (e & ERR_BUDGET) return fail(c, IUGKP_EBUDGET, "a particle exceeded the step budget and was dropped");
-    if (e & ERR_PCG) return fail(c, IUGKP_ENOCONV, "PCG reached cg_maxit before cg_rtol");
-    if (e & ERR_DEFER)
-      return fail(c, IUGKP_EDEVICE, "more particles than the replay queue holds needed the FP64 walk (queue overflow)");
-    return fail(c, IUGKP_EDEVICE, "device-side check failed (code " + std::to_string(e) + ")");
-  }
-  return IUGKP_OK;
+  const int e = *h;
+  const char* text;
+  const iugkp_status st = error_word_status(e, &text);
+  if (st == IUGKP_OK) return st;
+  CK(cudaMemsetAsync(c->d_err, 0, sizeof(int), s), "error reset");
+  return fail(c, st, text);
 }
 
 bool staged_path(const Ctx* c) {
@@ -1088,8 +1085,19 @@ iugkp_status pcg_status(Ctx* c, cudaStream_t s, int* iters) {
     worst = std::max(worst, h[k] < 0 ? c->opt.cg_maxit : h[k]);
   }
   if (iters) *iters = worst;
-  if (fail_) return fail(c, IUGKP_ENOCONV, "PCG reached cg_maxit before cg_rtol");
-  return IUGKP_OK;
+  if (!fail_) return IUGKP_OK;
+  // the cap, or a barrier that gave up (in the error word, whose bit must not stay for the next call)
+  int* e = reinterpret_cast<int*>(c->h_pinned + 15);
+  CK(cudaMemcpyAsync(e, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, s), "error readback");
+  CK(cudaStreamSynchronize(s), "stream synchronise");
+  const char* text;
+  const iugkp_status st = error_word_status((*e & ERR_WAIT) | ERR_PCG, &text);
+  if (*e & (ERR_WAIT | ERR_PCG)) {
+    *e = error_word_after_correction(*e);
+    CK(cudaMemcpyAsync(c->d_err, e, sizeof(int), cudaMemcpyHostToDevice, s), "error reset");
+    CK(cudaStreamSynchronize(s), "stream synchronise");
+  }
+  return fail(c, st, text);
 }
 
 // New relaxation times: every tau-dependent part of the context (band split of the particles,
