@@ -98,8 +98,8 @@ typedef struct {
   int blocks_per_sm;                  /* persistent blocks per SM (0 = auto) */
   int refill_lanes;                   /* staged sweep: a warp refills its idle lanes once at
                                          least this many (1..32) are idle; 0 = chosen per
-                                         instance from the expected events per particle.
-                                         0 or 32 in 2D when every instance's tallied faces
+                                         instance from the expected events per particle in 1D
+                                         and 2D, 4 in 3D. 0 or 32 in 2D when every instance's tallied faces
                                          fit the shared-memory window: pass-synchronous
                                          schedule (each pass of a warp emits up to 32
                                          particles, follows each to its end, then tallies
@@ -109,8 +109,11 @@ typedef struct {
                                          two iterations); 0: plain launches */
   int warp_grab;                      /* staged sweep: particles a warp claims at a time
                                          (0 = 256) */
-  int walk_k;                         /* staged sweep: crossings a lane walks between bulk
-                                         steps (0 = 16) */
+  int walk_k;                         /* staged sweep in 1D, and in 2D without the
+                                         pass-synchronous schedule: crossings a lane walks
+                                         between bulk steps (0 = 16); the same for the null
+                                         candidates of the steady loop, the averaging and the
+                                         adjoint */
 } iugkp_options;
 
 /* Fills *o with defaults: FP32 tracking, staged tallies, frozen draws, Newton on,
@@ -249,8 +252,8 @@ iugkp_status iugkp_persistent_step(iugkp_ctx *ctx, const double *T_dev, unsigned
  * length change speed, not results; the tally mode changes results by rounding only).
  * iugkp_autotune times full sweeps from T_dev (device FP64 [total_cells]) on the caller's
  * stream with CUDA events, searches refill_lanes in {auto, 4, 8, 16, 24}, warp_grab in
- * {128, 256, 512}, walk_k in {8, 16, 32} and, if allow_k32, tally in {STAGED, STAGED_K32}
- * one at a time, stores the fastest in the context's options and reports them in *out
+ * {128, 256, 512}, walk_k in {8, 16, 32} where the sweep reads it (see walk_k) and, if
+ * allow_k32, tally in {STAGED, STAGED_K32} one at a time, stores the fastest in the context's options and reports them in *out
  * (may be NULL). Synchronises the stream. The context must use FP32 tracking with a staged
  * tally mode (EINVAL otherwise). */
 typedef struct {

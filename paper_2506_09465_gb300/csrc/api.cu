@@ -1267,6 +1267,9 @@ iugkp_status iugkp_autotune(iugkp_ctx* ctx, const double* T_dev, unsigned epoch,
   const int* values[4] = {refills, grabs, walks, tallies};
   const int counts[4] = {5, 3, 3, 2};
   for (int kdx = 0; kdx < (allow_k32 ? 4 : 3); ++kdx) {
+    // walk_k is not read by the 3D sweep nor by the pass-synchronous one: its times would be noise, and
+    // the winner would change the steady loop's chains
+    if (kdx == 2 && (c->dim == 3 || sync_schedule(c))) continue;
     int keep = *knobs[kdx];
     for (int j = 0; j < counts[kdx]; ++j) {
       *knobs[kdx] = values[kdx][j];

@@ -258,6 +258,8 @@ cudaError_t launch_sweep_staged(const Ctx* c, const SweepArgs& a, cudaStream_t s
 // Allows a kernel all the dynamic shared memory a block may have. The limit belongs to the kernel, not
 // to a context: every context sets the same value, so that none lowers it for another that is alive.
 cudaError_t allow_shared(const void* kernel, size_t optin);
+// The pass-synchronous schedule (2D): refill only when all 32 lanes are idle, the default where it applies.
+inline bool sync_schedule(const Ctx* c) { return c->sync_ok && (c->opt.refill_lanes == 0 || c->opt.refill_lanes == 32); }
 cudaError_t configure_staged(Ctx* c);
 cudaError_t configure_chain(const Ctx* c);
 cudaError_t launch_chain(const Ctx* c, const SweepArgs& a, const StagedArgs& S, bool k32, cudaStream_t s);

@@ -962,9 +962,7 @@ cudaError_t launch_sweep_staged(const Ctx* c, const SweepArgs& a_in, cudaStream_
   S.R32 = k32 ? c->d_R32 : nullptr;
   S.W32 = k32 && a.W ? c->d_W32 : nullptr;
   S.F32 = k32 && a.F ? c->d_F32 : nullptr;
-  // pass-synchronous schedule: refill only when all 32 lanes are idle (the default where it
-  // applies)
-  const bool sync = c->sync_ok && a.F && (c->opt.refill_lanes == 0 || c->opt.refill_lanes == 32);
+  const bool sync = sync_schedule(c) && a.F;
   PrologueArgs P = {};
   auto clear = [&](void* p, size_t n) {
     if (!p || !n) return;
