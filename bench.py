@@ -30,6 +30,9 @@ SWEEP_DRAM_BYTES = 2.81e6  # dram__bytes_read.sum + dram__bytes_write.sum per la
 SWEEP_ISSUE_UTIL = 0.831   # smsp__issue_active of the same launch
 NGRID = 128
 NPART = 1024
+# The plain FP64 kernels (one thread per particle, cell by cell, global FP64 atomics): step budgets
+# below 2^24, the default, select them; from there up FP64 tracking filters its decisions in FP32.
+PLAIN_FP64 = {"precision": 0, "tally": 0, "schedule": 0, "step_budget": (1 << 24) - 1}
 
 
 def parse():
@@ -85,7 +88,7 @@ def run_profile(args):
     if args.workload == "box32":  # one box of the 3D two-material batch (32^3, 256 particles per cell)
         wl = WL.box_batch(16)
         wl.instances = [WL.two_material_box(32)]
-    opt = {"fast": {"refill_lanes": args.refill}, "plain64": {"precision": 0, "tally": 0, "schedule": 0},
+    opt = {"fast": {"refill_lanes": args.refill}, "plain64": PLAIN_FP64,
            "plain32": {"precision": 1, "tally": 0, "schedule": 0}}[args.mode]
     s = make_solver(wl, seed=0, **opt)
     T = torch.full((s.total_cells,), 0.3, dtype=torch.float64, device="cuda")
@@ -333,7 +336,7 @@ def adjoint_gradient_time(WL, make_solver, tuned, with_plain):
         co = 0
         for k, inst in enumerate(wl.instances):
             w1 = WL.Workload("one", wl.C, wl.v, [inst], wl.particles_per_cell, wl.particles_per_wall_face)
-            sp = make_solver(w1, seed=0, instance_base=k, precision=0, tally=0, schedule=0, use_graphs=0)
+            sp = make_solver(w1, seed=0, instance_base=k, use_graphs=0, **PLAIN_FP64)
             gk = g[co:co + inst.ncells].contiguous()
             torch.cuda.synchronize()
             t0 = time.perf_counter()
@@ -467,9 +470,8 @@ def newton_step_time(lib, L, solver, T, T_half, R, stream, sp, flush, reps):
 
 def slab_config(WL, make_solver):
     """Workload of the 1D gray slab: 50 cells on [0, 1], Kn = 1, black walls at +1 / -1, 1000
-    particles per cell and per wall face, FP64 walk (the plain one-thread-per-particle path),
-    plain iteration (no correction) to residual 1e-6, seed 0, frozen draws. GPU time and
-    iterations, the oracle's (one host core) on the same problem, and the largest difference
+    particles per cell and per wall face, FP64 tracking, plain iteration (no correction) to
+    residual 1e-6, seed 0, frozen draws. GPU time and iterations, the oracle's (one host core) on the same problem, and the largest difference
     of the two steady states (same draws, both FP64)."""
     import numpy as np
     import torch
@@ -709,7 +711,7 @@ def run_ours(args):
             nf1 = solver.total_faces // len(KNS)
             for j, kn in enumerate(KNS):
                 w1 = WL.cavity(NGRID, kn, NPART)
-                sp1 = make_solver(w1, seed=0, instance_base=j, precision=0, tally=0, schedule=0, use_graphs=0)
+                sp1 = make_solver(w1, seed=0, instance_base=j, use_graphs=0, **PLAIN_FP64)
                 T1 = torch.full((sp1.total_cells,), 0.3, dtype=torch.float64, device=dev)
                 R1 = torch.empty(sp1.total_cells, dtype=torch.float64, device=dev)
                 F1 = torch.empty(sp1.total_faces, dtype=torch.float64, device=dev)
@@ -768,7 +770,7 @@ def run_ours(args):
             if not args.no_steady:
                 configs["nongray_256x256_80bands_steady"] = steady_pair(
                     make_solver, WL.nongray_square(256, 40, 1024), dict(tuned),
-                    dict(precision=0, tally=0, schedule=0, use_graphs=0), max_iter=200)
+                    dict(use_graphs=0, **PLAIN_FP64), max_iter=200)
                 configs["nongray_256x256_80bands_steady"]["ref"] = "plain FP64 path"
                 configs["box_batch_16_steady"] = steady_pair(make_solver, WL.box_batch(16), dict(tally=1),
                                                              dict(tally=2), max_iter=200)
