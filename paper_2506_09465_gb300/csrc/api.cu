@@ -130,7 +130,7 @@ void free_all(Ctx* c) {
   void* ptrs[] = {c->d_vtm32, c->d_perm, c->d_wmax_bpre, c->d_inst, c->d_groups_all, c->d_groups_fwd, c->d_coef, c->d_ratio64, c->d_ratio32, c->d_ratio_nb32, c->d_taumaj,
                   c->d_v, c->d_wcoef, c->d_wallT, c->d_srcshift, c->d_source, c->d_m, c->d_Vm, c->d_invVm, c->d_VC,
                   c->d_theta, c->d_theta_m, c->d_diag, c->d_cx, c->d_cy, c->d_cz, c->d_pcg, c->d_work, c->d_T2,
-                  c->d_R, c->d_W, c->d_F, c->d_wall, c->d_red, c->d_counters, c->d_work_counter, c->d_err,
+                  c->d_R, c->d_W, c->d_F, c->d_wall, c->d_red, c->d_counters, c->d_err,
                   c->d_pcg_iters, c->d_scalar, c->d_adj, c->d_mg, c->d_mg_diag, c->d_mg_dinv, c->d_mg_cx,
                   c->d_mg_cy, c->d_mg_cz, c->d_mg_cinv, c->d_mg_b, c->d_mg_x, c->d_mg_t, c->d_fd_q, c->d_fd_lam,
                   c->d_inst_beg, c->d_inst_end, c->d_inst_next, c->d_cost_prefix, c->d_window, c->d_wmax,
@@ -138,7 +138,7 @@ void free_all(Ctx* c) {
                   c->d_all_group_mag, c->d_R32, c->d_W32, c->d_F32, c->d_m2, c->d_wallTf,
                   c->d_pslot_off, c->d_phome_off, c->d_pnband, c->d_pnwall, c->d_px, c->d_pband, c->d_phome,
                   c->d_pcount, c->d_pfcount, c->d_phome_w, c->d_wemit, c->d_DY, c->d_EY, c->d_GX, c->d_Fx, c->d_Fi, c->d_ticket, c->d_wpart,
-                  c->d_all_real, c->d_defer, c->d_defer_n, c->d_over, c->d_land_fwd, c->d_land_all, c->d_items, c->d_nodes, c->d_sync_groups, c->d_sync_beg,
+                  c->d_all_real, c->d_defer, c->d_defer_n, c->d_land_fwd, c->d_land_all, c->d_items, c->d_nodes, c->d_sync_groups, c->d_sync_beg,
                   c->d_sync_end, c->team_plan[0].d_buf, c->team_plan[1].d_buf};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -323,8 +323,8 @@ iugkp_status rebuild_forward_groups(Ctx* c) {
   iugkp_status s = upload(c, &c->d_groups_fwd, c->h_groups_fwd);
   if (s != IUGKP_OK) return s;
   {
-    // w_max pre-pass: each group's blocks in proportion to its emitters, about eight blocks per
-    // SM in all, at least WMAX_MIN_CHUNK emitters per block
+    // weights in the pass before the trace: each group's blocks in proportion to its emitters, about
+    // eight blocks per SM in all, at least WMAX_MIN_CHUNK emitters per block
     long long total = 0;
     for (const Group& g : c->h_groups_fwd) total += g.n_emitters;
     const long long nblk = 8 * (long long)std::max(1, c->sm_count);
@@ -352,7 +352,6 @@ iugkp_status rebuild_forward_groups(Ctx* c) {
   // them (the rest take global atomics).
   std::vector<int2> window(c->n_inst);
   c->any_two_group = false;
-  c->all_two_group = c->dim == 2;
   c->sync_ok = c->dim == 2;
   c->sync_partial = false;
   for (int k = 0; k < c->n_inst; ++k) {
@@ -363,7 +362,6 @@ iugkp_status rebuild_forward_groups(Ctx* c) {
       c->any_two_group = true;
       continue;
     }
-    c->all_two_group = false;
     // 3D: no face window (sweep_chain.cu tallies its faces in global memory)
     const long long len = c->dim == 3 ? 0 : std::min<long long>(X, c->staged_cap);
     window[k] = make_int2((int)((X - len) / 2), (int)len);
@@ -824,12 +822,12 @@ iugkp_status iugkp_create_batch(int n, const iugkp_grid* g, const double* const*
     const long long cap = std::min<long long>(c->total_particles / 32 + 65536, 1ll << 31);
     c->defer_cap = (unsigned)cap;
     if ((s = dalloc(c, &c->d_defer, (size_t)cap)) != IUGKP_OK) return bail(s);
-    if ((s = dalloc(c, &c->d_defer_n, 4)) != IUGKP_OK) return bail(s);
-    // landing sweeps (particle numbers are 32-bit there): a bit per particle for those beyond it
-    const size_t words = (size_t)(std::min<long long>(c->total_particles, 1ll << 31) + 31) / 32;
-    if ((s = dalloc(c, &c->d_over, words)) != IUGKP_OK) return bail(s);
-    if (cudaMemset(c->d_defer_n, 0, 4 * sizeof(unsigned)) != cudaSuccess ||
-        cudaMemset(c->d_over, 0, words * sizeof(unsigned)) != cudaSuccess) {
+    // after its counters, for landing sweeps (particle numbers are 32-bit there), a bit per particle
+    // for those beyond it
+    const size_t words = 4 + (size_t)(std::min<long long>(c->total_particles, 1ll << 31) + 31) / 32;
+    if ((s = dalloc(c, &c->d_defer_n, words)) != IUGKP_OK) return bail(s);
+    c->d_over = c->d_defer_n + 4;
+    if (cudaMemset(c->d_defer_n, 0, words * sizeof(unsigned)) != cudaSuccess) {
       cudaGetLastError();
       fail(c, IUGKP_ECUDA, "clear of the replay queue");
       return bail(IUGKP_ECUDA);
@@ -863,7 +861,6 @@ iugkp_status iugkp_create_batch(int n, const iugkp_grid* g, const double* const*
   if ((s = dalloc(c, &c->d_wall, c->total_walls)) != IUGKP_OK) return bail(s);
   if ((s = dalloc(c, &c->d_red, 1024)) != IUGKP_OK) return bail(s);
   if ((s = dalloc(c, &c->d_counters, CNT_N)) != IUGKP_OK) return bail(s);
-  if ((s = dalloc(c, &c->d_work_counter, 4)) != IUGKP_OK) return bail(s);
   if ((s = dalloc(c, &c->d_err, 1)) != IUGKP_OK) return bail(s);
   if ((s = dalloc(c, &c->d_pcg_iters, n)) != IUGKP_OK) return bail(s);
   if ((s = dalloc(c, &c->d_scalar, 16)) != IUGKP_OK) return bail(s);
@@ -941,7 +938,6 @@ SweepArgs base_args(Ctx* c) {
   a.seed = c->opt.seed;
   a.budget = c->opt.step_budget;
   a.err = c->d_err;
-  a.work_counter = c->d_work_counter;
   a.dim = c->dim;
   a.invVm = c->d_invVm;
   return a;

@@ -13,14 +13,14 @@
 
 namespace iugkp {
 
+// Fewest emitters per block of the weights in the pass before a trace (4 per thread); above that the
+// pass takes about eight blocks per SM.
+constexpr int WMAX_MIN_CHUNK = 1024;
+
 // Counts of particles absorbed through one boundary face are spread over this many copies
 // (by lane), summed when the face's power is shared out: a wall face receives far more
 // absorptions per iteration than a cell receives real collisions, and same-address atomics
 // serialise at the L2.
-// Fewest emitters per block of the w_max pre-pass of the staged sweep (4 per thread); above
-// that the pass takes about two blocks per SM.
-constexpr int WMAX_MIN_CHUNK = 1024;
-
 constexpr int PERS_FACE_REPLICAS = 32;
 
 struct InstMG;
@@ -59,7 +59,7 @@ struct SweepArgs {
   const float* vtm32;      // [inst * nb] v_b tau_maj in FP32
   const double* wcoef;     // [inst * nb * 6] C_b v_b A / (4 N_w) per wall
   const double* wallT;     // [walls]
-  double* wemit;           // [bc] staged sweep: weight of every thermal emitter (w_max pre-pass)
+  double* wemit;           // [bc] staged sweep: weight of every thermal emitter (pass before the trace)
   const double* wallTf;    // [boundary faces] temperature of every boundary face
   double* R;
   double* W;
@@ -74,7 +74,6 @@ struct SweepArgs {
   unsigned epoch;
   long long budget;
   int* err;
-  unsigned long long* work_counter;  // persistent schedule: next particle index
   int staged_faces;                  // staged schedule: faces held in shared memory (0 = none)
   int dim;
 };
@@ -107,7 +106,7 @@ struct Ctx {
   float* d_ratio32 = nullptr;
   float* d_ratio_nb32 = nullptr; // [nb * cells] largest FP32 ratio over each cell's neighbourhood
   int* d_perm = nullptr;         // emitter visiting orders of the groups (Group::perm_off)
-  int* d_wmax_bpre = nullptr;    // [forward groups + 1] first block of each group in the w_max pre-pass
+  int* d_wmax_bpre = nullptr;    // [forward groups + 1] first block of each group in the pass before the trace
                                  // (in proportion to its emitters)
   int wmax_blocks = 0;           // blocks of that pass
   int* d_all_real = nullptr;     // [inst * nb] tau = tau_maj in every cell of the band
@@ -128,7 +127,6 @@ struct Ctx {
   unsigned long long* d_wpart = nullptr;  // [wmax_blocks] largest weight of each block of the pass before it
   bool fp32_lengths = true;      // every cell size and mean free path well inside FP32 (fp32_range.h)
   bool any_two_group = false;    // some instance of the context uses the two-group tallies
-  bool all_two_group = false;    // ... every instance does (no face follows from a column walk)
   bool sync_ok = false;          // 2D: the pass-synchronous staged kernel applies
   bool sync_partial = false;     // ... and some instance's x-faces exceed the window
   double* d_wallTf = nullptr;    // [total_bfaces]
@@ -156,7 +154,6 @@ struct Ctx {
   float2* d_F32 = nullptr;
   double* d_red = nullptr;       // reduction scratch
   unsigned long long* d_counters = nullptr;
-  unsigned long long* d_work_counter = nullptr;
   int* d_err = nullptr;
   int* d_pcg_iters = nullptr;    // [n_inst]
   double* d_scalar = nullptr;    // [8] small results
@@ -208,7 +205,8 @@ struct Ctx {
   uint2* d_defer = nullptr;
   unsigned* d_defer_n = nullptr;     // [4] queue length, queued faces (exact.cu), 64-bit claim counter (land.cu, exact.cu)
   unsigned defer_cap = 0;
-  unsigned* d_over = nullptr;        // [particles / 32] landing sweeps: particles beyond the queue (0 between launches)
+  unsigned* d_over = nullptr;        // [particles / 32] landing sweeps: particles beyond the queue (0 between
+                                     // launches; in the buffer of d_defer_n)
   // tasks of the pass-synchronous 2D sweep and of the filtered FP64 sweep (as many particles per
   // emitter and task as warp_grab allows): the groups', and each instance's range
   LandGroup* d_sync_groups = nullptr;

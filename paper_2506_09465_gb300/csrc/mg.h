@@ -1,5 +1,5 @@
 // Multigrid hierarchy descriptor of one instance (device-resident), shared by the host
-// set-up (mg_setup.cu) and the cluster PCG kernel (mgpcg.cu).
+// set-up (mg_setup.cu) and the correction kernels (mgpcg.cu).
 #pragma once
 
 namespace iugkp {

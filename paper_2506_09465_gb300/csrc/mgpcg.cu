@@ -5,9 +5,9 @@
 // One team of thread blocks per instance, one block per SM. Small instances: a team is one thread-block
 // cluster (ClusterTeam). Larger or many ones: all blocks resident together (a cooperative launch: it
 // starts once a block fits on each SM it needs), the SMs dealt to the instances by their cost
-// (plan_teams). A team's blocks split each level's cells in contiguous ranges, exchange neighbour values through global
-// memory (L2) between team barriers, and reduce dot products in a fixed rank order (every block
-// gets the same value, so all take the same branch). With one 8-block cluster per instance
+// (plan_teams). A team's blocks split each level's cells in contiguous ranges, exchange neighbour
+// values through global memory (L2) between team barriers, and reduce dot products in a fixed rank
+// order (every block gets the same value, so all take the same branch). With one 8-block cluster per instance
 // the largest of four boxes (64^3, 64 cells per thread and phase) set the time on 8 of 152 SMs:
 // 5.5 ms per solve of 11 CG steps, now 1.4 ms (latency of L2 round trips and of the barriers, one
 // instruction in six cycles issued; the loads of two cells in flight at once cost 8 % in index
@@ -224,8 +224,9 @@ struct ClusterTeam {
 // The finest level's cells and the order of its FP32 sums. The cells are cut into MG_RANKS equal
 // ranges; unit (r, w) has the cells of range r whose offset modulo 32 MG_WARPS falls on 32 w .. 32 w
 // + 31, one per lane, in steps: a lane's products are added in FP32 over the steps, the lanes' sums
-// in FP64. A team's blocks take whole units, so that a sum does not depend on how many blocks share
-// the instance. The products are formed in parallel over units and steps and pass through shared
+// in FP64. A team's blocks take whole units, so that the FP32 part of a sum does not depend on how
+// many blocks share the instance (the order of the FP64 part does: last bits of the dot products).
+// The products are formed in parallel over units and steps and pass through shared
 // memory to the warp that adds a unit's.
 constexpr int MG_RANKS = 8, MG_WARPS = 16;
 constexpr int MG_STAGE = 128;  // unit steps staged at a time
@@ -590,8 +591,8 @@ __device__ __forceinline__ double fine_apply(const MGArgs& A, const InstMG& m, c
 // chunks of its rows (asynchronous copies, two chunks ahead), and each warp multiplies units of
 // 32 columns x 4 rows. The terms of an output are added one after the other, in ascending order,
 // or, where both axes have at most FD_QUAD_N cells, in ascending groups of four with the last of a
-// group first: sums as they have always been taken, so that a result does not depend on how many
-// blocks share the instance.
+// group first: a product does not depend on how many blocks share the instance (the order of the
+// residual norm's FP64 sum does).
 constexpr int FD_RB = 8;         // rows of a strip at most
 constexpr int FD_QUAD_N = 128;
 constexpr int FD_CHUNK = 8192;   // floats of a chunk (a multiple of 4 rows, 4 at least: FD_MAX_N <= 2048)

@@ -14,19 +14,17 @@
 //  * faces normal to y in 2D are not tallied, except on the low
 //    boundary: every particle conserves power, so in every cell the net inflow equals the
 //    absorbed minus emitted power, and the last-axis faces follow exactly by a prefix sum
-//    along each column (derive_last_axis_kernel);
+//    along each column (close_2d_kernel);
 //  * 2D instances whose faces all fit the window use two-group tallies instead: a particle
 //    tallies only the faces normal to the axis it crosses less often, and each group's
-//    other faces follow from that group's own per-cell balance (derive_two_group_kernel,
-//    assemble_two_group_kernel);
+//    other faces follow from that group's own per-cell balance (close_2d_kernel);
 //  * a warp tallies the face items of the particles that ended together: in the
 //    pass-synchronous kernel each lane takes segments of 8 items of one list, dealt
 //    round-robin; in the 2D per-lane-refill kernel each lane takes one contiguous chunk of the
 //    concatenated item lists;
 //  * nothing is tallied per particle for the walls: the power a wall emits enters through
 //    its faces deterministically (N particles of known weight per face), and the power it
-//    absorbs is its emission plus the outward net flux through its faces
-//    (boundary_emission_kernel, wall_absorbed_kernel).
+//    absorbs follows from its faces (closing.cu).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -40,13 +38,11 @@
 
 namespace iugkp {
 
-// Emits particle pid (global forward index) into lane state. Returns false for a
-// zero-weight particle (nothing to trace).
 // Per-lane cache of the group of the lane's previous particle (and of the weight of a
 // wall group, which is the same for all its particles).
 struct EmitCache {
   unsigned g_first, g_end;  // forward particle range of the cached group
-  int g_idx, g_ne, g_kind, g_band;
+  int g_ne, g_kind, g_band;
   int g_perm;               // perm_off of the group
   unsigned g_mag;           // division magic of n_emitters
   int e;
@@ -62,7 +58,6 @@ __device__ __forceinline__ bool staged_emit(const SweepArgs& A, const StagedArgs
   if (pid < ec.g_first || pid >= ec.g_end) {
     const int gi = find_group(A.groups, A.n_groups, (long long)pid);
     const Group G = A.groups[gi];
-    ec.g_idx = gi;
     ec.g_first = (unsigned)G.first_particle;
     ec.g_end = (unsigned)(G.first_particle + (long long)G.n_emitters * G.per_emitter);
     ec.g_ne = G.n_emitters;
@@ -83,22 +78,20 @@ __device__ __forceinline__ bool staged_emit(const SweepArgs& A, const StagedArgs
   const int q = (int)udiv(local, (unsigned)ec.g_ne, ec.g_mag);
   int e = (int)(local - (unsigned)q * (unsigned)ec.g_ne);
   if (ec.g_perm >= 0) e = A.perm[ec.g_perm + e];
-  const int n0 = in.n[0], n1 = in.n[1], n2 = in.n[2];
+  const int n0 = in.n[0], n1 = in.n[1];
   const int kind = ec.g_kind;
-  float xi0 = 0.5f, xi1 = 0.5f, xi2 = 0.5f, sx = 0.f, sy = 0.f, sz = 0.f;
+  float xi0 = 0.5f, xi1 = 0.5f, sx = 0.f, sy = 0.f;
   if (kind == 0) {
-    w = A.wemit[in.bc_off + (long long)b * in.ncells + e];  // from the w_max pre-pass
+    w = A.wemit[in.bc_off + (long long)b * in.ncells + e];  // from the pass before the trace
     if ((__double_as_longlong(w) << 1) == 0) return false;   // +-0: nothing to trace
     st.init(A.seed, in.inst_id, (uint32_t)b, A.epoch, (uint32_t)e, (uint32_t)q);
     if (DIM == 1) {
       f.i0 = e;
       f.i1 = 0;
-      f.i2 = 0;
     } else {
       const int r = (int)udiv((unsigned)e, (unsigned)n0, S.mag_n0[k]);
       f.i0 = e - r * n0;
       f.i1 = r;
-      f.i2 = 0;
     }
     float u_mu, u_phi = 0.5f;
     if (DIM == 1) {
@@ -117,7 +110,6 @@ __device__ __forceinline__ bool staged_emit(const SweepArgs& A, const StagedArgs
       float sp, cp;
       sincospif(2.f * u_phi, &sp, &cp);
       sy = sn * cp;
-      sz = sn * sp;
     }
     st.j = thermal_uniforms(DIM);
   } else {
@@ -129,30 +121,19 @@ __device__ __forceinline__ bool staged_emit(const SweepArgs& A, const StagedArgs
     w = ec.w * A.wallTf[in.bface_off + in.wface_off[wl] + e];
     if (w == 0.0) return false;
     const int a = wl >> 1, side = wl & 1;
-    // faces of wall a are enumerated over (o1, o2) = ((a+1)%3, (a+2)%3), o1 fastest
-    const int no1 = a == 0 ? n1 : (a == 1 ? n2 : n0);
-    const int j2 = (int)udiv((unsigned)e, (unsigned)no1, S.mag_wall[k * 3 + a]);
-    const int j1 = e - j2 * no1;
-    long long face;
+    long long face;  // a wall's faces run along the other axis (1D: one face)
     if (a == 0) {
       f.i0 = side ? n0 - 1 : 0;
-      f.i1 = j1;
-      f.i2 = j2;
-      face = in.fax_off[0] + (side ? n0 : 0) + (long long)(n0 + 1) * (j1 + (long long)n1 * j2);
-    } else if (a == 1) {
-      f.i0 = j2;
-      f.i1 = side ? n1 - 1 : 0;
-      f.i2 = j1;
-      face = in.fax_off[1] + j2 + (long long)n0 * ((side ? n1 : 0) + (long long)(n1 + 1) * j1);
+      f.i1 = e;
+      face = in.fax_off[0] + (side ? n0 : 0) + (long long)(n0 + 1) * e;
     } else {
-      f.i0 = j1;
-      f.i1 = j2;
-      f.i2 = side ? n2 - 1 : 0;
-      face = in.fax_off[2] + j1 + (long long)n0 * (j2 + (long long)n1 * (side ? n2 : 0));
+      f.i0 = e;
+      f.i1 = side ? n1 - 1 : 0;
+      face = in.fax_off[1] + e + (long long)n0 * (side ? n1 : 0);
     }
     st.init(A.seed, in.inst_id, (uint32_t)b, A.epoch, (uint32_t)(in.ncells + face), (uint32_t)q);
     float u_n, u_phi = 0.5f;
-    float t0 = 0.5f, t1 = 0.5f;  // tangential fractions, in axis order
+    float t0 = 0.5f;  // tangential fraction
     if (DIM == 1) {
       u_n = word_uniform<float>(st.buf.x);
     } else {
@@ -164,19 +145,19 @@ __device__ __forceinline__ bool staged_emit(const SweepArgs& A, const StagedArgs
     const float sn = DIM >= 2 ? sqrtf(1.f - u_n) : 0.f;
     float sp = 0.f, cp = 0.f;
     if (DIM >= 2) sincospif(2.f * u_phi, &sp, &cp);
-    const float nrm = side ? -mn : mn, ta = sn * cp, tb = sn * sp;  // tangential (o1, o2)
+    // the wall's tangential axes are (a+1)%3 (cosine) and (a+2)%3 (sine)
     if (a == 0) {
-      sx = nrm; sy = ta; sz = tb;
-      xi0 = side ? 1.f : 0.f; xi1 = t0; xi2 = t1;
-    } else if (a == 1) {
-      sy = nrm; sz = ta; sx = tb;
-      xi1 = side ? 1.f : 0.f; xi0 = t0; xi2 = t1;
+      sx = side ? -mn : mn;
+      sy = sn * cp;
+      xi0 = side ? 1.f : 0.f;
+      xi1 = t0;
     } else {
-      sz = nrm; sx = ta; sy = tb;
-      xi2 = side ? 1.f : 0.f; xi0 = t0; xi1 = t1;
+      sy = side ? -mn : mn;
+      sx = sn * sp;
+      xi1 = side ? 1.f : 0.f;
+      xi0 = t0;
     }
-    st.j = wall_uniforms(DIM);
-    (void)face;  // the power entering through wall faces is added by boundary_kernel
+    st.j = wall_uniforms(DIM);  // (the power entering through wall faces is added after the trace)
   }
   axis_init(sx, xi0, in.hf[0], f.t0, f.d0, f.s0);
   f.tex = axis_exit(f.i0, f.s0, n0, f.t0, f.d0);
@@ -249,17 +230,16 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
     const InstDesc& in = A.inst[k];
     // descriptor fields used inside the walk, held in registers (the atomics below would
     // otherwise force reloads)
-    const int n0 = in.n[0], n1 = in.n[1], n2 = in.n[2];
-    const long long face_off = in.face_off, fax1 = in.fax_off[1], fax2 = in.fax_off[2];
+    const int n0 = in.n[0], n1 = in.n[1];
+    const long long face_off = in.face_off, fax1 = in.fax_off[1];
     const long long bc_off = in.bc_off;
     const int ncells = in.ncells, refill = S.refill > 0 ? S.refill : in.refill;
-    const int sy_cell = n0, sz_cell = n0 * n1;           // cell index steps along y, z
-    const int sy_xf = n0 + 1, sz_xf = (n0 + 1) * n1;     // x-face index steps along y, z
+    const int sy_cell = n0, sy_xf = n0 + 1;  // cell and x-face index steps along y
     // x-faces [wbase, wbase + wlen) of this instance are tallied in the shared window
     const int2 wd = useF ? S.window[k] : make_int2(0, 0);
     const int wbase = wd.x;
     const unsigned wlen = (unsigned)wd.y;
-    const bool wfull = wbase == 0 && (long long)wlen == (long long)(n0 + 1) * n1 * n2;
+    const bool wfull = wbase == 0 && (long long)wlen == (long long)(n0 + 1) * n1;
     // 2D instance whose faces all fit the window: two-group tallies (see StagedArgs)
     const bool two = DIM == 2 && useF && wbase == 0 && (long long)wlen == in.nfaces;
     for (unsigned i = threadIdx.x; i < wlen; i += STAGED_NT) win[i] = WIN_BIAS;
@@ -277,7 +257,7 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
     uint32_t ub = 0;
     bool alive = false, exhausted = false;
     bool tally = false;     // the lane's particle has ended and tallies its faces
-    int kcur = 0, kend = 0; // face items of the tally phase (x-faces, then y-faces in 3D)
+    int kcur = 0, kend = 0; // face items of the tally phase
     EmitCache ec;
     ec.g_first = 1;
     ec.g_end = 0;  // empty: forces a lookup on the first emission
@@ -357,14 +337,14 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
           if (DIM >= 2) cell += sy_cell * clampi(f.i1 + f.s1 * fb1, n1);
           const long long ci = bcbase + cell;
           const int oc = candidate_outcome<DIM>(A, bcbase, ncells, f, base, fb0, fb1, 0, cell, all_real, near, ub,
-                                                n0, n1, n2, sy_cell, sz_cell);
+                                                n0, n1, 1, sy_cell, 0);
           if (oc == CAND_DEFER) {
             ended = deferred = true;
             break;
           }
           cnt.v[CNT_CANDIDATES] += 1;
           ++kc;
-          // W collects w here; the sweep scales it by tau_maj afterwards (scale_by_taumaj), and
+          // W collects w here; the sweep scales it by tau_maj afterwards, and
           // a band whose every candidate is real takes W = tau_maj R there instead
           if (K32 && S.W32 && !all_real) tally_k32(&S.W32[ci], w);
           else if (!K32 && A.W && !all_real) atomicAdd(&A.W[ci], w);
@@ -567,27 +547,17 @@ __global__ void __launch_bounds__(STAGED_NT, 1) sweep_staged_kernel(SweepArgs A,
             if (carry) add_units(S.Fi, face_off + xface, (long long)carry << 32);
           }
         };
-        if (DIM == 2 && (two || wfull)) {
-          // every face of the tallied axis is in the window at its instance index; the count
-          // along the other axis needs only the upper bound (the lower one holds by
-          // construction)
+        // (2D instances whose tallied faces are all in the window have tallied them above)
 #pragma unroll 1
-          for (; kcur < kstop; ++kcur, fk += 1.f) {
-            const int face = f.i0 + kcur * f.s0 + f.s1 * min(ceil_count(fmaf(fk, f.tex, f.D)), f.i2);
-            window_add(face, (unsigned)face);
+        for (; kcur < kstop; ++kcur, fk += 1.f) {
+          int xface = f.s0 > 0 ? f.i0 + 1 + kcur : f.i0 - kcur;
+          if (DIM == 2) {
+            xface += sy_xf * (f.i1 + f.s1 * min(ceil_count(fmaf(fk, f.tex, f.D)), f.i2));
           }
-        } else {
-#pragma unroll 1
-          for (; kcur < kstop; ++kcur, fk += 1.f) {
-            int xface = f.s0 > 0 ? f.i0 + 1 + kcur : f.i0 - kcur;
-            if (DIM == 2) {
-              xface += sy_xf * (f.i1 + f.s1 * min(ceil_count(fmaf(fk, f.tex, f.D)), f.i2));
-            }
-            const unsigned rel = (unsigned)(xface - wbase);
-            if (rel < wlen) window_add(xface, rel);
-            else if (K32) tally_k32(&S.F32[face_off + xface], f.s0 > 0 ? w : -w);
-            else atomicAdd(&A.F[face_off + xface], f.s0 > 0 ? w : -w);
-          }
+          const unsigned rel = (unsigned)(xface - wbase);
+          if (rel < wlen) window_add(xface, rel);
+          else if (K32) tally_k32(&S.F32[face_off + xface], f.s0 > 0 ? w : -w);
+          else atomicAdd(&A.F[face_off + xface], f.s0 > 0 ? w : -w);
         }
         if (kcur >= kend) {
           tally = false;
