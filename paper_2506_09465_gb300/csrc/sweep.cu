@@ -111,7 +111,9 @@ __device__ __noinline__ void replay_real(const SweepArgs& A, const StagedArgs& S
 // an exit through the low wall of an untallied axis goes to that wall's face (one-group
 // instances) or to the group's exit tally GX (two-group). Emission needs nothing: the staged
 // sweep and its post-passes account for it.
-template <int DIM>
+// LAND: after a landing sweep, whose particles beyond the queue follow (the full sweeps keep the kernel
+// without them: its stack is half as deep).
+template <int DIM, bool LAND>
 __global__ void __launch_bounds__(256)
     replay_kernel(const __grid_constant__ SweepArgs A, const __grid_constant__ StagedArgs S) {
   Counts cnt;
@@ -244,17 +246,23 @@ __global__ void __launch_bounds__(256)
     }
     (void)ex;
   }
-  for_overflow(S, [&](unsigned pid) { replay_real<DIM>(A, S, pid); });
+  if (LAND) for_overflow(S, [&](unsigned pid) { replay_real<DIM>(A, S, pid); });
   flush_counts(cnt, A.counters);
 }
 
-cudaError_t launch_replay(const Ctx* c, const SweepArgs& a, const StagedArgs& S, cudaStream_t s) {
+template <bool LAND>
+static void launch_replay_dim(const Ctx* c, const SweepArgs& a, const StagedArgs& S, cudaStream_t s) {
   const int blocks = c->sm_count * 8;
   switch (c->dim) {
-    case 1: replay_kernel<1><<<blocks, 256, 0, s>>>(a, S); break;
-    case 2: replay_kernel<2><<<blocks, 256, 0, s>>>(a, S); break;
-    default: replay_kernel<3><<<blocks, 256, 0, s>>>(a, S); break;
+    case 1: replay_kernel<1, LAND><<<blocks, 256, 0, s>>>(a, S); break;
+    case 2: replay_kernel<2, LAND><<<blocks, 256, 0, s>>>(a, S); break;
+    default: replay_kernel<3, LAND><<<blocks, 256, 0, s>>>(a, S); break;
   }
+}
+
+cudaError_t launch_replay(const Ctx* c, const SweepArgs& a, const StagedArgs& S, cudaStream_t s) {
+  if (S.over) launch_replay_dim<true>(c, a, S, s);
+  else launch_replay_dim<false>(c, a, S, s);
   return cudaGetLastError();
 }
 
