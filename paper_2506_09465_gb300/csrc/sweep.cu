@@ -84,7 +84,7 @@ __device__ __forceinline__ double shfl_d(double x, int src) {
 
 // The real collision of a landing sweep's particle (forward index pid, nothing tallied yet) in FP64.
 template <int DIM>
-__device__ __noinline__ void replay_real(const SweepArgs& A, const StagedArgs& S, unsigned pid) {
+__device__ __forceinline__ void replay_real(const SweepArgs& A, const StagedArgs& S, unsigned pid) {
   Counts cnt;  // a landing sweep's event counts are not read
   const Group G = A.groups[find_group(A.groups, A.n_groups, (long long)pid)];
   const InstDesc& in = A.inst[G.inst];
@@ -114,8 +114,7 @@ __device__ __noinline__ void replay_real(const SweepArgs& A, const StagedArgs& S
 // LAND: after a landing sweep, whose particles beyond the queue follow (the full sweeps keep the kernel
 // without them: its stack is half as deep).
 template <int DIM, bool LAND>
-__global__ void __launch_bounds__(256)
-    replay_kernel(const __grid_constant__ SweepArgs A, const __grid_constant__ StagedArgs S) {
+__global__ void __launch_bounds__(256) replay_kernel(SweepArgs A, StagedArgs S) {
   Counts cnt;
 #pragma unroll
   for (int k = 0; k < CNT_N; ++k) cnt.v[k] = 0;
