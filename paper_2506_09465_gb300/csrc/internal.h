@@ -205,8 +205,7 @@ struct Ctx {
   uint2* d_defer = nullptr;
   unsigned* d_defer_n = nullptr;     // [4] queue length, queued faces (exact.cu), 64-bit claim counter (land.cu, exact.cu)
   unsigned defer_cap = 0;
-  unsigned* d_over = nullptr;        // [particles / 32] landing sweeps: particles beyond the queue (0 between
-                                     // launches; in the buffer of d_defer_n)
+  unsigned* d_over = nullptr;        // [particles / 32] landing sweeps: particles beyond the queue (0 between launches)
   // tasks of the pass-synchronous 2D sweep and of the filtered FP64 sweep (as many particles per
   // emitter and task as warp_grab allows): the groups', and each instance's range
   LandGroup* d_sync_groups = nullptr;
