@@ -44,7 +44,8 @@ typedef enum {
   IUGKP_ECUDA = 3,    /* a CUDA runtime call failed (message has the CUDA error) */
   IUGKP_ENOCONV = 4,  /* an iteration hit its limit before its tolerance */
   IUGKP_EBUDGET = 5,  /* a particle exceeded the per-particle step budget (dropped) */
-  IUGKP_EDEVICE = 6   /* a device-side check failed (index out of range, bad state) */
+  IUGKP_EDEVICE = 6   /* a device-side check failed (replay queue overflow, a block of the
+                         correction solve that waited too long for its team, bad state) */
 } iugkp_status;
 
 typedef struct iugkp_ctx iugkp_ctx; /* opaque; owned by the library */
@@ -84,8 +85,10 @@ typedef struct {
   int draws;          /* IUGKP_DRAWS_FRESH: epoch = epoch0 + iteration;
                          IUGKP_DRAWS_FROZEN: epoch = epoch0 every iteration. */
   int newton;         /* 0: plain iteration; 1: inexact-Newton diffusion correction. */
-  int schedule;       /* IUGKP_SCHED_PLAIN: one thread per particle;
-                         IUGKP_SCHED_PERSISTENT: persistent warps that refill lanes. */
+  int schedule;       /* Read by no kernel any more: the schedule follows from precision, tally
+                         and step_budget. FP32 tracking with staged tallies, and FP64 tracking
+                         with step_budget >= 2^24: persistent warps; the others: one thread per
+                         particle. */
   long long particles_per_cell;       /* N_cell >= nb; split over bands (largest remainder) */
   long long particles_per_wall_face;  /* >= nb; split over bands by C_b v_b */
   unsigned long long seed;            /* Philox key (low, high words) */
@@ -93,7 +96,16 @@ typedef struct {
   unsigned instance_base;             /* instance k of a batch draws with id base + k */
   double cg_rtol;                     /* PCG relative tolerance (Newton step) */
   int cg_maxit;                       /* PCG iteration cap -> IUGKP_ENOCONV */
-  long long step_budget;              /* max crossings + candidates per particle */
+  long long step_budget;              /* max crossings + candidates per particle (EBUDGET). FP64
+                                         tracking: below 2^24 the plain kernels run (one thread
+                                         per particle, cell by cell, every step counted, about
+                                         five times slower); from 2^24 (the default) up decisions
+                                         are filtered in FP32 and a particle of more than 2^20
+                                         candidates is followed again with its steps counted
+                                         (its candidates only in the steady loop, the averaging
+                                         without faces and the adjoint).
+                                         FP32 tracking with staged tallies counts the candidates
+                                         of replayed particles only */
   int block_threads;                  /* threads per block of the trace kernel (0 = auto) */
   int blocks_per_sm;                  /* persistent blocks per SM (0 = auto) */
   int refill_lanes;                   /* staged sweep: a warp refills its idle lanes once at
@@ -198,12 +210,15 @@ iugkp_status iugkp_macro(iugkp_ctx *ctx, const double *R_dev, const double *W_de
 /* Inexact-Newton correction (Sec. 3.3): s = (sum_b R_b - sum_b C_b T_n V / tau_b) / V,
  * solves -div(kappa grad dT) = s to ||s - A dT|| <= cg_rtol ||s|| and sets T_half += theta dT
  * (theta = min(1, 1.5 / cell optical thickness)). Solver: CG preconditioned by one
- * aggregation-multigrid V-cycle in FP32, one thread-block cluster per instance. For
+ * aggregation-multigrid V-cycle in FP32 (fast diagonalization where the operator is separable),
+ * one team of thread blocks, or one cluster, per instance. Team launches are cooperative: they
+ * start when all their blocks fit beside what else runs on the device. For
  * cg_rtol >= 1e-5 (the default 1e-3) the CG iterates are FP32 inside FP64 iterative
  * refinement: the solution is accumulated in FP64 and its residual s - A dT is formed and
  * measured in FP64, which is what cg_rtol bounds; below 1e-5 the CG iterates and residual
  * are FP64. Synchronises the stream to read the CG status; *cg_iters_out (may be NULL) gets
- * the largest iteration count over instances. ENOCONV if cg_maxit is reached. */
+ * the largest iteration count over instances. ENOCONV if cg_maxit is reached; EDEVICE if a block
+ * waited too long for the others of its team. */
 iugkp_status iugkp_newton_step(iugkp_ctx *ctx, const double *T_n_dev, double *T_half_inout_dev,
                                const double *R_dev, void *cuda_stream, int *cg_iters_out);
 
@@ -253,9 +268,9 @@ iugkp_status iugkp_persistent_step(iugkp_ctx *ctx, const double *T_dev, unsigned
  * iugkp_autotune times full sweeps from T_dev (device FP64 [total_cells]) on the caller's
  * stream with CUDA events, searches refill_lanes in {auto, 4, 8, 16, 24}, warp_grab in
  * {128, 256, 512}, walk_k in {8, 16, 32} where the sweep reads it (see walk_k) and, if
- * allow_k32, tally in {STAGED, STAGED_K32} one at a time, stores the fastest in the context's options and reports them in *out
- * (may be NULL). Synchronises the stream. The context must use FP32 tracking with a staged
- * tally mode (EINVAL otherwise). */
+ * allow_k32, tally in {STAGED, STAGED_K32} one at a time, stores the fastest in the context's
+ * options and reports them in *out (may be NULL). Synchronises the stream. The context must
+ * use FP32 tracking with a staged tally mode (EINVAL otherwise). */
 typedef struct {
   int refill_lanes, warp_grab, walk_k, tally;
   double sweep_ms;      /* best sweep time found */
